@@ -268,3 +268,146 @@ def tolerance(case):
     if case["kind"] == "error":
         return {"rel": 1e-5, "max": 1e-4}
     return {"fp32": {"rel": 6e-4, "max": 5e-3}, "fp16": {"rel": 1e-3, "max": 6e-3}, "bf16": {"rel": 3e-3, "max": 2e-2}}[case["out"]]
+
+
+# ---------------------------------------------------------------------------------------------- the same in 64 bits
+def _hadamard(x, signs, inverse=False):
+    """Randomized Hadamard rotation of the last axis, stage by stage, in x's own precision."""
+    D = x.shape[-1]
+    y, h = (x if inverse else x * signs.to(x.dtype)), 1
+    while h < D:
+        p = y.reshape(*y.shape[:-1], D // (2 * h), 2, h)
+        y = torch.stack((p[..., 0, :] + p[..., 1, :], p[..., 0, :] - p[..., 1, :]), dim=-2).reshape(x.shape)
+        h *= 2
+    y = y * torch.tensor(1.0 / math.sqrt(D), dtype=x.dtype, device=x.device)
+    return y * signs.to(x.dtype) if inverse else y
+
+
+def _reconstructed(x, bits, dim):
+    """x (fp32, one group along `dim`) quantized with fp16 scale and minimum, and back in 64 bits."""
+    qmax = torch.tensor(2.0 ** bits - 1.0, device=x.device)
+    lo, hi = x.amin(dim, keepdim=True) + 0.0, x.amax(dim, keepdim=True) + 0.0
+    s = ((hi - lo) / qmax).clamp(-65504.0, 65504.0).half().float()
+    z = lo.clamp(-65504.0, 65504.0).half().float()
+    inv = torch.where(s != 0, torch.ones_like(s) / s, torch.zeros_like(s))
+    code = torch.minimum(torch.round((x - z) * inv).clamp(min=0.0), qmax)
+    return code.double() * s.double() + z.double()
+
+
+class _Sequence:
+    """One sequence of one layer: its tokens as the cache holds them, in 64 bits (keys rotated where the cache rotates)."""
+
+    def __init__(self, c, w, cap, signs, dev):
+        self.c, self.w, self.signs, self.n = c, w, signs, 0
+        shape = (w.n_kv_heads, cap, w.head_dim)
+        self.k, self.v = (torch.zeros(shape, dtype=torch.float64, device=dev) for _ in range(2))
+        self.win = torch.zeros((2, w.n_kv_heads, max(c["window"], 1), w.head_dim), device=dev)
+        self.tail = torch.zeros((w.n_kv_heads, PAGE, w.head_dim), device=dev)
+
+    def _tokenwise(self, x, bits, group):
+        return _reconstructed(x.reshape(*x.shape[:-1], -1, group), bits, -1).reshape(x.shape)
+
+    def append(self, k, v):
+        w, R, t0 = self.w, self.c["window"], self.n
+        end = self.n = t0 + k.shape[1]
+        k, v = k.float(), v.float()
+        qa, qb = (t0 // R * R, end // R * R) if R else (t0, end)
+        if R and qb > qa:
+            slots = torch.arange(qa, t0, device=k.device) % R
+            kq, vq = (torch.cat((self.win[i][:, slots], x), 1)[:, :qb - qa] for i, x in enumerate((k, v)))
+        else:
+            kq, vq = k[:, :qb - qa], v[:, :qb - qa]
+        kr = _hadamard(kq, self.signs) if self.signs is not None else kq
+        if qb > qa:
+            self.v[:, qa:qb] = self._tokenwise(vq, w.vb, w.gv)
+        if w.k_axis == 1:
+            first = t0 // PAGE * PAGE
+            x = torch.cat((self.tail[:, :t0 - first], kr.clamp(-65504.0, 65504.0).half().float()), 1)
+            full = x.shape[1] // PAGE * PAGE
+            blocks = x[:, :full].reshape(x.shape[0], -1, PAGE, x.shape[2])
+            if full:
+                self.k[:, first:first + full] = _reconstructed(blocks, w.kb, 2).flatten(1, 2)
+            self.tail[:, :x.shape[1] - full] = x[:, full:]
+            self.k[:, first + full:end] = x[:, full:].double()
+        elif qb > qa:
+            self.k[:, qa:qb] = self._tokenwise(kr, w.kb, w.gk)
+        if R:
+            keep = torch.arange(max(t0, qb), end, device=k.device)
+            self.win[0][:, keep % R], self.win[1][:, keep % R] = k[:, keep - t0], v[:, keep - t0]
+
+    def attend(self, q):
+        """q [rows, Hq, D]: causal rows over the last positions."""
+        w, R, n = self.w, self.c["window"], self.n
+        rows, H, D = q.shape[0], w.n_kv_heads, w.head_dim
+        q = q.double().reshape(rows, H, -1, D).transpose(0, 1)                       # [H, rows, G, D]
+        qr = _hadamard(q, self.signs) if self.signs is not None else q
+        packed = n // R * R if R else n
+        logits = torch.einsum("hrgd,htd->hrgt", qr, self.k[:, :packed])
+        values = self.v[:, :packed]
+        if R:
+            slots = torch.arange(packed, n, device=q.device) % R
+            logits = torch.cat((logits, torch.einsum("hrgd,htd->hrgt", q, self.win[0][:, slots].double())), -1)
+            values = torch.cat((values, self.win[1][:, slots].double()), 1)
+        seen = torch.arange(n, device=q.device) <= n - rows + torch.arange(rows, device=q.device)[:, None]
+        p = torch.softmax(logits.div(math.sqrt(D)).masked_fill(~seen[None, :, None], -math.inf), -1)
+        return torch.einsum("hrgt,htd->hrgd", p, values).transpose(0, 1).reshape(rows, -1, D)
+
+
+def exact(case, seed):
+    """What `run` returns in 64 bits over the same codes; packed bytes, tails, windows and lengths have no such value."""
+    c, dev = case, "cuda"
+    w = _workload(c, seed)
+    T, B, H, D = c["tokens"], w.batch, w.n_kv_heads, w.head_dim
+    if c["kind"] == "append":
+        return None
+    if c["kind"] == "error":
+        sums = torch.zeros((w.layers, 3, B, H, 4), dtype=torch.float64, device=dev)
+        for i in range(w.layers):
+            for side, x in enumerate(wl.make_kv(w, i, dev, tokens=T)):
+                x = x.float()
+                for j, bits in enumerate((2, 3, 4)):
+                    g = x.reshape(B, H, T, -1, (w.gk, w.gv)[side])
+                    sums[i, j, :, :, 2 * side] = x.double().square().sum((2, 3))
+                    sums[i, j, :, :, 2 * side + 1] = (g.double() - _reconstructed(g, bits, -1)).square().sum((2, 3, 4))
+        return sums
+    cap = _config(c, w).capacity_tokens
+    signs = None
+    if c["rotated"]:
+        g = torch.Generator().manual_seed(abs(int(seed)) + 1)
+        signs = (torch.randint(0, 2, (D,), generator=g, dtype=torch.int8) * 2 - 1).to(dev)
+    base = None if c["kind"] == "restore" else _base_lens(c, w, abs(int(seed)))
+    n, lead = c["append"], 0 if base is None else min(PAGE, int(base.min()))
+    page0 = (T - 1) // PAGE * PAGE
+    outs, written = [], []
+    for i in range(w.layers):
+        k, v = wl.make_kv(w, i, dev, tokens=T)
+        if base is None:
+            back = tuple(torch.zeros((B, H, cap, D), dtype=torch.float64, device=dev) for _ in range(2))
+        else:
+            new = wl.make_kv(w, 100 + i, dev, tokens=n)
+            q = wl.make_q(w, i, dev, batch=B * c["rows"]).view(B, c["rows"], w.n_q_heads, D)
+            out = torch.zeros(q.shape, dtype=torch.float64, device=dev)
+            back = tuple(torch.zeros((B, H, T - page0, D), dtype=torch.float64, device=dev) for _ in range(2))
+        for b in range(B):
+            s = _Sequence(c, w, cap, signs, dev)
+            s.append(k[b], v[b])
+            if base is not None:
+                if lead:
+                    s.n = int(base[b]) - lead
+                    s.append(k[b][:, T - lead:], v[b][:, T - lead:])
+                s.n = int(base[b])
+                s.append(new[0][b], new[1][b])
+                out[b] = s.attend(q[b])
+            if base is None or c["restore"]:
+                at = slice(0, T) if base is None else slice(page0, T)
+                unrotated = s.k[:, at] if signs is None else _hadamard(s.k[:, at], signs, inverse=True)
+                back[0][b, :, :at.stop - at.start], back[1][b, :, :at.stop - at.start] = unrotated, s.v[:, at]
+        if base is None:
+            outs.append(back)
+        else:
+            outs.append(out.view(B, w.n_q_heads, D) if c["rows"] == 1 else out)
+            written = list(back) if c["restore"] else []
+    if base is None:
+        return outs
+    none = [None] * w.layers
+    return [outs, none, none, none, None, written]
