@@ -674,69 +674,183 @@ __device__ __forceinline__ void pack_k_rows(const uint8_t* codes, int code_strid
   }
 }
 
-// Channel-wise quantization of one complete 128-token block held as fp16 in shared memory, head_dim 128, 4- or
-// 8-bit codes.  Thread = (token quarter, slice pair rp, channel pair pi): the four channels 32 rp + 2 pi + {0, 1}
-// and 32 rp + 16 + 2 pi + {0, 1}, whose codes share two adjacent bytes (4 bits) or two adjacent byte pairs
-// (8 bits) of every token row.  Minimum and maximum are taken two channels at a time in fp16 (exact), the
-// parameters once per channel, and the codes are written as whole bytes into a shared image of the page's key
-// region, which leaves with 16-byte stores.
-template <int KB>
-__device__ __forceinline__ void kchan_block_fast(const uint16_t* sX, uint8_t* sImg, uint8_t* pg, const Geom& g, int tid) {
-  constexpr int D = 128, ROW = D * KB / 8;
-  const __half2* sX2 = reinterpret_cast<const __half2*>(sX);            // [128][64]
-  __half2* sRed = reinterpret_cast<__half2*>(sImg);                    // [4 quarters][32][4], dead before the image is written
-  const int q = tid >> 5, l32 = tid & 31, rp = l32 >> 3, pi = l32 & 7;
-  const int w_lo = 16 * rp + pi, w_hi = w_lo + 8;
-  const float qmax = (float)((1 << KB) - 1);
-  __half2 mn_lo = sX2[(32 * q) * 64 + w_lo], mx_lo = mn_lo, mn_hi = sX2[(32 * q) * 64 + w_hi], mx_hi = mn_hi;
-#pragma unroll 8
-  for (int t = 32 * q + 1; t < 32 * q + 32; ++t) {
-    const __half2 a = sX2[t * 64 + w_lo], b = sX2[t * 64 + w_hi];
-    mn_lo = __hmin2(mn_lo, a); mx_lo = __hmax2(mx_lo, a);
-    mn_hi = __hmin2(mn_hi, b); mx_hi = __hmax2(mx_hi, b);
-  }
-  sRed[(q * 32 + l32) * 4 + 0] = mn_lo; sRed[(q * 32 + l32) * 4 + 1] = mx_lo;
-  sRed[(q * 32 + l32) * 4 + 2] = mn_hi; sRed[(q * 32 + l32) * 4 + 3] = mx_hi;
-  __syncthreads();
+// The 16-byte pieces (eight channels 8 v .. 8 v + 7, v = tid % 16) of new key rows as saturated fp16, rotated if asked.
+// The 16 lanes of a row take part together (the rotation shuffles between them).
+template <int DTYPE, bool ROT>
+__device__ __forceinline__ uint4 key_row_fp16(uint4 val, const int8_t* __restrict__ signs, int v) {
+  if constexpr (DTYPE == KVQ_BF16 || ROT) {
+    uint32_t w[4] = {val.x, val.y, val.z, val.w};
+    float x[8];
 #pragma unroll
-  for (int qq = 0; qq < 4; ++qq) {
-    mn_lo = __hmin2(mn_lo, sRed[(qq * 32 + l32) * 4 + 0]); mx_lo = __hmax2(mx_lo, sRed[(qq * 32 + l32) * 4 + 1]);
-    mn_hi = __hmin2(mn_hi, sRed[(qq * 32 + l32) * 4 + 2]); mx_hi = __hmax2(mx_hi, sRed[(qq * 32 + l32) * 4 + 3]);
-  }
-  const GroupParams p0 = group_params(__low2float(mn_lo), __low2float(mx_lo), qmax);     // channel 32 rp + 2 pi
-  const GroupParams p1 = group_params(__high2float(mn_lo), __high2float(mx_lo), qmax);   // ... + 1
-  const GroupParams p2 = group_params(__low2float(mn_hi), __low2float(mx_hi), qmax);     // ... + 16
-  const GroupParams p3 = group_params(__high2float(mn_hi), __high2float(mx_hi), qmax);   // ... + 17
-  if (q == 0) {
-    uint32_t* meta = reinterpret_cast<uint32_t*>(pg + g.k_meta_off);
-    const int d0 = 32 * rp + 2 * pi;
-    meta[d0] = p0.meta; meta[d0 + 1] = p1.meta; meta[d0 + 16] = p2.meta; meta[d0 + 17] = p3.meta;
-  }
-  __syncthreads();                       // every thread has read the reduction scratch: the image may overwrite it
-#pragma unroll 4
-  for (int t = 32 * q; t < 32 * q + 32; ++t) {
-    const float2 a = __half22float2(sX2[t * 64 + w_lo]), b = __half22float2(sX2[t * 64 + w_hi]);
-    const uint32_t c0 = code_of_fast(a.x, p0, qmax), c1 = code_of_fast(a.y, p1, qmax);
-    const uint32_t c2 = code_of_fast(b.x, p2, qmax), c3 = code_of_fast(b.y, p3, qmax);
-    if constexpr (KB == 4) {
-      // bytes 2 (pi % 2) + {0, 1} of word rp in chunk pi / 2: low nibble slice 2 rp, high nibble slice 2 rp + 1
-      *reinterpret_cast<uint16_t*>(sImg + t * ROW + (pi >> 1) * 16 + rp * 4 + 2 * (pi & 1)) =
-          (uint16_t)((c0 | (c2 << 4)) | ((c1 | (c3 << 4)) << 8));
-    } else {
-      const int wa = 2 * rp, wb = 2 * rp + 1;                      // words = slices 2 rp and 2 rp + 1
-      *reinterpret_cast<uint16_t*>(sImg + t * ROW + (wa >> 2) * 64 + (pi >> 1) * 16 + (wa & 3) * 4 + 2 * (pi & 1)) =
-          (uint16_t)(c0 | (c1 << 8));
-      *reinterpret_cast<uint16_t*>(sImg + t * ROW + (wb >> 2) * 64 + (pi >> 1) * 16 + (wb & 3) * 4 + 2 * (pi & 1)) =
-          (uint16_t)(c2 | (c3 << 8));
+    for (int i = 0; i < 4; ++i) {
+      if constexpr (DTYPE == KVQ_BF16) {
+        x[2 * i] = __uint_as_float(w[i] << 16);
+        x[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+      } else {
+        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[i]));
+        x[2 * i] = f.x;
+        x[2 * i + 1] = f.y;
+      }
     }
+    if constexpr (ROT) rotate_row8<128>(x, signs, v);
+    // saturating: the conversion rounds to nearest (infinity from 65520 on), the packed clamp brings infinities to 65504
+    const __half2 top = __half2half2(__ushort_as_half(0x7BFF)), bottom = __half2half2(__ushort_as_half(0xFBFF));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const __half2 h = __hmin2(__hmax2(__floats2half2_rn(x[2 * i], x[2 * i + 1]), bottom), top);
+      w[i] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+  } else {
+    return val;
   }
-  __syncthreads();
-  for (int i = tid; i < kPageTokens * ROW / 16; i += kThreads)
-    reinterpret_cast<uint4*>(pg)[i] = reinterpret_cast<const uint4*>(sImg)[i];
 }
 
-// Channel-wise quantization of K over 128-token blocks with the fp16 tail.
-// CTA j of a stream handles the j-th block touched by this append.  CTA 0 also
+// Codes of four values as the four bytes of a word: rint(clamp((x - z) * inv, 0, qmax)), the fixed formula.  `inv_q` is
+// inv * 2^-BITS (exact), so that the saturation of a multiplication to [0, 1] is the clamp to [0, 2^BITS] (a NaN becomes
+// 0); the fused multiply-add by 2^BITS onto 1.5 * 2^23 rounds to nearest-even, and the upper clamp follows on two codes at a time.
+template <int BITS>
+__device__ __forceinline__ uint32_t code_word4(const float (&x)[4], const float (&z)[4], const float (&inv_q)[4]) {
+  uint32_t n[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    n[j] = __float_as_uint(__fmaf_rn(__saturatef(__fmul_rn(__fsub_rn(x[j], z[j]), inv_q[j])), (float)(1 << BITS), kRoundMagic));
+  constexpr uint32_t TOP = ((1u << BITS) - 1u) * 0x00010001u;
+  const uint32_t even = __vminu2(prmt(n[0], n[2], 0x5410), TOP), odd = __vminu2(prmt(n[1], n[3], 0x5410), TOP);
+  return even + odd * 256u;
+}
+
+// Channel-wise quantization of one complete 128-token block, head_dim 128, 4- or 8-bit codes, held in the registers of
+// 256 threads: thread (tr = tid / 16, v = tid % 16) has channels 8 v .. 8 v + 7 of tokens tr + 16 i as fp16.  Minimum and
+// maximum are taken two channels at a time in fp16 (exact), first in the thread, then over the warps through 4 KB of
+// shared memory; the parameters are made once per channel.  At 4 bits the lanes whose codes share bytes (v and v ^ 2) swap one word
+// per token, and each stores one word of the row: the 16 lanes of a row write its 64 (8 bits: 128) bytes whole.
+struct KchanShared {
+  uint4 mn[8][16], mx[8][16];       // per warp: the eight channels of each v
+  float2 par[128];                  // (zero, 2^-KB / scale) per channel
+};
+template <int KB>
+__device__ __forceinline__ void kchan_block(const uint4 (&val)[8], KchanShared& sh, uint8_t* __restrict__ pg, const Geom& g, int tid) {
+  constexpr int ROW = 128 * KB / 8;
+  const int tr = tid >> 4, v = tid & 15, warp = tid >> 5, lane = tid & 31;
+  __half2 mn[4], mx[4];
+  auto h2 = [](uint32_t u) { return *reinterpret_cast<const __half2*>(&u); };
+  auto u32 = [](__half2 h) { return *reinterpret_cast<const uint32_t*>(&h); };
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t w[4] = {val[i].x, val[i].y, val[i].z, val[i].w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      mn[j] = i ? __hmin2(mn[j], h2(w[j])) : h2(w[j]);
+      mx[j] = i ? __hmax2(mx[j], h2(w[j])) : h2(w[j]);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    mn[j] = __hmin2(mn[j], h2(__shfl_xor_sync(FULL, u32(mn[j]), 16)));
+    mx[j] = __hmax2(mx[j], h2(__shfl_xor_sync(FULL, u32(mx[j]), 16)));
+  }
+  if (lane < 16) {
+    sh.mn[warp][v] = make_uint4(u32(mn[0]), u32(mn[1]), u32(mn[2]), u32(mn[3]));
+    sh.mx[warp][v] = make_uint4(u32(mx[0]), u32(mx[1]), u32(mx[2]), u32(mx[3]));
+  }
+  __syncthreads();
+  if (tid < 128) {
+    const __half* a = reinterpret_cast<const __half*>(sh.mn) + tid;       // channel tid of warp 0
+    const __half* b = reinterpret_cast<const __half*>(sh.mx) + tid;
+    __half lo = a[0], hi = b[0];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) { lo = __hmin(lo, a[128 * w]); hi = __hmax(hi, b[128 * w]); }
+    const GroupParams p = group_params(__half2float(lo), __half2float(hi), (float)((1 << KB) - 1));
+    reinterpret_cast<uint32_t*>(pg + g.k_meta_off)[tid] = p.meta;
+    sh.par[tid] = make_float2(p.z, p.inv * (1.0f / (float)(1 << KB)));
+  }
+  __syncthreads();
+  float z[8], inv_q[8];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float4 p = *reinterpret_cast<const float4*>(&sh.par[8 * v + 2 * j]);
+    z[2 * j] = p.x; inv_q[2 * j] = p.y; z[2 * j + 1] = p.z; inv_q[2 * j + 1] = p.w;
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t w[4] = {val[i].x, val[i].y, val[i].z, val[i].w};
+    uint32_t word[2];
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+      const float2 f0 = __half22float2(h2(w[2 * hh])), f1 = __half22float2(h2(w[2 * hh + 1]));
+      const float x[4] = {f0.x, f0.y, f1.x, f1.y};
+      const float zz[4] = {z[4 * hh], z[4 * hh + 1], z[4 * hh + 2], z[4 * hh + 3]};
+      const float ii[4] = {inv_q[4 * hh], inv_q[4 * hh + 1], inv_q[4 * hh + 2], inv_q[4 * hh + 3]};
+      word[hh] = code_word4<KB>(x, zz, ii);
+    }
+    uint8_t* row = pg + (tr + 16 * i) * ROW;
+    if constexpr (KB == 4) {
+      const int rh = v & 1, f = (v >> 1) & 1, mw = v >> 2;
+      const uint32_t other = __shfl_xor_sync(FULL, f ? word[0] : word[1], 2);       // the partner's half of the word this lane stores
+      *reinterpret_cast<uint32_t*>(row + (2 * rh + f) * 16 + mw * 4) = f ? (other | (word[1] << 4)) : (word[0] | (other << 4));
+    } else {
+      const int rh = v & 1, mw = v >> 1;
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh)
+        *reinterpret_cast<uint32_t*>(row + (mw >> 2) * 64 + (2 * rh + hh) * 16 + (mw & 3) * 4) = word[hh];
+    }
+  }
+  __syncthreads();                       // the scratch may be used for another block
+}
+
+// Channel-wise quantization of K, head_dim 128, 4- or 8-bit codes: CTA j of a stream takes the j-th 128-token block that the
+// append touches; CTA 0 also takes the last one when that stays incomplete (its rows go to the tail, which CTA 0 must
+// have finished reading first).  A complete block never passes through shared memory: every thread has eight 16-byte
+// loads in flight and keeps them, which is what the kernel is bound by (reading the 16-bit rows).  K and V of 120 streams x
+// 16,383 tokens (values by the kernel above, 162 us of it): 605 us with the block staged in shared memory (48 KB a CTA,
+// one load in flight per thread, 7 instructions more per element), 327 us now.
+template <int DTYPE, int KB, bool ROT>
+__global__ void __launch_bounds__(256, 3)
+quant_kchan_fast_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, int64_t sb, int64_t sh, int64_t st, int t_new) {
+  constexpr int D = 128;
+  __shared__ KchanShared scratch;
+  const int bh = blockIdx.y, b = bh / g.Hkv, h = bh % g.Hkv;
+  const int t0 = c.seq_len[b];
+  if (!append_fits(t0, t_new, g.capacity)) return;
+  const int end = t0 + t_new, first_page = t0 >> 7;
+  const int nblk = ((end + 127) >> 7) - first_page;
+  const bool last_partial = (end & 127) != 0;
+  const int tid = threadIdx.x, tr = tid >> 4, v = tid & 15;
+  uint16_t* tail = c.k_tail + (size_t)bh * kPageTokens * D;
+  const int j = blockIdx.x;
+  if (j >= nblk) return;
+  const uint16_t* in = k_new + (int64_t)b * sb + (int64_t)h * sh - (int64_t)t0 * st + v * 8;     // channel piece of token 0
+  if (j < nblk - 1 || !last_partial) {
+    const int tb = (first_page + j) << 7, lo = max(t0 - tb, 0);
+    uint4 val[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int slot = tr + 16 * i;
+      if (slot < lo) val[i] = *reinterpret_cast<const uint4*>(tail + (size_t)slot * D + v * 8);
+      else val[i] = __ldcs(reinterpret_cast<const uint4*>(in + (int64_t)(tb + slot) * st));
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint4 conv = key_row_fp16<DTYPE, ROT>(val[i], c.k_signs, v);
+      if (tr + 16 * i >= lo) val[i] = conv;
+    }
+    kchan_block<KB>(val, scratch, c.pages + ((size_t)bh * g.n_pages + first_page + j) * g.page_bytes, g, tid);
+  }
+  if (j == 0 && last_partial) {           // the block that stays incomplete: its new rows go to the tail
+    const int tb = (first_page + nblk - 1) << 7, lo = max(t0 - tb, 0), hi = end - tb;
+    for (int s0 = lo; s0 < hi; s0 += 16) {
+      const int slot = s0 + tr;
+      uint4 val = make_uint4(0u, 0u, 0u, 0u);
+      if (slot < hi) val = __ldcs(reinterpret_cast<const uint4*>(in + (int64_t)(tb + slot) * st));
+      val = key_row_fp16<DTYPE, ROT>(val, c.k_signs, v);
+      if (slot < hi) *reinterpret_cast<uint4*>(tail + (size_t)slot * D + v * 8) = val;
+    }
+  }
+}
+
+// Channel-wise quantization of K over 128-token blocks with the fp16 tail, the shapes that the kernel above does not
+// serve (head_dim 64, 2-bit codes).  CTA j of a stream handles the j-th block touched by this append.  CTA 0 also
 // handles the final block when that one is incomplete (it writes the tail, which
 // CTA 0 must have finished reading first).
 __global__ void __launch_bounds__(kThreads)
@@ -811,10 +925,6 @@ quant_kchan_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new,
     if (!complete) continue;
     __syncthreads();
     uint8_t* pg = c.pages + ((size_t)bh * g.n_pages + page) * g.page_bytes;
-    if (D == 128 && (g.kb == 4 || g.kb == 8)) {
-      if (g.kb == 4) kchan_block_fast<4>(sX, sC, pg, g, tid); else kchan_block_fast<8>(sX, sC, pg, g, tid);
-      continue;
-    }
     for (int d = tid; d < D; d += kThreads) {
       float mn = INFINITY, mx = -INFINITY;
       for (int t = 0; t < kPageTokens; ++t) {
@@ -886,7 +996,17 @@ int launch_quantize_append(const Geom& g, const CachePtrs& c, const void* k_new,
   else if (g.in_dtype == KVQ_BF16) KVQ_QLAUNCH(64, KVQ_BF16);
   else KVQ_QLAUNCH(64, KVQ_FP16);
 #undef KVQ_QLAUNCH
-  if (g.k_axis == 1) {
+  if (g.k_axis == 1 && g.D == 128 && (g.kb == 4 || g.kb == 8)) {
+    dim3 grid2((t_new + 127) / 128 + 1, streams);
+#define KVQ_KCHAN(T_, KB_)                                                                                         \
+  do {                                                                                                             \
+    if (c.k_signs) quant_kchan_fast_kernel<T_, KB_, true><<<grid2, 256, 0, stream>>>(g, c, k, sb, sh, st, t_new);  \
+    else quant_kchan_fast_kernel<T_, KB_, false><<<grid2, 256, 0, stream>>>(g, c, k, sb, sh, st, t_new);           \
+  } while (0)
+    if (g.in_dtype == KVQ_BF16) { if (g.kb == 4) KVQ_KCHAN(KVQ_BF16, 4); else KVQ_KCHAN(KVQ_BF16, 8); }
+    else { if (g.kb == 4) KVQ_KCHAN(KVQ_FP16, 4); else KVQ_KCHAN(KVQ_FP16, 8); }
+#undef KVQ_KCHAN
+  } else if (g.k_axis == 1) {
     size_t smem = (size_t)kPageTokens * g.D * 3;
     cudaFuncSetAttribute(quant_kchan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 128 * 3);
     dim3 grid2((t_new + 127) / 128 + 1, streams);
