@@ -11,7 +11,7 @@
 // atomics, no read-modify-write; a token that is not new is simply not stored (byte stores for
 // values).  Group minima and maxima are reduced with a few shuffles between the lanes of a row.
 // The kernel is bound by reading the 16-bit inputs from HBM.
-#include "kvq_internal.h"
+#include "kvq_quantize.cuh"
 
 namespace kvq {
 
@@ -19,8 +19,6 @@ namespace {
 
 constexpr int kThreads = 128;
 constexpr int kWarps = kThreads / 32;
-constexpr uint32_t FULL = 0xffffffffu;
-constexpr float kRoundMagic = 12582912.0f;   // 1.5 * 2^23: adding it rounds to nearest-even at integer precision
 
 // Where the 16-bit row of a task-local token comes from: the call's input, or - for the first n_win tokens of a task
 // when a residual window is kept - the window's ring of rows (token t in slot t % R; a task never wraps the ring).
@@ -38,12 +36,6 @@ struct RowSrc {
 // Tokens handled by one warp task: 32, or 64 where 32 tokens would leave a lane fewer than the four tokens
 // that make up a word of value codes.
 __host__ __device__ constexpr int task_tokens(int D, int bits) { return (D == 64 && bits == 2) ? 64 : 32; }
-
-__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
-  uint32_t d;
-  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
-  return d;
-}
 
 // Four byte values held as exact float integers (0..255) -> one little-endian word.
 __device__ __forceinline__ uint32_t pack_bytes(float b0, float b1, float b2, float b3) {
@@ -559,11 +551,6 @@ __device__ __forceinline__ void copy_task_side(const RowSrc& rsrc, int D, int lo
         *reinterpret_cast<const uint4*>(rsrc.row(row) + l * 8);
 }
 
-// An append of t_new tokens at position t0 fits the cache; written without a sum that could overflow.
-__host__ __device__ __forceinline__ bool append_fits(int t0, int t_new, int capacity) {
-  return t0 >= 0 && t0 <= capacity - t_new;
-}
-
 // Token-wise quantization of V (blockIdx.z == 0) and of K (blockIdx.z == 1).  grid.y = stream, grid.x strides
 // over the warp tasks touched by this append.
 template <int D, int DTYPE, bool ROT>
@@ -674,131 +661,6 @@ __device__ __forceinline__ void pack_k_rows(const uint8_t* codes, int code_strid
   }
 }
 
-// The 16-byte pieces (eight channels 8 v .. 8 v + 7, v = tid % 16) of new key rows as saturated fp16, rotated if asked.
-// The 16 lanes of a row take part together (the rotation shuffles between them).
-template <int DTYPE, bool ROT>
-__device__ __forceinline__ uint4 key_row_fp16(uint4 val, const int8_t* __restrict__ signs, int v) {
-  if constexpr (DTYPE == KVQ_BF16 || ROT) {
-    uint32_t w[4] = {val.x, val.y, val.z, val.w};
-    float x[8];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if constexpr (DTYPE == KVQ_BF16) {
-        x[2 * i] = __uint_as_float(w[i] << 16);
-        x[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
-      } else {
-        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[i]));
-        x[2 * i] = f.x;
-        x[2 * i + 1] = f.y;
-      }
-    }
-    if constexpr (ROT) rotate_row8<128>(x, signs, v);
-    // saturating: the conversion rounds to nearest (infinity from 65520 on), the packed clamp brings infinities to 65504
-    const __half2 top = __half2half2(__ushort_as_half(0x7BFF)), bottom = __half2half2(__ushort_as_half(0xFBFF));
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const __half2 h = __hmin2(__hmax2(__floats2half2_rn(x[2 * i], x[2 * i + 1]), bottom), top);
-      w[i] = *reinterpret_cast<const uint32_t*>(&h);
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
-  } else {
-    return val;
-  }
-}
-
-// Codes of four values as the four bytes of a word: rint(clamp((x - z) * inv, 0, qmax)), the fixed formula.  `inv_q` is
-// inv * 2^-BITS (exact), so that the saturation of a multiplication to [0, 1] is the clamp to [0, 2^BITS] (a NaN becomes
-// 0); the fused multiply-add by 2^BITS onto 1.5 * 2^23 rounds to nearest-even, and the upper clamp follows on two codes at a time.
-template <int BITS>
-__device__ __forceinline__ uint32_t code_word4(const float (&x)[4], const float (&z)[4], const float (&inv_q)[4]) {
-  uint32_t n[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-    n[j] = __float_as_uint(__fmaf_rn(__saturatef(__fmul_rn(__fsub_rn(x[j], z[j]), inv_q[j])), (float)(1 << BITS), kRoundMagic));
-  constexpr uint32_t TOP = ((1u << BITS) - 1u) * 0x00010001u;
-  const uint32_t even = __vminu2(prmt(n[0], n[2], 0x5410), TOP), odd = __vminu2(prmt(n[1], n[3], 0x5410), TOP);
-  return even + odd * 256u;
-}
-
-// Channel-wise quantization of one complete 128-token block, head_dim 128, 4- or 8-bit codes, held in the registers of
-// 256 threads: thread (tr = tid / 16, v = tid % 16) has channels 8 v .. 8 v + 7 of tokens tr + 16 i as fp16.  Minimum and
-// maximum are taken two channels at a time in fp16 (exact), first in the thread, then over the warps through 4 KB of
-// shared memory; the parameters are made once per channel.  At 4 bits the lanes whose codes share bytes (v and v ^ 2) swap one word
-// per token, and each stores one word of the row: the 16 lanes of a row write its 64 (8 bits: 128) bytes whole.
-struct KchanShared {
-  uint4 mn[8][16], mx[8][16];       // per warp: the eight channels of each v
-  float2 par[128];                  // (zero, 2^-KB / scale) per channel
-};
-template <int KB>
-__device__ __forceinline__ void kchan_block(const uint4 (&val)[8], KchanShared& sh, uint8_t* __restrict__ pg, const Geom& g, int tid) {
-  constexpr int ROW = 128 * KB / 8;
-  const int tr = tid >> 4, v = tid & 15, warp = tid >> 5, lane = tid & 31;
-  __half2 mn[4], mx[4];
-  auto h2 = [](uint32_t u) { return *reinterpret_cast<const __half2*>(&u); };
-  auto u32 = [](__half2 h) { return *reinterpret_cast<const uint32_t*>(&h); };
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const uint32_t w[4] = {val[i].x, val[i].y, val[i].z, val[i].w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      mn[j] = i ? __hmin2(mn[j], h2(w[j])) : h2(w[j]);
-      mx[j] = i ? __hmax2(mx[j], h2(w[j])) : h2(w[j]);
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    mn[j] = __hmin2(mn[j], h2(__shfl_xor_sync(FULL, u32(mn[j]), 16)));
-    mx[j] = __hmax2(mx[j], h2(__shfl_xor_sync(FULL, u32(mx[j]), 16)));
-  }
-  if (lane < 16) {
-    sh.mn[warp][v] = make_uint4(u32(mn[0]), u32(mn[1]), u32(mn[2]), u32(mn[3]));
-    sh.mx[warp][v] = make_uint4(u32(mx[0]), u32(mx[1]), u32(mx[2]), u32(mx[3]));
-  }
-  __syncthreads();
-  if (tid < 128) {
-    const __half* a = reinterpret_cast<const __half*>(sh.mn) + tid;       // channel tid of warp 0
-    const __half* b = reinterpret_cast<const __half*>(sh.mx) + tid;
-    __half lo = a[0], hi = b[0];
-#pragma unroll
-    for (int w = 1; w < 8; ++w) { lo = __hmin(lo, a[128 * w]); hi = __hmax(hi, b[128 * w]); }
-    const GroupParams p = group_params(__half2float(lo), __half2float(hi), (float)((1 << KB) - 1));
-    reinterpret_cast<uint32_t*>(pg + g.k_meta_off)[tid] = p.meta;
-    sh.par[tid] = make_float2(p.z, p.inv * (1.0f / (float)(1 << KB)));
-  }
-  __syncthreads();
-  float z[8], inv_q[8];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float4 p = *reinterpret_cast<const float4*>(&sh.par[8 * v + 2 * j]);
-    z[2 * j] = p.x; inv_q[2 * j] = p.y; z[2 * j + 1] = p.z; inv_q[2 * j + 1] = p.w;
-  }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const uint32_t w[4] = {val[i].x, val[i].y, val[i].z, val[i].w};
-    uint32_t word[2];
-#pragma unroll
-    for (int hh = 0; hh < 2; ++hh) {
-      const float2 f0 = __half22float2(h2(w[2 * hh])), f1 = __half22float2(h2(w[2 * hh + 1]));
-      const float x[4] = {f0.x, f0.y, f1.x, f1.y};
-      const float zz[4] = {z[4 * hh], z[4 * hh + 1], z[4 * hh + 2], z[4 * hh + 3]};
-      const float ii[4] = {inv_q[4 * hh], inv_q[4 * hh + 1], inv_q[4 * hh + 2], inv_q[4 * hh + 3]};
-      word[hh] = code_word4<KB>(x, zz, ii);
-    }
-    uint8_t* row = pg + (tr + 16 * i) * ROW;
-    if constexpr (KB == 4) {
-      const int rh = v & 1, f = (v >> 1) & 1, mw = v >> 2;
-      const uint32_t other = __shfl_xor_sync(FULL, f ? word[0] : word[1], 2);       // the partner's half of the word this lane stores
-      *reinterpret_cast<uint32_t*>(row + (2 * rh + f) * 16 + mw * 4) = f ? (other | (word[1] << 4)) : (word[0] | (other << 4));
-    } else {
-      const int rh = v & 1, mw = v >> 1;
-#pragma unroll
-      for (int hh = 0; hh < 2; ++hh)
-        *reinterpret_cast<uint32_t*>(row + (mw >> 2) * 64 + (2 * rh + hh) * 16 + (mw & 3) * 4) = word[hh];
-    }
-  }
-  __syncthreads();                       // the scratch may be used for another block
-}
-
 // Channel-wise quantization of K, head_dim 128, 4- or 8-bit codes: CTA j of a stream takes the j-th 128-token block that the
 // append touches; CTA 0 also takes the last one when that stays incomplete (its rows go to the tail, which CTA 0 must
 // have finished reading first).  A complete block never passes through shared memory: every thread has eight 16-byte
@@ -808,7 +670,6 @@ __device__ __forceinline__ void kchan_block(const uint4 (&val)[8], KchanShared& 
 template <int DTYPE, int KB, bool ROT>
 __global__ void __launch_bounds__(256, 3)
 quant_kchan_fast_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, int64_t sb, int64_t sh, int64_t st, int t_new) {
-  constexpr int D = 128;
   __shared__ KchanShared scratch;
   const int bh = blockIdx.y, b = bh / g.Hkv, h = bh % g.Hkv;
   const int t0 = c.seq_len[b];
@@ -816,37 +677,12 @@ quant_kchan_fast_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new,
   const int end = t0 + t_new, first_page = t0 >> 7;
   const int nblk = ((end + 127) >> 7) - first_page;
   const bool last_partial = (end & 127) != 0;
-  const int tid = threadIdx.x, tr = tid >> 4, v = tid & 15;
-  uint16_t* tail = c.k_tail + (size_t)bh * kPageTokens * D;
+  const int tid = threadIdx.x;
   const int j = blockIdx.x;
   if (j >= nblk) return;
-  const uint16_t* in = k_new + (int64_t)b * sb + (int64_t)h * sh - (int64_t)t0 * st + v * 8;     // channel piece of token 0
-  if (j < nblk - 1 || !last_partial) {
-    const int tb = (first_page + j) << 7, lo = max(t0 - tb, 0);
-    uint4 val[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int slot = tr + 16 * i;
-      if (slot < lo) val[i] = *reinterpret_cast<const uint4*>(tail + (size_t)slot * D + v * 8);
-      else val[i] = __ldcs(reinterpret_cast<const uint4*>(in + (int64_t)(tb + slot) * st));
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const uint4 conv = key_row_fp16<DTYPE, ROT>(val[i], c.k_signs, v);
-      if (tr + 16 * i >= lo) val[i] = conv;
-    }
-    kchan_block<KB>(val, scratch, c.pages + ((size_t)bh * g.n_pages + first_page + j) * g.page_bytes, g, tid);
-  }
-  if (j == 0 && last_partial) {           // the block that stays incomplete: its new rows go to the tail
-    const int tb = (first_page + nblk - 1) << 7, lo = max(t0 - tb, 0), hi = end - tb;
-    for (int s0 = lo; s0 < hi; s0 += 16) {
-      const int slot = s0 + tr;
-      uint4 val = make_uint4(0u, 0u, 0u, 0u);
-      if (slot < hi) val = __ldcs(reinterpret_cast<const uint4*>(in + (int64_t)(tb + slot) * st));
-      val = key_row_fp16<DTYPE, ROT>(val, c.k_signs, v);
-      if (slot < hi) *reinterpret_cast<uint4*>(tail + (size_t)slot * D + v * 8) = val;
-    }
-  }
+  const uint16_t* in = k_new + (int64_t)b * sb + (int64_t)h * sh - (int64_t)t0 * st + (tid & 15) * 8;
+  if (j < nblk - 1 || !last_partial) kchan_complete_block<DTYPE, KB, ROT>(g, c, bh, first_page + j, t0, in, st, scratch, tid);
+  if (j == 0 && last_partial) kchan_tail_rows<DTYPE, ROT>(c, bh, first_page + nblk - 1, t0, end, in, st, tid);
 }
 
 // Channel-wise quantization of K over 128-token blocks with the fp16 tail, the shapes that the kernel above does not
@@ -976,6 +812,7 @@ __global__ void bump_seq_len_kernel(Geom g, CachePtrs c, int t_new) {
 
 int launch_quantize_append(const Geom& g, const CachePtrs& c, const void* k_new, const void* v_new,
                            int64_t sb, int64_t sh, int64_t st, int t_new, cudaStream_t stream) {
+  if (append_rows_serves(g, t_new)) return launch_append_rows(g, c, k_new, v_new, sb, sh, st, t_new, stream);
   const uint16_t* k = static_cast<const uint16_t*>(k_new);
   const uint16_t* v = static_cast<const uint16_t*>(v_new);
   // warp tasks touched per stream: at most ceil(t_new / 32) + 1; one warp per task, CTAs stride over them

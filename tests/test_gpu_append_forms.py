@@ -20,10 +20,10 @@ def kvq():
     return mod
 
 
-def edge_values(w, T, B, seed):
+def edge_values(w, T, B, seed, rotated=False):
     """Keys and values with constant groups, signed zeros, subnormal ranges and entries at the ends of the 16-bit type."""
     k, v = wl.make_kv(w.with_(number=seed), tokens=T, batch=B)
-    big = 65504.0 if w.dtype == "fp16" else 3.0e38
+    big = 65504.0 if w.dtype == "fp16" else 1.0e30 if rotated else 3.0e38      # (a rotation sums 128 of them: finite)
     for x in (k, v):
         x[:, :, 0] = 0.25                                   # a constant row
         if T > 3:
@@ -38,7 +38,7 @@ def edge_values(w, T, B, seed):
 def check(kvq, w, B, chunks, signs=None, residual=0, strided=False, seed=1):
     T = sum(chunks)
     cap = -(-T // 128) * 128 + 128
-    k, v = edge_values(w, T, B, seed)
+    k, v = edge_values(w, T, B, seed, signs is not None)
     if strided:                                              # [B, T, H, D] in memory, as a projection leaves it
         k, v = (x.transpose(1, 2).contiguous().transpose(1, 2) for x in (k, v))
     cfg, gc, oc = tl.build_both(kvq, w, k, v, chunks, cap, k_signs=signs, residual=residual)
@@ -57,3 +57,28 @@ SIGNS = np.random.default_rng(3).choice([-1, 1], 128).astype(np.int8)
 def test_channelwise_keys(kvq, chunks, kb, dtype, rotated):
     w = wl.SHAPED_14B.with_(n_kv_heads=3, n_q_heads=3, kb=kb, dtype=dtype)
     check(kvq, w, 2, CHUNKS[chunks], SIGNS if rotated else None, strided=chunks == "over")
+
+
+FEW = [1, 1, 2, 5, 16, 17, 103, 1, 15]          # single tokens and short runs around the page's 16-, 32- and 128-token marks
+
+
+@pytest.mark.parametrize("kb,vb", [(2, 8), (4, 2), (8, 4)])
+@pytest.mark.parametrize("D,gk,gv", [(128, 128, 32), (128, 32, 64), (64, 64, 32), (64, 32, 64)])
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+@pytest.mark.parametrize("form", ["plain", "rotated", "window", "rotated window"])
+def test_few_tokens(kvq, kb, vb, D, gk, gv, dtype, form):
+    heads = 9 if D == 64 else 3                  # more and fewer heads than CTAs of a cluster
+    w = wl.LLAMA_8B.with_(n_kv_heads=heads, n_q_heads=heads, head_dim=D, kb=kb, vb=vb, gk=gk, gv=gv, dtype=dtype)
+    check(kvq, w, 2, FEW, SIGNS[:D] if "rotated" in form else None, 64 if "window" in form else 0, strided=D == 64)
+
+
+def test_few_tokens_beyond_the_capacity(kvq):
+    """A sequence without room keeps its bytes and its length and sets the status; the others take their tokens."""
+    w = wl.LLAMA_8B.with_(n_kv_heads=2, n_q_heads=2)
+    k, v = edge_values(w, 128, 2, 1)
+    cfg, gc, _ = tl.build_both(kvq, w, k, v, [128], 256)
+    gc.seq_len.copy_(torch.tensor([255, 128], dtype=torch.int32))
+    before = gc.pages_view()[0].clone()
+    kvq.kvq_quantize_append(cfg, gc, k[:, :, :2].cuda(), v[:, :, :2].cuda())
+    assert gc.seq_len.tolist() == [255, 130] and torch.equal(gc.pages_view()[0], before)
+    assert kvq.kvq_check_status(gc) == -5
