@@ -90,3 +90,17 @@ def test_window_improves_attention_accuracy(kvq):
         cfg, gc, _ = tl.build_both(kvq, w, k, v, [T], 512, residual=R)
         errs.append(np.linalg.norm(tl.gpu_decode(kvq, cfg, gc, q) - exact))
     assert errs[1] < errs[0]
+
+
+@pytest.mark.parametrize("D,heads,rows", [(128, 1, 1), (128, 3, 1), (128, 2, 2), (128, 4, 2), (128, 7, 1), (128, 8, 1),
+                                          (64, 1, 1), (64, 3, 1), (64, 2, 2)])      # (head_dim 64 serves four pairs)
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+@pytest.mark.parametrize("R,T", [(64, 1), (64, 63), (64, 128 + 33), (128, 127), (128, 128 + 65)])
+def test_window_tokens_only_and_with_pages(kvq, D, heads, rows, dtype, R, T):
+    """Window lengths around the kernel's token passes, every number of (row, head) pairs, with and without pages."""
+    g = 128 if D == 128 else 64
+    w = wl.LLAMA_8B.with_(n_kv_heads=2, n_q_heads=2 * heads, head_dim=D, gk=g, gv=g, dtype=dtype)
+    k, v = wl.make_kv(w, tokens=T, batch=2)
+    cfg, gc, oc = tl.build_both(kvq, w, k, v, [T], 384, residual=R)
+    q = make_q_rows(w, 2, rows, T)
+    tl.assert_attention_close(decode_rows(kvq, cfg, gc, q), oc.decode_rows(tl.bits_of(q)))
