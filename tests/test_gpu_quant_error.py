@@ -74,3 +74,21 @@ def test_channel_wise_keys_are_rejected(kvq):
     with pytest.raises(kvq.KvqError) as e:
         kvq.kvq_quant_error(cfg, k.cuda(), v.cuda(), sums)
     assert e.value.code == -2
+
+
+@pytest.mark.parametrize("T", [1, 31, 64, 65, 130, 700])
+@pytest.mark.parametrize("D,gk,gv", [(128, 128, 32), (128, 64, 128), (64, 32, 64)])
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+def test_error_sums_at_the_ends_of_the_row_turns(kvq, T, D, gk, gv, dtype):
+    """Token counts around a CTA's turn of rows, every group size, strided inputs; same bound as above (fp32 squares of at
+    most 8 elements, then double precision: far below 1e-5)."""
+    for kb, vb in ((2, 8), (4, 6), (16, 1)) if D == 128 else ((2, 8), (4, 6)):
+        w = wl.LLAMA_8B.with_(n_kv_heads=3, n_q_heads=3, head_dim=D, gk=gk, gv=gv, dtype=dtype, kb=kb, vb=vb)
+        k, v = wl.make_kv(w, tokens=T, batch=2)
+        k[:, :, 0] = 0.5                                   # a constant row: scale 0
+        cfg = tl.gpu_config_for(kvq, w, 2, 128)
+        sums = torch.zeros((2, 3, 4), dtype=torch.float64, device="cuda")
+        kd, vd = (x.transpose(1, 2).contiguous().transpose(1, 2).cuda() for x in (k, v))
+        kvq.kvq_quant_error(cfg, kd, vd, sums)
+        want = oe.quant_error_sums(tl.bits_of(k), tl.bits_of(v), w.dtype, w.kb, w.vb, w.gk, w.gv)
+        assert np.allclose(sums.cpu().numpy(), want, rtol=1e-5, atol=0.0)
