@@ -37,22 +37,49 @@ struct RowSrc {
 // that make up a word of value codes.
 __host__ __device__ constexpr int task_tokens(int D, int bits) { return (D == 64 && bits == 2) ? 64 : 32; }
 
-// Four byte values held as exact float integers (0..255) -> one little-endian word.
-__device__ __forceinline__ uint32_t pack_bytes(float b0, float b1, float b2, float b3) {
-  const float lo = __fmaf_rn(b1, 256.0f, b0), hi = __fmaf_rn(b3, 256.0f, b2);        // < 65536: exact
-  return prmt(__float_as_uint(__fadd_rn(lo, 8388608.0f)), __float_as_uint(__fadd_rn(hi, 8388608.0f)), 0x5410);
+// Two 16-bit inputs as a packed pair of their own type, for exact minima and maxima.
+template <int DTYPE> struct Pair16 { using type = __half2; };
+template <> struct Pair16<KVQ_BF16> { using type = __nv_bfloat162; };
+__device__ __forceinline__ float2 pair_to_f32(__half2 h) { return __half22float2(h); }
+__device__ __forceinline__ float2 pair_to_f32(__nv_bfloat162 h) { return __bfloat1622float2(h); }
+__device__ __forceinline__ __half2 lows(__half2 a, __half2 b) { return __lows2half2(a, b); }
+__device__ __forceinline__ __half2 highs(__half2 a, __half2 b) { return __highs2half2(a, b); }
+__device__ __forceinline__ __nv_bfloat162 lows(__nv_bfloat162 a, __nv_bfloat162 b) { return __lows2bfloat162(a, b); }
+__device__ __forceinline__ __nv_bfloat162 highs(__nv_bfloat162 a, __nv_bfloat162 b) { return __highs2bfloat162(a, b); }
+
+// (minimum, - maximum) of the eight values of a 16-byte piece.
+template <int DTYPE>
+__device__ __forceinline__ typename Pair16<DTYPE>::type minmax8(const uint4& r) {
+  using H2 = typename Pair16<DTYPE>::type;
+  const H2* h = reinterpret_cast<const H2*>(&r);
+  const H2 lo = __hmin2(__hmin2(h[0], h[1]), __hmin2(h[2], h[3]));
+  const H2 hi = __hneg2(__hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3])));
+  return __hmin2(lows(lo, hi), highs(lo, hi));
 }
 
-// Quantize one side of a task of TT tokens.  src: row of the task's first token in the input; tokens
-// [lo, hi) of the task are new.  codes: keys - the page's key row of the task's first token; values - the
-// page's value block of the task's first token.  meta_out: metadata row of the task's first token.
+// Value e (0..7) of a 16-byte piece in fp32.
+template <int DTYPE>
+__device__ __forceinline__ float piece_value(const uint4& r, int e) {
+  const uint32_t w = e < 2 ? r.x : e < 4 ? r.y : e < 6 ? r.z : r.w;
+  if constexpr (DTYPE == KVQ_BF16) return __uint_as_float((e & 1) ? (w & 0xFFFF0000u) : (w << 16));
+  else { const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w)); return (e & 1) ? f.y : f.x; }
+}
+
+// Quantize one side of a task of TT tokens, four tokens of a lane per pass.  rsrc: the task's rows; tokens [lo, hi) of the
+// task are new (FULLBLK: all of them).  codes: keys - the page's key row of the task's first token; values - the page's
+// value block of the task's first token.  meta_out: metadata row of the task's first token.
 //
-// Lane = (row slot rs, word column mw, row half rh): it owns, for each of its tokens, the FPB pieces of
-// 8 channels 16 (FPB mw + f) + 8 rh + {0..7}, f < FPB, whose codes share bytes.
-template <int BITS, bool IS_V, int D, int DTYPE, bool ROT>
-__device__ __forceinline__ void quantize_task(const RowSrc& rsrc, int gsz, int lo, int hi,
-                                              uint8_t* __restrict__ codes, uint32_t* __restrict__ meta_out,
-                                              int lane, const int8_t* __restrict__ signs) {
+// Lane = (row slot rs, word column mw, row half rh): it owns, for each of its tokens, the FPB pieces of 8 channels
+// 16 (FPB mw + f) + 8 rh + {0..7}, f < FPB, whose codes share bytes.  The minima / maxima of the four tokens are reduced
+// with a shuffle reduce-scatter, so that the group parameters (two divisions) are computed once per group rather than once
+// per lane, and are then broadcast to the lanes of the group.  Minimum and negated maximum travel as one pair of the 16-bit type,
+// the clamp is the saturation of a multiplication: 10.6 instructions per element instead of 14.  K and V of 64 streams x
+// 32,768 tokens (K4V2, 1.29 GB) 333 -> 275 us; in a replayed graph 335 -> 250 us at five CTAs per SM (four 259, three 298, six 270: registers spill);
+// bound by issue (60 %) and load latency.  8-byte pieces at 2 bits (half the registers, twice the loads): 276 us.
+template <int BITS, bool IS_V, int D, int DTYPE, bool FULLBLK>
+__device__ __forceinline__ void quantize_task(const RowSrc& rsrc, int gsz, int lo, int hi, uint8_t* __restrict__ codes,
+                                              uint32_t* __restrict__ meta_out, int lane) {
+  using H2 = typename Pair16<DTYPE>::type;
   constexpr int FPB = 8 / BITS;
   constexpr int NMW = (D / 16) / FPB;        // word columns per row half
   constexpr int LR = 2 * NMW;                // lanes per token row
@@ -60,13 +87,17 @@ __device__ __forceinline__ void quantize_task(const RowSrc& rsrc, int gsz, int l
   constexpr int TT = task_tokens(D, BITS);
   constexpr int TPL = TT / RS;               // tokens per lane
   constexpr int K_ROW_BYTES = D * BITS / 8;
+  constexpr int NSET = FPB == 4 ? 2 : 1;      // a lane's fields may belong to two groups (groups of 32 at 2 bits)
+  constexpr float DOWN = 1.0f / (float)(1 << BITS);
   static_assert(TPL % 4 == 0, "a lane holds whole groups of four tokens");
   const int rs = lane / LR, cs = lane % LR, mw = cs >> 1, rh = cs & 1;
   const float qmax = (float)((1 << BITS) - 1);
   const int spg = gsz >> 4;                                  // 16-channel slices per group
-  const bool split = FPB > spg;                              // a lane's fields belong to two groups (FPB 4, groups of 32)
-  const int lpg = split ? 2 : 2 * spg / FPB;                 // lanes per group
+  const bool split = FPB > spg;
+  const int lpg = split ? 2 : 2 * spg / FPB;                 // lanes per group: 2, 4, 8 or 16
   const int ng = D / gsz;
+  const int b0 = cs & 1, b1 = (cs >> 1) & 1;
+  const int gbase = lane & ~(lpg - 1);                       // first lane of this lane's group
 
   // block-local token of token slot k
   auto token_of = [&](int k) {
@@ -77,255 +108,9 @@ __device__ __forceinline__ void quantize_task(const RowSrc& rsrc, int gsz, int l
       return k * RS + rs;
     }
   };
-
-  // ---- all loads first (TPL * FPB 16-byte loads in flight per lane)
-  uint4 raw[TPL][FPB];
-#pragma unroll
-  for (int k = 0; k < TPL; ++k) {
-    const int tau = token_of(k);
-    const bool valid = tau >= lo && tau < hi;
-#pragma unroll
-    for (int f = 0; f < FPB; ++f) {
-      raw[k][f] = make_uint4(0u, 0u, 0u, 0u);
-      if (valid) raw[k][f] = __ldcs(reinterpret_cast<const uint4*>(rsrc.row(tau) + 16 * (FPB * mw + f) + 8 * rh));
-    }
-  }
-
-  float vbyte[4][8];      // values: byte values (exact float integers) of the four tokens of the words being built
-#pragma unroll
-  for (int k = 0; k < TPL; ++k) {
-    const int tau = token_of(k);
-    const bool valid = tau >= lo && tau < hi;
-    float x[FPB][8];
-#pragma unroll
-    for (int f = 0; f < FPB; ++f) {
-      const uint32_t rw[4] = {raw[k][f].x, raw[k][f].y, raw[k][f].z, raw[k][f].w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if constexpr (DTYPE == KVQ_BF16) {
-          x[f][2 * i] = __uint_as_float(rw[i] << 16);
-          x[f][2 * i + 1] = __uint_as_float(rw[i] & 0xFFFF0000u);
-        } else {
-          const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&rw[i]));
-          x[f][2 * i] = v.x;
-          x[f][2 * i + 1] = v.y;
-        }
-      }
-    }
-    if constexpr (ROT) {
-      // keys only: y = H (signs * x) / sqrt(D); channel d = 16 (FPB mw + f) + 8 rh + i.  Butterfly stages in
-      // the order h = 1, 2, 4, ...: bits of i in the lane, rh across lanes, bits of f in the lane, bits of mw across lanes.
-#pragma unroll
-      for (int f = 0; f < FPB; ++f) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) x[f][i] = __fmul_rn(x[f][i], (float)signs[16 * (FPB * mw + f) + 8 * rh + i]);
-#pragma unroll
-        for (int h = 1; h < 8; h <<= 1) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            if ((i & h) == 0) {
-              const float a = x[f][i], b = x[f][i + h];
-              x[f][i] = __fadd_rn(a, b);
-              x[f][i + h] = __fsub_rn(a, b);
-            }
-          }
-        }
-      }
-#pragma unroll
-      for (int f = 0; f < FPB; ++f) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float o = __shfl_xor_sync(FULL, x[f][i], 1);
-          x[f][i] = rh ? __fsub_rn(o, x[f][i]) : __fadd_rn(x[f][i], o);
-        }
-      }
-#pragma unroll
-      for (int hf = 1; hf < FPB; hf <<= 1) {
-#pragma unroll
-        for (int f = 0; f < FPB; ++f) {
-          if ((f & hf) == 0) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const float a = x[f][i], b = x[f + hf][i];
-              x[f][i] = __fadd_rn(a, b);
-              x[f + hf][i] = __fsub_rn(a, b);
-            }
-          }
-        }
-      }
-#pragma unroll
-      for (int hm = 1; hm < NMW; hm <<= 1) {
-        const bool upper = (mw & hm) != 0;
-#pragma unroll
-        for (int f = 0; f < FPB; ++f) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const float o = __shfl_xor_sync(FULL, x[f][i], 2 * hm);
-            x[f][i] = upper ? __fsub_rn(o, x[f][i]) : __fadd_rn(x[f][i], o);
-          }
-        }
-      }
-#pragma unroll
-      for (int f = 0; f < FPB; ++f) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) x[f][i] = __fmul_rn(x[f][i], inv_sqrt_dim<D>());
-      }
-    }
-
-    // ---- group minimum / maximum: fields in the lane, then the lanes of the group
-    float mnf[FPB], mxf[FPB];
-#pragma unroll
-    for (int f = 0; f < FPB; ++f) {
-      mnf[f] = fminf(fminf(fminf(x[f][0], x[f][1]), fminf(x[f][2], x[f][3])),
-                     fminf(fminf(x[f][4], x[f][5]), fminf(x[f][6], x[f][7])));
-      mxf[f] = fmaxf(fmaxf(fmaxf(x[f][0], x[f][1]), fmaxf(x[f][2], x[f][3])),
-                     fmaxf(fmaxf(x[f][4], x[f][5]), fmaxf(x[f][6], x[f][7])));
-    }
-    float mnA = mnf[0], mxA = mxf[0], mnB = mnf[FPB - 1], mxB = mxf[FPB - 1];
-    if constexpr (FPB == 2) {
-      mnA = mnB = fminf(mnf[0], mnf[1]);
-      mxA = mxB = fmaxf(mxf[0], mxf[1]);
-    }
-    if constexpr (FPB == 4) {
-      mnA = fminf(mnf[0], mnf[1]); mxA = fmaxf(mxf[0], mxf[1]);
-      mnB = fminf(mnf[2], mnf[3]); mxB = fmaxf(mxf[2], mxf[3]);
-      if (!split) {
-        mnA = mnB = fminf(mnA, mnB);
-        mxA = mxB = fmaxf(mxA, mxB);
-      }
-    }
-#pragma unroll
-    for (int off = 1; off < LR; off <<= 1) {
-      if (off < lpg) {
-        mnA = fminf(mnA, __shfl_xor_sync(FULL, mnA, off));
-        mxA = fmaxf(mxA, __shfl_xor_sync(FULL, mxA, off));
-        if constexpr (FPB == 4) {
-          if (split) {
-            mnB = fminf(mnB, __shfl_xor_sync(FULL, mnB, off));
-            mxB = fmaxf(mxB, __shfl_xor_sync(FULL, mxB, off));
-          }
-        }
-      }
-    }
-    const GroupParams pA = group_params(mnA, mxA, qmax);
-    GroupParams pB = pA;
-    if constexpr (FPB == 4) {
-      if (split) pB = group_params(mnB, mxB, qmax);
-    }
-    if (valid && (cs & (lpg - 1)) == 0) {
-      const int gi = (16 * FPB * mw) / gsz;                 // group of the lane's first field
-      meta_out[tau * ng + gi] = pA.meta;
-      if constexpr (FPB == 4) {
-        if (split) meta_out[tau * ng + gi + 1] = pB.meta;
-      }
-    }
-
-    // ---- codes as exact float integers, the FPB fields of a byte combined: byte = sum_f code_f * 2^(BITS f)
-    float bytev[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) bytev[i] = 0.f;
-#pragma unroll
-    for (int f = FPB - 1; f >= 0; --f) {
-      const GroupParams& p = (FPB == 4 && f >= 2) ? pB : pA;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        float u = __fmul_rn(__fsub_rn(x[f][i], p.z), p.inv);
-        u = fminf(fmaxf(u, 0.0f), qmax);
-        const float r = __fsub_rn(__fadd_rn(u, kRoundMagic), kRoundMagic);      // rint(u), exact
-        bytev[i] = __fmaf_rn(bytev[i], (float)(1 << BITS), r);                  // exact: < 256
-      }
-    }
-
-    if constexpr (!IS_V) {
-      // keys: bytes 0..3 of a word are channels 4 hh + {0..3} of this lane's 8, chunk 2 rh + hh, word mw of the row
-      if (valid) {
-        constexpr int wpc = D * BITS / 128;
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-          const uint32_t w = pack_bytes(bytev[4 * hh], bytev[4 * hh + 1], bytev[4 * hh + 2], bytev[4 * hh + 3]);
-          *reinterpret_cast<uint32_t*>(codes + (size_t)tau * K_ROW_BYTES + chunk_word_byte(2 * rh + hh, mw, wpc, 4)) = w;
-        }
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) vbyte[k & 3][i] = bytev[i];
-      if ((k & 3) == 3) {
-        // the four tokens (bytes) of this lane's words are complete: word of channel slot i at lane chunk 4 i + t
-        const int cmb = (k >> 2) * RS + rs;
-        uint8_t* wbase = codes + (size_t)(cmb >> 3) * (4 * D * BITS) + mw * 512 + (cmb & 3) * 16 +
-                         4 * (2 * rh + ((cmb >> 2) & 1));
-        const int t4 = 32 * (cmb >> 3) + 16 * ((cmb >> 2) & 1) + 2 * (cmb & 3);   // token of byte 0; bytes 1..3: +8, +1, +9
-        const bool v0 = t4 >= lo && t4 < hi, v1 = t4 + 8 >= lo && t4 + 8 < hi;
-        const bool v2 = t4 + 1 >= lo && t4 + 1 < hi, v3 = t4 + 9 >= lo && t4 + 9 < hi;
-        if (v0 && v1 && v2 && v3) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            *reinterpret_cast<uint32_t*>(wbase + 64 * i) = pack_bytes(vbyte[0][i], vbyte[1][i], vbyte[2][i], vbyte[3][i]);
-        } else if (v0 || v1 || v2 || v3) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            if (v0) wbase[64 * i + 0] = (uint8_t)vbyte[0][i];
-            if (v1) wbase[64 * i + 1] = (uint8_t)vbyte[1][i];
-            if (v2) wbase[64 * i + 2] = (uint8_t)vbyte[2][i];
-            if (v3) wbase[64 * i + 3] = (uint8_t)vbyte[3][i];
-          }
-        }
-      }
-    }
-  }
-}
-
-// Minimum and maximum of the eight 16-bit values of a 16-byte piece, taken in the 16-bit type itself (two at a
-// time; exact, since every 16-bit value is an fp32 value and the order is the same).
-template <int DTYPE>
-__device__ __forceinline__ void minmax8(const uint4& r, float& mn, float& mx) {
-  if constexpr (DTYPE == KVQ_BF16) {
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&r);
-    const __nv_bfloat162 lo = __hmin2(__hmin2(h[0], h[1]), __hmin2(h[2], h[3]));
-    const __nv_bfloat162 hi = __hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3]));
-    mn = fminf(__low2float(lo), __high2float(lo));
-    mx = fmaxf(__low2float(hi), __high2float(hi));
-  } else {
-    const __half2* h = reinterpret_cast<const __half2*>(&r);
-    const __half2 lo = __hmin2(__hmin2(h[0], h[1]), __hmin2(h[2], h[3]));
-    const __half2 hi = __hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3]));
-    mn = fminf(__low2float(lo), __high2float(lo));
-    mx = fmaxf(__low2float(hi), __high2float(hi));
-  }
-}
-
-// quantize_task without rotation, four tokens per pass: the group minima / maxima of the four tokens are
-// reduced with a shuffle reduce-scatter, so that the group parameters (two divisions) are computed once per
-// group rather than once per lane, and are then broadcast to the lanes of the group.  FULLBLK: every token of
-// the task is new (no predicates).  Same results as quantize_task, bit for bit.
-template <int BITS, bool IS_V, int D, int DTYPE, bool FULLBLK>
-__device__ __forceinline__ void quantize_task_fast(const RowSrc& rsrc, int gsz, int lo,
-                                                   int hi, uint8_t* __restrict__ codes,
-                                                   uint32_t* __restrict__ meta_out, int lane) {
-  constexpr int FPB = 8 / BITS;
-  constexpr int NMW = (D / 16) / FPB;
-  constexpr int LR = 2 * NMW;
-  constexpr int RS = 32 / LR;
-  constexpr int TT = task_tokens(D, BITS);
-  constexpr int TPL = TT / RS;
-  constexpr int K_ROW_BYTES = D * BITS / 8;
-  constexpr int NSET = FPB == 4 ? 2 : 1;      // a lane's fields may belong to two groups (groups of 32 at 2 bits)
-  const int rs = lane / LR, cs = lane % LR, mw = cs >> 1, rh = cs & 1;
-  const float qmax = (float)((1 << BITS) - 1);
-  const int spg = gsz >> 4;
-  const bool split = FPB > spg;
-  const int lpg = split ? 2 : 2 * spg / FPB;                 // lanes per group: 2, 4, 8 or 16
-  const int ng = D / gsz;
-  const int b0 = cs & 1, b1 = (cs >> 1) & 1;
-  const int gbase = lane & ~(lpg - 1);                       // first lane of this lane's group
-
-  auto token_of = [&](int k) {
-    if constexpr (IS_V) {
-      const int cmb = (k >> 2) * RS + rs, j = k & 3;
-      return 32 * (cmb >> 3) + 16 * ((cmb >> 2) & 1) + 2 * (cmb & 3) + (j >> 1) + 8 * (j & 1);
-    } else {
-      return k * RS + rs;
-    }
+  auto swap = [](H2 x, int off) {
+    const uint32_t o = __shfl_xor_sync(FULL, *reinterpret_cast<uint32_t*>(&x), off);
+    return *reinterpret_cast<const H2*>(&o);
   };
 
 #pragma unroll 1
@@ -342,59 +127,38 @@ __device__ __forceinline__ void quantize_task_fast(const RowSrc& rsrc, int gsz, 
         if (valid[kk]) raw[kk][f] = __ldcs(reinterpret_cast<const uint4*>(rsrc.row(tau) + 16 * (FPB * mw + f) + 8 * rh));
       }
     }
-    // ---- phase 1: minima / maxima of the lane's fields, per token and per set
-    float mn[NSET][4], mx[NSET][4];
+    // ---- minima / maxima of the lane's fields, per token and per set
+    H2 m[NSET][4];
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
-      float fm[FPB], fx[FPB];
-#pragma unroll
-      for (int f = 0; f < FPB; ++f) minmax8<DTYPE>(raw[kk][f], fm[f], fx[f]);
-      if constexpr (FPB == 1) { mn[0][kk] = fm[0]; mx[0][kk] = fx[0]; }
-      if constexpr (FPB == 2) { mn[0][kk] = fminf(fm[0], fm[1]); mx[0][kk] = fmaxf(fx[0], fx[1]); }
+      m[0][kk] = minmax8<DTYPE>(raw[kk][0]);
+      if constexpr (FPB == 2) m[0][kk] = __hmin2(m[0][kk], minmax8<DTYPE>(raw[kk][1]));
       if constexpr (FPB == 4) {
-        mn[0][kk] = fminf(fm[0], fm[1]); mx[0][kk] = fmaxf(fx[0], fx[1]);
-        mn[1][kk] = fminf(fm[2], fm[3]); mx[1][kk] = fmaxf(fx[2], fx[3]);
-        if (!split) {
-          mn[0][kk] = mn[1][kk] = fminf(mn[0][kk], mn[1][kk]);
-          mx[0][kk] = mx[1][kk] = fmaxf(mx[0][kk], mx[1][kk]);
-        }
+        m[0][kk] = __hmin2(m[0][kk], minmax8<DTYPE>(raw[kk][1]));
+        m[1][kk] = __hmin2(minmax8<DTYPE>(raw[kk][2]), minmax8<DTYPE>(raw[kk][3]));
+        if (!split) m[0][kk] = __hmin2(m[0][kk], m[1][kk]);
       }
     }
     // ---- reduce-scatter over the lanes of the group: after lane bit 0 a lane holds tokens 2 b0 + {0, 1}, after
     // bit 1 (groups of 4 lanes or more) token 2 b0 + b1; higher bits are plain butterflies
     float pz[NSET][2], pinv[NSET][2];
-    uint32_t pmeta[NSET][2];
 #pragma unroll
     for (int e = 0; e < NSET; ++e) {
       if (e == 1 && !split) break;
-      float a0, a1, c0, c1;
-      {
-        const float sm0 = b0 ? mn[e][0] : mn[e][2], sm1 = b0 ? mn[e][1] : mn[e][3];
-        const float sx0 = b0 ? mx[e][0] : mx[e][2], sx1 = b0 ? mx[e][1] : mx[e][3];
-        a0 = fminf(b0 ? mn[e][2] : mn[e][0], __shfl_xor_sync(FULL, sm0, 1));
-        a1 = fminf(b0 ? mn[e][3] : mn[e][1], __shfl_xor_sync(FULL, sm1, 1));
-        c0 = fmaxf(b0 ? mx[e][2] : mx[e][0], __shfl_xor_sync(FULL, sx0, 1));
-        c1 = fmaxf(b0 ? mx[e][3] : mx[e][1], __shfl_xor_sync(FULL, sx1, 1));
-      }
-      if (lpg >= 4) {
-        const float sm = b1 ? a0 : a1, sx = b1 ? c0 : c1;
-        a0 = fminf(b1 ? a1 : a0, __shfl_xor_sync(FULL, sm, 2));
-        c0 = fmaxf(b1 ? c1 : c0, __shfl_xor_sync(FULL, sx, 2));
-      }
-      if (lpg >= 8) {
-        a0 = fminf(a0, __shfl_xor_sync(FULL, a0, 4));
-        c0 = fmaxf(c0, __shfl_xor_sync(FULL, c0, 4));
-      }
-      if (lpg >= 16) {
-        a0 = fminf(a0, __shfl_xor_sync(FULL, a0, 8));
-        c0 = fmaxf(c0, __shfl_xor_sync(FULL, c0, 8));
-      }
-      const GroupParams p0 = group_params(a0, c0, qmax);
-      pz[e][0] = p0.z; pinv[e][0] = p0.inv; pmeta[e][0] = p0.meta;
-      pz[e][1] = 0.f; pinv[e][1] = 0.f; pmeta[e][1] = 0u;
+      H2 a0 = __hmin2(b0 ? m[e][2] : m[e][0], swap(b0 ? m[e][0] : m[e][2], 1));
+      H2 a1 = __hmin2(b0 ? m[e][3] : m[e][1], swap(b0 ? m[e][1] : m[e][3], 1));
+      if (lpg >= 4) a0 = __hmin2(b1 ? a1 : a0, swap(b1 ? a0 : a1, 2));
+      if (lpg >= 8) a0 = __hmin2(a0, swap(a0, 4));
+      if (lpg >= 16) a0 = __hmin2(a0, swap(a0, 8));
+      uint32_t pmeta[2];
+      const float2 f0 = pair_to_f32(a0);
+      const GroupParams p0 = group_params(f0.x, -f0.y, qmax);
+      pz[e][0] = p0.z; pinv[e][0] = p0.inv * DOWN; pmeta[0] = p0.meta;
+      pz[e][1] = 0.f; pinv[e][1] = 0.f; pmeta[1] = 0u;
       if (lpg == 2) {
-        const GroupParams p1 = group_params(a1, c1, qmax);
-        pz[e][1] = p1.z; pinv[e][1] = p1.inv; pmeta[e][1] = p1.meta;
+        const float2 f1 = pair_to_f32(a1);
+        const GroupParams p1 = group_params(f1.x, -f1.y, qmax);
+        pz[e][1] = p1.z; pinv[e][1] = p1.inv * DOWN; pmeta[1] = p1.meta;
       }
       // the lane (one per group) that holds a token's parameters stores its metadata word
       if ((cs & (lpg - 1) & ~3) == 0) {
@@ -404,83 +168,201 @@ __device__ __forceinline__ void quantize_task_fast(const RowSrc& rsrc, int gsz, 
           if (i == 1 && lpg != 2) break;
           const int kk = 2 * b0 + (lpg >= 4 ? b1 : i);
           const int tau = token_of(4 * pass + kk);
-          if (FULLBLK || (tau >= lo && tau < hi)) meta_out[tau * ng + gi] = pmeta[e][i];
+          if (FULLBLK || (tau >= lo && tau < hi)) meta_out[tau * ng + gi] = pmeta[i];
         }
       }
     }
-    // ---- phase 2: codes, token by token, with the group's parameters fetched from the lane that made them
-    float vbyte[4][8];
+    // ---- the group's parameters, fetched from the lane that made them
+    float z[NSET][4], inv[NSET][4];
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
-      const int tau = token_of(4 * pass + kk);
       const int srcl = gbase + (lpg >= 4 ? (kk >> 1) + 2 * (kk & 1) : (kk >> 1));
       const int el = (lpg >= 4) ? 0 : (kk & 1);
-      float zA, iA, zB, iB;
-      zA = __shfl_sync(FULL, el ? pz[0][1] : pz[0][0], srcl);
-      iA = __shfl_sync(FULL, el ? pinv[0][1] : pinv[0][0], srcl);
-      zB = zA; iB = iA;
+      z[0][kk] = __shfl_sync(FULL, el ? pz[0][1] : pz[0][0], srcl);
+      inv[0][kk] = __shfl_sync(FULL, el ? pinv[0][1] : pinv[0][0], srcl);
       if constexpr (NSET == 2) {
+        z[1][kk] = z[0][kk]; inv[1][kk] = inv[0][kk];
         if (split) {
-          zB = __shfl_sync(FULL, el ? pz[1][1] : pz[1][0], srcl);
-          iB = __shfl_sync(FULL, el ? pinv[1][1] : pinv[1][0], srcl);
+          z[1][kk] = __shfl_sync(FULL, el ? pz[1][1] : pz[1][0], srcl);
+          inv[1][kk] = __shfl_sync(FULL, el ? pinv[1][1] : pinv[1][0], srcl);
         }
-      }
-      float bytev[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) bytev[i] = 0.f;
-#pragma unroll
-      for (int f = FPB - 1; f >= 0; --f) {
-        const float z = (FPB == 4 && f >= 2) ? zB : zA, inv = (FPB == 4 && f >= 2) ? iB : iA;
-        const uint32_t rw[4] = {raw[kk][f].x, raw[kk][f].y, raw[kk][f].z, raw[kk][f].w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          float xa, xb;
-          if constexpr (DTYPE == KVQ_BF16) {
-            xa = __uint_as_float(rw[i] << 16);
-            xb = __uint_as_float(rw[i] & 0xFFFF0000u);
-          } else {
-            const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&rw[i]));
-            xa = v.x; xb = v.y;
-          }
-          float ua = __fmul_rn(__fsub_rn(xa, z), inv), ub = __fmul_rn(__fsub_rn(xb, z), inv);
-          ua = fminf(fmaxf(ua, 0.0f), qmax);
-          ub = fminf(fmaxf(ub, 0.0f), qmax);
-          const float ra = __fsub_rn(__fadd_rn(ua, kRoundMagic), kRoundMagic);
-          const float rb = __fsub_rn(__fadd_rn(ub, kRoundMagic), kRoundMagic);
-          bytev[2 * i] = __fmaf_rn(bytev[2 * i], (float)(1 << BITS), ra);
-          bytev[2 * i + 1] = __fmaf_rn(bytev[2 * i + 1], (float)(1 << BITS), rb);
-        }
-      }
-      if constexpr (!IS_V) {
-        if (valid[kk]) {
-          constexpr int wpc = D * BITS / 128;
-#pragma unroll
-          for (int hh = 0; hh < 2; ++hh) {
-            const uint32_t w = pack_bytes(bytev[4 * hh], bytev[4 * hh + 1], bytev[4 * hh + 2], bytev[4 * hh + 3]);
-            *reinterpret_cast<uint32_t*>(codes + (size_t)tau * K_ROW_BYTES + chunk_word_byte(2 * rh + hh, mw, wpc, 4)) = w;
-          }
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) vbyte[kk][i] = bytev[i];
       }
     }
-    if constexpr (IS_V) {
+    if constexpr (!IS_V) {
+      // ---- keys: the four bytes of a word are channels 4 hh + {0..3} of this lane's 8, chunk 2 rh + hh, word mw of the row
+      constexpr int wpc = D * BITS / 128;
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        const int tau = token_of(4 * pass + kk);
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+          uint32_t w = 0;
+#pragma unroll
+          for (int f = FPB - 1; f >= 0; --f) {
+            const int e = NSET == 2 ? f >> 1 : 0;
+            float x[4], zz[4], ii[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) { x[j] = piece_value<DTYPE>(raw[kk][f], 4 * hh + j); zz[j] = z[e][kk]; ii[j] = inv[e][kk]; }
+            w = w * (1u << BITS) + code_word4<BITS>(x, zz, ii);
+          }
+          if (valid[kk])
+            *reinterpret_cast<uint32_t*>(codes + (size_t)tau * K_ROW_BYTES + chunk_word_byte(2 * rh + hh, mw, wpc, 4)) = w;
+        }
+      }
+    } else {
+      // ---- values: the four bytes of a word are this lane's four tokens; word of channel slot i at lane chunk 4 i + t
       const int cmb = pass * RS + rs;
       uint8_t* wbase = codes + (size_t)(cmb >> 3) * (4 * D * BITS) + mw * 512 + (cmb & 3) * 16 +
                        4 * (2 * rh + ((cmb >> 2) & 1));
-      if (FULLBLK || (valid[0] && valid[1] && valid[2] && valid[3])) {
+      const bool all = FULLBLK || (valid[0] && valid[1] && valid[2] && valid[3]);
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-          *reinterpret_cast<uint32_t*>(wbase + 64 * i) = pack_bytes(vbyte[0][i], vbyte[1][i], vbyte[2][i], vbyte[3][i]);
-      } else if (valid[0] || valid[1] || valid[2] || valid[3]) {
+      for (int i = 0; i < 8; ++i) {
+        uint32_t w = 0;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int f = FPB - 1; f >= 0; --f) {
+          const int e = NSET == 2 ? f >> 1 : 0;
+          float x[4];
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) x[kk] = piece_value<DTYPE>(raw[kk][f], i);
+          w = w * (1u << BITS) + code_word4<BITS>(x, z[e], inv[e]);
+        }
+        if (all) {
+          *reinterpret_cast<uint32_t*>(wbase + 64 * i) = w;
+        } else {
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
-            if (valid[kk]) wbase[64 * i + kk] = (uint8_t)vbyte[kk][i];
+            if (valid[kk]) wbase[64 * i + kk] = (uint8_t)(w >> (8 * kk));
         }
       }
+    }
+  }
+}
+
+// Rotated keys (y = H (signs * x) / sqrt(D), then token-wise groups): tokens [lo, hi) of a task, one token of a lane at a time with
+// the next one's loads in flight (bound by fetching instructions beside the value side's code; two tokens at a time were slower, 32
+// streams x 2,047 tokens 24.8 us against 24; with the signs converted for every token and lanes' own divisions 36 us).
+// Lanes and fields as in quantize_task; butterfly stages in the order h = 1, 2, 4, ...: bits of i in the lane, rh across
+// lanes, bits of f in the lane, bits of mw across lanes.
+template <int BITS, int D, int DTYPE>
+__device__ __forceinline__ void quantize_task_rotated(const RowSrc& rsrc, int gsz, int lo, int hi, uint8_t* __restrict__ codes,
+                                                      uint32_t* __restrict__ meta_out, int lane, const int8_t* __restrict__ signs) {
+  constexpr int FPB = 8 / BITS, NMW = (D / 16) / FPB, LR = 2 * NMW, RS = 32 / LR;
+  constexpr int K_ROW_BYTES = D * BITS / 8, NSET = FPB == 4 ? 2 : 1, wpc = D * BITS / 128;
+  constexpr float DOWN = 1.0f / (float)(1 << BITS);
+  const int rs = lane / LR, cs = lane % LR, mw = cs >> 1, rh = cs & 1;
+  const float qmax = (float)((1 << BITS) - 1);
+  const int spg = gsz >> 4, lpg = FPB > spg ? 2 : 2 * spg / FPB, ng = D / gsz;
+  const bool split = FPB > spg;
+  float sg[FPB][8];
+#pragma unroll
+  for (int f = 0; f < FPB; ++f) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sg[f][i] = (float)signs[16 * (FPB * mw + f) + 8 * rh + i];
+  }
+  const float srh = rh ? -1.0f : 1.0f;             // a butterfly between lanes: o + s x (the product with +-1 is exact)
+  uint4 next[FPB];
+  auto fetch = [&](int tau) {
+#pragma unroll
+    for (int f = 0; f < FPB; ++f) {
+      next[f] = make_uint4(0u, 0u, 0u, 0u);
+      if (tau < hi) next[f] = __ldcs(reinterpret_cast<const uint4*>(rsrc.row(tau) + 16 * (FPB * mw + f) + 8 * rh));
+    }
+  };
+  fetch(lo + rs);
+#pragma unroll 1
+  for (int base = lo; base < hi; base += RS) {
+    const int tau = base + rs;
+    float x[FPB][8];
+#pragma unroll
+    for (int f = 0; f < FPB; ++f) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[f][i] = __fmul_rn(piece_value<DTYPE>(next[f], i), sg[f][i]);
+    }
+    fetch(tau + RS);
+#pragma unroll
+    for (int f = 0; f < FPB; ++f) {
+#pragma unroll
+      for (int h = 1; h < 8; h <<= 1) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          if ((i & h) == 0) {
+            const float a = x[f][i], c = x[f][i + h];
+            x[f][i] = __fadd_rn(a, c);
+            x[f][i + h] = __fsub_rn(a, c);
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[f][i] = __fmaf_rn(srh, x[f][i], __shfl_xor_sync(FULL, x[f][i], 1));
+    }
+#pragma unroll
+    for (int hf = 1; hf < FPB; hf <<= 1) {
+#pragma unroll
+      for (int f = 0; f < FPB; ++f) {
+        if ((f & hf) == 0) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const float a = x[f][i], c = x[f + hf][i];
+            x[f][i] = __fadd_rn(a, c);
+            x[f + hf][i] = __fsub_rn(a, c);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int hm = 1; hm < NMW; hm <<= 1) {
+      const float sm = (mw & hm) ? -1.0f : 1.0f;
+#pragma unroll
+      for (int f = 0; f < FPB; ++f) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[f][i] = __fmaf_rn(sm, x[f][i], __shfl_xor_sync(FULL, x[f][i], 2 * hm));
+      }
+    }
+    float mn[NSET], mx[NSET];
+#pragma unroll
+    for (int e = 0; e < NSET; ++e) { mn[e] = INFINITY; mx[e] = -INFINITY; }
+#pragma unroll
+    for (int f = 0; f < FPB; ++f) {
+      const int e = NSET == 2 ? f >> 1 : 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        x[f][i] = __fmul_rn(x[f][i], inv_sqrt_dim<D>());
+        mn[e] = fminf(mn[e], x[f][i]);
+        mx[e] = fmaxf(mx[e], x[f][i]);
+      }
+    }
+    if constexpr (NSET == 2) {
+      if (!split) {
+        mn[0] = mn[1] = fminf(mn[0], mn[1]);
+        mx[0] = mx[1] = fmaxf(mx[0], mx[1]);
+      }
+    }
+    float z[NSET], inv[NSET];
+#pragma unroll
+    for (int e = 0; e < NSET; ++e) {
+#pragma unroll
+      for (int off = 1; off < LR; off <<= 1) {
+        const float oa = __shfl_xor_sync(FULL, mn[e], off), oc = __shfl_xor_sync(FULL, mx[e], off);
+        if (off < lpg) { mn[e] = fminf(mn[e], oa); mx[e] = fmaxf(mx[e], oc); }
+      }
+      const GroupParams p = group_params(mn[e], mx[e], qmax);
+      z[e] = p.z;
+      inv[e] = p.inv * DOWN;
+      if (tau < hi && (cs & (lpg - 1)) == 0 && (e == 0 || split)) meta_out[tau * ng + (16 * FPB * mw) / gsz + e] = p.meta;
+    }
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+      uint32_t w = 0;
+#pragma unroll
+      for (int f = FPB - 1; f >= 0; --f) {
+        const int e = NSET == 2 ? f >> 1 : 0;
+        float v[4], zz[4], ii[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { v[j] = x[f][4 * hh + j]; zz[j] = z[e]; ii[j] = inv[e]; }
+        w = w * (1u << BITS) + code_word4<BITS>(v, zz, ii);
+      }
+      if (tau < hi)
+        *reinterpret_cast<uint32_t*>(codes + (size_t)tau * K_ROW_BYTES + chunk_word_byte(2 * rh + hh, mw, wpc, 4)) = w;
     }
   }
 }
@@ -554,7 +436,7 @@ __device__ __forceinline__ void copy_task_side(const RowSrc& rsrc, int D, int lo
 // Token-wise quantization of V (blockIdx.z == 0) and of K (blockIdx.z == 1).  grid.y = stream, grid.x strides
 // over the warp tasks touched by this append.
 template <int D, int DTYPE, bool ROT>
-__global__ void __launch_bounds__(kThreads, ROT ? 1 : 3)
+__global__ void __launch_bounds__(kThreads, ROT ? 4 : 5)
 quant_token_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
                    int64_t sb, int64_t sh, int64_t st, int t_new) {
   const bool is_v = blockIdx.z == 0;
@@ -601,14 +483,14 @@ quant_token_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, cons
       uint32_t* vm = reinterpret_cast<uint32_t*>(pg + g.v_meta_off) + tp0 * (D / gsz);
       const bool full = lo == 0 && hi == TT;
       if (bits == 2) {
-        if (full) quantize_task_fast<2, true, D, DTYPE, true>(rs, gsz, lo, hi, vb, vm, lane);
-        else quantize_task_fast<2, true, D, DTYPE, false>(rs, gsz, lo, hi, vb, vm, lane);
+        if (full) quantize_task<2, true, D, DTYPE, true>(rs, gsz, lo, hi, vb, vm, lane);
+        else quantize_task<2, true, D, DTYPE, false>(rs, gsz, lo, hi, vb, vm, lane);
       } else if (bits == 4) {
-        if (full) quantize_task_fast<4, true, D, DTYPE, true>(rs, gsz, lo, hi, vb, vm, lane);
-        else quantize_task_fast<4, true, D, DTYPE, false>(rs, gsz, lo, hi, vb, vm, lane);
+        if (full) quantize_task<4, true, D, DTYPE, true>(rs, gsz, lo, hi, vb, vm, lane);
+        else quantize_task<4, true, D, DTYPE, false>(rs, gsz, lo, hi, vb, vm, lane);
       } else {
-        if (full) quantize_task_fast<8, true, D, DTYPE, true>(rs, gsz, lo, hi, vb, vm, lane);
-        else quantize_task_fast<8, true, D, DTYPE, false>(rs, gsz, lo, hi, vb, vm, lane);
+        if (full) quantize_task<8, true, D, DTYPE, true>(rs, gsz, lo, hi, vb, vm, lane);
+        else quantize_task<8, true, D, DTYPE, false>(rs, gsz, lo, hi, vb, vm, lane);
       }
     } else {
       if (bits == 16) {
@@ -623,20 +505,20 @@ quant_token_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, cons
       uint8_t* kr = pg + (size_t)tp0 * (D * bits / 8);
       uint32_t* km = reinterpret_cast<uint32_t*>(pg + g.k_meta_off) + tp0 * (D / gsz);
       if constexpr (ROT) {
-        if (bits == 2) quantize_task<2, false, D, DTYPE, true>(rs, gsz, lo, hi, kr, km, lane, c.k_signs);
-        else if (bits == 4) quantize_task<4, false, D, DTYPE, true>(rs, gsz, lo, hi, kr, km, lane, c.k_signs);
-        else quantize_task<8, false, D, DTYPE, true>(rs, gsz, lo, hi, kr, km, lane, c.k_signs);
+        if (bits == 2) quantize_task_rotated<2, D, DTYPE>(rs, gsz, lo, hi, kr, km, lane, c.k_signs);
+        else if (bits == 4) quantize_task_rotated<4, D, DTYPE>(rs, gsz, lo, hi, kr, km, lane, c.k_signs);
+        else quantize_task_rotated<8, D, DTYPE>(rs, gsz, lo, hi, kr, km, lane, c.k_signs);
       } else {
         const bool full = lo == 0 && hi == TT;
         if (bits == 2) {
-          if (full) quantize_task_fast<2, false, D, DTYPE, true>(rs, gsz, lo, hi, kr, km, lane);
-          else quantize_task_fast<2, false, D, DTYPE, false>(rs, gsz, lo, hi, kr, km, lane);
+          if (full) quantize_task<2, false, D, DTYPE, true>(rs, gsz, lo, hi, kr, km, lane);
+          else quantize_task<2, false, D, DTYPE, false>(rs, gsz, lo, hi, kr, km, lane);
         } else if (bits == 4) {
-          if (full) quantize_task_fast<4, false, D, DTYPE, true>(rs, gsz, lo, hi, kr, km, lane);
-          else quantize_task_fast<4, false, D, DTYPE, false>(rs, gsz, lo, hi, kr, km, lane);
+          if (full) quantize_task<4, false, D, DTYPE, true>(rs, gsz, lo, hi, kr, km, lane);
+          else quantize_task<4, false, D, DTYPE, false>(rs, gsz, lo, hi, kr, km, lane);
         } else {
-          if (full) quantize_task_fast<8, false, D, DTYPE, true>(rs, gsz, lo, hi, kr, km, lane);
-          else quantize_task_fast<8, false, D, DTYPE, false>(rs, gsz, lo, hi, kr, km, lane);
+          if (full) quantize_task<8, false, D, DTYPE, true>(rs, gsz, lo, hi, kr, km, lane);
+          else quantize_task<8, false, D, DTYPE, false>(rs, gsz, lo, hi, kr, km, lane);
         }
       }
     }

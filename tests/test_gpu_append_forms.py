@@ -82,3 +82,15 @@ def test_few_tokens_beyond_the_capacity(kvq):
     kvq.kvq_quantize_append(cfg, gc, k[:, :, :2].cuda(), v[:, :, :2].cuda())
     assert gc.seq_len.tolist() == [255, 130] and torch.equal(gc.pages_view()[0], before)
     assert kvq.kvq_check_status(gc) == -5
+
+
+RUNS = {"odd": [131, 70, 259], "exact": [256, 160], "inside": [200, 65, 66]}       # whole, partial and interior 32-token tasks
+
+
+@pytest.mark.parametrize("kb,vb", [(2, 8), (4, 2), (8, 4)])
+@pytest.mark.parametrize("D,gk,gv", [(128, 128, 32), (128, 32, 128), (128, 64, 64), (64, 64, 32), (64, 32, 64)])
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+@pytest.mark.parametrize("runs,form", [("odd", "plain"), ("exact", "plain"), ("odd", "rotated"), ("inside", "rotated window")])
+def test_runs_of_tokens(kvq, kb, vb, D, gk, gv, dtype, runs, form):
+    w = wl.LLAMA_8B.with_(n_kv_heads=2, n_q_heads=2, head_dim=D, kb=kb, vb=vb, gk=gk, gv=gv, dtype=dtype)
+    check(kvq, w, 2, RUNS[runs], SIGNS[:D] if "rotated" in form else None, 64 if "window" in form else 0, strided=runs == "odd")
