@@ -8,8 +8,8 @@ namespace kvq {
 namespace mma {
 
 // Instantiation units (kvq_decode_mma_inst_*.cu).
-#define KVQ_MMA_DECL(D, KB, VB, KAXIS, NGK, NGV, NH, NW, MINB)                                                  \
-  extern template int launch_mma_inst<D, KB, VB, KAXIS, NGK, NGV, NH, NW, MINB>(                                   \
+#define KVQ_MMA_DECL(D, KB, VB, KAXIS, NGK, NGV, NH, MINB)                                                  \
+  extern template int launch_mma_inst<D, KB, VB, KAXIS, NGK, NGV, NH, MINB>(                                   \
       const Geom&, const CachePtrs&, const void*, float, float*, int, void*, int, unsigned long long,              \
       unsigned long long, long long, cudaStream_t);
 #include "kvq_decode_mma_list.inc"
@@ -48,12 +48,12 @@ static int pick(const Geom& g, const CachePtrs& c, const void* q, float c1, floa
   const int ngk = (g.k_axis == 1 || g.kb == 16) ? 1 : g.D / g.gk;
   const int ngv = (g.vb == 16) ? 1 : g.D / g.gv;
   const int nh = g.G * g.rows <= 4 ? 1 : 2;                                // (virtual) query heads per lane
-#define KVQ_MMA_DECL(D_, KB_, VB_, KAXIS_, NGK_, NGV_, NH_, NW_, MINB_)                                      \
+#define KVQ_MMA_DECL(D_, KB_, VB_, KAXIS_, NGK_, NGV_, NH_, MINB_)                                      \
   if (g.D == D_ && g.kb == KB_ && g.vb == VB_ && g.k_axis == KAXIS_ && ngk == NGK_ && ngv == NGV_ &&          \
       NH_ == nh) {                                                                                            \
     *grid = 148 * MINB_;                                                                                      \
     if (probe) return KVQ_OK;                                                                                 \
-    return mma::launch_mma_inst<D_, KB_, VB_, KAXIS_, NGK_, NGV_, NH_, NW_, MINB_>(                          \
+    return mma::launch_mma_inst<D_, KB_, VB_, KAXIS_, NGK_, NGV_, NH_, MINB_>(                          \
         g, c, q, c1, ws, s_cap, out, out_dtype, next_call_id(),                                               \
         dbg.wait_us ? 1000ull * dbg.wait_us : mma::kWaitTimeoutNs, dbg.skip_page, stream);                    \
   }

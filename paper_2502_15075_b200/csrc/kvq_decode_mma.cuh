@@ -6,13 +6,13 @@
 //  * the producer streams whole 128-token pages into a four-stage shared-memory ring
 //    with cp.async.bulk (one bulk copy per page with an L2 evict-first policy,
 //    completion on an mbarrier);
-//  * each consumer warp owns one 32-token block of every page and loads its operand
-//    fragments with 16-byte shared loads (the page layout already is fragment order);
+//  * each consumer warp owns one 32-token block of every page for the logits and softmax weights, and a quarter of the
+//    channels for PV; the weights change hands through shared memory as MMA operands; fragments are 16-byte shared loads
+//    (the page layout already is fragment order);
 //  * both contractions are integer tensor-core MMAs on the raw code bytes
 //    (mma.m16n8k32, int32 accumulate; one mask per operand register): q enters as 16-bit
 //    fixed point in two signed bytes (channel-wise keys: q*s per page in three), the softmax
-//    weight times the value scale as 31-bit fixed point in four unsigned bytes (24 bits in
-//    three for 8 heads); the 8 MMA columns carry (head, limb) pairs;
+//    weight times the value scale as 32-bit fixed point in four unsigned bytes; the 8 MMA columns carry (head, limb) pairs;
 //  * scale and zero-point never touch the codes:  q.K^_t = s_t (q.c_t) + z_t sum(q)
 //    and  o = sum_t (p_t s_t) c_t + sum_t p_t z_t ;
 //  * the sequence is split flat over the grid: CTA i takes the i-th share of all pages

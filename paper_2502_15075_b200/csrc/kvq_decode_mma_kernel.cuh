@@ -8,25 +8,27 @@
 namespace kvq {
 namespace mma {
 
-// Shared-memory carve-up (dynamic): ring | barriers | prefix | misc | per-warp fp32 masters | (m, l) | channel-wise scratch
+// Shared-memory carve-up (dynamic): ring | barriers | prefix | misc | weights | reductions | channel-wise scratch
 struct SmemLayout {
-  int page_stride, ring_bytes, bar_off, pref_off, misc_off, master_off, ml_off, chan_off, total;
+  int page_stride, ring_bytes, bar_off, pref_off, misc_off, w_off, red_off, chan_off, total;
 };
-// master: per consumer warp, 4 NH heads x (D + 8) floats (the row padding keeps a warp's accesses conflict-free).
+// weights: the PV operands of a page as the owners of its four 32-token blocks leave them, per value group and block
+// (16 NH bytes per lane), for two pages in turn.
 // chan: channel-wise keys keep, per ring stage, the page's q operands made by the preparation warp
 // (NH x 2 x D/16 x 32 words) followed by 8 zero-point sums and 8 fixed-point scales (one per head).
+__host__ __device__ constexpr int weight_block_bytes(int nh) { return 512 * nh; }
+__host__ __device__ constexpr int reduction_bytes(int ngv) { return 4 * (8 * ngv * 8 + (8 + 4 + 8) * 4); }   // per warp: p z sums (64 bits), maxima, scale limit, l
 __host__ __device__ inline int chan_stage_bytes(int D, int nh) { return nh * 2 * (D / 16) * 32 * 4 + 64; }
-__host__ __device__ inline SmemLayout smem_layout(int page_bytes, int stages, int nw, int batch, int D, int nh,
-                                                  bool chan) {
+__host__ __device__ inline SmemLayout smem_layout(int page_bytes, int stages, int batch, int D, int nh, int ngv, bool chan) {
   SmemLayout s;
   s.page_stride = (page_bytes + 127) & ~127;
   s.ring_bytes = s.page_stride * stages;
   s.bar_off = s.ring_bytes;
   s.pref_off = s.bar_off + 16 * 8 * 2;                      // up to 32 barriers: (full, empty[, ready]) per stage
   s.misc_off = (s.pref_off + 2 * (batch + 1) * 4 + 15) & ~15;      // two prefixes: pages, and pages + stream gaps
-  s.master_off = s.misc_off + 64;
-  s.ml_off = s.master_off + nw * 4 * nh * (D + 8) * 4;
-  s.chan_off = s.ml_off + nw * 4 * nh * 2 * 4;
+  s.w_off = s.misc_off + 64;
+  s.red_off = s.w_off + 2 * ngv * 4 * weight_block_bytes(nh);
+  s.chan_off = s.red_off + reduction_bytes(ngv);
   s.total = s.chan_off + (chan ? stages * chan_stage_bytes(D, nh) : 0);
   return s;
 }
@@ -45,6 +47,34 @@ __device__ __forceinline__ void mma16832_u8u8(int (&d)[4], uint32_t a0, uint32_t
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// The same with a zero accumulator: D = A B.
+__device__ __forceinline__ void mma16832_u8u8_zero(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                                   uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k32.row.col.s32.u8.u8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(0));
+}
+__device__ __forceinline__ void mma16832_u8s8_zero(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                                   uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(0));
+}
+__device__ __forceinline__ void mbar_arrive_if(uint32_t bar, bool p) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"((uint32_t)p) : "memory");
+}
+// Barrier of `nthreads` threads that also says whether any of them came with p.
+__device__ __forceinline__ bool named_bar_any(int id, int nthreads, bool p) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.or.pred q, %2, %3, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r) : "r"((uint32_t)p), "r"(id), "r"(nthreads) : "memory");
+  return r != 0;
+}
+
 // Four values times `scale` rounded to integers |Q| <= 32512 and split into two balanced signed bytes,
 // Q = hi * 256 + lo; returns the four hi bytes (lo_limb = 0) or the four lo bytes (lo_limb = 1) as one word
 // and adds the four Q to `qsum`.
@@ -61,20 +91,14 @@ __device__ __forceinline__ uint32_t fixed_point_limb(const float (&t)[4], float 
   return w;
 }
 
-// The split balances time, not pages.  Ending one stream and starting the next (fold and combine the warps'
-// state, store and publish the partial, perhaps merge; load and convert the next queries) costs a CTA as much as
-// ~9 pages (8.4 us on the 8B-shaped layer: CTAs whose share crosses a stream boundary ended at 81.2 us, the others
-// at 72.8 us), and of the three CTAs that share an SM the hardware favours the older ones (launch waves ended at
-// 68.9 / 72.7 / 76.8 us with equal work).  So every stream is given kGapPages virtual pages in front of its real
-// ones and the shares of the launch waves are weighted; the split is taken on that virtual axis.
-#ifndef KVQ_GAP_PAGES
-#define KVQ_GAP_PAGES 10
-#endif
-#ifndef KVQ_WAVE_W0
-#define KVQ_WAVE_W0 1040
-#endif
-constexpr int kGapPages = KVQ_GAP_PAGES;
-constexpr int kWaveWeight0 = KVQ_WAVE_W0;  // share of a first-wave CTA in thousandths of the mean (third wave: 2000 - this)
+// The split balances time, not pages.  Ending one stream and starting the next costs a CTA about as much as six to eight pages
+// (load and convert the next queries, publish a partial, perhaps merge), so every stream is given kGapPages virtual pages in front
+// of its real ones and the split is taken on that virtual axis; with many CTAs per stream the gap also keeps shares from
+// crossing into the next stream for a page or two (40 ragged streams of 36 to 70 K4V4 pages: gap 8 16.5 us, 6 19.8, 0 28).
+// Channel-wise keys, whose pages take longer: gap 2 (ragged 14B shape 119 us; 10: 131 us).  Of the CTAs that
+// share an SM the hardware favours the older ones (0.85 / 0.91 / 0.99 us per page at three per SM, 0.96 / 1.01 at two),
+// so the launch waves are weighted (8B shape K4V2: 1040 76.1 us, 1080 77.3, equal 80.4).
+constexpr int kGapPages = 8, kGapPagesChan = 2;
 constexpr float kQFix = 32512.0f;          // largest |Q| of the 16-bit fixed-point q (hi limb stays within +-127)
 constexpr float kQFix3 = 8300000.0f;       // ... of the 24-bit fixed-point q * s of channel-wise keys (three limbs)
 
@@ -95,11 +119,12 @@ __device__ __forceinline__ void fixed_point_bytes3(const float (&t)[4], float sc
 }
 // The softmax weights enter PV as fixed point P = rint(p * s_V * 2^PBITS / s_lim), p = 2^(logit - reference) with the
 // reference kHeadroom bits above the largest logit seen so far, so that a larger logit rarely forces a rescale.
-// Tokens whose P falls below one unit vanish, so the width matters over long contexts: four byte limbs (31 bits)
-// where one lane serves one head, three (24 bits, less headroom) where it serves two.
-template <int NH> constexpr int kPBits = NH == 1 ? 31 : 24;
-template <int NH> constexpr float kHeadroom = NH == 1 ? 6.0f : 1.0f;
-constexpr int kFlushBlocks = 512;          // fold the int32 value accumulators at least this often (no overflow)
+// Tokens whose P falls below one unit vanish, so the width matters over long contexts: four byte limbs, all 32 bits of them.  The
+// reference is common to the CTA's four warps, so headroom is kept to four bits: a unit is 2^-28 of the largest weight (heavy-tailed
+// channel-wise keys, 64-bit comparison: 31 bits and 6 of headroom 2.1e-5, against 6.7e-6 with a reference per warp).
+constexpr int kPBits = 32;
+constexpr float kHeadroom = 4.0f;
+constexpr int kFlushPages = 128;           // fold the int32 value accumulators at least this often: 128 x 128 tokens x 255 x 255 < 2^31
 
 // The query values a lane needs as MMA operand: head hb (a (row, head) pair when several rows are served), channels
 // 16 r + 4 tid + {0..3} for every slot r, in fp32, rotated like the keys if the cache rotates them; heads >= G are
@@ -170,12 +195,9 @@ __device__ __forceinline__ float load_q_lane(const Geom& g, const CachePtrs& c, 
 
 // Weighted position of a CTA on the virtual axis in units of 1 / (148 * 1000 * waves) of the whole: two or three launch
 // waves of 148 CTAs (one per CTA that an SM holds) with weights W0, [1000,] 2000 - W0.
-#ifndef KVQ_WAVE2_W0
-#define KVQ_WAVE2_W0 1000   /* two CTAs per SM: weighting the waves did not pay (70B-shaped layer: 147.8 us equal, 149.9 us at 1040, 154.1 us at 1080) */
-#endif
 template <int WAVES> struct WaveWeights;
-template <> struct WaveWeights<3> { static constexpr int w[3] = {kWaveWeight0, 1000, 2000 - kWaveWeight0}; };
-template <> struct WaveWeights<2> { static constexpr int w[3] = {KVQ_WAVE2_W0, 2000 - KVQ_WAVE2_W0, 0}; };
+template <> struct WaveWeights<3> { static constexpr int w[3] = {1040, 1000, 960}; };
+template <> struct WaveWeights<2> { static constexpr int w[3] = {1010, 990, 0}; };
 template <int WAVES>
 __device__ __forceinline__ long long wave_prefix(int cta) {
   constexpr int W0 = WaveWeights<WAVES>::w[0], W1 = WaveWeights<WAVES>::w[1], W2 = WaveWeights<WAVES>::w[2];
@@ -218,29 +240,41 @@ static __device__ __forceinline__ long long share_start(const FlatPlan& plan, bo
 }
 
 // Template parameters: head_dim, key bits, value bits, key axis (0 token-wise, 1 channel-wise), key / value groups
-// per row, NH = query heads per lane (1: up to 4 heads per KV head, 2: up to 8), consumer warps (4: one per
-// 32-token block of a page), resident CTAs per SM.
+// per row, NH = query heads per lane (1: up to 4 heads per KV head, 2: up to 8), resident CTAs per SM.
 //
 // Both contractions run on integer tensor-core MMAs over the raw code bytes (m16n8k32, int32 accumulate).
 // The 8 columns of an MMA carry (head, limb) pairs: q as 16-bit fixed point in two signed bytes for QK^T, the
-// softmax weight times the value scale as 31-bit (NH = 2: 24-bit) fixed point in unsigned bytes for PV.  Lane (g, t) of a
+// softmax weight times the value scale as 32-bit fixed point in four unsigned bytes for PV.  Lane (g, t) of a
 // warp (g = lane / 4, t = lane % 4) owns query heads t (and t + 4 when NH = 2): its accumulator columns 2t, 2t+1
 // are the limbs of that head, so logits, softmax and the fixed-point weights need no exchange between lanes.
-template <int D, int KB, int VB, int KAXIS, int NGK, int NGV, int NH, int NW, int MINB>
-__global__ void __launch_bounds__((NW + 1 + (KAXIS == 1 ? 1 : 0)) * 32, MINB)
+//
+// The four consumer warps share a page twice: for logits and weights each takes 32 of its tokens, for PV each takes a quarter of the
+// channels of all 128.  In between the weights pass through shared memory as ready MMA operands, behind the page's one
+// barrier, which also says whether any warp saw a logit above the common reference (or a value scale above the common
+// limit; then all move it and make their weights again).  A warp's accumulators are a quarter of what whole rows per warp take
+// (32 registers for 8 heads, where 24-bit weights alone took 96 and spilled): 8 heads have 32-bit weights and four bits of
+// headroom too, channel-wise keys three CTAs per SM instead of two, and a stream's end needs no sum over the warps but two scalars per head.
+// Bound by the length of the instruction stream: a warp issues every 6 to 7 cycles, so what counts is instructions per page.  A page
+// without masks (all but a stream's last) runs code without a condition.  Against whole rows per warp, one layer:
+// 8B K4V2 81.2 -> 76.8 us, K2V4 85 -> 79, K4V4 93 -> 90, K8V4 131 -> 127; 8 heads per KV head (70B shape) 152 -> 120; channel-wise
+// 14B K4V2 182 -> 153, K8V2 192 -> 161; groups of 32 / 64 59 / 60 -> 52 / 51; 4 x 8 streams of 4,000 tokens 22.8 -> 17.5.
+constexpr int kConsumerWarps = 4;
+template <int D, int KB, int VB, int KAXIS, int NGK, int NGV, int NH, int MINB>
+__global__ void __launch_bounds__((kConsumerWarps + 1 + (KAXIS == 1 ? 1 : 0)) * 32, MINB)
 decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1, float* __restrict__ ws,
                   int s_cap, int stages, void* __restrict__ out, int out_dtype, unsigned long long call_id,
                   unsigned long long wait_ns, long long skip_x) {
+  constexpr int NW = kConsumerWarps;
   constexpr int NR = D / 16;                // 16-channel register slots per key row
   constexpr int KS32 = D / 32;              // k-steps of an 8-bit MMA over the channels
   constexpr int MT = D / 16;                // m-tiles of PV (16 channels each)
+  constexpr int MTW = MT / NW;              // ... of one warp
   constexpr int KW = D * KB / 128;          // key words per lane per token row
   constexpr int FPBV = 8 / VB;              // value codes per byte (channels 16 apart)
-  constexpr int VQ = MT / FPBV;             // quads of value words per lane per 32-token block
-  constexpr int NTV = NH == 1 ? 2 : 3;      // n-tiles of PV: (head, limb) columns
+  constexpr int QPW = MTW > FPBV ? MTW / FPBV : 1;   // quads of value words per lane, warp and 32-token block
+  constexpr int TPQ = MTW / QPW;            // m-tiles of the warp in a quad
+  constexpr int NTV = 2 * NH;               // n-tiles of PV: (head, limb) columns, four limbs
   constexpr int NTK = KAXIS == 1 ? 2 : 1;   // n-tiles of QK^T per head set: two byte limbs of q, or three of q * s
-  constexpr int NHEADS = 4 * NH;
-  constexpr int MSTRIDE = D + 8;
   constexpr int K_ROW_BYTES = D * KB / 8;
   constexpr int V_BLOCK_BYTES = 4 * D * VB;
   // page geometry (the same numbers the host put into Geom)
@@ -248,27 +282,27 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   constexpr int V_CODES_OFF = K_META_OFF + (KAXIS == 1 ? 4 * D : kPageTokens * NGK * 4);
   constexpr int V_META_OFF = V_CODES_OFF + 4 * V_BLOCK_BYTES;
   constexpr int NCONS = NW * 32;
-  constexpr int NG = NW / 4;                // groups of four consumer warps; a group takes every NG-th page
   constexpr uint32_t FULL = 0xffffffffu;
-  // The time-balanced split (stream gaps, wave weights) pays where the arithmetic per page limits the kernel
-  // (token-wise and channel-wise keys alike: 14B-shaped channel-wise K4V2 188 -> 184 us); pages of 10 bits per
-  // element pair and more lose with it (channel-wise K8V2 193 -> 197 us) and keep the plain split by pages.
-  constexpr int GAP = (KB + VB <= 8) ? kGapPages : 0;
-  constexpr int WAVES = MINB == 2 ? 2 : 3;          // CTAs per SM = launch waves (the weights apply to a grid of 148 * WAVES)
-  static_assert(NW % 4 == 0, "four consumer warps per page, one per 32-token block");
+  // The time-balanced split (stream gaps) pays where the arithmetic per page limits the kernel (token-wise and
+  // channel-wise keys alike); pages of 10 bits per element pair and more lose with it and keep the plain split by pages.
+  constexpr int GAP = (KB + VB <= 8) ? (KAXIS == 1 ? kGapPagesChan : kGapPages) : 0;
+  constexpr int WAVES = MINB;               // CTAs per SM = launch waves (the weights apply to a grid of 148 * WAVES)
+  static_assert(MT % NW == 0 && (MT / NGV) % MTW == 0, "a warp's channels are whole m-tiles of one value group");
   static_assert(KAXIS == 0 || KB != 2, "channel-wise 2-bit keys are not instantiated");
   static_assert(MT % FPBV == 0, "value m-tiles come in groups that share a byte");
 
   extern __shared__ __align__(128) uint8_t smem[];
-  const SmemLayout sl = smem_layout(g.page_bytes, stages, NW, g.B, D, NH, KAXIS == 1);
+  const SmemLayout sl = smem_layout(g.page_bytes, stages, g.B, D, NH, NGV, KAXIS == 1);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + sl.bar_off);   // full[0..stages), empty[0..stages)
   int* sPref = reinterpret_cast<int*>(smem + sl.pref_off);
   int* sVPref = sPref + (g.B + 1);                                   // the same prefix with kGapPages more per stream
   int* sMisc = reinterpret_cast<int*>(smem + sl.misc_off);           // [0] pages_max, [1] abort flag, [2] published count, [4..7] share ends, [8..9] segment slot / partials, [10..13] CTAs taking part, cursor
-  float* sMaster = reinterpret_cast<float*>(smem + sl.master_off);   // [NW][NHEADS][MSTRIDE]
-  float* sML = reinterpret_cast<float*>(smem + sl.ml_off);           // [NW][NHEADS][2] = (reference, l)
+  double* sZ = reinterpret_cast<double*>(smem + sl.red_off);         // [NW][8][NGV] sums of weight x zero-point
+  float* sMax = reinterpret_cast<float*>(sZ + NW * 8 * NGV);         // [NW][8] block maxima
+  float* sLim = sMax + NW * 8;                                       // [NW][4] value scales (one used)
+  float* sSum = sLim + NW * 4;                                       // [NW][8] sums of weights
 
-  const int tid_ = threadIdx.x, lane = tid_ & 31, warp = tid_ >> 5;
+  const int tid_ = threadIdx.x, lane = tid_ & 31, warp = __shfl_sync(FULL, tid_ >> 5, 0);     // (known to be the same in a warp)
   const int gid = lane >> 2, tid = lane & 3;
   // Several query rows per head (g.rows > 1) are served as virtual heads: row r of head j is virtual head
   // r * Gq + j, with its own causal limit on the tokens it may see.
@@ -514,58 +548,62 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   float hs[NH];                // c1 / fixed-point scale of q, own heads (tid + 4 nh)
   float qsum[NH][NGK];         // c1 * sum of q over each key group, own heads
   float zq[NH];                // channel-wise keys: c1 * sum_d q_d z_d of the current page, own heads
-  float m_ref[NH], l[NH], zacc[NH][NGV];
-  int Oi[NTV][MT][4];          // PV accumulators: NH = 1: n-tiles (limb 3, 2 | limb 1, 0) of head tid; NH = 2: (head tid:
-                               // limb 2, 1 | head tid + 4: limb 2, 1 | limb 0 of both)
-  constexpr float PONE = (float)(1u << (kPBits<NH> - 1)) * 2.0f;     // 2^PBITS
+  float m_ref[NH], l[NH], zacc[NH][NGV];     // reference: the same in all warps; sums: over this warp's tokens
+  int Oi[NTV][MTW][4];         // PV accumulators: n-tiles 2 nh, 2 nh + 1 hold limbs (3, 2) and (1, 0) of head tid + 4 nh
+  double acc[NH][MTW][2];      // what has been folded out of them: channel 16 (MTW warp + i) + 8 r + gid
+  constexpr float PONE = (float)(1u << (kPBits - 1)) * 2.0f;     // 2^PBITS
   // sscale = 2^PBITS / s_lim, s_lim a power of two above every value scale folded into the weights so far (2^-40 at first)
   float sscale = PONE / 9.094947e-13f;
-  float* myM = sMaster + warp * NHEADS * MSTRIDE;
-  const int grp = warp >> 2, wq = warp & 3;       // page group of this warp, and its 32-token block inside a page
-  int page_no = 0;
-  int stage = grp;             // ring slot and parity of this group's next page (pages go to the groups in turn)
+  int page_no = 0, stage = 0;
   uint32_t phase = 0;
-  int turn = 0;                // CTA-wide page counter modulo NG
   bool aborted = false;
   constexpr int KCB = (KW < 4 ? KW : 4) * 4;     // bytes of a lane chunk's first quad of key words
-  const int lane_k = (wq * 32 + gid) * K_ROW_BYTES + tid * KCB;
-  const int lane_km = K_META_OFF + (wq * 32 + gid) * 4 * NGK;
-  const int lane_v = V_CODES_OFF + wq * V_BLOCK_BYTES + lane * 16;
-  const int lane_vm = V_META_OFF + (wq * 32 + gid) * 4 * NGV;
+  const int lane_k = (warp * 32 + gid) * K_ROW_BYTES + tid * KCB;
+  const int lane_km = K_META_OFF + (warp * 32 + gid) * 4 * NGK;
+  const int lane_vm = V_META_OFF + (warp * 32 + gid) * 4 * NGV;
+  const int mt0 = MTW * warp;                    // first m-tile of this warp, its field of a value byte, its value group
+  const int f0 = mt0 % FPBV, jw = mt0 / (MT / NGV);
+  const int lane_v = V_CODES_OFF + (mt0 / FPBV) * 512 + lane * 16;
+  constexpr int WB = weight_block_bytes(NH);
 
-  // Fold the int32 accumulators into the warp's fp32 master (each (head, channel) belongs to one lane) and clear them.
+  // A page that is not there yet (the whole warp comes here): wait for it, bounded; on expiry set the status and go on without waiting (the barriers keep their
+  // protocol, what is computed no longer matters and reads nothing out of range).
+  auto wait_slowly = [&](uint32_t bar) {
+    if (aborted) return;
+    const bool got = mbar_wait_slow(bar, phase, wait_ns);
+    if (!__all_sync(FULL, got)) {
+      aborted = true;
+      *abort_flag = 1;
+      if (lane == 0) atomicOr(c.status, KVQ_STATUS_DEVICE_TIMEOUT);
+    }
+  };
+  // Fold the int32 accumulators into 64-bit sums and clear them (the sum of code terms and the sum of zero-points that meets it at
+  // the segment's end are each up to a few hundred times their difference).
   auto flush_acc = [&]() {
 #pragma unroll
-    for (int mt = 0; mt < MT; ++mt) {
-      const float fw = (1.0f / sscale) / (float)(1 << (VB * (mt % FPBV)));      // sscale is a power of two
+    for (int i = 0; i < MTW; ++i) {
+      const double fw = (double)((1.0f / sscale) / (float)(1 << (VB * ((f0 + i) % FPBV))));      // sscale is a power of two
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-        const int d = 16 * mt + 8 * r + gid;
-        if constexpr (NH == 1) {
-          const float v = fmaf((float)Oi[0][mt][2 * r], 16777216.f,
-                               fmaf((float)Oi[0][mt][2 * r + 1], 65536.f,
-                                    fmaf((float)Oi[1][mt][2 * r], 256.f, (float)Oi[1][mt][2 * r + 1])));
-          myM[tid * MSTRIDE + d] += v * fw;
-        } else {
-          const float v0 = fmaf((float)Oi[0][mt][2 * r], 65536.f, fmaf((float)Oi[0][mt][2 * r + 1], 256.f,
-                                                                        (float)Oi[2][mt][2 * r]));
-          const float v1 = fmaf((float)Oi[1][mt][2 * r], 65536.f, fmaf((float)Oi[1][mt][2 * r + 1], 256.f,
-                                                                        (float)Oi[2][mt][2 * r + 1]));
-          myM[tid * MSTRIDE + d] += v0 * fw;
-          myM[(tid + 4) * MSTRIDE + d] += v1 * fw;
+#pragma unroll
+        for (int nh = 0; nh < NH; ++nh) {
+          const long long v = (((long long)Oi[2 * nh][i][2 * r] << 24) + ((long long)Oi[2 * nh][i][2 * r + 1] << 16)) +
+                              (((long long)Oi[2 * nh + 1][i][2 * r] << 8) + Oi[2 * nh + 1][i][2 * r + 1]);
+          acc[nh][i][r] += (double)v * fw;
         }
       }
 #pragma unroll
-      for (int nt = 0; nt < NTV; ++nt) { Oi[nt][mt][0] = Oi[nt][mt][1] = Oi[nt][mt][2] = Oi[nt][mt][3] = 0; }
+      for (int nt = 0; nt < NTV; ++nt) { Oi[nt][i][0] = Oi[nt][i][1] = Oi[nt][i][2] = Oi[nt][i][3] = 0; }
     }
   };
 
   for (long long x = x_lo; x < x_hi;) {
     const int seg_pages = (int)min((long long)(pages_b - page), x_hi - x);
-    const int n_tok = paged_len(c.seq_len, b, g.capacity, g.R);   // tokens of the sequence that are in the pages
+    const int n_all = clamped_len(c.seq_len, b, g.capacity);
+    const int n_tok = g.R ? (n_all / g.R) * g.R : n_all;          // tokens of the sequence that are in the pages
     // a block is unmasked when all of its 32 tokens exist and every query row may see them (several causal rows:
     // row r sees the first n - (rows - 1 - r) tokens of the n the sequence holds, window included)
-    const int n_unmasked = min(n_tok, clamped_len(c.seq_len, b, g.capacity) - (g.rows - 1));
+    const int n_unmasked = min(n_tok, n_all - (g.rows - 1));
     const int stream = b * Hkv + h;
     // which of the stream's partials this CTA writes, and how many there are: one thread works it out now, everybody
     // reads it after the barrier at the segment's end (the barrier that closed the last segment keeps its readers apart)
@@ -577,85 +615,67 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
     }
 
     // ---- segment start: q operands, group sums and a clean state for this stream's heads
-    {
 #pragma unroll
-      for (int nh = 0; nh < NH; ++nh) {
-        const int hb = (gid >> 1) + 4 * nh;                          // head of this lane's operand column
+    for (int nh = 0; nh < NH; ++nh) {
+      const int hb = (gid >> 1) + 4 * nh;                          // head of this lane's operand column
+      hs[nh] = 0.f;
+      if constexpr (KAXIS == 0) {       // (channel-wise keys: the preparation warp makes the operands, per page)
         float qv[NR][4];
-        float amax = 0.f;
-        if constexpr (KAXIS == 0) amax = load_q_lane<D>(g, c, q, b, h, hb, tid, qv);
+        float amax = load_q_lane<D>(g, c, q, b, h, hb, tid, qv);
         amax = fmaxf(amax, __shfl_xor_sync(FULL, amax, 1));
         amax = fmaxf(amax, __shfl_xor_sync(FULL, amax, 2));
-        if constexpr (KAXIS == 1) {
-          // channel-wise keys: the operands depend on the page's scales; the preparation warp makes them per page
-          hs[nh] = 0.f;
-        } else {
-          // 16-bit fixed point relative to the head's largest entry: Q = rint(q * scale), |Q| <= 32512
-          const float scale = amax > 0.f ? kQFix / amax : 0.f;
-          const float hsb = amax > 0.f ? c1 / scale : 0.f;
-          int qs[NGK];
+        // 16-bit fixed point relative to the head's largest entry: Q = rint(q * scale), |Q| <= 32512
+        const float scale = amax > 0.f ? kQFix / amax : 0.f;
+        const float hsb = amax > 0.f ? c1 / scale : 0.f;
+        int qs[NGK];
 #pragma unroll
-          for (int j = 0; j < NGK; ++j) qs[j] = 0;
+        for (int j = 0; j < NGK; ++j) qs[j] = 0;
 #pragma unroll
-          for (int r = 0; r < NR; ++r) qB[nh][0][r] = fixed_point_limb(qv[r], scale, gid & 1, qs[r / (NR / NGK)]);
-          hs[nh] = __shfl_sync(FULL, hsb, 8 * tid);
-          // the zero-point term uses the sum of the same fixed-point q the MMAs see: the two large terms
-          // s (q . c) and z sum(q) of a logit then cancel exactly as they do for the exact q
+        for (int r = 0; r < NR; ++r) qB[nh][0][r] = fixed_point_limb(qv[r], scale, gid & 1, qs[r / (NR / NGK)]);
+        hs[nh] = __shfl_sync(FULL, hsb, 8 * tid);
+        // the zero-point term uses the sum of the same fixed-point q the MMAs see: the two large terms
+        // s (q . c) and z sum(q) of a logit then cancel exactly as they do for the exact q
 #pragma unroll
-          for (int j = 0; j < NGK; ++j) {
-            int v = qs[j];
-            v += __shfl_xor_sync(FULL, v, 1);
-            v += __shfl_xor_sync(FULL, v, 2);
-            qsum[nh][j] = hs[nh] * (float)__shfl_sync(FULL, v, 8 * tid);
-          }
-        }
-        m_ref[nh] = -INFINITY;
-        l[nh] = 0.f;
-        zq[nh] = 0.f;
-#pragma unroll
-        for (int j = 0; j < NGV; ++j) zacc[nh][j] = 0.f;
-      }
-#pragma unroll
-      for (int mt = 0; mt < MT; ++mt) {
-#pragma unroll
-        for (int nt = 0; nt < NTV; ++nt) { Oi[nt][mt][0] = Oi[nt][mt][1] = Oi[nt][mt][2] = Oi[nt][mt][3] = 0; }
-#pragma unroll
-        for (int nh = 0; nh < NH; ++nh) {
-          myM[(tid + 4 * nh) * MSTRIDE + 16 * mt + gid] = 0.f;
-          myM[(tid + 4 * nh) * MSTRIDE + 16 * mt + 8 + gid] = 0.f;
+        for (int j = 0; j < NGK; ++j) {
+          int v = qs[j];
+          v += __shfl_xor_sync(FULL, v, 1);
+          v += __shfl_xor_sync(FULL, v, 2);
+          qsum[nh][j] = hs[nh] * (float)__shfl_sync(FULL, v, 8 * tid);
         }
       }
+      m_ref[nh] = -INFINITY;
+      l[nh] = 0.f;
+      zq[nh] = 0.f;
+#pragma unroll
+      for (int j = 0; j < NGV; ++j) zacc[nh][j] = 0.f;
+#pragma unroll
+      for (int i = 0; i < MTW; ++i) acc[nh][i][0] = acc[nh][i][1] = 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < MTW; ++i) {
+#pragma unroll
+      for (int nt = 0; nt < NTV; ++nt) { Oi[nt][i][0] = Oi[nt][i][1] = Oi[nt][i][2] = Oi[nt][i][3] = 0; }
     }
 
-    for (int pp = 0; pp < seg_pages; ++pp) {
-      const bool mine = turn == grp;
-      if (++turn == NG) turn = 0;
-      if (!mine) continue;
-      const int nv = min(kPageTokens, n_tok - (page + pp) * kPageTokens);
+    auto process = [&](auto full_tag, int pp) {
+      constexpr bool FULL_PAGE = decltype(full_tag)::value;
+      const int nv = FULL_PAGE ? kPageTokens : min(kPageTokens, n_tok - (page + pp) * kPageTokens);
       const bool tail_k = (KAXIS == 1) && (nv < kPageTokens);
-      if (!aborted) {
-        const bool got = mbar_wait(bar0 + 8 * stage, phase, wait_ns);
-        if (!__all_sync(FULL, got)) {
-          aborted = true;
-          *abort_flag = 1;
-          if (lane == 0) atomicOr(c.status, KVQ_STATUS_DEVICE_TIMEOUT);
-        }
-      }
       const uint8_t* sp = smem + stage * sl.page_stride;
-
-      // ---- channel-wise keys: the page's operands come from the preparation warp (stage buffer, `ready` barrier)
-      if constexpr (KAXIS == 1) {
-        if (!aborted) {
-          const bool got = mbar_wait(bar0 + 8 * (2 * stages + stage), phase, wait_ns);
-          if (!__all_sync(FULL, got)) {
-            aborted = true;
-            *abort_flag = 1;
-            if (lane == 0) atomicOr(c.status, KVQ_STATUS_DEVICE_TIMEOUT);
-          }
-        }
-        if (!aborted) {
-          constexpr int CSB = NH * 2 * NR * 32 * 4 + 64;
-          const uint32_t* ops = reinterpret_cast<const uint32_t*>(smem + sl.chan_off + stage * CSB);
+      uint8_t* wbuf = smem + sl.w_off + (page_no & 1) * (NGV * 4 * WB);
+      // ---- logits of the warp's 32 tokens, two tiles of 16; (scale, zero) of their values
+      float L[2][2][NH];                 // [tile][row gid / gid + 8][head]
+      float sv[2][2][NGV], zv[2][2][NGV];
+      const bool active = FULL_PAGE || warp * 32 < nv;
+      const bool masked = !FULL_PAGE && (page + pp) * kPageTokens + warp * 32 + 32 > n_unmasked;
+      bool trig = false;
+      float bmax[NH], smax = 0.f;
+#pragma unroll
+      for (int nh = 0; nh < NH; ++nh) bmax[nh] = -INFINITY;
+      if (active) {
+        [[maybe_unused]] const uint32_t* ops = nullptr;      // channel-wise keys: the page's operands
+        if constexpr (KAXIS == 1) {
+          ops = reinterpret_cast<const uint32_t*>(smem + sl.chan_off + stage * (NH * 2 * NR * 32 * 4 + 64));
           const float* opf = reinterpret_cast<const float*>(ops + NH * 2 * NR * 32);
 #pragma unroll
           for (int nh = 0; nh < NH; ++nh) {
@@ -668,259 +688,282 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
             hs[nh] = opf[8 + tid + 4 * nh];
           }
         }
-      }
-
-      if (!aborted && wq * 32 < nv) {
-        const uint8_t* sp_k = sp + lane_k;
-        const uint8_t* sp_km = sp + lane_km;
-        const uint8_t* sp_v = sp + lane_v;
-        const uint8_t* sp_vm = sp + lane_vm;
-
-        auto do_block = [&](auto masked_tag) {
-          constexpr bool MASKED = decltype(masked_tag)::value;
-          float L[2][2][NH];                 // [tile][row gid / gid + 8][head]
-          bool vld[2][2];
-          // ------------------------------------------------------------ logits of the block's two 16-token tiles
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int tok0 = wq * 32 + 16 * u + gid;        // page-local tokens of this lane's two rows: tok0, tok0 + 8
-            vld[u][0] = !MASKED || tok0 < nv;
-            vld[u][1] = !MASKED || tok0 + 8 < nv;
-            if (KAXIS == 1 && tail_k) {
-              // tokens of the incomplete block: fp16 keys from the tail against q as fp16 high + low parts (operand
-              // column gid = (head gid/2 + 4 nh, part gid%2), so lane columns 2 tid, 2 tid + 1 are the two parts of
-              // head tid + 4 nh)
-              const uint16_t* tl = c.k_tail + ((size_t)stream * kPageTokens + tok0) * D;
+        for (int u = 0; u < 2; ++u) {
+          const int tok0 = warp * 32 + 16 * u + gid;        // page-local tokens of this lane's two rows: tok0, tok0 + 8
+          if (KAXIS == 1 && tail_k) {
+            // tokens of the incomplete block: fp16 keys from the tail against q as fp16 high + low parts (operand
+            // column gid = (head gid/2 + 4 nh, part gid%2), so lane columns 2 tid, 2 tid + 1 are the two parts of
+            // head tid + 4 nh)
+            const uint16_t* tl = c.k_tail + ((size_t)stream * kPageTokens + tok0) * D;
+            const bool v0 = tok0 < nv, v1 = tok0 + 8 < nv;
+#pragma unroll
+            for (int nh = 0; nh < NH; ++nh) {
+              float S[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+              for (int r = 0; r < NR; ++r) {
+                uint2 ra = make_uint2(0u, 0u), rb = make_uint2(0u, 0u);
+                if (v0) ra = *reinterpret_cast<const uint2*>(tl + 16 * r + 4 * tid);
+                if (v1) rb = *reinterpret_cast<const uint2*>(tl + 8 * D + 16 * r + 4 * tid);
+                const uint32_t a0 = __byte_perm(ra.x, ra.y, 0x5410), a1 = __byte_perm(rb.x, rb.y, 0x5410);
+                const uint32_t a2 = __byte_perm(ra.x, ra.y, 0x7632), a3 = __byte_perm(rb.x, rb.y, 0x7632);
+                mma16816(S, a0, a1, a2, a3, qB[nh][0][r], qB[nh][NTK - 1][r]);    // q's fp16 parts, made by the preparation warp
+              }
+              L[u][0][nh] = c1 * (S[0] + S[1]);
+              L[u][1][nh] = c1 * (S[2] + S[3]);
+            }
+          } else {
+            uint32_t ka[KW], kb2[KW];
+            const uint8_t* krow = sp + lane_k + u * (16 * K_ROW_BYTES);           // this lane's chunk of row tok0
+            load_words<KW>(krow, 64, ka);
+            load_words<KW>(krow + 8 * K_ROW_BYTES, 64, kb2);
+            int S[NGK][NH][NTK][4];
+#pragma unroll
+            for (int s = 0; s < KS32; ++s) {
+              const int j = s / (KS32 / NGK);
+              const bool first = s % (KS32 / NGK) == 0;
+              const uint32_t a0 = key_slot<KB, KW>(ka, 2 * s), a1 = key_slot<KB, KW>(kb2, 2 * s);
+              const uint32_t a2 = key_slot<KB, KW>(ka, 2 * s + 1), a3 = key_slot<KB, KW>(kb2, 2 * s + 1);
 #pragma unroll
               for (int nh = 0; nh < NH; ++nh) {
-                float S[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                  uint2 ra = make_uint2(0u, 0u), rb = make_uint2(0u, 0u);
-                  if (vld[u][0]) ra = *reinterpret_cast<const uint2*>(tl + 16 * r + 4 * tid);
-                  if (vld[u][1]) rb = *reinterpret_cast<const uint2*>(tl + 8 * D + 16 * r + 4 * tid);
-                  const uint32_t a0 = __byte_perm(ra.x, ra.y, 0x5410), a1 = __byte_perm(rb.x, rb.y, 0x5410);
-                  const uint32_t a2 = __byte_perm(ra.x, ra.y, 0x7632), a3 = __byte_perm(rb.x, rb.y, 0x7632);
-                  mma16816(S, a0, a1, a2, a3, qB[nh][0][r], qB[nh][NTK - 1][r]);    // q's fp16 parts, made by the preparation warp
-                }
-                L[u][0][nh] = c1 * (S[0] + S[1]);
-                L[u][1][nh] = c1 * (S[2] + S[3]);
-              }
-            } else {
-              uint32_t ka[KW], kb2[KW];
-              const uint8_t* krow = sp_k + u * (16 * K_ROW_BYTES);           // this lane's chunk of row tok0
-              load_words<KW>(krow, 64, ka);
-              load_words<KW>(krow + 8 * K_ROW_BYTES, 64, kb2);
-              int S[NGK][NH][NTK][4];
-#pragma unroll
-              for (int j = 0; j < NGK; ++j) {
-#pragma unroll
-                for (int nh = 0; nh < NH; ++nh) {
-#pragma unroll
-                  for (int nt = 0; nt < NTK; ++nt) { S[j][nh][nt][0] = S[j][nh][nt][1] = S[j][nh][nt][2] = S[j][nh][nt][3] = 0; }
-                }
-              }
-#pragma unroll
-              for (int s = 0; s < KS32; ++s) {
-                const int j = s / (KS32 / NGK);
-                const uint32_t a0 = key_slot<KB, KW>(ka, 2 * s), a1 = key_slot<KB, KW>(kb2, 2 * s);
-                const uint32_t a2 = key_slot<KB, KW>(ka, 2 * s + 1), a3 = key_slot<KB, KW>(kb2, 2 * s + 1);
-#pragma unroll
-                for (int nh = 0; nh < NH; ++nh) {
-#pragma unroll
-                  for (int nt = 0; nt < NTK; ++nt) {
-                    if (nt == 0) mma16832_u8s8(S[j][nh][nt], a0, a1, a2, a3, qB[nh][nt][2 * s], qB[nh][nt][2 * s + 1]);
-                    else mma16832_u8u8(S[j][nh][nt], a0, a1, a2, a3, qB[nh][nt][2 * s], qB[nh][nt][2 * s + 1]);
-                  }
-                }
-              }
-              // accumulator columns 2 tid, 2 tid + 1 = (hi, lo) limbs of head tid + 4 nh: sum_d code_d Q_d = 256 hi + lo
-              // (channel-wise keys: the signed top byte in n-tile 0, the two unsigned lower bytes in n-tile 1, combined in fp32)
-              if constexpr (KAXIS == 1) {
-#pragma unroll
-                for (int nh = 0; nh < NH; ++nh) {
-                  const float t0 = fmaf((float)S[0][nh][0][0], 65536.f, fmaf((float)S[0][nh][NTK - 1][0], 256.f, (float)S[0][nh][NTK - 1][1]));
-                  const float t1 = fmaf((float)S[0][nh][0][2], 65536.f, fmaf((float)S[0][nh][NTK - 1][2], 256.f, (float)S[0][nh][NTK - 1][3]));
-                  L[u][0][nh] = fmaf(t0, hs[nh], zq[nh]);
-                  L[u][1][nh] = fmaf(t1, hs[nh], zq[nh]);
-                }
-              } else {
-                const uint32_t* km = reinterpret_cast<const uint32_t*>(sp_km + u * (16 * 4 * NGK));   // row tok0
-#pragma unroll
-                for (int nh = 0; nh < NH; ++nh) { L[u][0][nh] = 0.f; L[u][1][nh] = 0.f; }
-#pragma unroll
-                for (int j = 0; j < NGK; ++j) {
-                  const float2 ma = __half22float2(as_h2(km[j]));                       // (scale, zero) of row tok0
-                  const float2 mb = __half22float2(as_h2(km[8 * NGK + j]));             // ... of row tok0 + 8
-#pragma unroll
-                  for (int nh = 0; nh < NH; ++nh) {
-                    const float t0 = (float)(S[j][nh][0][0] * 256 + S[j][nh][0][1]);
-                    const float t1 = (float)(S[j][nh][0][2] * 256 + S[j][nh][0][3]);
-                    L[u][0][nh] += fmaf(ma.x * hs[nh], t0, ma.y * qsum[nh][j]);
-                    L[u][1][nh] += fmaf(mb.x * hs[nh], t1, mb.y * qsum[nh][j]);
-                  }
+                for (int nt = 0; nt < NTK; ++nt) {
+                  const uint32_t b0 = qB[nh][nt][2 * s], b1 = qB[nh][nt][2 * s + 1];
+                  if (nt == 0) { if (first) mma16832_u8s8_zero(S[j][nh][nt], a0, a1, a2, a3, b0, b1); else mma16832_u8s8(S[j][nh][nt], a0, a1, a2, a3, b0, b1); }
+                  else { if (first) mma16832_u8u8_zero(S[j][nh][nt], a0, a1, a2, a3, b0, b1); else mma16832_u8u8(S[j][nh][nt], a0, a1, a2, a3, b0, b1); }
                 }
               }
             }
-            if (MASKED) {
-              const int tokg = (page + pp) * kPageTokens + tok0;        // position of row tok0 in the sequence
-              const int n_all = clamped_len(c.seq_len, b, g.capacity);
+            // accumulator columns 2 tid, 2 tid + 1 = (hi, lo) limbs of head tid + 4 nh: sum_d code_d Q_d = 256 hi + lo
+            // (channel-wise keys: the signed top byte in n-tile 0, the two unsigned lower bytes in n-tile 1, combined in fp32)
+            if constexpr (KAXIS == 1) {
+#pragma unroll
+              for (int nh = 0; nh < NH; ++nh) {
+                const float t0 = fmaf((float)S[0][nh][0][0], 65536.f, fmaf((float)S[0][nh][NTK - 1][0], 256.f, (float)S[0][nh][NTK - 1][1]));
+                const float t1 = fmaf((float)S[0][nh][0][2], 65536.f, fmaf((float)S[0][nh][NTK - 1][2], 256.f, (float)S[0][nh][NTK - 1][3]));
+                L[u][0][nh] = fmaf(t0, hs[nh], zq[nh]);
+                L[u][1][nh] = fmaf(t1, hs[nh], zq[nh]);
+              }
+            } else {
+              const uint32_t* km = reinterpret_cast<const uint32_t*>(sp + lane_km + u * (16 * 4 * NGK));   // row tok0
+#pragma unroll
+              for (int nh = 0; nh < NH; ++nh) { L[u][0][nh] = 0.f; L[u][1][nh] = 0.f; }
+#pragma unroll
+              for (int j = 0; j < NGK; ++j) {
+                const float2 ma = __half22float2(as_h2(km[j]));                       // (scale, zero) of row tok0
+                const float2 mb = __half22float2(as_h2(km[8 * NGK + j]));             // ... of row tok0 + 8
+#pragma unroll
+                for (int nh = 0; nh < NH; ++nh) {
+                  const float t0 = (float)(S[j][nh][0][0] * 256 + S[j][nh][0][1]);
+                  const float t1 = (float)(S[j][nh][0][2] * 256 + S[j][nh][0][3]);
+                  L[u][0][nh] += fmaf(ma.x * hs[nh], t0, ma.y * qsum[nh][j]);
+                  L[u][1][nh] += fmaf(mb.x * hs[nh], t1, mb.y * qsum[nh][j]);
+                }
+              }
+            }
+          }
+          const uint32_t* vm = reinterpret_cast<const uint32_t*>(sp + lane_vm + u * (16 * 4 * NGV));
+#pragma unroll
+          for (int j = 0; j < NGV; ++j) {
+            const float2 fa = __half22float2(as_h2(vm[j])), fb = __half22float2(as_h2(vm[8 * NGV + j]));
+            sv[u][0][j] = fa.x; zv[u][0][j] = fa.y;
+            sv[u][1][j] = fb.x; zv[u][1][j] = fb.y;
+          }
+          if (masked) {
+            const int tokg = (page + pp) * kPageTokens + tok0;        // position of row tok0 in the sequence
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+              const bool there = tok0 + 8 * r < nv;
 #pragma unroll
               for (int nh = 0; nh < NH; ++nh) {
                 // tokens the lane's head may attend to: the causal limit of its query row
                 const int lim = n_all - (g.rows - 1 - min((tid + 4 * nh) / Gq, g.rows - 1));
-                if (!vld[u][0] || tokg >= lim) L[u][0][nh] = -INFINITY;
-                if (!vld[u][1] || tokg + 8 >= lim) L[u][1][nh] = -INFINITY;
+                if (!there || tokg + 8 * r >= lim) L[u][r][nh] = -INFINITY;
+              }
+#pragma unroll
+              for (int j = 0; j < NGV; ++j) {
+                if (!there) sv[u][r][j] = zv[u][r][j] = 0.f;
               }
             }
           }
-
-          // ------------------------------------------------------------ value scales and zero-points of the four rows
-          float sv[2][2][NGV], zv[2][2][NGV];
-          float smax = 0.f;
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const uint32_t* vm = reinterpret_cast<const uint32_t*>(sp_vm + u * (16 * 4 * NGV));
+          for (int j = 0; j < NGV; ++j) smax = fmaxf(smax, fmaxf(sv[u][0][j], sv[u][1][j]));
+        }
+        // ---- softmax reference / scale check (rarely true)
+        trig = smax * sscale >= PONE;
 #pragma unroll
-            for (int j = 0; j < NGV; ++j) {
-              const uint32_t ma = vld[u][0] ? vm[j] : 0u;
-              const uint32_t mb = vld[u][1] ? vm[8 * NGV + j] : 0u;
-              const float2 fa = __half22float2(as_h2(ma)), fb = __half22float2(as_h2(mb));
-              sv[u][0][j] = fa.x; zv[u][0][j] = fa.y;
-              sv[u][1][j] = fb.x; zv[u][1][j] = fb.y;
-              smax = fmaxf(smax, fmaxf(fa.x, fb.x));
-            }
-          }
+        for (int nh = 0; nh < NH; ++nh) {
+          bmax[nh] = fmaxf(fmaxf(L[0][0][nh], L[0][1][nh]), fmaxf(L[1][0][nh], L[1][1][nh]));
+          trig |= bmax[nh] > m_ref[nh];
+        }
+      }
 
-          // ------------------------------------------------------------ softmax reference / scale check (rarely taken)
-          float bmax[NH];
-          // (the int32 accumulators are also folded every kFlushBlocks pages, long before they can overflow)
-          bool trig = (smax * sscale >= PONE) | ((page_no & (kFlushBlocks - 1)) == kFlushBlocks - 1);
+      // ---- weights: p = 2^(logit - reference) <= 2^-headroom, P = rint(p * s_V * sscale) < 2^PBITS, left for all warps as
+      // the B operands of the block; the sums over the warp's own tokens are kept apart until the reference holds
+      float psum[NH], zsum[NH][NGV];
+      auto make_weights = [&]() {
+#pragma unroll
+        for (int nh = 0; nh < NH; ++nh) {
+          psum[nh] = 0.f;
+#pragma unroll
+          for (int j = 0; j < NGV; ++j) zsum[nh][j] = 0.f;
+        }
+        uint32_t bV[NGV][NTV][2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          float p[2][NH];
 #pragma unroll
           for (int nh = 0; nh < NH; ++nh) {
-            bmax[nh] = fmaxf(fmaxf(L[0][0][nh], L[0][1][nh]), fmaxf(L[1][0][nh], L[1][1][nh]));
-            trig |= bmax[nh] > m_ref[nh];
+            p[0][nh] = ex2(L[u][0][nh] - m_ref[nh]);
+            p[1][nh] = ex2(L[u][1][nh] - m_ref[nh]);
           }
-          if (__any_sync(FULL, trig)) {
-            flush_acc();                                   // with the scale the accumulated weights were made with
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) smax = fmaxf(smax, __shfl_xor_sync(FULL, smax, off));
-            if (smax * sscale >= PONE) {
-              // next power of two above the largest value scale: p * s * sscale < 2^PBITS for every p <= 1
-              sscale = PONE / __uint_as_float((__float_as_uint(smax) & 0x7F800000u) + 0x00800000u);
-            }
+          if (masked) {       // a head that has seen no token yet has no reference: its weights are zero
 #pragma unroll
             for (int nh = 0; nh < NH; ++nh) {
-              float bm = bmax[nh];
-#pragma unroll
-              for (int off = 4; off < 32; off <<= 1) bm = fmaxf(bm, __shfl_xor_sync(FULL, bm, off));
-              if (bm > m_ref[nh]) {
-                const float nref = bm + kHeadroom<NH>;
-                const float a = (m_ref[nh] == -INFINITY) ? 0.f : ex2(m_ref[nh] - nref);
-                m_ref[nh] = nref;
-                l[nh] *= a;
-#pragma unroll
-                for (int j = 0; j < NGV; ++j) zacc[nh][j] *= a;
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt) {
-                  myM[(tid + 4 * nh) * MSTRIDE + 16 * mt + gid] *= a;
-                  myM[(tid + 4 * nh) * MSTRIDE + 16 * mt + 8 + gid] *= a;
-                }
-              }
+              if (L[u][0][nh] == -INFINITY) p[0][nh] = 0.f;
+              if (L[u][1][nh] == -INFINITY) p[1][nh] = 0.f;
             }
           }
-
-          // ------------------------------------------------------------ weights: p = 2^(logit - reference) <= 2^-headroom,
-          // P = rint(p * s_V * sscale) < 2^PBITS
-          uint32_t bV[NGV][NTV][2];
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            float p[2][NH];
+          for (int nh = 0; nh < NH; ++nh) psum[nh] += p[0][nh] + p[1][nh];
+#pragma unroll
+          for (int j = 0; j < NGV; ++j) {
+            const float sa = sv[u][0][j] * sscale, sb = sv[u][1][j] * sscale;
+            uint32_t Pa[NH], Pb[NH];
 #pragma unroll
             for (int nh = 0; nh < NH; ++nh) {
-              p[0][nh] = ex2(L[u][0][nh] - m_ref[nh]);
-              p[1][nh] = ex2(L[u][1][nh] - m_ref[nh]);
-              if (MASKED) {       // a head that has seen no token yet has no reference: its weights are zero
-                if (L[u][0][nh] == -INFINITY) p[0][nh] = 0.f;
-                if (L[u][1][nh] == -INFINITY) p[1][nh] = 0.f;
-              }
-              l[nh] += p[0][nh] + p[1][nh];
+              zsum[nh][j] = fmaf(p[0][nh], zv[u][0][j], fmaf(p[1][nh], zv[u][1][j], zsum[nh][j]));
+              Pa[nh] = __float2uint_rn(p[0][nh] * sa);      // token tok0
+              Pb[nh] = __float2uint_rn(p[1][nh] * sb);      // token tok0 + 8
             }
+            // one 16-bit element per (column, lane row) = that column's limb of tokens (tok0, tok0 + 8); the 8x8
+            // transpose turns lane columns into the B operand (column = lane/4, tokens 2t, 2t+8, 2t+1, 2t+9)
 #pragma unroll
-            for (int j = 0; j < NGV; ++j) {
-              const float sa = sv[u][0][j] * sscale, sb = sv[u][1][j] * sscale;
-              uint32_t Pa[NH], Pb[NH];
-#pragma unroll
-              for (int nh = 0; nh < NH; ++nh) {
-                zacc[nh][j] = fmaf(p[0][nh], zv[u][0][j], fmaf(p[1][nh], zv[u][1][j], zacc[nh][j]));
-                Pa[nh] = __float2uint_rn(p[0][nh] * sa);      // token tok0
-                Pb[nh] = __float2uint_rn(p[1][nh] * sb);      // token tok0 + 8
-              }
-              // one 16-bit element per (column, lane row) = that column's limb of tokens (tok0, tok0 + 8); the 8x8
-              // transpose turns lane columns into the B operand (column = lane/4, tokens 2t, 2t+8, 2t+1, 2t+9)
-              if constexpr (NH == 1) {
-                bV[j][0][u] = movmatrix_trans(prmt(Pa[0], Pb[0], 0x6273));       // limbs (3, 2): bytes a3 b3 a2 b2
-                bV[j][1][u] = movmatrix_trans(prmt(Pa[0], Pb[0], 0x4051));       // limbs (1, 0): bytes a1 b1 a0 b0
-              } else {
-                bV[j][0][u] = movmatrix_trans(prmt(Pa[0], Pb[0], 0x5162));       // head tid: (hi, mid)
-                bV[j][1][u] = movmatrix_trans(prmt(Pa[1], Pb[1], 0x5162));       // head tid + 4: (hi, mid)
-                bV[j][2][u] = movmatrix_trans(prmt(prmt(Pa[0], Pb[0], 0x0040), prmt(Pa[1], Pb[1], 0x0040), 0x5410));
-              }
+            for (int nh = 0; nh < NH; ++nh) {
+              bV[j][2 * nh][u] = movmatrix_trans(prmt(Pa[nh], Pb[nh], 0x6273));         // limbs (3, 2): bytes a3 b3 a2 b2
+              bV[j][2 * nh + 1][u] = movmatrix_trans(prmt(Pa[nh], Pb[nh], 0x4051));     // limbs (1, 0): bytes a1 b1 a0 b0
             }
           }
+        }
+#pragma unroll
+        for (int j = 0; j < NGV; ++j) {
+          uint8_t* w = wbuf + (j * 4 + warp) * WB;
+#pragma unroll
+          for (int nh = 0; nh < NH; ++nh)
+            *reinterpret_cast<uint4*>(w + 512 * nh + lane * 16) = make_uint4(bV[j][2 * nh][0], bV[j][2 * nh][1], bV[j][2 * nh + 1][0], bV[j][2 * nh + 1][1]);
+        }
+      };
+      if (active) make_weights();
+      if (named_bar_any(1, NCONS, trig)) {
+        // somebody saw a larger logit or value scale: all warps move to the new reference and limit together
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) smax = fmaxf(smax, __shfl_xor_sync(FULL, smax, off));
+#pragma unroll
+        for (int nh = 0; nh < NH; ++nh) {
+#pragma unroll
+          for (int off = 4; off < 32; off <<= 1) bmax[nh] = fmaxf(bmax[nh], __shfl_xor_sync(FULL, bmax[nh], off));
+          if (gid == 0) sMax[warp * 8 + tid + 4 * nh] = bmax[nh];
+        }
+        if (lane == 0) sLim[warp * 4] = smax;
+        named_bar_sync(1, NCONS);
+        flush_acc();                                   // with the scale the accumulated weights were made with
+        smax = fmaxf(fmaxf(sLim[0], sLim[4]), fmaxf(sLim[8], sLim[12]));
+        if (smax * sscale >= PONE) {
+          // next power of two above the largest value scale: p * s * sscale < 2^PBITS for every p <= 1
+          sscale = PONE / __uint_as_float((__float_as_uint(smax) & 0x7F800000u) + 0x00800000u);
+        }
+#pragma unroll
+        for (int nh = 0; nh < NH; ++nh) {
+          const float* mx = sMax + tid + 4 * nh;
+          const float bm = fmaxf(fmaxf(mx[0], mx[8]), fmaxf(mx[16], mx[24]));
+          if (bm > m_ref[nh]) {
+            const float nref = bm + kHeadroom;
+            const float a = (m_ref[nh] == -INFINITY) ? 0.f : ex2(m_ref[nh] - nref);
+            m_ref[nh] = nref;
+            l[nh] *= a;
+#pragma unroll
+            for (int j = 0; j < NGV; ++j) zacc[nh][j] *= a;
+#pragma unroll
+            for (int i = 0; i < MTW; ++i) { acc[nh][i][0] *= (double)a; acc[nh][i][1] *= (double)a; }
+          }
+        }
+        if (active) make_weights();
+        named_bar_sync(1, NCONS);
+      }
+      if (active) {
+#pragma unroll
+        for (int nh = 0; nh < NH; ++nh) {
+          l[nh] += psum[nh];
+#pragma unroll
+          for (int j = 0; j < NGV; ++j) zacc[nh][j] += zsum[nh][j];
+        }
+      }
 
-          // ------------------------------------------------------------ PV on the raw code bytes: one mask per register.
-          // Field f of every byte belongs to m-tile FPBV q + f, whose accumulators carry the factor 2^(VB f).
+      // ---- PV of the warp's channels over the page's blocks, on the raw code bytes: one mask per register.  Field f of every
+      // byte belongs to m-tile FPBV q + f, whose accumulators carry the factor 2^(VB f).
 #pragma unroll
-          for (int qd = 0; qd < VQ; ++qd) {
-            const uint4 vw = *reinterpret_cast<const uint4*>(sp_v + qd * 512);
+      for (int blk = 0; blk < 4; ++blk) {
+        if (FULL_PAGE || blk * 32 < nv) {
+          const uint8_t* w = wbuf + (jw * 4 + blk) * WB;
+          uint32_t bw[NTV][2];
 #pragma unroll
-            for (int f = 0; f < FPBV; ++f) {
-              const int mt = FPBV * qd + f;
-              const int j = mt / (MT / NGV);
+          for (int nh = 0; nh < NH; ++nh) {
+            const uint4 w4 = *reinterpret_cast<const uint4*>(w + 512 * nh + lane * 16);
+            bw[2 * nh][0] = w4.x; bw[2 * nh][1] = w4.y; bw[2 * nh + 1][0] = w4.z; bw[2 * nh + 1][1] = w4.w;
+          }
+#pragma unroll
+          for (int qd = 0; qd < QPW; ++qd) {
+            const uint4 vw = *reinterpret_cast<const uint4*>(sp + lane_v + blk * V_BLOCK_BYTES + qd * 512);
+#pragma unroll
+            for (int t = 0; t < TPQ; ++t) {
+              const int i = qd * TPQ + t;
               uint32_t a0 = vw.x, a2 = vw.y, a1 = vw.z, a3 = vw.w;     // words (rh, kh) = (0,0), (0,1), (1,0), (1,1)
               if constexpr (VB != 8) {
                 constexpr uint32_t M0 = ((1u << VB) - 1u) * 0x01010101u;
-                const uint32_t mask = M0 << (VB * f);
+                const uint32_t mask = M0 << (VB * (TPQ == FPBV ? t : f0 + t));
                 a0 &= mask; a1 &= mask; a2 &= mask; a3 &= mask;
               }
 #pragma unroll
-              for (int nt = 0; nt < NTV; ++nt) mma16832_u8u8(Oi[nt][mt], a0, a1, a2, a3, bV[j][nt][0], bV[j][nt][1]);
+              for (int nt = 0; nt < NTV; ++nt) mma16832_u8u8(Oi[nt][i], a0, a1, a2, a3, bw[nt][0], bw[nt][1]);
             }
           }
-        };
-
-        // the masked variant also serves the last tokens when several causal query rows see different prefixes
-        if ((page + pp) * kPageTokens + wq * 32 + 32 <= n_unmasked) do_block(std::false_type{});
-        else do_block(std::true_type{});
+        }
       }
+    };
+
+#pragma unroll 1
+    for (int pp = 0; pp < seg_pages; ++pp) {
+      if (!__all_sync(FULL, mbar_try_wait(bar0 + 8 * stage, phase))) wait_slowly(bar0 + 8 * stage);
+      if constexpr (KAXIS == 1) {         // the operands of the page
+        if (!__all_sync(FULL, mbar_try_wait(bar0 + 8 * (2 * stages + stage), phase))) wait_slowly(bar0 + 8 * (2 * stages + stage));
+      }
+      // a page whose tokens all exist and may be seen by every query row needs no masks
+      if ((page + pp + 1) * kPageTokens <= n_unmasked) process(std::true_type{}, pp);
+      else process(std::false_type{}, pp);
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar0 + 8 * (stages + stage));
-      stage += NG;
-      if (stage >= stages) { stage -= stages; phase ^= 1; }
-      ++page_no;
+      mbar_arrive_if(bar0 + 8 * (stages + stage), lane == 0);
+      if (++stage == stages) { stage = 0; phase ^= 1; }
+      if ((++page_no & (kFlushPages - 1)) == 0) flush_acc();      // long before the int32 accumulators can overflow
     }
 
-    // ---- segment end: finish this warp's state, combine the NW warps, write the partial
+    // ---- segment end: sum over the warps' tokens, write this warp's channels of the partial
     {
       flush_acc();
 #pragma unroll
       for (int nh = 0; nh < NH; ++nh) {
+        double z[NGV];
+#pragma unroll
+        for (int j = 0; j < NGV; ++j) z[j] = (double)zacc[nh][j];
 #pragma unroll
         for (int off = 4; off < 32; off <<= 1) {
           l[nh] += __shfl_xor_sync(FULL, l[nh], off);
 #pragma unroll
-          for (int j = 0; j < NGV; ++j) zacc[nh][j] += __shfl_xor_sync(FULL, zacc[nh][j], off);
-        }
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-          const int j = mt / (MT / NGV);
-          myM[(tid + 4 * nh) * MSTRIDE + 16 * mt + gid] += zacc[nh][j];
-          myM[(tid + 4 * nh) * MSTRIDE + 16 * mt + 8 + gid] += zacc[nh][j];
+          for (int j = 0; j < NGV; ++j) z[j] += __shfl_xor_sync(FULL, z[j], off);
         }
         if (gid == 0) {
-          sML[(warp * NHEADS + tid + 4 * nh) * 2 + 0] = m_ref[nh];
-          sML[(warp * NHEADS + tid + 4 * nh) * 2 + 1] = l[nh];
+          sSum[warp * 8 + tid + 4 * nh] = l[nh];
+#pragma unroll
+          for (int j = 0; j < NGV; ++j) sZ[(warp * 8 + tid + 4 * nh) * NGV + j] = z[j];
         }
       }
       named_bar_sync(1, NCONS);
@@ -928,75 +971,96 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       // whole stream writes the output at once; otherwise it stores its partial, counts itself in, and the CTA
       // that completes the count merges all partials of the stream by log-sum-exp and stores the output.
       const int slot = sMisc[8], n_part = sMisc[9];
-      const bool has_win = clamped_len(c.seq_len, b, g.capacity) > n_tok;    // the window kernel left a partial in slot s_cap - 1
+      const bool has_win = n_all > n_tok;                 // the window kernel left a partial in slot s_cap - 1
       if (slot >= 0 && slot < s_plan) {
-        for (int idx = tid_; idx < G * D; idx += NCONS) {
-          const int head = idx / D, d = idx % D;
-          float mstar = -INFINITY;
+        const bool direct = n_part == 1 && !has_win;
 #pragma unroll
-          for (int w = 0; w < NW; ++w) mstar = fmaxf(mstar, sML[(w * NHEADS + head) * 2]);
-          float o = 0.f, lsum = 0.f;
+        for (int nh = 0; nh < NH; ++nh) {
+          const int head = tid + 4 * nh;
+          if (head < G) {
+            float lsum = 0.f;
+            double zsum = 0.0;
 #pragma unroll
-          for (int w = 0; w < NW; ++w) {
-            const float mw = sML[(w * NHEADS + head) * 2];
-            const float f = (mw == -INFINITY) ? 0.f : ex2(mw - mstar);
-            o = fmaf(f, sMaster[(w * NHEADS + head) * MSTRIDE + d], o);
-            lsum = fmaf(f, sML[(w * NHEADS + head) * 2 + 1], lsum);
-          }
-          if (n_part == 1 && !has_win) {
-            const float r = lsum > 0.f ? o / lsum : 0.f;
-            const size_t oi = (((size_t)b * g.rows + head / Gq) * g.Hq + (size_t)h * Gq + head % Gq) * D + d;
-            if (out_dtype == KVQ_FP32) static_cast<float*>(out)[oi] = r;
-            else static_cast<uint16_t*>(out)[oi] = f32_to_bits16(r, out_dtype);
-          } else {
+            for (int w = 0; w < NW; ++w) {
+              lsum += sSum[w * 8 + head];
+              zsum += sZ[(w * 8 + head) * NGV + jw];
+            }
+            const size_t oi = (((size_t)b * g.rows + head / Gq) * g.Hq + (size_t)h * Gq + head % Gq) * D;
             float* dst = ws + (((size_t)stream * s_cap + slot) * G + head) * (D + 2);
-            if (d == 0) { dst[0] = mstar; dst[1] = lsum; }
-            dst[2 + d] = o;
+            if (!direct && warp == 0 && gid == 0) { dst[0] = m_ref[nh]; dst[1] = lsum; }
+#pragma unroll
+            for (int i = 0; i < MTW; ++i) {
+#pragma unroll
+              for (int r = 0; r < 2; ++r) {
+                const int d = 16 * (mt0 + i) + 8 * r + gid;
+                const float o = (float)(acc[nh][i][r] + zsum);
+                if (direct) {
+                  const float v = lsum > 0.f ? o / lsum : 0.f;
+                  if (out_dtype == KVQ_FP32) static_cast<float*>(out)[oi + d] = v;
+                  else static_cast<uint16_t*>(out)[oi + d] = f32_to_bits16(v, out_dtype);
+                } else {
+                  dst[2 + d] = o;
+                }
+              }
+            }
           }
         }
-        if (n_part > 1 || has_win) {
+        if (!direct) {
           __threadfence();
           named_bar_sync(1, NCONS);
           if (tid_ == 0) *n_published = (int)tagged_count(counts + stream, id40);
           named_bar_sync(1, NCONS);
           if (*n_published == n_part) {
             __threadfence();
-            for (int idx = tid_; idx < G * D; idx += NCONS) {
-              const int head = idx / D, d = idx % D;
+            // a warp per head, two or four channels per lane; eight partials' loads are in flight at a time
+            constexpr int C2 = D / 64;
+#pragma unroll 1
+            for (int head = warp; head < G; head += NW) {
               const float* base = ws + (((size_t)stream * s_cap) * G + head) * (D + 2);
               const size_t slot_stride = (size_t)G * (D + 2);
-              float mstar = -INFINITY, num = 0.f, den = 0.f;
-              const int n_merge = n_part + (has_win ? 1 : 0);
-              for (int j0 = 0; j0 < n_merge; j0 += 4) {
-                float mj[4], lj[4], oj[4];
+              float mstar = -INFINITY, den = 0.f;
+              float2 num[C2];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {                   // issue the loads of a batch before using any
+              for (int e = 0; e < C2; ++e) num[e] = make_float2(0.f, 0.f);
+              const int n_merge = n_part + (has_win ? 1 : 0);
+#pragma unroll 1
+              for (int j0 = 0; j0 < n_merge; j0 += 8) {
+                float2 ml[8], oj[8][C2];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {                   // issue the loads of a batch before using any
                   const bool on = j0 + u < n_merge;
                   const int sj = (j0 + u < n_part) ? j0 + u : s_cap - 1;      // the window's partial comes last
-                  const float* pj = base + (size_t)(on ? sj : 0) * slot_stride;
-                  mj[u] = on ? __ldcg(pj) : -INFINITY;
-                  lj[u] = on ? __ldcg(pj + 1) : 0.f;
-                  oj[u] = on ? __ldcg(pj + 2 + d) : 0.f;
+                  const float2* pj = reinterpret_cast<const float2*>(base + (size_t)(on ? sj : 0) * slot_stride);
+                  ml[u] = on ? __ldcg(pj) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+                  for (int e = 0; e < C2; ++e) oj[u][e] = on ? __ldcg(pj + 1 + lane + 32 * e) : make_float2(0.f, 0.f);
                 }
                 float mb = mstar;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) mb = fmaxf(mb, mj[u]);
+                for (int u = 0; u < 8; ++u) mb = fmaxf(mb, ml[u].x);
                 if (mb == -INFINITY) continue;
                 const float keep = (mstar == -INFINITY) ? 0.f : ex2(mstar - mb);
-                num *= keep;
                 den *= keep;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                  const float wgt = (mj[u] == -INFINITY) ? 0.f : ex2(mj[u] - mb);
-                  num = fmaf(wgt, oj[u], num);
-                  den = fmaf(wgt, lj[u], den);
+                for (int e = 0; e < C2; ++e) { num[e].x *= keep; num[e].y *= keep; }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                  const float wgt = (ml[u].x == -INFINITY) ? 0.f : ex2(ml[u].x - mb);
+                  den = fmaf(wgt, ml[u].y, den);
+#pragma unroll
+                  for (int e = 0; e < C2; ++e) { num[e].x = fmaf(wgt, oj[u][e].x, num[e].x); num[e].y = fmaf(wgt, oj[u][e].y, num[e].y); }
                 }
                 mstar = mb;
               }
-              const float r = den > 0.f ? num / den : 0.f;
-              const size_t oi = (((size_t)b * g.rows + head / Gq) * g.Hq + (size_t)h * Gq + head % Gq) * D + d;
-              if (out_dtype == KVQ_FP32) static_cast<float*>(out)[oi] = r;
-              else static_cast<uint16_t*>(out)[oi] = f32_to_bits16(r, out_dtype);
+              const size_t oi = (((size_t)b * g.rows + head / Gq) * g.Hq + (size_t)h * Gq + head % Gq) * D;
+#pragma unroll
+              for (int e = 0; e < C2; ++e) {
+                const float rx = den > 0.f ? num[e].x / den : 0.f, ry = den > 0.f ? num[e].y / den : 0.f;
+                const int d = 2 * (lane + 32 * e);
+                if (out_dtype == KVQ_FP32) *reinterpret_cast<float2*>(static_cast<float*>(out) + oi + d) = make_float2(rx, ry);
+                else *reinterpret_cast<uint32_t*>(static_cast<uint16_t*>(out) + oi + d) =
+                         (uint32_t)f32_to_bits16(rx, out_dtype) | ((uint32_t)f32_to_bits16(ry, out_dtype) << 16);
+              }
             }
             if (tid_ == 0) counts[stream] = 0ull;
           }
@@ -1020,22 +1084,23 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
 }
 
 // Launches one instantiation; defined per instantiation unit.
-template <int D, int KB, int VB, int KAXIS, int NGK, int NGV, int NH, int NW, int MINB>
+template <int D, int KB, int VB, int KAXIS, int NGK, int NGV, int NH, int MINB>
 int launch_mma_inst(const Geom& g, const CachePtrs& c, const void* q, float c1, float* ws, int s_cap,
                     void* out, int out_dtype, unsigned long long call_id, unsigned long long wait_ns, long long skip_x,
                     cudaStream_t stream) {
   const int budget = (227 * 1024) / MINB - 1024;            // shared memory per CTA for MINB resident CTAs per SM
-  int stages = (budget - smem_layout(0, 0, NW, g.B, D, NH, KAXIS == 1).total) /
+  int stages = (budget - smem_layout(0, 0, g.B, D, NH, NGV, KAXIS == 1).total) /
                (((g.page_bytes + 127) & ~127) + (KAXIS == 1 ? chan_stage_bytes(D, NH) : 0));
-  // Deeper rings do not help: the kernel is bound by its arithmetic, not by copy latency, and more bytes in
-  // flight cost DRAM efficiency (8B shape, K4V2: 5 stages 95 us, 3-4 stages 91-92 us, 2 stages 97 us).
+  // Deeper rings do not help, and more bytes in flight cost DRAM efficiency: at most four stages and 54 KB (K4V4, 17 KB pages, 8B
+  // shape: four stages 97.9 us, three 89.8 us; K4V2, 13 KB pages: four 76.8 us, three 77.3 us).
   if (stages > 4) stages = 4;
-  if (stages < 2 || stages < NW / 4) return KVQ_ERR_UNSUPPORTED;
-  const SmemLayout sl = smem_layout(g.page_bytes, stages, NW, g.B, D, NH, KAXIS == 1);
-  auto kern = decode_mma_kernel<D, KB, VB, KAXIS, NGK, NGV, NH, NW, MINB>;
+  if (stages > 2 && stages * ((g.page_bytes + 127) & ~127) > 54 * 1024) stages = 3;
+  if (stages < 2) return KVQ_ERR_UNSUPPORTED;
+  const SmemLayout sl = smem_layout(g.page_bytes, stages, g.B, D, NH, NGV, KAXIS == 1);
+  auto kern = decode_mma_kernel<D, KB, VB, KAXIS, NGK, NGV, NH, MINB>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sl.total) != cudaSuccess)
     return KVQ_ERR_CUDA_LAUNCH;
-  kern<<<148 * MINB, (NW + 1 + (KAXIS == 1 ? 1 : 0)) * 32, sl.total, stream>>>(g, c, static_cast<const uint16_t*>(q), c1, ws, s_cap,
+  kern<<<148 * MINB, (kConsumerWarps + 1 + (KAXIS == 1 ? 1 : 0)) * 32, sl.total, stream>>>(g, c, static_cast<const uint16_t*>(q), c1, ws, s_cap,
                                                          stages, out, out_dtype, call_id, wait_ns, skip_x);
   return cudaGetLastError() == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
 }

@@ -1,0 +1,43 @@
+"""Decode attention where the fast kernel's pages and blocks end: lengths around a 32-token block and a 128-token page, keys and
+values that keep growing (the common reference and the scale limit move on every page), every number of heads it
+serves, against the fp64 oracle on the same codes."""
+import pytest
+import torch
+
+from paper_2502_15075_b200 import workloads as wl
+
+import kvq_testlib as tl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def kvq():
+    from paper_2502_15075_b200 import build
+    build.build()
+    from paper_2502_15075_b200 import kvq as mod
+    return mod
+
+
+FORMS = {
+    "k4v2": wl.LLAMA_8B, "k2v4": wl.LLAMA_8B.with_(kb=2, vb=4), "k8v4": wl.LLAMA_8B.with_(kb=8, vb=4),
+    "k4v4": wl.LLAMA_8B.with_(vb=4), "k4v2-g32": wl.LLAMA_8B.with_(gk=32), "k4v2-g64": wl.LLAMA_8B.with_(gk=64, gv=64),
+    "d64": wl.LLAMA_1B, "d64-g32": wl.TINY, "channel-k4v2": wl.SHAPED_14B, "channel-k8v2": wl.SHAPED_14B.with_(kb=8),
+}
+
+
+@pytest.mark.parametrize("T", [1, 31, 33, 96, 127, 128, 129, 500])
+@pytest.mark.parametrize("form,heads", [(f, h) for f in FORMS for h in (1, 4)] + [("k4v2", 8), ("k4v2-g32", 5), ("k4v2-g64", 8)])
+def test_growing_logits_and_values(kvq, form, heads, T):
+    w = FORMS[form].with_(n_kv_heads=2, n_q_heads=2 * heads)
+    k, v = wl.make_kv(w, tokens=T, batch=2)
+    ramp = torch.linspace(0.05, 4.0, T).view(1, 1, T, 1)             # later tokens: larger logits, larger value scales
+    k, v = (x.float().mul(ramp).to(w.torch_dtype) for x in (k, v))
+    cfg, gc, _ = tl.build_both(kvq, w, k, v, [T], 512)
+    oc = tl.oracle_on_gpu_codes(gc, w)
+    # The absolute bound is for values of unit size: an error d of the logits moves an output by up to 2 d max|v|, and d comes
+    # from q in 16-bit fixed point, half a unit of max|q| / 32512 per channel whatever the values are.
+    scale = max(1.0, float(v.float().abs().max()))
+    for variant in ("normal", "peaked"):
+        q = wl.make_q(w, batch=2, variant=variant, k=k)
+        tl.assert_attention_close(tl.gpu_decode(kvq, cfg, gc, q), oc.decode(tl.bits_of(q)), mabs=tl.MAX_ABS_TOL * scale)
