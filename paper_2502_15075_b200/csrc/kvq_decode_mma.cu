@@ -69,6 +69,48 @@ bool decode_mma_supported(const Geom& g) {
   return pick(g, none, nullptr, 0.f, nullptr, 0, nullptr, 0, DecodeDebug{}, nullptr, true, &grid) == KVQ_OK;
 }
 
+namespace {
+// The kernel's plan for given lengths, worked out on the host by the same functions.
+template <int WAVES>
+void host_plan(const Geom& g, int gap, const int32_t* seq_len, int32_t* parts, int64_t* starts, int32_t* info) {
+  int pref[mma::kMaxBatchFlat + 1] = {}, vpref[mma::kMaxBatchFlat + 1] = {};
+  int pmax = 0;
+  for (int b = 0; b < g.B; ++b) {
+    const int n = seq_len[b] < 0 ? 0 : seq_len[b] > g.capacity ? g.capacity : seq_len[b];
+    const int pages = ((g.R ? n / g.R * g.R : n) + kPageTokens - 1) / kPageTokens;
+    pmax = pages > pmax ? pages : pmax;
+    pref[b + 1] = pref[b] + pages * g.Hkv;
+    vpref[b + 1] = vpref[b] + (pages ? (pages + gap) * g.Hkv : 0);
+  }
+  const int slots = flat_slot_cap(g) - (g.R ? 1 : 0);
+  const mma::FlatPlan plan = mma::make_plan(vpref[g.B], pmax + gap, WAVES * 148, slots);
+  const bool waves = mma::weighted_shares<WAVES>(plan, gap, WAVES * 148, pmax, slots);
+  info[0] = slots; info[1] = plan.c_eff; info[2] = waves;
+  for (int c = 0; c <= plan.c_eff && plan.N; ++c)
+    starts[c] = mma::first_page<WAVES>(plan, waves, c, pref, vpref, g.B, g.Hkv, gap);
+  for (int b = 0; b < g.B; ++b) {
+    const int pages = (pref[b + 1] - pref[b]) / g.Hkv;
+    for (int h = 0; h < g.Hkv; ++h) {
+      int32_t* p = parts + 2 * (b * g.Hkv + h);
+      p[0] = p[1] = 0;
+      if (pages) mma::stream_ctas<WAVES>(plan, waves, (long long)vpref[b] + (long long)h * (pages + gap) + gap, pages, p, p + 1);
+    }
+  }
+}
+}  // namespace
+
+int decode_mma_plan(const Geom& g, const int32_t* seq_len, int32_t* parts, int64_t* starts, int32_t* info) {
+  CachePtrs none{};
+  int grid = 0;
+  if (g.B > mma::kMaxBatchFlat) return KVQ_ERR_UNSUPPORTED;
+  const int rc = pick(g, none, nullptr, 0.f, nullptr, 0, nullptr, 0, DecodeDebug{}, nullptr, true, &grid);
+  if (rc != KVQ_OK) return rc;
+  const int gap = mma::gap_pages(g.kb, g.vb, g.k_axis);
+  if (grid == 3 * 148) host_plan<3>(g, gap, seq_len, parts, starts, info);
+  else host_plan<2>(g, gap, seq_len, parts, starts, info);
+  return KVQ_OK;
+}
+
 int launch_decode_mma(const Geom& g, const CachePtrs& c, const void* q, void* out, int out_dtype, float c1,
                       float* ws, const DecodeDebug& dbg, cudaStream_t stream) {
   const int s_cap = flat_slot_cap(g);

@@ -180,11 +180,11 @@ constexpr int kMaxBatchFlat = 1024;   // the flat partition keeps a per-batch pr
 struct FlatPlan {
   long long N;       // total pages over all streams
   int c_eff;         // CTAs that take part
-  __device__ __forceinline__ int cta_of(long long x) const { return (int)(((x + 1) * c_eff - 1) / N); }
-  __device__ __forceinline__ long long lo(int c) const { return (long long)c * N / c_eff; }
+  __host__ __device__ __forceinline__ int cta_of(long long x) const { return (int)(((x + 1) * c_eff - 1) / N); }
+  __host__ __device__ __forceinline__ long long lo(int c) const { return (long long)c * N / c_eff; }
 };
 
-__device__ __forceinline__ FlatPlan make_plan(long long N, int pages_max, int grid, int s_cap) {
+__host__ __device__ __forceinline__ FlatPlan make_plan(long long N, int pages_max, int grid, int s_cap) {
   FlatPlan p;
   p.N = N;
   long long cap = pages_max > 0 ? (long long)(s_cap - 1) * N / pages_max : 0;

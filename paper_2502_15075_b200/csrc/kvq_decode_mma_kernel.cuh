@@ -199,21 +199,21 @@ template <int WAVES> struct WaveWeights;
 template <> struct WaveWeights<3> { static constexpr int w[3] = {1040, 1000, 960}; };
 template <> struct WaveWeights<2> { static constexpr int w[3] = {1010, 990, 0}; };
 template <int WAVES>
-__device__ __forceinline__ long long wave_prefix(int cta) {
+__host__ __device__ __forceinline__ long long wave_prefix(int cta) {
   constexpr int W0 = WaveWeights<WAVES>::w[0], W1 = WaveWeights<WAVES>::w[1], W2 = WaveWeights<WAVES>::w[2];
   const int k = cta / 148, r = cta % 148;
   return (k == 0 ? 0 : k == 1 ? W0 : k == 2 ? W0 + W1 : W0 + W1 + W2) * 148ll + (long long)r * (k == 0 ? W0 : k == 1 ? W1 : W2);
 }
 // First virtual page of a CTA's share: equal shares, or shares weighted by launch wave.
 template <int WAVES>
-static __device__ __forceinline__ long long share_start_virtual(const FlatPlan& plan, bool waves, int cta) {
+static __host__ __device__ __forceinline__ long long share_start_virtual(const FlatPlan& plan, bool waves, int cta) {
   if (!waves) return plan.lo(cta);
   return plan.N * wave_prefix<WAVES>(cta) / (148ll * 1000 * WAVES);
 }
 // The CTA whose share holds virtual page v: the largest c with N prefix(c) < (v + 1) U, found wave by wave (the
 // prefix is linear inside a wave), one division.
 template <int WAVES>
-static __device__ __forceinline__ int cta_of_virtual(const FlatPlan& plan, bool waves, long long v) {
+static __host__ __device__ __forceinline__ int cta_of_virtual(const FlatPlan& plan, bool waves, long long v) {
   if (!waves) return plan.cta_of(v);
   constexpr int W0 = WaveWeights<WAVES>::w[0], W1 = WaveWeights<WAVES>::w[1], W2 = WaveWeights<WAVES>::w[2];
   const long long a = (v + 1) * (148ll * 1000 * WAVES) - 1;      // N prefix(c) <= a
@@ -225,7 +225,7 @@ static __device__ __forceinline__ int cta_of_virtual(const FlatPlan& plan, bool 
 }
 // Flat index of the first real page at or after the start of a CTA's share (sPref: pages, sVPref: pages + gaps).
 template <int WAVES>
-static __device__ __forceinline__ long long share_start(const FlatPlan& plan, bool waves, int cta, const int* sPref,
+static __host__ __device__ __forceinline__ long long share_start(const FlatPlan& plan, bool waves, int cta, const int* sPref,
                                                      const int* sVPref, int B, int Hkv, int gap) {
   const long long v = share_start_virtual<WAVES>(plan, waves, cta);
   if (v >= plan.N) return sPref[B];
@@ -236,7 +236,34 @@ static __device__ __forceinline__ long long share_start(const FlatPlan& plan, bo
   }
   const int pb = (sPref[lo_ + 1] - sPref[lo_]) / Hkv, len = pb + gap;
   const int vs = (int)(v - sVPref[lo_]), hh = vs / len, off = vs % len;
-  return (long long)sPref[lo_] + (long long)hh * pb + max(0, off - gap);
+  return (long long)sPref[lo_] + (long long)hh * pb + (off > gap ? off - gap : 0);
+}
+// The CTAs that hold pages of a stream: the first one, and how many (its partials).  xs: the stream's first page, virtual axis.
+template <int WAVES>
+static __host__ __device__ __forceinline__ void stream_ctas(const FlatPlan& plan, bool waves, long long xs, int pages, int* first, int* count) {
+  *first = cta_of_virtual<WAVES>(plan, waves, xs);
+  *count = cta_of_virtual<WAVES>(plan, waves, xs + pages - 1) - *first + 1;
+}
+// First page (real, flat) of a CTA's share; the CTA behind the last one that takes part starts where the pages end.
+template <int WAVES>
+static __host__ __device__ __forceinline__ long long first_page(const FlatPlan& plan, bool waves, int cta, const int* sPref,
+                                                             const int* sVPref, int B, int Hkv, int gap) {
+  return gap == 0 ? plan.lo(cta) : share_start<WAVES>(plan, waves, cta, sPref, sVPref, B, Hkv, gap);
+}
+// The time-balanced split (stream gaps) pays where the arithmetic per page limits the kernel (token-wise and
+// channel-wise keys alike); pages of 10 bits per element pair and more lose with it and keep the plain split by pages.
+__host__ __device__ constexpr int gap_pages(int kb, int vb, int k_axis) {
+  return kb + vb <= 8 ? (k_axis == 1 ? kGapPagesChan : kGapPages) : 0;
+}
+// Whether the shares of a full grid are weighted by launch wave: only where every stream's partials fit its slots all the
+// same.  A stream of P pages touches fewer than 2 + (P - 1) / s CTAs when no share is smaller than s virtual pages (the shares
+// between its first and its last one lie within its pages), so P - 1 <= (slots - 1) s keeps it within its slots; make_plan
+// bounds equal shares the same way, which are larger than the lightest weighted one.
+template <int WAVES>
+static __host__ __device__ __forceinline__ bool weighted_shares(const FlatPlan& plan, int gap, int grid, int pages_max, int slots) {
+  constexpr int WMIN = WaveWeights<WAVES>::w[WAVES - 1];      // lightest wave; s = N WMIN / (1000 grid)
+  return gap != 0 && grid == WAVES * 148 && plan.c_eff == grid && plan.N >= 8ll * grid &&
+         (pages_max - 1) * 1000ll * grid <= (slots - 1) * plan.N * WMIN;
 }
 
 // Template parameters: head_dim, key bits, value bits, key axis (0 token-wise, 1 channel-wise), key / value groups
@@ -283,9 +310,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   constexpr int V_META_OFF = V_CODES_OFF + 4 * V_BLOCK_BYTES;
   constexpr int NCONS = NW * 32;
   constexpr uint32_t FULL = 0xffffffffu;
-  // The time-balanced split (stream gaps) pays where the arithmetic per page limits the kernel (token-wise and
-  // channel-wise keys alike); pages of 10 bits per element pair and more lose with it and keep the plain split by pages.
-  constexpr int GAP = (KB + VB <= 8) ? (KAXIS == 1 ? kGapPagesChan : kGapPages) : 0;
+  constexpr int GAP = gap_pages(KB, VB, KAXIS);
   constexpr int WAVES = MINB;               // CTAs per SM = launch waves (the weights apply to a grid of 148 * WAVES)
   static_assert(MT % NW == 0 && (MT / NGV) % MTW == 0, "a warp's channels are whole m-tiles of one value group");
   static_assert(KAXIS == 0 || KB != 2, "channel-wise 2-bit keys are not instantiated");
@@ -296,7 +321,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + sl.bar_off);   // full[0..stages), empty[0..stages)
   int* sPref = reinterpret_cast<int*>(smem + sl.pref_off);
   int* sVPref = sPref + (g.B + 1);                                   // the same prefix with kGapPages more per stream
-  int* sMisc = reinterpret_cast<int*>(smem + sl.misc_off);           // [0] pages_max, [1] abort flag, [2] published count, [4..7] share ends, [8..9] segment slot / partials, [10..13] CTAs taking part, cursor
+  int* sMisc = reinterpret_cast<int*>(smem + sl.misc_off);           // [0] pages_max, [1] abort flag, [2] published count, [4..7] share ends, [8..9] segment slot / partials, [10..13] CTAs taking part, cursor, [14] weighted shares
   double* sZ = reinterpret_cast<double*>(smem + sl.red_off);         // [NW][8][NGV] sums of weight x zero-point
   float* sMax = reinterpret_cast<float*>(sZ + NW * 8 * NGV);         // [NW][8] block maxima
   float* sLim = sMax + NW * 8;                                       // [NW][4] value scales (one used)
@@ -341,15 +366,10 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
     if (lane < 2) {
       // lane 0: the share's first page, the CTAs that take part and the cursor; lane 1: the share's end
       const FlatPlan p0 = make_plan(vcarry, pmax + GAP, gridDim.x, s_plan);
+      const bool w0 = weighted_shares<WAVES>(p0, GAP, gridDim.x, pmax, s_plan);
       long long x0 = 0;
-      if (p0.N != 0 && (int)blockIdx.x < p0.c_eff) {
-        if constexpr (GAP == 0) {
-          x0 = p0.lo(blockIdx.x + lane);
-        } else {
-          const bool w0 = gridDim.x == WAVES * 148 && p0.c_eff == (int)gridDim.x && p0.N >= 8ll * gridDim.x;
-          x0 = share_start<WAVES>(p0, w0, (int)blockIdx.x + lane, sPref, sVPref, B, Hkv, GAP);
-        }
-      }
+      if (p0.N != 0 && (int)blockIdx.x < p0.c_eff)
+        x0 = first_page<WAVES>(p0, w0, (int)blockIdx.x + lane, sPref, sVPref, B, Hkv, GAP);
       *reinterpret_cast<long long*>(sMisc + 4 + 2 * lane) = x0;
       if (lane == 0) {
         int cb = 0, ch = 0, cp = 0;
@@ -363,7 +383,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
           const int pb = (sPref[cb + 1] - sPref[cb]) / Hkv, r = (int)x0 - sPref[cb];
           if (pb > 0) { ch = r / pb; cp = r % pb; }
         }
-        sMisc[10] = p0.c_eff; sMisc[11] = cb; sMisc[12] = ch; sMisc[13] = cp;
+        sMisc[10] = p0.c_eff; sMisc[11] = cb; sMisc[12] = ch; sMisc[13] = cp; sMisc[14] = w0;
       }
     }
   }
@@ -385,7 +405,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   plan.c_eff = sMisc[10];
   if (plan.N == 0 || (int)blockIdx.x >= plan.c_eff) return;
   unsigned long long* counts = reinterpret_cast<unsigned long long*>(ws + tag_offset_floats(B * Hkv, s_cap, G, D));
-  const bool waves = GAP != 0 && gridDim.x == WAVES * 148 && plan.c_eff == (int)gridDim.x && plan.N >= 8ll * gridDim.x;
+  const bool waves = GAP != 0 && sMisc[14] != 0;
   const long long x_lo = *reinterpret_cast<const long long*>(sMisc + 4), x_hi = *reinterpret_cast<const long long*>(sMisc + 6);
   if (x_lo >= x_hi) return;                          // a share that lies inside a gap (tiny problems only)
 
@@ -609,9 +629,10 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
     // reads it after the barrier at the segment's end (the barrier that closed the last segment keeps its readers apart)
     if (tid_ == 0) {
       const long long xs = (long long)sVPref[b] + (long long)h * (pages_b + GAP) + GAP;   // first real page of this stream, virtual axis
-      const int c_first = cta_of_virtual<WAVES>(plan, waves, xs);
-      sMisc[8] = (int)blockIdx.x - c_first;
-      sMisc[9] = cta_of_virtual<WAVES>(plan, waves, xs + pages_b - 1) - c_first + 1;
+      int first, count;
+      stream_ctas<WAVES>(plan, waves, xs, pages_b, &first, &count);
+      sMisc[8] = (int)blockIdx.x - first;
+      sMisc[9] = count;
     }
 
     // ---- segment start: q operands, group sums and a clean state for this stream's heads

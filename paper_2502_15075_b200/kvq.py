@@ -71,13 +71,15 @@ _lib.kvq_debug_decode_impl.argtypes = [_P(kvq_config), _P(kvq_cache), ctypes.c_v
 _lib.kvq_debug_decode_stall_impl.argtypes = [_P(kvq_config), _P(kvq_cache), ctypes.c_void_p, ctypes.c_void_p,
                                              ctypes.c_int32, ctypes.c_float, ctypes.c_void_p, ctypes.c_size_t,
                                              ctypes.c_int64, ctypes.c_uint32, ctypes.c_int32, ctypes.c_void_p]
+_lib.kvq_debug_decode_plan.argtypes = [_P(kvq_config), ctypes.c_int32, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
+                                       ctypes.c_void_p]
 _lib.kvq_check_status.argtypes = [_P(kvq_cache), ctypes.c_void_p]
 _lib.kvq_strerror.argtypes = [ctypes.c_int]
 _lib.kvq_strerror.restype = ctypes.c_char_p
 for _f in ("kvq_page_bytes", "kvq_cache_bytes", "kvq_workspace_bytes", "kvq_quantize_append",
            "kvq_decode_attention", "kvq_decode_attention_static", "kvq_dequantize", "kvq_check_status",
            "kvq_quant_error", "kvq_bit_balance", "kvq_debug_decode_generic", "kvq_debug_decode_stall",
-           "kvq_debug_decode_impl", "kvq_debug_decode_stall_impl", "kvq_workspace_bytes_rows", "kvq_decode_attention_rows"):
+           "kvq_debug_decode_impl", "kvq_debug_decode_stall_impl", "kvq_debug_decode_plan", "kvq_workspace_bytes_rows", "kvq_decode_attention_rows"):
     getattr(_lib, _f).restype = ctypes.c_int
 
 EXPORTS = ("kvq_layout_version", "kvq_page_bytes", "kvq_cache_bytes", "kvq_workspace_bytes",
@@ -321,6 +323,18 @@ def kvq_debug_decode_stall_impl(cfg: kvq_config, cache: Cache, q: torch.Tensor, 
                                             _dtype_code(out.dtype), 0.0, workspace.data_ptr(),
                                             workspace.numel() * workspace.element_size(), int(skip_page), int(wait_us),
                                             int(impl), _stream_ptr(None)), "kvq_debug_decode_stall_impl")
+
+
+def kvq_debug_decode_plan(cfg: kvq_config, seq_len, n_rows: int = 1):
+    """Test hook, host only: the split of the fast decode kernel for a list of lengths.  Returns (partial slots per stream,
+    weighted shares?, first page of every share [CTAs + 1], (first CTA, partials) per stream)."""
+    lens = torch.tensor(list(seq_len), dtype=torch.int32)
+    assert lens.numel() == cfg.batch
+    parts = torch.zeros((cfg.batch * cfg.n_kv_heads, 2), dtype=torch.int32)
+    starts, info = torch.zeros(512, dtype=torch.int64), torch.zeros(3, dtype=torch.int32)
+    _check(_lib.kvq_debug_decode_plan(ctypes.byref(cfg), int(n_rows), lens.data_ptr(), parts.data_ptr(), starts.data_ptr(),
+                                      info.data_ptr()), "kvq_debug_decode_plan")
+    return int(info[0]), bool(info[2]), starts[:int(info[1]) + 1].numpy(), parts.numpy()
 
 
 def kvq_check_status(cache: Cache, stream: Optional[torch.cuda.Stream] = None) -> int:

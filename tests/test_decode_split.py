@@ -1,0 +1,84 @@
+"""The decode kernel's split of the pages over its CTAs: every page in one share, every stream's partials counted as the
+shares hold them, and never more of them than a stream has slots (a partial without a slot would leave the output unwritten).
+The library works the split out on the host with the kernel's own functions.  No GPU needed."""
+import random
+
+import numpy as np
+import pytest
+
+from paper_2502_15075_b200 import build as kvq_build
+
+PAGE = 128
+
+
+@pytest.fixture(scope="module")
+def kvq():
+    kvq_build.build()
+    from paper_2502_15075_b200 import kvq as mod
+    return mod
+
+
+def check_split(kvq, cfg, pages, rows=1):
+    lens = [PAGE * p - (7 * i) % PAGE if p else 0 for i, p in enumerate(pages)]        # p pages, the last one incomplete
+    slots, weighted, starts, parts = kvq.kvq_debug_decode_plan(cfg, lens, rows)
+    H, first = cfg.n_kv_heads, 0
+    assert starts[0] == 0 and starts[-1] == H * sum(pages) and np.all(np.diff(starts) >= 0)
+    for b, p in enumerate(pages):
+        for h in range(H):
+            c0, n = parts[b * H + h]
+            if p:
+                holds = np.nonzero((starts[1:] > first) & (starts[:-1] < first + p) & (starts[1:] > starts[:-1]))[0]
+                assert holds.tolist() == list(range(c0, c0 + n)), f"sequence {b} head {h}: partials {c0}+{n}, shares {holds}"
+                assert n <= slots, f"sequence {b} head {h} ({p} pages): {n} partials, {slots} slots"
+            else:
+                assert (c0, n) == (0, 0)
+            first += p
+    return weighted
+
+
+# (key bits, value bits, key axis, query heads per KV head): three weighted waves with the stream gap of token-wise and of
+# channel-wise keys, two weighted waves, equal shares
+FORMS = {"token": (4, 2, 0, 4), "channel": (4, 2, 1, 4), "eight heads": (4, 2, 0, 8), "wide pages": (8, 4, 0, 4)}
+
+
+def config(kvq, form, batch, heads, max_pages, residual=0):
+    kb, vb, axis, group = FORMS[form]
+    return kvq.make_config(batch, heads * group, heads, 128, kb, vb, 128, 128, axis, "bf16", PAGE * max_pages, residual)
+
+
+@pytest.mark.parametrize("form,heads,pages", [
+    ("channel", 10, [95, 63, 37, 57, 58, 70, 35, 110, 117, 93]),
+    ("token", 8, [472, 1024]),
+    ("token", 1, [3000, 900, 5]),
+    ("wide pages", 8, [472, 1024])])
+def test_long_streams_of_uneven_batches(kvq, form, heads, pages):
+    check_split(kvq, config(kvq, form, len(pages), heads, max(pages)), pages)
+
+
+@pytest.mark.parametrize("form", list(FORMS))
+def test_random_uneven_batches(kvq, form):
+    rng, weighted = random.Random(form), 0
+    for _ in range(1500):
+        heads, batch = rng.randint(1, 10), rng.randint(1, 24)
+        top = rng.choice([4, 40, 150, 1200])
+        pages = [rng.choice([0, 1, rng.randint(1, top), rng.randint(top // 2, top)]) for _ in range(batch)]
+        residual = rng.choice([0, 0, 128]) if form != "channel" else 0
+        if residual:            # whole blocks of the window are pages: no incomplete ones
+            pages = [max(0, p - 1) for p in pages]
+            cfg = config(kvq, form, batch, heads, top, residual)
+            slots, _, starts, parts = kvq.kvq_debug_decode_plan(cfg, [PAGE * p + 5 if p else 0 for p in pages])
+            assert parts[:, 1].max() <= slots and (sum(pages) == 0 or starts[-1] == heads * sum(pages))
+        elif sum(pages):
+            weighted += check_split(kvq, config(kvq, form, batch, heads, top), pages)
+    assert (weighted > 0) == (form != "wide pages")         # the weighted split is among what was checked
+
+
+def test_empty_caches_have_no_split(kvq):
+    slots, weighted, starts, parts = kvq.kvq_debug_decode_plan(config(kvq, "token", 3, 2, 4), [0, 0, 0])
+    assert len(starts) == 1 and not parts.any() and not weighted
+
+
+def test_a_split_is_refused_where_the_kernel_does_not_serve(kvq):
+    with pytest.raises(kvq.KvqError) as e:
+        kvq.kvq_debug_decode_plan(kvq.make_config(1, 4, 1, 128, 16, 16, 128, 128, 0, "bf16", 256), [5])
+    assert e.value.code == -2

@@ -41,3 +41,20 @@ def test_growing_logits_and_values(kvq, form, heads, T):
     for variant in ("normal", "peaked"):
         q = wl.make_q(w, batch=2, variant=variant, k=k)
         tl.assert_attention_close(tl.gpu_decode(kvq, cfg, gc, q), oc.decode(tl.bits_of(q)), mabs=tl.MAX_ABS_TOL * scale)
+
+
+@pytest.mark.parametrize("form,pages", [("channel-k4v2", [95, 63, 37, 57, 58, 70, 35, 110, 117, 93]), ("k4v2", [472, 1024])])
+def test_every_row_of_an_uneven_batch_is_written(kvq, form, pages):
+    """Full grids over uneven lengths, where a long stream's partials come close to its slots: against the plain kernel."""
+    w = FORMS[form].with_(n_q_heads=FORMS[form].n_kv_heads)
+    T, B = 128 * max(pages), len(pages)
+    cfg = tl.gpu_config_for(kvq, w, B, T)
+    gc = kvq.Cache(cfg)
+    kvq.kvq_quantize_append(cfg, gc, *wl.make_kv(w, 0, "cuda", tokens=T, batch=B))
+    gc.seq_len.copy_(torch.tensor(pages, dtype=torch.int32) * 128)
+    q = wl.make_q(w, batch=B)
+    got = tl.gpu_decode(kvq, cfg, gc, q)
+    ws = torch.empty(kvq.kvq_workspace_bytes(cfg), dtype=torch.uint8, device="cuda")
+    want = torch.empty(tuple(q.shape), dtype=torch.float32, device="cuda")
+    kvq.kvq_debug_decode_generic(cfg, gc, q.cuda(), want, ws)
+    tl.assert_attention_close(got, want.double().cpu().numpy())
