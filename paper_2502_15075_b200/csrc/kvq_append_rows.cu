@@ -17,6 +17,7 @@ constexpr int kMaxThreads = 512;
 constexpr int kChanThreads = 256;       // channel-wise keys: what a block's registers are laid out for
 
 __device__ __forceinline__ void cluster_barrier() {
+  __syncwarp();                         // (.aligned takes whole warps; loops before it end lane by lane)
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }

@@ -95,6 +95,7 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar), "l"(policy) : "memory");
 }
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
+  __syncwarp();                         // (bar.sync takes whole warps; single lanes store and count before it)
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 

@@ -595,6 +595,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       aborted = true;
       *abort_flag = 1;
       if (lane == 0) atomicOr(c.status, KVQ_STATUS_DEVICE_TIMEOUT);
+      __syncwarp();
     }
   };
   // Fold the int32 accumulators into 64-bit sums and clear them (the sum of code terms and the sum of zero-points that meets it at
