@@ -572,8 +572,9 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   int Oi[NTV][MTW][4];         // PV accumulators: n-tiles 2 nh, 2 nh + 1 hold limbs (3, 2) and (1, 0) of head tid + 4 nh
   double acc[NH][MTW][2];      // what has been folded out of them: channel 16 (MTW warp + i) + 8 r + gid
   constexpr float PONE = (float)(1u << (kPBits - 1)) * 2.0f;     // 2^PBITS
-  // sscale = 2^PBITS / s_lim, s_lim a power of two above every value scale folded into the weights so far (2^-40 at first)
-  float sscale = PONE / 9.094947e-13f;
+  // sscale = 2^PBITS / s_lim, s_lim a power of two above every value scale of the stream folded into the weights so far (2^-40 at first)
+  constexpr float SSCALE0 = PONE / 9.094947e-13f;
+  float sscale = SSCALE0;
   int page_no = 0, stage = 0;
   uint32_t phase = 0;
   bool aborted = false;
@@ -636,7 +637,9 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       sMisc[9] = count;
     }
 
-    // ---- segment start: q operands, group sums and a clean state for this stream's heads
+    // ---- segment start: q operands, group sums and a clean state for this stream's heads (the scale limit too: under one
+    // of another stream with larger values this stream's weights would vanish)
+    sscale = SSCALE0;
 #pragma unroll
     for (int nh = 0; nh < NH; ++nh) {
       const int hb = (gid >> 1) + 4 * nh;                          // head of this lane's operand column

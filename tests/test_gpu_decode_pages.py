@@ -1,6 +1,7 @@
 """Decode attention where the fast kernel's pages and blocks end: lengths around a 32-token block and a 128-token page, keys and
 values that keep growing (the common reference and the scale limit move on every page), every number of heads it
 serves, against the fp64 oracle on the same codes."""
+import numpy as np
 import pytest
 import torch
 
@@ -58,3 +59,21 @@ def test_every_row_of_an_uneven_batch_is_written(kvq, form, pages):
     want = torch.empty(tuple(q.shape), dtype=torch.float32, device="cuda")
     kvq.kvq_debug_decode_generic(cfg, gc, q.cuda(), want, ws)
     tl.assert_attention_close(got, want.double().cpu().numpy())
+
+
+@pytest.mark.parametrize("form,heads", [("k4v2", 1), ("k4v4", 4), ("k4v2-g64", 1), ("k4v2", 8), ("channel-k4v2", 1)])
+def test_streams_of_very_different_values_share_a_cta(kvq, form, heads):
+    """More streams than CTAs, neighbours' values a factor of 2^24 apart: a stream's weights are fixed point below the largest
+    value scale of that stream, not of the one its CTA served before it."""
+    H, B, T = 8, 75, 200
+    w = FORMS[form].with_(n_kv_heads=H, n_q_heads=H * heads)
+    k, v = wl.make_kv(w, tokens=T, batch=B)
+    v = (v.float() * torch.where(torch.arange(B * H) % 2 == 0, 2.0 ** 12, 2.0 ** -12).view(B, H, 1, 1)).to(w.torch_dtype)
+    cfg = tl.gpu_config_for(kvq, w, B, 256)
+    gc = kvq.Cache(cfg)
+    kvq.kvq_quantize_append(cfg, gc, k.cuda(), v.cuda())
+    q = wl.make_q(w, batch=B)
+    got = tl.gpu_decode(kvq, cfg, gc, q).reshape(B * H, -1)
+    want = tl.oracle_on_gpu_codes(gc, w).decode(tl.bits_of(q)).reshape(B * H, -1)
+    err = np.linalg.norm(got - want, axis=1) / np.linalg.norm(want, axis=1)
+    assert err.max() <= tl.REL_L2_TOL, f"stream {err.argmax()}: rel-L2 {err.max():.2e}"
