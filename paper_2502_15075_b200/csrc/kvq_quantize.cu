@@ -318,17 +318,17 @@ __device__ __forceinline__ void quantize_task_rotated(const RowSrc& rsrc, int gs
         for (int i = 0; i < 8; ++i) x[f][i] = __fmaf_rn(sm, x[f][i], __shfl_xor_sync(FULL, x[f][i], 2 * hm));
       }
     }
+    // (from the first value on, as everywhere: a row of NaN has the same parameters in every kernel)
     float mn[NSET], mx[NSET];
-#pragma unroll
-    for (int e = 0; e < NSET; ++e) { mn[e] = INFINITY; mx[e] = -INFINITY; }
 #pragma unroll
     for (int f = 0; f < FPB; ++f) {
       const int e = NSET == 2 ? f >> 1 : 0;
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         x[f][i] = __fmul_rn(x[f][i], inv_sqrt_dim<D>());
-        mn[e] = fminf(mn[e], x[f][i]);
-        mx[e] = fmaxf(mx[e], x[f][i]);
+        const bool first = i == 0 && f == (FPB / NSET) * e;
+        mn[e] = first ? x[f][i] : fminf(mn[e], x[f][i]);
+        mx[e] = first ? x[f][i] : fmaxf(mx[e], x[f][i]);
       }
     }
     if constexpr (NSET == 2) {

@@ -94,3 +94,23 @@ RUNS = {"odd": [131, 70, 259], "exact": [256, 160], "inside": [200, 65, 66]}    
 def test_runs_of_tokens(kvq, kb, vb, D, gk, gv, dtype, runs, form):
     w = wl.LLAMA_8B.with_(n_kv_heads=2, n_q_heads=2, head_dim=D, kb=kb, vb=vb, gk=gk, gv=gv, dtype=dtype)
     check(kvq, w, 2, RUNS[runs], SIGNS[:D] if "rotated" in form else None, 64 if "window" in form else 0, strided=runs == "odd")
+
+
+@pytest.mark.parametrize("kb", [2, 4, 8])
+@pytest.mark.parametrize("rotated", [False, True])
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+def test_a_nan_row_gives_the_same_bytes_at_once_and_in_pieces(kvq, kb, rotated, dtype):
+    """Non-finite inputs are outside of what the quantizer defines, but the bytes must not depend on how many tokens a call has."""
+    w = wl.LLAMA_8B.with_(n_kv_heads=2, n_q_heads=2, kb=kb, dtype=dtype)
+    k, v = wl.make_kv(w, tokens=140, batch=1)
+    for t in (3, 70, 139):
+        k[:, :, t, 17] = float("nan")
+    k[:, 0, 40] = v[:, 1, 41] = float("nan")
+    pages = []
+    for chunks in ([140], [64, 12, 64]):
+        cfg = tl.gpu_config_for(kvq, w, 1, 256)
+        gc = kvq.Cache(cfg, k_signs=torch.from_numpy(SIGNS) if rotated else None)
+        for part in torch.split(torch.arange(140), chunks):
+            kvq.kvq_quantize_append(cfg, gc, k[:, :, part].cuda(), v[:, :, part].cuda())
+        pages.append(gc.pages.cpu())
+    assert torch.equal(*pages)
