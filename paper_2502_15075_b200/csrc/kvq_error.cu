@@ -1,7 +1,7 @@
 // kvq_quant_error: the reconstruction-error analysis of the cache quantizer in one pass over new K and V
 // (Sec. 4.1 experiment (i); MSE(A, A^) = ||A - A^||_F^2 / entries, App. B.4).  Every token row is quantized in
 // registers exactly as kvq_quantize_append would (same group parameters, same codes), reconstructed as
-// x^ = z + code s and compared with the input; nothing packed is written.  Per (batch, kv-head)
+// x^ = fmaf(code, scale, zero) and compared with the input; nothing packed is written.  Per (batch, kv-head)
 // the kernel adds sum x^2 and sum (x - x^)^2 of keys and of values to four doubles.
 #include <math.h>
 
@@ -94,10 +94,9 @@ quant_error_kernel(Geom g, const uint16_t* __restrict__ k, const uint16_t* __res
         for (int e = 0; e < 2; ++e) {
           const float x = e ? x2.y : x2.x;
           s2 = fmaf(x, x, s2);
-          const float y = __fsub_rn(x, zi);
-          const float r = __fmaf_rn(__saturatef(__fmul_rn(y, ii)), up, 12582912.0f);
+          const float r = __fmaf_rn(__saturatef(__fmul_rn(__fsub_rn(x, zi), ii)), up, 12582912.0f);
           const float code = fminf(__fsub_rn(r, 12582912.0f), qmax);
-          const float d = __fmaf_rn(-code, si, y);             // x - (z + code s), rounded at the size of x - z
+          const float d = __fsub_rn(x, __fmaf_rn(code, si, zi));      // (the rounding of x^ belongs to the error)
           se = fmaf(d, d, se);
         }
       }

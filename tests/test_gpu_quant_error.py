@@ -92,3 +92,19 @@ def test_error_sums_at_the_ends_of_the_row_turns(kvq, T, D, gk, gv, dtype):
         kvq.kvq_quant_error(cfg, kd, vd, sums)
         want = oe.quant_error_sums(tl.bits_of(k), tl.bits_of(v), w.dtype, w.kb, w.vb, w.gk, w.gv)
         assert np.allclose(sums.cpu().numpy(), want, rtol=1e-5, atol=0.0)
+
+
+@pytest.mark.parametrize("D,gk,gv", [(128, 128, 32), (64, 32, 64)])
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+def test_error_sums_of_values_far_from_zero(kvq, D, gk, gv, dtype):
+    """A group far from zero for its range: the fp32 rounding of the reconstructed value is then part of the error, as the
+    definition has it.  The fp32 operations are the oracle's own; only the squares' sums differ (8 elements in fp32: below 1e-6)."""
+    for kb, vb in ((8, 4), (6, 8)) if D == 128 else ((8, 4),):
+        w = wl.LLAMA_8B.with_(n_kv_heads=2, n_q_heads=2, head_dim=D, gk=gk, gv=gv, dtype=dtype, kb=kb, vb=vb)
+        k, v = wl.make_kv(w, tokens=130, batch=1)
+        k, v = ((x.float() + 1000.0).to(w.torch_dtype) for x in (k, v))
+        cfg = tl.gpu_config_for(kvq, w, 1, 128)
+        sums = torch.zeros((1, 2, 4), dtype=torch.float64, device="cuda")
+        kvq.kvq_quant_error(cfg, k.cuda(), v.cuda(), sums)
+        want = oe.quant_error_sums(tl.bits_of(k), tl.bits_of(v), w.dtype, w.kb, w.vb, w.gk, w.gv)
+        assert np.allclose(sums.cpu().numpy(), want, rtol=1e-5, atol=0.0), (sums.cpu().numpy() / want - 1)
