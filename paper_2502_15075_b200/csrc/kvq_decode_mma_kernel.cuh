@@ -399,14 +399,8 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       }
     }
   }
-  // the plan lives on the virtual axis (pages + a gap in front of every stream)
-  FlatPlan plan;
-  plan.N = sVPref[B];
-  plan.c_eff = sMisc[10];
-  if (plan.N == 0 || (int)blockIdx.x >= plan.c_eff) return;
-  unsigned long long* counts = reinterpret_cast<unsigned long long*>(ws + tag_offset_floats(B * Hkv, s_cap, G, D));
-  const bool waves = GAP != 0 && sMisc[14] != 0;
-  const long long x_lo = *reinterpret_cast<const long long*>(sMisc + 4), x_hi = *reinterpret_cast<const long long*>(sMisc + 6);
+  if (sVPref[B] == 0 || (int)blockIdx.x >= sMisc[10]) return;
+  const int x_lo = (int)*reinterpret_cast<const long long*>(sMisc + 4), x_hi = (int)*reinterpret_cast<const long long*>(sMisc + 6);
   if (x_lo >= x_hi) return;                          // a share that lies inside a gap (tiny problems only)
 
   // ---- cursor: first page of this CTA -> (b, h, page)
@@ -425,7 +419,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       uint32_t phase = 1;                // parity of the previous round of `empty`
       bool ok = true;
       const uint64_t policy = l2_evict_first_policy();
-      for (long long x = x_lo; x < x_hi; ++x, ++it) {
+      for (int x = x_lo; x < x_hi; ++x, ++it) {
         if (it >= stages) {
           ok = mbar_wait(bar0 + 8 * (stages + stage), phase, wait_ns);
           if (!ok || *abort_flag) { ok = false; break; }
@@ -474,7 +468,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       float qv[NH][NR][4];
       float amaxB[NH];
       int cur_b = -1, cur_h = -1;
-      for (long long x = x_lo; x < x_hi; ++x) {
+      for (int x = x_lo; x < x_hi; ++x) {
         if (b != cur_b || h != cur_h) {          // a new stream: its queries
           cur_b = b; cur_h = h;
 #pragma unroll
@@ -619,8 +613,8 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
     }
   };
 
-  for (long long x = x_lo; x < x_hi;) {
-    const int seg_pages = (int)min((long long)(pages_b - page), x_hi - x);
+  for (int x = x_lo; x < x_hi;) {
+    const int seg_pages = min(pages_b - page, x_hi - x);
     const int n_all = clamped_len(c.seq_len, b, g.capacity);
     const int n_tok = g.R ? (n_all / g.R) * g.R : n_all;          // tokens of the sequence that are in the pages
     // a block is unmasked when all of its 32 tokens exist and every query row may see them (several causal rows:
@@ -630,6 +624,10 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
     // which of the stream's partials this CTA writes, and how many there are: one thread works it out now, everybody
     // reads it after the barrier at the segment's end (the barrier that closed the last segment keeps its readers apart)
     if (tid_ == 0) {
+      FlatPlan plan;                         // on the virtual axis (pages + a gap in front of every stream); kept in shared memory
+      plan.N = sVPref[B];
+      plan.c_eff = sMisc[10];
+      const bool waves = GAP != 0 && sMisc[14] != 0;
       const long long xs = (long long)sVPref[b] + (long long)h * (pages_b + GAP) + GAP;   // first real page of this stream, virtual axis
       int first, count;
       stream_ctas<WAVES>(plan, waves, xs, pages_b, &first, &count);
@@ -1033,6 +1031,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
         if (!direct) {
           __threadfence();
           named_bar_sync(1, NCONS);
+          unsigned long long* counts = reinterpret_cast<unsigned long long*>(ws + tag_offset_floats(B * Hkv, s_cap, G, D));
           if (tid_ == 0) *n_published = (int)tagged_count(counts + stream, id40);
           named_bar_sync(1, NCONS);
           if (*n_published == n_part) {
