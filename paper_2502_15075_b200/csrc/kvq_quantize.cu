@@ -10,7 +10,7 @@
 // word, is then assembled in that lane's registers and stored directly - no shared memory, no
 // atomics, no read-modify-write; a token that is not new is simply not stored (byte stores for
 // values).  Group minima and maxima are reduced with a few shuffles between the lanes of a row.
-// The kernel is bound by reading the 16-bit inputs from HBM.
+// Bound by instruction issue and load latency in long calls, by fetching instructions in short ones.
 #include "kvq_quantize.cuh"
 
 namespace kvq {
@@ -74,8 +74,11 @@ __device__ __forceinline__ float piece_value(const uint4& r, int e) {
 // with a shuffle reduce-scatter, so that the group parameters (two divisions) are computed once per group rather than once
 // per lane, and are then broadcast to the lanes of the group.  Minimum and negated maximum travel as one pair of the 16-bit type,
 // the clamp is the saturation of a multiplication: 10.6 instructions per element instead of 14.  K and V of 64 streams x
-// 32,768 tokens (K4V2, 1.29 GB) 333 -> 275 us; in a replayed graph 335 -> 250 us at five CTAs per SM (four 259, three 298, six 270: registers spill);
-// bound by issue (60 %) and load latency.  8-byte pieces at 2 bits (half the registers, twice the loads): 276 us.
+// 32,768 tokens (K4V2, 1.29 GB) 333 -> 272 us; in a replayed graph 335 -> 250 us at five CTAs per SM (four 259, three 298, six 270;
+// registers spill at five as well, 168 / 368 bytes); bound by issue (60 %) and load latency.  8-byte pieces at 2 bits (half
+// the registers, twice the loads): 276 us.  A short call is bound by fetching instructions (6.6 of 10 cycles between two of a warp), so
+// a value word's two ways of leaving, whole or byte by byte, are one branch behind all eight words: a branch per word made the
+// partial tasks longer (8 streams x 500 tokens K4V2 11.8 -> 8.7 us, K2V4 11.1 -> 8.3, head_dim 64 12.2 -> 8.7; 64 x 2,047 19.5 -> 18.9).
 template <int BITS, bool IS_V, int D, int DTYPE, bool FULLBLK>
 __device__ __forceinline__ void quantize_task(const RowSrc& rsrc, int gsz, int lo, int hi, uint8_t* __restrict__ codes,
                                               uint32_t* __restrict__ meta_out, int lane) {
@@ -214,24 +217,29 @@ __device__ __forceinline__ void quantize_task(const RowSrc& rsrc, int gsz, int l
       const int cmb = pass * RS + rs;
       uint8_t* wbase = codes + (size_t)(cmb >> 3) * (4 * D * BITS) + mw * 512 + (cmb & 3) * 16 +
                        4 * (2 * rh + ((cmb >> 2) & 1));
-      const bool all = FULLBLK || (valid[0] && valid[1] && valid[2] && valid[3]);
+      uint32_t w[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        uint32_t w = 0;
+        w[i] = 0;
 #pragma unroll
         for (int f = FPB - 1; f >= 0; --f) {
           const int e = NSET == 2 ? f >> 1 : 0;
           float x[4];
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) x[kk] = piece_value<DTYPE>(raw[kk][f], i);
-          w = w * (1u << BITS) + code_word4<BITS>(x, z[e], inv[e]);
+          w[i] = w[i] * (1u << BITS) + code_word4<BITS>(x, z[e], inv[e]);
         }
-        if (all) {
-          *reinterpret_cast<uint32_t*>(wbase + 64 * i) = w;
-        } else {
+      }
+      if (FULLBLK || (valid[0] && valid[1] && valid[2] && valid[3])) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            if (valid[kk]) wbase[64 * i + kk] = (uint8_t)(w >> (8 * kk));
+        for (int i = 0; i < 8; ++i) *reinterpret_cast<uint32_t*>(wbase + 64 * i) = w[i];
+      } else {
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+          if (valid[kk]) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) wbase[64 * i + kk] = (uint8_t)(w[i] >> (8 * kk));
+          }
         }
       }
     }
