@@ -77,3 +77,25 @@ def test_streams_of_very_different_values_share_a_cta(kvq, form, heads):
     want = tl.oracle_on_gpu_codes(gc, w).decode(tl.bits_of(q)).reshape(B * H, -1)
     err = np.linalg.norm(got - want, axis=1) / np.linalg.norm(want, axis=1)
     assert err.max() <= tl.REL_L2_TOL, f"stream {err.argmax()}: rel-L2 {err.max():.2e}"
+
+
+def test_value_sums_over_more_pages_than_an_integer_accumulator_holds(kvq):
+    """Over 350 pages per CTA of equal weights and largest codes: without the fold every 128 pages the 32-bit sums would overflow
+    (the second weight byte is 254, the upper code field 192: 344 pages of 128 tokens).  All values of a head are equal, so the
+    output is that value whatever the weights; the folds also fall at different distances behind a change of stream."""
+    H, P = 8, 22000
+    cfg = kvq.make_config(1, H, H, 64, 4, 2, 64, 64, 0, "fp16", 128 * P)
+    starts = kvq.kvq_debug_decode_plan(cfg, [128 * P])[2]
+    assert np.diff(starts).min() > 344
+    gc = kvq.Cache(cfg)
+    pages = gc.pages_view()                                  # key codes and metadata stay zero: every logit is 0
+    k_bytes, v_codes = 128 * 64 // 2 + 128 * 4, 128 * 64 // 4
+    pages[..., k_bytes:k_bytes + v_codes] = 0xFF             # code 3 everywhere
+    scales = [0x3FFF, 0x3BFF, 0x3FFF, 0x33FF, 0x3FFF, 0x3FFF, 0x2FFF, 0x3FFF]     # 1.999 and smaller ones, mantissas all ones
+    for h, s in enumerate(scales):
+        meta = pages[0, h, :, k_bytes + v_codes:].view(P, 128, 4)
+        meta[..., 0], meta[..., 1] = s & 255, s >> 8         # (zero-points stay 0)
+    gc.seq_len.fill_(128 * P)
+    got = tl.gpu_decode(kvq, cfg, gc, torch.ones((1, H, 64), dtype=torch.float16))[0]
+    want = 3.0 * torch.tensor(scales, dtype=torch.int16).view(torch.float16).double().numpy()
+    assert np.allclose(got, want[:, None], rtol=1e-5, atol=0.0)
