@@ -5,8 +5,8 @@
 // (cluster barrier) one thread stores the new one.  A token row is spread over D / 8 lanes, eight consecutive channels each; lanes whose
 // codes share bytes merge them with shuffles.  The call is bound by latency, not by bytes: the code is kept short and is
 // the same for every width, because in a step the instructions come from L2 each time.  The task kernels of
-// kvq_quantize.cu (32 tokens a warp, several thousand instructions) and a launch for the lengths take 6 to 8 us for one token
-// (10 to 11 with channel-wise keys), this kernel 2.5 to 3 (4).
+// kvq_quantize.cu (32 tokens a warp, several thousand instructions) and a launch for the lengths take 7 to 8 us for one token
+// (9 to 10 with channel-wise keys), this kernel 3.0 to 3.5 (4).
 #include "kvq_quantize.cuh"
 
 namespace kvq {
@@ -14,6 +14,7 @@ namespace kvq {
 namespace {
 
 constexpr int kMaxThreads = 512;
+inline int heads_per_cta(int n_kv_heads) { return (n_kv_heads + 7) / 8; }
 constexpr int kChanThreads = 256;       // channel-wise keys: what a block's registers are laid out for
 
 __device__ __forceinline__ void cluster_barrier() {
@@ -139,20 +140,30 @@ append_rows_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, cons
 
 }  // namespace
 
-// Up to 64 tokens at head_dim 128 and 128 at head_dim 64.  Both sides measured, one call alone on the GPU, rows / tasks + lengths:
-// 8 KV heads x 16 sequences, head_dim 128: 8 tokens 3.2 / 7.9 us, 32 tokens 6.0 / 7.8, 64 tokens 9.4 / 13.6, 128 tokens 16.9 / 17.4,
-// 256 tokens 31 / 18 (one sequence 64 tokens 6.5 / 7.7, 128 tokens 10.7 / 9.1); channel-wise keys, 10 heads x 32 sequences:
-// 64 tokens 13.4 / 14.8, 128 tokens 25.4 / 23.4; head_dim 64, 8 x 8: 128 tokens 6.6 / 11.6, 256 tokens 10.8 / 11.8 (one
-// sequence 10.5 / 7.0).  A channel-wise append of at most 128 tokens completes at most one block.
-bool append_rows_serves(const Geom& g, int t_new) {
+// A sequence has at most eight CTAs, so the time goes with the rows of one of them: its KV heads x new tokens.  Both sides measured
+// from an uneven position, one call alone on the GPU, rows / tasks + lengths, for 1 and 16 sequences (K4V2, head_dim 128):
+//    8 KV heads:  64 tokens 7.4 / 8.7 us, 10.3 / 13.4;   96 tokens 9.5 / 8.8, 14.0 / 13.5
+//   16 KV heads:  32 tokens 7.3 / 8.3, 10.2 / 9.8;       48 tokens 9.5 / 8.7, 13.9 / 12.5
+//   32 KV heads:  16 tokens 7.2 / 7.8, 10.2 / 13.1;      32 tokens 11.7 / 8.0, 17.6 / 14.0
+//   64 KV heads:   8 tokens 7.0 / 7.8, 10.0 / 17.3;      16 tokens 11.2 / 8.0, 17.2 / 18.3
+// so 64 rows a CTA at head_dim 128 and 128 at head_dim 64 (16 heads, 64 tokens 7.2 / 7.5; 128 tokens 11.1 / 8.7).  Rotated keys and a
+// residual window cost more a row: 40 rows beyond eight heads (16 heads, 16 tokens rotated 5.8 / 7.1, 8.1 / 8.0, 32 tokens
+// 8.8 / 8.3, 13.2 / 9.4; with a window 16 tokens 6.2 / 7.2, 8.5 / 8.2, 32 tokens 8.8 / 8.8, 13.1 / 10.2).  Channel-wise keys also
+// pay for a block a head (10 heads, 1 and 32 sequences: 48 tokens 10.7 / 12.7, 14.5 / 14.8, 64 tokens 13.8 / 12.9, 17.5 / 16.3; 32
+// heads: 16 tokens 9.0 / 9.4, 11.5 / 18.1, 32 tokens 14.9 / 10.6, 19.4 / 21.8; 64 heads: 4 tokens 7.5 / 9.6, 8 tokens 11.4 / 9.7).
+// An append of at most 64 tokens of channel-wise keys completes at most one block.
+bool append_rows_serves(const Geom& g, bool rotated, int t_new) {
   auto width = [](int b) { return b == 2 || b == 4 || b == 8; };
   if (t_new > 64 * 128 / g.D || !width(g.kb) || !width(g.vb)) return false;
-  return g.k_axis == 0 || (g.D == 128 && g.kb != 2);
+  const long long heads = heads_per_cta(g.Hkv);
+  if (g.k_axis == 1) return g.D == 128 && g.kb != 2 && heads * (t_new + 12) <= 128;
+  const int limit = heads > 1 && (rotated || g.R) ? 40 : 64;
+  return heads * t_new * g.D <= limit * 128;
 }
 
 int launch_append_rows(const Geom& g, const CachePtrs& c, const void* k_new, const void* v_new, int64_t sb, int64_t sh,
                        int64_t st, int t_new, cudaStream_t stream) {
-  const int per_cta = (g.Hkv + 7) / 8, ranks = (g.Hkv + per_cta - 1) / per_cta;        // at most 8 CTAs, evenly loaded
+  const int per_cta = heads_per_cta(g.Hkv), ranks = (g.Hkv + per_cta - 1) / per_cta;        // at most 8 CTAs, evenly loaded
   const bool chan = g.k_axis == 1, rot = c.k_signs != nullptr;
   int threads = per_cta * 2 * (t_new + g.R) * (g.D / 8);
   threads = chan ? kChanThreads : threads > kMaxThreads ? kMaxThreads : (threads + 31) / 32 * 32;

@@ -9,7 +9,7 @@ int launch_quantize_append(const Geom& g, const CachePtrs& c, const void* k_new,
                            int64_t sb, int64_t sh, int64_t st, int t_new, cudaStream_t stream);
 
 // the append of a few tokens (kvq_append_rows.cu): whole call in one launch
-bool append_rows_serves(const Geom& g, int t_new);
+bool append_rows_serves(const Geom& g, bool rotated, int t_new);
 int launch_append_rows(const Geom& g, const CachePtrs& c, const void* k_new, const void* v_new, int64_t sb, int64_t sh,
                        int64_t st, int t_new, cudaStream_t stream);
 

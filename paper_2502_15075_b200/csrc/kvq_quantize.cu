@@ -702,7 +702,7 @@ __global__ void bump_seq_len_kernel(Geom g, CachePtrs c, int t_new) {
 
 int launch_quantize_append(const Geom& g, const CachePtrs& c, const void* k_new, const void* v_new,
                            int64_t sb, int64_t sh, int64_t st, int t_new, cudaStream_t stream) {
-  if (append_rows_serves(g, t_new)) return launch_append_rows(g, c, k_new, v_new, sb, sh, st, t_new, stream);
+  if (append_rows_serves(g, c.k_signs != nullptr, t_new)) return launch_append_rows(g, c, k_new, v_new, sb, sh, st, t_new, stream);
   const uint16_t* k = static_cast<const uint16_t*>(k_new);
   const uint16_t* v = static_cast<const uint16_t*>(v_new);
   // warp tasks touched per stream: at most ceil(t_new / 32) + 1; one warp per task, CTAs stride over them

@@ -114,3 +114,49 @@ def test_a_nan_row_gives_the_same_bytes_at_once_and_in_pieces(kvq, kb, rotated, 
             kvq.kvq_quantize_append(cfg, gc, k[:, :, part].cuda(), v[:, :, part].cuda())
         pages.append(gc.pages.cpu())
     assert torch.equal(*pages)
+
+
+# appends of at most 64 tokens that complete a block and leave tokens behind it, or end with it
+BLOCKS = {"behind": [120, 20, 64, 60], "behind and ahead": [100, 64, 1, 64], "exact": [64, 64, 1, 63, 64]}
+
+
+@pytest.mark.parametrize("chunks", list(BLOCKS))
+@pytest.mark.parametrize("heads", [9, 10])              # two heads for some or all CTAs of a cluster: the scratch is used again
+@pytest.mark.parametrize("kb", [4, 8])
+@pytest.mark.parametrize("rotated", [False, True])
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+def test_short_appends_of_channelwise_keys_over_blocks(kvq, chunks, heads, kb, rotated, dtype):
+    w = wl.SHAPED_14B.with_(n_kv_heads=heads, n_q_heads=heads, kb=kb, dtype=dtype)
+    check(kvq, w, 2, BLOCKS[chunks], SIGNS if rotated else None, strided=chunks == "exact")
+
+
+@pytest.mark.parametrize("D,heads,n", [(128, 1, 64), (64, 8, 128), (128, 16, 32), (64, 16, 64), (128, 24, 21)])
+@pytest.mark.parametrize("form", ["plain", "rotated", "window"])
+def test_both_sides_of_the_short_append(kvq, D, heads, n, form):
+    """The largest append that takes one launch and the one beyond it, for few and many heads."""
+    if form != "plain" and heads > 8:
+        n = n * 40 // 64
+    w = wl.LLAMA_8B.with_(n_kv_heads=heads, n_q_heads=heads, head_dim=D, gk=64, gv=64)
+    check(kvq, w, 1, [13, n, n + 1, 3, n, n + 1], SIGNS[:D] if form == "rotated" else None, 64 if form == "window" else 0)
+
+
+@pytest.mark.parametrize("heads,n", [(8, 64), (10, 52), (17, 30)])
+def test_both_sides_of_the_short_append_of_channelwise_keys(kvq, heads, n):
+    w = wl.SHAPED_14B.with_(n_kv_heads=heads, n_q_heads=heads)
+    check(kvq, w, 1, [13, n, n + 1, 3, n, n + 1])
+
+
+@pytest.mark.parametrize("shape,kb", [("channel", 4), ("channel", 8), ("token", 4)])
+@pytest.mark.parametrize("n", [1, 20, 64, 90])
+def test_append_to_sequences_of_different_lengths(kvq, shape, kb, n):
+    """One sequence completes a block and leaves tokens behind it, one ends with the block, one stays inside it."""
+    w = (wl.SHAPED_14B if shape == "channel" else wl.LLAMA_8B).with_(n_kv_heads=9, n_q_heads=9, kb=kb)
+    k, v = edge_values(w, 120 + n, 3, 5)
+    cfg, gc, oc = tl.build_both(kvq, w, k[:, :, :120], v[:, :, :120], [120], 256)
+    lens = [120, 128 - n, 3]
+    gc.seq_len.copy_(torch.tensor(lens, dtype=torch.int32))
+    oc.seq_len[:] = lens
+    kvq.kvq_quantize_append(cfg, gc, k[:, :, 120:].cuda(), v[:, :, 120:].cuda())
+    oc.append(tl.bits_of(k)[:, :, 120:], tl.bits_of(v)[:, :, 120:])
+    assert kvq.kvq_check_status(gc) == 0
+    tl.assert_caches_equal(gc, oc)
