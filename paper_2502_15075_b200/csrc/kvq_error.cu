@@ -5,7 +5,7 @@
 // the kernel adds sum x^2 and sum (x - x^)^2 of keys and of values to four doubles.
 #include <math.h>
 
-#include "kvq_internal.h"
+#include "kvq_quantize.cuh"
 
 namespace kvq {
 
@@ -13,24 +13,14 @@ namespace {
 
 constexpr int kThreads = 128;
 constexpr int kPerSm = 12;
-constexpr uint32_t FULL = 0xffffffffu;
-
-template <int DTYPE> struct Pair16 { using type = __half2; };
-template <> struct Pair16<KVQ_BF16> { using type = __nv_bfloat162; };
-__device__ __forceinline__ __half2 lows(__half2 a, __half2 b) { return __lows2half2(a, b); }
-__device__ __forceinline__ __half2 highs(__half2 a, __half2 b) { return __highs2half2(a, b); }
-__device__ __forceinline__ __nv_bfloat162 lows(__nv_bfloat162 a, __nv_bfloat162 b) { return __lows2bfloat162(a, b); }
-__device__ __forceinline__ __nv_bfloat162 highs(__nv_bfloat162 a, __nv_bfloat162 b) { return __highs2bfloat162(a, b); }
-__device__ __forceinline__ float2 pair_to_f32(__half2 h) { return __half22float2(h); }
-__device__ __forceinline__ float2 pair_to_f32(__nv_bfloat162 h) { return __bfloat1622float2(h); }
 
 // One side (keys: blockIdx.z = 0, values: 1).  A row of D channels is spread over D/8 lanes, 8 channels each, and a lane
 // takes the same channels of four rows at a time.  Minimum and negated maximum of a group travel as one pair of the 16-bit
 // input type (exact), reduced so that every lane of a group ends up with one of the four rows: the parameters (two
 // divisions) are made once per lane and row and fetched from there.  The codes are rounded by the fused multiply-add of the
-// magic number after a saturating multiplication (see code_word4).  Bound by arithmetic (about 17 instructions per
+// magic number after a saturating multiplication (see code_word4).  Bound by arithmetic (about 18 instructions per
 // element, 0.66 issued per cycle) and by whole waves: 20 M elements (80 streams x 1000 tokens x 128, K and V) 23 us with parameters
-// per lane and 30 instructions per element, 15.6 us now; eight rows per lane were no faster (fewer, longer turns).
+// per lane and 30 instructions per element, 16.3 us now; eight rows per lane were no faster (fewer, longer turns).
 template <int D, int DTYPE>
 __global__ void __launch_bounds__(kThreads, kPerSm)
 quant_error_kernel(Geom g, const uint16_t* __restrict__ k, const uint16_t* __restrict__ v, int64_t sb, int64_t sh,
@@ -60,11 +50,7 @@ quant_error_kernel(Geom g, const uint16_t* __restrict__ k, const uint16_t* __res
     if (bits != 16) {
       H2 m[ROWS];                                        // (minimum, - maximum) of the lane's channels
 #pragma unroll
-      for (int i = 0; i < ROWS; ++i) {
-        const H2* p = reinterpret_cast<const H2*>(&raw[i]);
-        const H2 lo = __hmin2(__hmin2(p[0], p[1]), __hmin2(p[2], p[3])), hi = __hmax2(__hmax2(p[0], p[1]), __hmax2(p[2], p[3]));
-        m[i] = __hmin2(lows(lo, __hneg2(hi)), highs(lo, __hneg2(hi)));
-      }
+      for (int i = 0; i < ROWS; ++i) m[i] = minmax8<DTYPE>(raw[i]);
       auto swap = [](H2 x, int off) {
         const uint32_t o = __shfl_xor_sync(FULL, *reinterpret_cast<uint32_t*>(&x), off);
         return *reinterpret_cast<const H2*>(&o);
@@ -94,8 +80,8 @@ quant_error_kernel(Geom g, const uint16_t* __restrict__ k, const uint16_t* __res
         for (int e = 0; e < 2; ++e) {
           const float x = e ? x2.y : x2.x;
           s2 = fmaf(x, x, s2);
-          const float r = __fmaf_rn(__saturatef(__fmul_rn(__fsub_rn(x, zi), ii)), up, 12582912.0f);
-          const float code = fminf(__fsub_rn(r, 12582912.0f), qmax);
+          const float r = __fmaf_rn(__saturatef(__fmul_rn(__fsub_rn(x, zi), ii)), up, kRoundMagic);
+          const float code = fminf(__fsub_rn(r, kRoundMagic), qmax);
           const float d = __fsub_rn(x, __fmaf_rn(code, si, zi));      // (the rounding of x^ belongs to the error)
           se = fmaf(d, d, se);
         }
@@ -127,7 +113,8 @@ int launch_quant_error(const Geom& g, const void* k, const void* v, int64_t sb, 
   const int streams = g.B * g.Hkv;
   const uint16_t* kk = static_cast<const uint16_t*>(k);
   const uint16_t* vv = static_cast<const uint16_t*>(v);
-  // one wave of CTAs, no more of them than turns of rows (12 CTAs of 128 threads per SM 188 us for twelve calls, 8: 198 us)
+  // one wave of CTAs, no more of them than turns of rows (twelve calls when this was chosen: 12 CTAs of 128 threads per SM
+  // 188 us, 8: 198 us)
   const int step = (kThreads / 32) * (32 / (g.D / 8)) * 4;
   int gx = (n_tokens + step - 1) / step, want = 148 * kPerSm / (2 * streams);
   if (want < 1) want = 1;

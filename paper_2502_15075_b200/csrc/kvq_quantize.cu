@@ -37,26 +37,6 @@ struct RowSrc {
 // that make up a word of value codes.
 __host__ __device__ constexpr int task_tokens(int D, int bits) { return (D == 64 && bits == 2) ? 64 : 32; }
 
-// Two 16-bit inputs as a packed pair of their own type, for exact minima and maxima.
-template <int DTYPE> struct Pair16 { using type = __half2; };
-template <> struct Pair16<KVQ_BF16> { using type = __nv_bfloat162; };
-__device__ __forceinline__ float2 pair_to_f32(__half2 h) { return __half22float2(h); }
-__device__ __forceinline__ float2 pair_to_f32(__nv_bfloat162 h) { return __bfloat1622float2(h); }
-__device__ __forceinline__ __half2 lows(__half2 a, __half2 b) { return __lows2half2(a, b); }
-__device__ __forceinline__ __half2 highs(__half2 a, __half2 b) { return __highs2half2(a, b); }
-__device__ __forceinline__ __nv_bfloat162 lows(__nv_bfloat162 a, __nv_bfloat162 b) { return __lows2bfloat162(a, b); }
-__device__ __forceinline__ __nv_bfloat162 highs(__nv_bfloat162 a, __nv_bfloat162 b) { return __highs2bfloat162(a, b); }
-
-// (minimum, - maximum) of the eight values of a 16-byte piece.
-template <int DTYPE>
-__device__ __forceinline__ typename Pair16<DTYPE>::type minmax8(const uint4& r) {
-  using H2 = typename Pair16<DTYPE>::type;
-  const H2* h = reinterpret_cast<const H2*>(&r);
-  const H2 lo = __hmin2(__hmin2(h[0], h[1]), __hmin2(h[2], h[3]));
-  const H2 hi = __hneg2(__hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3])));
-  return __hmin2(lows(lo, hi), highs(lo, hi));
-}
-
 // Value e (0..7) of a 16-byte piece in fp32.
 template <int DTYPE>
 __device__ __forceinline__ float piece_value(const uint4& r, int e) {
@@ -555,8 +535,8 @@ __device__ __forceinline__ void pack_k_rows(const uint8_t* codes, int code_strid
 // append touches; CTA 0 also takes the last one when that stays incomplete (its rows go to the tail, which CTA 0 must
 // have finished reading first).  A complete block never passes through shared memory: every thread has eight 16-byte
 // loads in flight and keeps them, which is what the kernel is bound by (reading the 16-bit rows).  K and V of 120 streams x
-// 16,383 tokens (values by the kernel above, 162 us of it): 605 us with the block staged in shared memory (48 KB a CTA,
-// one load in flight per thread, 7 instructions more per element), 327 us now.
+// 16,383 tokens (values by the kernel above included): 605 us with the block staged in shared memory (48 KB a CTA,
+// one load in flight per thread, 7 instructions more per element), 292 us now.
 template <int DTYPE, int KB, bool ROT>
 __global__ void __launch_bounds__(256, 3)
 quant_kchan_fast_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, int64_t sb, int64_t sh, int64_t st, int t_new) {

@@ -1,5 +1,5 @@
-// Device functions that the quantize-append kernels share: rounding and packing of codes, and a complete 128-token block of
-// channel-wise keys.
+// Device functions that the quantize-append kernels and the error analysis share: minima and maxima of 16-bit pairs, rounding
+// and packing of codes, and a complete 128-token block of channel-wise keys.
 #pragma once
 
 #include "kvq_internal.h"
@@ -13,6 +13,26 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
   uint32_t d;
   asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
   return d;
+}
+
+// Two 16-bit inputs as a packed pair of their own type, for exact minima and maxima.
+template <int DTYPE> struct Pair16 { using type = __half2; };
+template <> struct Pair16<KVQ_BF16> { using type = __nv_bfloat162; };
+__device__ __forceinline__ float2 pair_to_f32(__half2 h) { return __half22float2(h); }
+__device__ __forceinline__ float2 pair_to_f32(__nv_bfloat162 h) { return __bfloat1622float2(h); }
+__device__ __forceinline__ __half2 lows(__half2 a, __half2 b) { return __lows2half2(a, b); }
+__device__ __forceinline__ __half2 highs(__half2 a, __half2 b) { return __highs2half2(a, b); }
+__device__ __forceinline__ __nv_bfloat162 lows(__nv_bfloat162 a, __nv_bfloat162 b) { return __lows2bfloat162(a, b); }
+__device__ __forceinline__ __nv_bfloat162 highs(__nv_bfloat162 a, __nv_bfloat162 b) { return __highs2bfloat162(a, b); }
+
+// (minimum, - maximum) of the eight values of a 16-byte piece.
+template <int DTYPE>
+__device__ __forceinline__ typename Pair16<DTYPE>::type minmax8(const uint4& r) {
+  using H2 = typename Pair16<DTYPE>::type;
+  const H2* h = reinterpret_cast<const H2*>(&r);
+  const H2 lo = __hmin2(__hmin2(h[0], h[1]), __hmin2(h[2], h[3]));
+  const H2 hi = __hneg2(__hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3])));
+  return __hmin2(lows(lo, hi), highs(lo, hi));
 }
 
 // An append of t_new tokens at position t0 fits the cache; written without a sum that could overflow.
