@@ -2,9 +2,10 @@
 // (App. A.1) over the packed cache, with K^ = z + s*code and V^ likewise
 // reconstructed inside the contraction.
 //
-// Structure (one CTA = 4 consumer warps + 1 producer warp, several CTAs per SM):
-//  * the producer streams whole 128-token pages into a four-stage shared-memory ring
-//    with cp.async.bulk (one bulk copy per page with an L2 evict-first policy,
+// Structure (one CTA = 4 consumer warps + 1 producer warp, with channel-wise keys also a warp that prepares
+// every page's query operands; two or three CTAs per SM):
+//  * the producer streams whole 128-token pages into a shared-memory ring of two to four stages (as the
+//    pages' size allows) with cp.async.bulk (one bulk copy per page with an L2 evict-first policy,
 //    completion on an mbarrier);
 //  * each consumer warp owns one 32-token block of every page for the logits and softmax weights, and a quarter of the
 //    channels for PV; the weights change hands through shared memory as MMA operands; fragments are 16-byte shared loads
@@ -17,12 +18,14 @@
 //    and  o = sum_t (p_t s_t) c_t + sum_t p_t z_t ;
 //  * the sequence is split flat over the grid: CTA i takes the i-th share of all pages
 //    of all streams (shares balanced by time where the arithmetic limits the kernel: a
-//    stream boundary counts as ten pages, the launch waves of an SM are weighted) and
+//    stream boundary counts as eight pages, two with channel-wise keys; the launch waves of
+//    an SM are weighted where every stream's partials fit its slots all the same) and
 //    writes one unnormalised partial (m, l, o) per stream it touches; the CTA that
 //    publishes the last partial of a stream merges them by log-sum-exp and writes the
 //    output (no second kernel, nobody waits).
-// Every wait on an mbarrier is bounded in time; on expiry the kernel sets
-// KVQ_STATUS_DEVICE_TIMEOUT, keeps arriving at its barriers without computing, and returns.
+// Every wait on an mbarrier is bounded in time; on expiry the kernel sets KVQ_STATUS_DEVICE_TIMEOUT and
+// goes on without waiting: it keeps its barrier protocol, reads nothing out of range, and returns (the
+// output is undefined then).
 #pragma once
 
 #include "kvq_internal.h"

@@ -97,7 +97,7 @@ __device__ __forceinline__ uint32_t fixed_point_limb(const float (&t)[4], float 
 // crossing into the next stream for a page or two (40 ragged streams of 36 to 70 K4V4 pages: gap 8 16.5 us, 6 19.8, 0 28).
 // Channel-wise keys, whose pages take longer: gap 2 (ragged 14B shape 119 us; 10: 131 us).  Of the CTAs that
 // share an SM the hardware favours the older ones (0.85 / 0.91 / 0.99 us per page at three per SM, 0.96 / 1.01 at two),
-// so the launch waves are weighted (8B shape K4V2: 1040 76.1 us, 1080 77.3, equal 80.4).
+// so the launch waves are weighted (8B shape K4V2 when the weights were chosen: 1040 76.1 us, 1080 77.3, equal 80.4).
 constexpr int kGapPages = 8, kGapPagesChan = 2;
 constexpr float kQFix = 32512.0f;          // largest |Q| of the 16-bit fixed-point q (hi limb stays within +-127)
 constexpr float kQFix3 = 8300000.0f;       // ... of the 24-bit fixed-point q * s of channel-wise keys (three limbs)
@@ -282,9 +282,11 @@ static __host__ __device__ __forceinline__ bool weighted_shares(const FlatPlan& 
 // (32 registers for 8 heads, where 24-bit weights alone took 96 and spilled): 8 heads have 32-bit weights and four bits of
 // headroom too, channel-wise keys three CTAs per SM instead of two, and a stream's end needs no sum over the warps but two scalars per head.
 // Bound by the length of the instruction stream: a warp issues every 6 to 7 cycles, so what counts is instructions per page.  A page
-// without masks (all but a stream's last) runs code without a condition.  Against whole rows per warp, one layer:
-// 8B K4V2 81.2 -> 76.8 us, K2V4 85 -> 79, K4V4 93 -> 90, K8V4 131 -> 127; 8 heads per KV head (70B shape) 152 -> 120; channel-wise
-// 14B K4V2 182 -> 153, K8V2 192 -> 161; groups of 32 / 64 59 / 60 -> 52 / 51; 4 x 8 streams of 4,000 tokens 22.8 -> 17.5.
+// without masks (all but a stream's last) runs code without a condition.  Against whole rows per warp, one layer, 24 calls in a
+// replayed graph: 8B shape 32k K4V2 80.0 -> 78.5 us (16k: 48.7 -> 45.4, K2V4 49.6 -> 45.8, K4V4 54.8 -> 51.5, K8V4 75.2 -> 70.7, groups of
+// 32 / 64 57.9 / 59.4 -> 52.4 / 52.7); 8 heads per KV head 16 x 16,384 tokens 84 -> 68; channel-wise 16 x 32,768 tokens K4V2 183 -> 154,
+// 16,384 tokens K8V2 101.6 -> 88.4; 4 x 8 streams of 4,000 tokens 22.5 -> 18.0.  Slower only for channel-wise keys of short streams, whose
+// page code spills at three CTAs per SM: 10 streams of 200 tokens 9.7 -> 10.4 us, 1,280 of 1,000 tokens 68.5 -> 72.6.
 constexpr int kConsumerWarps = 4;
 template <int D, int KB, int VB, int KAXIS, int NGK, int NGV, int NH, int MINB>
 __global__ void __launch_bounds__((kConsumerWarps + 1 + (KAXIS == 1 ? 1 : 0)) * 32, MINB)
