@@ -500,8 +500,10 @@ def run_workload(kvq, w: wl.Workload, dev, rank: int, world: int, steps: int, wa
         deq_launches = 1 if B * w.n_kv_heads <= 148 * 8 else 2     # a short range takes both sides in one launch
     else:
         deq_launches += 1                                           # the general kernel serves what is left
-    # append (quantize [+ channel-wise K] + bump), decode, dequantize of the newest page
-    kern_per_layer = (2 if w.k_axis == 0 else 3) + 1 + deq_launches
+    # append of one token (one launch for 2/4/8-bit codes; else quantize [+ channel-wise K] + lengths), decode, dequantize of
+    # the newest page
+    short = fast_bits(w.kb) and fast_bits(w.vb) and (w.k_axis == 0 or (w.head_dim == 128 and w.kb != 2))
+    kern_per_layer = (1 if short else 2 if w.k_axis == 0 else 3) + 1 + deq_launches
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": steps,
             "warmup": warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "int32 accumulate over 8-bit operands (fp32 softmax and merge)",
