@@ -18,8 +18,8 @@ constexpr int kPerSm = 12;
 // takes the same channels of four rows at a time.  Minimum and negated maximum of a group travel as one pair of the 16-bit
 // input type (exact), reduced so that every lane of a group ends up with one of the four rows: the parameters (two
 // divisions) are made once per lane and row and fetched from there.  The codes are rounded by the fused multiply-add of the
-// magic number after a saturating multiplication (see code_word4).  Bound by arithmetic (about 18 instructions per
-// element, 0.66 issued per cycle) and by whole waves: 20 M elements (80 streams x 1000 tokens x 128, K and V) 23 us with parameters
+// magic number after a saturating multiplication (see code_word4).  Bound by arithmetic (about 18.5 instructions per
+// element, 0.76 issued per cycle) and by whole waves: 20 M elements (80 streams x 1000 tokens x 128, K and V) 23 us with parameters
 // per lane and 30 instructions per element, 16.3 us now; eight rows per lane were no faster (fewer, longer turns).
 template <int D, int DTYPE>
 __global__ void __launch_bounds__(kThreads, kPerSm)
