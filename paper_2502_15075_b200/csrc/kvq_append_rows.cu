@@ -31,6 +31,7 @@ append_rows_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, cons
   constexpr int LPR = D / 8, RPW = 32 / LPR;             // lanes per row, rows per warp
   const int b = blockIdx.y, rank = blockIdx.x, ranks = gridDim.x;
   const int tid = threadIdx.x, lane = tid & 31, l = lane % LPR;
+  begin_after_predecessor();
   const int t0 = c.seq_len[b];
   const bool fits = append_fits(t0, t_new, g.capacity);
   if (fits) {
@@ -167,21 +168,12 @@ int launch_append_rows(const Geom& g, const CachePtrs& c, const void* k_new, con
   const bool chan = g.k_axis == 1, rot = c.k_signs != nullptr;
   int threads = per_cta * 2 * (t_new + g.R) * (g.D / 8);
   threads = chan ? kChanThreads : threads > kMaxThreads ? kMaxThreads : (threads + 31) / 32 * 32;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ranks, g.B);
-  cfg.blockDim = dim3(threads);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = ranks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   const uint16_t* k = static_cast<const uint16_t*>(k_new);
   const uint16_t* v = static_cast<const uint16_t*>(v_new);
   cudaError_t e;
-#define KVQ_ROWS(D_, T_, C_)                                                                                         \
-  (rot ? cudaLaunchKernelEx(&cfg, append_rows_kernel<D_, T_, true, C_>, g, c, k, v, sb, sh, st, t_new)               \
-       : cudaLaunchKernelEx(&cfg, append_rows_kernel<D_, T_, false, C_>, g, c, k, v, sb, sh, st, t_new))
+#define KVQ_ROWS(D_, T_, C_)                                                                                             \
+  launch_dependent(rot ? append_rows_kernel<D_, T_, true, C_> : append_rows_kernel<D_, T_, false, C_>, dim3(ranks, g.B), \
+                   threads, 0, stream, ranks, g, c, k, v, sb, sh, st, t_new)
   const bool bf = g.in_dtype == KVQ_BF16;
   if (chan) e = bf ? KVQ_ROWS(128, KVQ_BF16, true) : KVQ_ROWS(128, KVQ_FP16, true);
   else if (g.D == 128) e = bf ? KVQ_ROWS(128, KVQ_BF16, false) : KVQ_ROWS(128, KVQ_FP16, false);

@@ -48,6 +48,14 @@ __device__ __forceinline__ int paged_len(const int32_t* seq_len, int b, int capa
   return R ? (n / R) * R : n;
 }
 
+// Dependent launches: a kernel started by launch_dependent may begin before the one in front of it on the stream has ended, so
+// every thread waits here before it touches global memory; behind the wait everything that the stream ran before is complete and
+// visible.  No kernel lets the next one in earlier than its own end (griddepcontrol.launch_dependents): blocks that wait beside a
+// running kernel take places on its multiprocessors, and those of a decode call then no longer spread one launch wave after the
+// other (16 layers of the 1B shape, append and decode 424 us; with dependent launches 357; with the signal at each kernel's start 392;
+// channel-wise 14B shape, two layers 272, 265, 277; twelve error analyses 223, 191, 198).
+__device__ __forceinline__ void begin_after_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------- conversions
 __device__ __forceinline__ float bits16_to_f32(uint16_t u, int dtype) {
   if (dtype == KVQ_FP16) return __half2float(__ushort_as_half(u));

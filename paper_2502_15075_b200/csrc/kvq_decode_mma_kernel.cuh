@@ -323,7 +323,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + sl.bar_off);   // full[0..stages), empty[0..stages)
   int* sPref = reinterpret_cast<int*>(smem + sl.pref_off);
   int* sVPref = sPref + (g.B + 1);                                   // the same prefix with kGapPages more per stream
-  int* sMisc = reinterpret_cast<int*>(smem + sl.misc_off);           // [0] pages_max, [1] abort flag, [2] published count, [4..7] share ends, [8..9] segment slot / partials, [10..13] CTAs taking part, cursor, [14] weighted shares
+  int* sMisc = reinterpret_cast<int*>(smem + sl.misc_off);           // [1] abort flag, [2] published count, [4..7] share ends, [8..9] segment slot / partials, [10..13] CTAs taking part, cursor, [14] weighted shares
   double* sZ = reinterpret_cast<double*>(smem + sl.red_off);         // [NW][8][NGV] sums of weight x zero-point
   float* sMax = reinterpret_cast<float*>(sZ + NW * 8 * NGV);         // [NW][8] block maxima
   float* sLim = sMax + NW * 8;                                       // [NW][4] value scales (one used)
@@ -338,6 +338,19 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   // ---- plan, all of it on warp 0 (the others wait at one barrier): pages per sequence, prefix over the batch,
   // this CTA's share of the pages and the stream its first page lies in
   const int s_plan = s_cap - (g.R ? 1 : 0);       // the last partial slot of a stream belongs to its residual window
+  if (warp == 0) {
+    if (lane == 0) {
+      sPref[0] = 0; sVPref[0] = 0; sMisc[1] = 0;
+      for (int s = 0; s < stages; ++s) {
+        mbar_init(smem_u32(&bars[s]), 1);
+        mbar_init(smem_u32(&bars[stages + s]), 4);
+        if constexpr (KAXIS == 1) mbar_init(smem_u32(&bars[2 * stages + s]), 1);     // ready: operands of the page made
+      }
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+  }
+  begin_after_predecessor();
   if (warp == 0) {
     int carry = 0, vcarry = 0, pmax = 0;
     for (int base = 0; base < B; base += 32) {
@@ -355,15 +368,6 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       vcarry += __shfl_sync(FULL, vv, 31);
     }
     for (int off = 16; off; off >>= 1) pmax = max(pmax, __shfl_xor_sync(FULL, pmax, off));
-    if (lane == 0) {
-      sPref[0] = 0; sVPref[0] = 0; sMisc[0] = pmax; sMisc[1] = 0;
-      for (int s = 0; s < stages; ++s) {
-        mbar_init(smem_u32(&bars[s]), 1);
-        mbar_init(smem_u32(&bars[stages + s]), 4);
-        if constexpr (KAXIS == 1) mbar_init(smem_u32(&bars[2 * stages + s]), 1);     // ready: operands of the page made
-      }
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
     __syncwarp();
     if (lane < 2) {
       // lane 0: the share's first page, the CTAs that take part and the cursor; lane 1: the share's end
@@ -1126,9 +1130,9 @@ int launch_mma_inst(const Geom& g, const CachePtrs& c, const void* q, float c1, 
   auto kern = decode_mma_kernel<D, KB, VB, KAXIS, NGK, NGV, NH, MINB>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sl.total) != cudaSuccess)
     return KVQ_ERR_CUDA_LAUNCH;
-  kern<<<148 * MINB, (kConsumerWarps + 1 + (KAXIS == 1 ? 1 : 0)) * 32, sl.total, stream>>>(g, c, static_cast<const uint16_t*>(q), c1, ws, s_cap,
-                                                         stages, out, out_dtype, call_id, wait_ns, skip_x);
-  return cudaGetLastError() == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
+  const cudaError_t e = launch_dependent(kern, dim3(148 * MINB), (kConsumerWarps + 1 + (KAXIS == 1 ? 1 : 0)) * 32, sl.total, stream, 1, g, c,
+                                         static_cast<const uint16_t*>(q), c1, ws, s_cap, stages, out, out_dtype, call_id, wait_ns, skip_x);
+  return e == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
 }
 
 }  // namespace mma

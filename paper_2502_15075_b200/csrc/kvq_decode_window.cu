@@ -34,6 +34,7 @@ decode_window_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float 
   const int stream = blockIdx.x, b = stream / g.Hkv, h = stream % g.Hkv;
   const int R = g.R, Gq = g.G, nvh = g.G * g.rows;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  begin_after_predecessor();
   const int n = clamped_len(c.seq_len, b, g.capacity);
   const int f = (n / R) * R, nw = n - f;     // tokens f .. n-1 are in the window, in the ring's slots 0 .. nw-1
   auto out_index = [&](int vh, int d) {
@@ -193,10 +194,11 @@ int launch_decode_window(const Geom& g, const CachePtrs& c, const void* q, void*
                          float* ws, int s_cap, cudaStream_t stream) {
   const uint16_t* qq = static_cast<const uint16_t*>(q);
   const dim3 grid(g.B * g.Hkv);
-  auto launch = [&](auto kern) { kern<<<grid, kThreads, 0, stream>>>(g, c, qq, c1, ws, s_cap, out, out_dtype); };
-  if (g.D == 128) launch(g.in_dtype == KVQ_BF16 ? decode_window_kernel<128, KVQ_BF16> : decode_window_kernel<128, KVQ_FP16>);
-  else launch(g.in_dtype == KVQ_BF16 ? decode_window_kernel<64, KVQ_BF16> : decode_window_kernel<64, KVQ_FP16>);
-  return cudaGetLastError() == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
+  auto launch = [&](auto kern) { return launch_dependent(kern, grid, kThreads, 0, stream, 1, g, c, qq, c1, ws, s_cap, out, out_dtype); };
+  const bool bf = g.in_dtype == KVQ_BF16;
+  const cudaError_t e = g.D == 128 ? launch(bf ? decode_window_kernel<128, KVQ_BF16> : decode_window_kernel<128, KVQ_FP16>)
+                                   : launch(bf ? decode_window_kernel<64, KVQ_BF16> : decode_window_kernel<64, KVQ_FP16>);
+  return e == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
 }
 
 }  // namespace kvq

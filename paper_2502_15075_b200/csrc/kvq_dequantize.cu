@@ -277,6 +277,7 @@ template <int KB, int VB, int DTYPE>
 __global__ void __launch_bounds__(kThreads)
 dequant_fast_kernel(Geom g, CachePtrs c, uint16_t* k_out, uint16_t* v_out, int t_begin, int t_end, int page0, int side0) {
   extern __shared__ __align__(16) uint8_t smem[];
+  begin_after_predecessor();
   const int tid = threadIdx.x;
   const int bh = blockIdx.y, b = bh / g.Hkv;
   const int n = paged_len(c.seq_len, b, g.capacity, g.R);
@@ -299,17 +300,16 @@ int launch_fast(const Geom& g, const CachePtrs& c, uint16_t* k_out, uint16_t* v_
                 int n_pages, int side0, int n_sides, cudaStream_t stream) {
   const size_t smem = (size_t)kPageTokens * (128 + kTilePad) * 2;
   dim3 grid(n_pages, g.B * g.Hkv, n_sides);
-  if (g.in_dtype == KVQ_FP16)
-    dequant_fast_kernel<KB, VB, KVQ_FP16><<<grid, kThreads, smem, stream>>>(g, c, k_out, v_out, t_begin, t_end, page0, side0);
-  else
-    dequant_fast_kernel<KB, VB, KVQ_BF16><<<grid, kThreads, smem, stream>>>(g, c, k_out, v_out, t_begin, t_end, page0, side0);
-  return cudaGetLastError() == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
+  const cudaError_t e = launch_dependent(g.in_dtype == KVQ_FP16 ? dequant_fast_kernel<KB, VB, KVQ_FP16> : dequant_fast_kernel<KB, VB, KVQ_BF16>,
+                                         grid, kThreads, smem, stream, 1, g, c, k_out, v_out, t_begin, t_end, page0, side0);
+  return e == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
 }
 
 __global__ void __launch_bounds__(kThreads)
 dequant_kernel(Geom g, CachePtrs c, uint16_t* k_out, uint16_t* v_out,
                int t_begin, int t_end, int page0, int side0) {
   extern __shared__ __align__(16) uint8_t smem[];
+  begin_after_predecessor();
   const int D = g.D, tid = threadIdx.x;
   uint8_t* spage = smem;
   uint16_t* tile = reinterpret_cast<uint16_t*>(smem + ((g.page_bytes + 15) & ~15));   // [128][D]
@@ -380,6 +380,7 @@ dequant_kernel(Geom g, CachePtrs c, uint16_t* k_out, uint16_t* v_out,
 // Tokens still in the residual window are the 16-bit inputs themselves: copy their rows out.
 __global__ void __launch_bounds__(kThreads)
 window_dequant_kernel(Geom g, CachePtrs c, uint16_t* k_out, uint16_t* v_out, int t_begin, int t_end) {
+  begin_after_predecessor();
   const int bh = blockIdx.x, b = bh / g.Hkv;
   const int D = g.D, R = g.R, vpr = D / 8;
   const int n = clamped_len(c.seq_len, b, g.capacity);
@@ -411,6 +412,10 @@ int launch_dequantize(const Geom& g, const CachePtrs& c, void* k_out, void* v_ou
   const bool fast_v = vo && g.D == 128 && fast_bits(g.vb);
   const bool fast_k = ko && g.D == 128 && g.k_axis == 0 && !c.k_signs && fast_bits(g.kb);
   int rc = KVQ_OK;
+  auto window_rows = [&]() {      // tokens that are still in the residual window
+    return g.R == 0 || launch_dependent(window_dequant_kernel, dim3(g.B * g.Hkv), kThreads, 0, stream, 1, g, c, ko, vo, t_begin, t_end) == cudaSuccess
+               ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
+  };
   // A short range (the newest page of every stream in a decode step) is one launch for both sides; a long one
   // keeps a launch per side, where the key CTAs run without the value side's shared-memory tile.
   if (fast_v && fast_k && (long long)np * g.B * g.Hkv <= 148 * 8) {
@@ -421,10 +426,7 @@ int launch_dequantize(const Geom& g, const CachePtrs& c, void* k_out, void* v_ou
     KVQ_DQ_BOTH(8, 2) KVQ_DQ_BOTH(8, 4) KVQ_DQ_BOTH(8, 8)
 #undef KVQ_DQ_BOTH
     if (rc != KVQ_OK) return rc;
-    if (g.R)
-      window_dequant_kernel<<<g.B * g.Hkv, kThreads, 0, stream>>>(g, c, static_cast<uint16_t*>(k_out),
-                                                                  static_cast<uint16_t*>(v_out), t_begin, t_end);
-    return cudaGetLastError() == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
+    return window_rows();
   }
   if (fast_v) {
     if (g.vb == 2) rc = launch_fast<0, 2>(g, c, ko, vo, t_begin, t_end, page0, np, 0, 1, stream);
@@ -442,12 +444,10 @@ int launch_dequantize(const Geom& g, const CachePtrs& c, void* k_out, void* v_ou
   const bool gen_v = vo && !fast_v, gen_k = ko && !fast_k;
   if (gen_v || gen_k) {
     dim3 grid(np, g.B * g.Hkv, (gen_v && gen_k) ? 2 : 1);
-    dequant_kernel<<<grid, kThreads, smem, stream>>>(g, c, ko, vo, t_begin, t_end, page0, gen_v ? 0 : 1);
+    if (launch_dependent(dequant_kernel, grid, kThreads, smem, stream, 1, g, c, ko, vo, t_begin, t_end, page0, gen_v ? 0 : 1) != cudaSuccess)
+      return KVQ_ERR_CUDA_LAUNCH;
   }
-  if (g.R)
-    window_dequant_kernel<<<g.B * g.Hkv, kThreads, 0, stream>>>(g, c, static_cast<uint16_t*>(k_out),
-                                                                static_cast<uint16_t*>(v_out), t_begin, t_end);
-  return cudaGetLastError() == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
+  return window_rows();
 }
 
 }  // namespace kvq

@@ -39,6 +39,7 @@ quant_error_kernel(Geom g, const uint16_t* __restrict__ k, const uint16_t* __res
   const int b0 = lane & 1, b1 = (lane >> 1) & 1, gbase = lane & ~(lpg - 1);
   const float qmax = (float)((1 << (bits & 15)) - 1), up = (float)(1 << (bits & 15)), down = 1.0f / up;
   double acc2 = 0.0, acce = 0.0;
+  begin_after_predecessor();
   for (int base = blockIdx.x * kStep; base < n_tokens; base += gridDim.x * kStep) {
     uint4 raw[ROWS];
 #pragma unroll
@@ -120,12 +121,12 @@ int launch_quant_error(const Geom& g, const void* k, const void* v, int64_t sb, 
   if (want < 1) want = 1;
   if (gx > want) gx = want;
   auto launch = [&](auto kern) {
-    kern<<<dim3(gx, streams, 2), kThreads, 0, stream>>>(g, kk, vv, sb, sh, st, n_tokens, sums);
+    return launch_dependent(kern, dim3(gx, streams, 2), kThreads, 0, stream, 1, g, kk, vv, sb, sh, st, n_tokens, sums);
   };
   const bool bf = g.in_dtype == KVQ_BF16;
-  if (g.D == 128) launch(bf ? quant_error_kernel<128, KVQ_BF16> : quant_error_kernel<128, KVQ_FP16>);
-  else launch(bf ? quant_error_kernel<64, KVQ_BF16> : quant_error_kernel<64, KVQ_FP16>);
-  return cudaGetLastError() == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
+  const cudaError_t e = g.D == 128 ? launch(bf ? quant_error_kernel<128, KVQ_BF16> : quant_error_kernel<128, KVQ_FP16>)
+                                   : launch(bf ? quant_error_kernel<64, KVQ_BF16> : quant_error_kernel<64, KVQ_FP16>);
+  return e == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
 }
 
 }  // namespace kvq

@@ -427,6 +427,7 @@ template <int D, int DTYPE, bool ROT>
 __global__ void __launch_bounds__(kThreads, ROT ? 4 : 5)
 quant_token_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
                    int64_t sb, int64_t sh, int64_t st, int t_new) {
+  begin_after_predecessor();
   const bool is_v = blockIdx.z == 0;
   const int bh = blockIdx.y;
   const int b = bh / g.Hkv, h = bh % g.Hkv;
@@ -541,6 +542,7 @@ template <int DTYPE, int KB, bool ROT>
 __global__ void __launch_bounds__(256, 3)
 quant_kchan_fast_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, int64_t sb, int64_t sh, int64_t st, int t_new) {
   __shared__ KchanShared scratch;
+  begin_after_predecessor();
   const int bh = blockIdx.y, b = bh / g.Hkv, h = bh % g.Hkv;
   const int t0 = c.seq_len[b];
   if (!append_fits(t0, t_new, g.capacity)) return;
@@ -563,6 +565,7 @@ __global__ void __launch_bounds__(kThreads)
 quant_kchan_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new,
                    int64_t sb, int64_t sh, int64_t st, int t_new) {
   extern __shared__ __align__(16) uint8_t smem[];
+  begin_after_predecessor();
   const int D = g.D;
   uint16_t* sX = reinterpret_cast<uint16_t*>(smem);          // [128][D] fp16 bits
   uint8_t* sC = smem + (size_t)kPageTokens * D * 2;           // [128][D] codes
@@ -654,6 +657,7 @@ quant_kchan_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new,
 __global__ void __launch_bounds__(kThreads)
 window_store_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
                     int64_t sb, int64_t sh, int64_t st, int t_new) {
+  begin_after_predecessor();
   const int bh = blockIdx.y, b = bh / g.Hkv, h = bh % g.Hkv;
   const int t0 = c.seq_len[b];
   if (!append_fits(t0, t_new, g.capacity)) return;
@@ -668,6 +672,7 @@ window_store_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, con
 }
 
 __global__ void bump_seq_len_kernel(Geom g, CachePtrs c, int t_new) {
+  begin_after_predecessor();
   int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= g.B) return;
   int t0 = c.seq_len[b];
@@ -693,38 +698,33 @@ int launch_quantize_append(const Geom& g, const CachePtrs& c, const void* k_new,
   if (gx > want) gx = want;
   dim3 grid1(gx, streams, g.k_axis == 0 ? 2 : 1);            // z = 0 values, z = 1 token-wise keys
   const bool rot = c.k_signs != nullptr && g.k_axis == 0;
-#define KVQ_QLAUNCH(D_, T_)                                                                                  \
-  do {                                                                                                       \
-    if (rot) quant_token_kernel<D_, T_, true><<<grid1, kThreads, 0, stream>>>(g, c, k, v, sb, sh, st, t_new); \
-    else quant_token_kernel<D_, T_, false><<<grid1, kThreads, 0, stream>>>(g, c, k, v, sb, sh, st, t_new);    \
-  } while (0)
+  cudaError_t e = cudaSuccess;
+  auto run = [&](auto kern, dim3 grid, unsigned threads, size_t smem, auto... args) {      // (the first failure ends the call)
+    if (e == cudaSuccess) e = launch_dependent(kern, grid, threads, smem, stream, 1, args...);
+  };
+#define KVQ_QLAUNCH(D_, T_) \
+  run(rot ? quant_token_kernel<D_, T_, true> : quant_token_kernel<D_, T_, false>, grid1, kThreads, 0, g, c, k, v, sb, sh, st, t_new)
   if (g.D == 128 && g.in_dtype == KVQ_BF16) KVQ_QLAUNCH(128, KVQ_BF16);
   else if (g.D == 128) KVQ_QLAUNCH(128, KVQ_FP16);
   else if (g.in_dtype == KVQ_BF16) KVQ_QLAUNCH(64, KVQ_BF16);
   else KVQ_QLAUNCH(64, KVQ_FP16);
 #undef KVQ_QLAUNCH
+  const dim3 grid2((t_new + 127) / 128 + 1, streams);
   if (g.k_axis == 1 && g.D == 128 && (g.kb == 4 || g.kb == 8)) {
-    dim3 grid2((t_new + 127) / 128 + 1, streams);
-#define KVQ_KCHAN(T_, KB_)                                                                                         \
-  do {                                                                                                             \
-    if (c.k_signs) quant_kchan_fast_kernel<T_, KB_, true><<<grid2, 256, 0, stream>>>(g, c, k, sb, sh, st, t_new);  \
-    else quant_kchan_fast_kernel<T_, KB_, false><<<grid2, 256, 0, stream>>>(g, c, k, sb, sh, st, t_new);           \
-  } while (0)
+#define KVQ_KCHAN(T_, KB_)                                                                                           \
+  run(c.k_signs ? quant_kchan_fast_kernel<T_, KB_, true> : quant_kchan_fast_kernel<T_, KB_, false>, grid2, 256, 0, g, c, k, \
+      sb, sh, st, t_new)
     if (g.in_dtype == KVQ_BF16) { if (g.kb == 4) KVQ_KCHAN(KVQ_BF16, 4); else KVQ_KCHAN(KVQ_BF16, 8); }
     else { if (g.kb == 4) KVQ_KCHAN(KVQ_FP16, 4); else KVQ_KCHAN(KVQ_FP16, 8); }
 #undef KVQ_KCHAN
   } else if (g.k_axis == 1) {
     size_t smem = (size_t)kPageTokens * g.D * 3;
     cudaFuncSetAttribute(quant_kchan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 128 * 3);
-    dim3 grid2((t_new + 127) / 128 + 1, streams);
-    quant_kchan_kernel<<<grid2, kThreads, smem, stream>>>(g, c, k, sb, sh, st, t_new);
+    run(quant_kchan_kernel, grid2, kThreads, smem, g, c, k, sb, sh, st, t_new);
   }
-  if (g.R) {
-    dim3 grid3(1, streams);
-    window_store_kernel<<<grid3, kThreads, 0, stream>>>(g, c, k, v, sb, sh, st, t_new);
-  }
-  bump_seq_len_kernel<<<(g.B + 127) / 128, 128, 0, stream>>>(g, c, t_new);
-  return cudaGetLastError() == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
+  if (g.R) run(window_store_kernel, dim3(1, streams), kThreads, 0, g, c, k, v, sb, sh, st, t_new);
+  run(bump_seq_len_kernel, dim3((g.B + 127) / 128), 128, 0, g, c, t_new);
+  return e == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
 }
 
 }  // namespace kvq
