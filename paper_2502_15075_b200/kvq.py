@@ -100,13 +100,19 @@ def _check(code: int, where: str):
         raise KvqError(code, where)
 
 
+_DTYPE_CODES = {torch.float16: KVQ_FP16, torch.bfloat16: KVQ_BF16, torch.float32: KVQ_FP32}
+
+
 def _dtype_code(dt: torch.dtype) -> int:
-    return {torch.float16: KVQ_FP16, torch.bfloat16: KVQ_BF16, torch.float32: KVQ_FP32}[dt]
+    return _DTYPE_CODES[dt]
 
 
 def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    """The stream's handle: the given one's, or the current device's current stream's (read as a number; making a
+    torch.cuda.Stream object for it took 3.1 of the 10 us of a call; the CUDA tensors of the call have initialised CUDA)."""
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def kvq_strerror(code: int) -> str:
@@ -195,13 +201,14 @@ def kvq_quantize_append(cfg: kvq_config, cache: Cache, k_new: torch.Tensor, v_ne
                         stream: Optional[torch.cuda.Stream] = None):
     """k_new, v_new: CUDA tensors [B, Hkv, t_new, D] of the config's dtype, last dim contiguous,
     identical strides."""
-    assert k_new.is_cuda and v_new.is_cuda and k_new.shape == v_new.shape and k_new.dim() == 4
-    assert k_new.stride() == v_new.stride() and k_new.stride(3) == 1
+    shape, strides = k_new.shape, k_new.stride()
+    assert k_new.is_cuda and v_new.is_cuda and shape == v_new.shape and len(shape) == 4
+    assert strides == v_new.stride() and strides[3] == 1
     assert _dtype_code(k_new.dtype) == cfg.in_dtype and v_new.dtype == k_new.dtype
-    assert k_new.shape[0] == cfg.batch and k_new.shape[1] == cfg.n_kv_heads and k_new.shape[3] == cfg.head_dim
+    assert shape[0] == cfg.batch and shape[1] == cfg.n_kv_heads and shape[3] == cfg.head_dim
     _check(_lib.kvq_quantize_append(ctypes.byref(cfg), ctypes.byref(cache.c), k_new.data_ptr(), v_new.data_ptr(),
-                                    k_new.stride(0), k_new.stride(1), k_new.stride(2), k_new.shape[2],
-                                    _stream_ptr(stream)), "kvq_quantize_append")
+                                    strides[0], strides[1], strides[2], shape[2], _stream_ptr(stream)),
+           "kvq_quantize_append")
 
 
 def kvq_decode_attention(cfg: kvq_config, cache: Cache, q: torch.Tensor, out: torch.Tensor,
