@@ -11,6 +11,8 @@ namespace kvq {
 
 namespace {
 
+__device__ __forceinline__ __half2 as_half2(uint32_t u) { return *reinterpret_cast<const __half2*>(&u); }
+
 constexpr int kThreads = 128;
 constexpr int kPerSm = 12;
 
@@ -18,9 +20,11 @@ constexpr int kPerSm = 12;
 // takes the same channels of four rows at a time.  Minimum and negated maximum of a group travel as one pair of the 16-bit
 // input type (exact), reduced so that every lane of a group ends up with one of the four rows: the parameters (two
 // divisions) are made once per lane and row and fetched from there.  The codes are rounded by the fused multiply-add of the
-// magic number after a saturating multiplication (see code_word4).  Bound by arithmetic (about 18.5 instructions per
-// element, 0.76 issued per cycle) and by whole waves: 20 M elements (80 streams x 1000 tokens x 128, K and V) 23 us with parameters
-// per lane and 30 instructions per element, 16.3 us now; eight rows per lane were no faster (fewer, longer turns).
+// magic number after a saturating multiplication (see code_word4); two neighbouring channels share every fp32 operation that has a
+// packed form, and a row's squares are added as two chains of four.  20 M elements a call (80 streams x 1000 tokens x 128, K and V),
+// twelve calls in a row: 191 us without packed operations, 173 now; 64-bit comparison of the sums 1.2e-8 before, 1.0e-8 now.  Bound by
+// latency (twelve CTAs per SM, each three turns of rows): longer fp32 sums 171 us, compensated fp32 sums in place of doubles 180, the next
+// turn's rows in flight at eight CTAs per SM 196; eight rows per lane were no faster (fewer, longer turns).
 template <int D, int DTYPE>
 __global__ void __launch_bounds__(kThreads, kPerSm)
 quant_error_kernel(Geom g, const uint16_t* __restrict__ k, const uint16_t* __restrict__ v, int64_t sb, int64_t sh,
@@ -37,7 +41,7 @@ quant_error_kernel(Geom g, const uint16_t* __restrict__ k, const uint16_t* __res
   const uint16_t* in = (side ? v : k) + (int64_t)b * sb + (int64_t)h * sh + 8 * l;
   const int lpg = gsz >> 3;                              // lanes per group: 4, 8 or 16
   const int b0 = lane & 1, b1 = (lane >> 1) & 1, gbase = lane & ~(lpg - 1);
-  const float qmax = (float)((1 << (bits & 15)) - 1), up = (float)(1 << (bits & 15)), down = 1.0f / up;
+  const float qmax = (float)((1 << (bits & 15)) - 1), up = (float)(1 << (bits & 15)), down = 1.0f / up, rtop = kRoundMagic + qmax;
   double acc2 = 0.0, acce = 0.0;
   begin_after_predecessor();
   for (int base = blockIdx.x * kStep; base < n_tokens; base += gridDim.x * kStep) {
@@ -47,7 +51,8 @@ quant_error_kernel(Geom g, const uint16_t* __restrict__ k, const uint16_t* __res
       const int t = base + i * (kStep / ROWS) + r0;      // rows beyond the end are zeros and add nothing
       raw[i] = t < n_tokens ? *reinterpret_cast<const uint4*>(in + (int64_t)t * st) : make_uint4(0u, 0u, 0u, 0u);
     }
-    float z = 0.f, s = 0.f, inv = 0.f;                   // of the lane's row
+    uint32_t meta = 0u;                                  // of the lane's row: scale and zero, 2^-bits / scale
+    float inv = 0.f;
     if (bits != 16) {
       H2 m[ROWS];                                        // (minimum, - maximum) of the lane's channels
 #pragma unroll
@@ -66,29 +71,34 @@ quant_error_kernel(Geom g, const uint16_t* __restrict__ k, const uint16_t* __res
       if (lpg >= 16) a = __hmin2(a, a8);
       const float2 f = pair_to_f32(a);
       const GroupParams p = group_params(f.x, -f.y, qmax);
-      z = p.z; s = p.s; inv = p.inv * down;
+      meta = p.meta; inv = p.inv * down;
     }
+    f32x2 s2[ROWS], se[ROWS];                            // sums over the even and the odd channels of a row
 #pragma unroll
     for (int i = 0; i < ROWS; ++i) {
       const int src = gbase + (i >> 1) + 2 * (i & 1);    // the lane of the group that holds row i
-      const float zi = __shfl_sync(FULL, z, src), si = __shfl_sync(FULL, s, src), ii = __shfl_sync(FULL, inv, src);
+      const float2 sz = __half22float2(as_half2(__shfl_sync(FULL, meta, src)));
+      const float ii = __shfl_sync(FULL, inv, src);
+      const f32x2 si = pack2(sz.x, sz.x), zi = pack2(sz.y, sz.y), nz = pack2(-sz.y, -sz.y);
       const H2* p = reinterpret_cast<const H2*>(&raw[i]);
-      float s2 = 0.f, se = 0.f;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float2 x2 = pair_to_f32(p[j]);
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const float x = e ? x2.y : x2.x;
-          s2 = fmaf(x, x, s2);
-          const float r = __fmaf_rn(__saturatef(__fmul_rn(__fsub_rn(x, zi), ii)), up, kRoundMagic);
-          const float code = fminf(__fsub_rn(r, kRoundMagic), qmax);
-          const float d = __fsub_rn(x, __fmaf_rn(code, si, zi));      // (the rounding of x^ belongs to the error)
-          se = fmaf(d, d, se);
-        }
+        const float2 f = pair_to_f32(p[j]);
+        const f32x2 x = pack2(f.x, f.y);
+        s2[i] = j ? fma2(x, x, s2[i]) : mul2(x, x);
+        const float2 t = unpack2(add2(x, nz));
+        const f32x2 r = fma2(pack2(__saturatef(__fmul_rn(t.x, ii)), __saturatef(__fmul_rn(t.y, ii))), pack2(up, up), pack2(kRoundMagic, kRoundMagic));
+        const float2 rf = unpack2(r);
+        const f32x2 code = add2(pack2(fminf(rf.x, rtop), fminf(rf.y, rtop)), pack2(-kRoundMagic, -kRoundMagic));
+        const f32x2 d = fma2(fma2(code, si, zi), pack2(-1.0f, -1.0f), x);      // (the rounding of x^ belongs to the error)
+        se[i] = j ? fma2(d, d, se[i]) : mul2(d, d);
       }
-      acc2 += (double)s2;
-      acce += (double)se;
+    }
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+      const float2 ts = unpack2(s2[i]), te = unpack2(se[i]);
+      acc2 += (double)__fadd_rn(ts.x, ts.y);
+      acce += (double)__fadd_rn(te.x, te.y);
     }
   }
   if (bits == 16) acce = 0.0;                            // passed through: no error
