@@ -2,7 +2,7 @@
 // (App. A.1) over the packed cache, with K^ = z + s*code and V^ likewise
 // reconstructed inside the contraction.
 //
-// Structure (one CTA = 4 consumer warps + 1 producer warp, with channel-wise keys also a warp that prepares
+// Structure (one CTA = 4 consumer warps + 1 producer warp, which with channel-wise keys also prepares
 // every page's query operands; two or three CTAs per SM):
 //  * the producer streams whole 128-token pages into a shared-memory ring of two to four stages (as the
 //    pages' size allows) with cp.async.bulk (one bulk copy per page with an L2 evict-first policy,
@@ -56,7 +56,17 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
-// Same, letting the hardware park the thread for up to `hint_ns` while the phase is pending.
+// Whether the phase is complete, without waiting for it.
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0;
+}
+// mbar_try_wait, letting the hardware park the thread for up to `hint_ns` while the phase is pending.
 __device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity, uint32_t hint_ns) {
   uint32_t ok;
   asm volatile(

@@ -14,7 +14,7 @@ struct SmemLayout {
 };
 // weights: the PV operands of a page as the owners of its four 32-token blocks leave them, per value group and block
 // (16 NH bytes per lane), for two pages in turn.
-// chan: channel-wise keys keep, per ring stage, the page's q operands made by the preparation warp
+// chan: channel-wise keys keep, per ring stage, the page's q operands made by the producer warp
 // (NH x 2 x D/16 x 32 words) followed by 8 zero-point sums and 8 fixed-point scales (one per head).
 __host__ __device__ constexpr int weight_block_bytes(int nh) { return 512 * nh; }
 __host__ __device__ constexpr int reduction_bytes(int ngv) { return 4 * (8 * ngv * 8 + (8 + 4 + 8) * 4); }   // per warp: p z sums (64 bits), maxima, scale limit, l
@@ -103,19 +103,15 @@ constexpr float kQFix = 32512.0f;          // largest |Q| of the 16-bit fixed-po
 constexpr float kQFix3 = 8300000.0f;       // ... of the 24-bit fixed-point q * s of channel-wise keys (three limbs)
 
 // Four values times `scale` rounded to integers |Q| <= kQFix3 and taken apart as two's-complement bytes,
-// Q = b2 * 65536 + b1 * 256 + b0 with b2 signed and b1, b0 unsigned.  Operand words of a lane: even operand
-// columns (odd = 0) carry b2 in n-tile 0 (signed bytes) and b1 in n-tile 1 (unsigned bytes), odd columns nothing in
-// n-tile 0 and b0 in n-tile 1.  Byte j of a word belongs to t[j].
-__device__ __forceinline__ void fixed_point_bytes3(const float (&t)[4], float scale, int odd, uint32_t& w_nt0,
-                                                   uint32_t& w_nt1) {
+// Q = b2 * 65536 + b1 * 256 + b0 with b2 signed and b1, b0 unsigned; byte j of w[k] is b_k of t[j].  The even operand
+// columns carry b2 in n-tile 0 (signed bytes) and b1 in n-tile 1 (unsigned bytes), the odd ones nothing in n-tile 0 and b0 in n-tile 1.
+__device__ __forceinline__ void fixed_point_bytes3(const float (&t)[4], float scale, uint32_t (&w)[3]) {
   const uint32_t q0 = (uint32_t)__float2int_rn(t[0] * scale), q1 = (uint32_t)__float2int_rn(t[1] * scale);
   const uint32_t q2 = (uint32_t)__float2int_rn(t[2] * scale), q3 = (uint32_t)__float2int_rn(t[3] * scale);
-  // byte k of each of the four integers -> one word: selectors pick byte k of (q0, q1) and of (q2, q3)
-  const uint32_t sel = odd ? 0x0040u : 0x0051u;                  // odd: byte 0; even: byte 1
-  const uint32_t lo01 = prmt(q0, q1, sel), lo23 = prmt(q2, q3, sel);
-  w_nt1 = prmt(lo01, lo23, 0x5410u);
-  const uint32_t hi01 = prmt(q0, q1, 0x0062u), hi23 = prmt(q2, q3, 0x0062u);   // byte 2 of each
-  w_nt0 = odd ? 0u : prmt(hi01, hi23, 0x5410u);
+  const uint32_t lo01 = prmt(q0, q1, 0x5140u), lo23 = prmt(q2, q3, 0x5140u);      // bytes (0, 0), (1, 1) of a pair
+  w[0] = prmt(lo01, lo23, 0x5410u);
+  w[1] = prmt(lo01, lo23, 0x7632u);
+  w[2] = prmt(prmt(q0, q1, 0x0062u), prmt(q2, q3, 0x0062u), 0x5410u);
 }
 // The softmax weights enter PV as fixed point P = rint(p * s_V * 2^PBITS / s_lim), p = 2^(logit - reference) with the
 // reference kHeadroom bits above the largest logit seen so far, so that a larger logit rarely forces a rescale.
@@ -285,11 +281,10 @@ static __host__ __device__ __forceinline__ bool weighted_shares(const FlatPlan& 
 // without masks (all but a stream's last) runs code without a condition.  Against whole rows per warp, one layer, 24 calls in a
 // replayed graph: 8B shape 32k K4V2 80.0 -> 78.5 us (16k: 48.7 -> 45.4, K2V4 49.6 -> 45.8, K4V4 54.8 -> 51.5, K8V4 75.2 -> 70.7, groups of
 // 32 / 64 57.9 / 59.4 -> 52.4 / 52.7); 8 heads per KV head 16 x 16,384 tokens 84 -> 68; channel-wise 16 x 32,768 tokens K4V2 183 -> 154,
-// 16,384 tokens K8V2 101.6 -> 88.4; 4 x 8 streams of 4,000 tokens 22.5 -> 18.0.  Slower only for channel-wise keys of short streams, whose
-// page code spills at three CTAs per SM: 10 streams of 200 tokens 9.7 -> 10.4 us, 1,280 of 1,000 tokens 68.5 -> 72.6.
+// 16,384 tokens K8V2 101.6 -> 88.4; 4 x 8 streams of 4,000 tokens 22.5 -> 18.0.
 constexpr int kConsumerWarps = 4;
 template <int D, int KB, int VB, int KAXIS, int NGK, int NGV, int NH, int MINB>
-__global__ void __launch_bounds__((kConsumerWarps + 1 + (KAXIS == 1 ? 1 : 0)) * 32, MINB)
+__global__ void __launch_bounds__((kConsumerWarps + 1) * 32, MINB)
 decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1, float* __restrict__ ws,
                   int s_cap, int stages, void* __restrict__ out, int out_dtype, unsigned long long call_id,
                   unsigned long long wait_ns, long long skip_x) {
@@ -419,7 +414,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   const unsigned long long id40 = (call_id & 0xFFFFFFFFFFull) ? (call_id & 0xFFFFFFFFFFull) : 1ull;
 
   // =========================================================== producer warp
-  if (warp == NW) {
+  if (KAXIS == 0 && warp == NW) {
     if (lane == 0) {
       int it = 0, stage = 0;
       uint32_t phase = 1;                // parity of the previous round of `empty`
@@ -460,38 +455,80 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
     return;
   }
 
-  // =========================================================== preparation warp (channel-wise keys)
+  // =========================================================== producer and preparation warp (channel-wise keys)
   // Per page, the operand of the integer QK^T MMAs is q_d * s_d in 24-bit fixed point (scale from max|q| of the head
-  // times the page's largest channel scale), and sum_d q_d z_d is one fp32 scalar per head.  One warp makes both for
-  // every page, in the lane arrangement the consumers' B fragments have, leaves them in the stage's operand buffer
-  // and signals the stage's `ready` barrier; for the incomplete last block it leaves q split into fp16 high and
-  // low parts instead (operands of the fp16 MMAs on the tail keys).
+  // times the page's largest channel scale), and sum_d q_d z_d is one fp32 scalar per head.  The warp that issues the copies makes
+  // both for every page that has landed, in the lane arrangement the consumers' B fragments have, leaves them in the stage's operand
+  // buffer and signals the stage's `ready` barrier; for the incomplete last block it leaves q split into fp16 high and low parts
+  // instead (operands of the fp16 MMAs on the tail keys).  Copies come first: it issues into every stage that is free before it takes
+  // the next page.  Its time per page bounds the kernel, so the two lanes that share a head split the channel slots (147 instructions a
+  // page instead of 270): two ragged 14B-shaped layers 265 -> 231 us, 240 with a sixth warp for the operands, which leaves 96 registers
+  // per thread at three CTAs per SM instead of 128, so that the page code spills (270 us without the split work).
   if constexpr (KAXIS == 1) {
-    if (warp == NW + 1) {
+    if (warp == NW) {
       constexpr int CSB = NH * 2 * NR * 32 * 4 + 64;
-      int stage = 0;
+      const uint64_t policy = l2_evict_first_policy();
+      int istage = 0, ib = b, ih = h, ipage = page, ipages = pages_b, ix = x_lo;       // the next page to copy
+      uint32_t iphase = 1;               // parity of the previous round of `empty`
+      int stage = 0, x = x_lo;           // the next page to prepare
       uint32_t phase = 0;
-      float qv[NH][NR][4];
+      // the lanes of an even and of the odd operand column share a head: each takes half of the channel slots for both columns
+      constexpr int HR = NR / 2;
+      const int r0 = HR * (gid & 1), even = lane & ~4;
+      float qv[NH][HR][4];
       float amaxB[NH];
       int cur_b = -1, cur_h = -1;
-      for (int x = x_lo; x < x_hi; ++x) {
+      bool ok = true;
+      unsigned long long t_idle = 0;
+      auto next_of = [&](int& bb, int& hh, int& pg, int& np) {
+        if (++pg == np) {
+          pg = 0;
+          if (++hh == Hkv) {
+            hh = 0;
+            do { ++bb; } while (bb < B && sPref[bb + 1] == sPref[bb]);
+            if (bb < B) np = (sPref[bb + 1] - sPref[bb]) / Hkv;
+          }
+        }
+      };
+      while (x < x_hi) {
+        if (ix < x_hi && (ix - x_lo < stages || __all_sync(FULL, mbar_test_wait(bar0 + 8 * (stages + istage), iphase)))) {
+          if (lane == 0 && ix != skip_x) {          // (skip_x: test hook - a page that never arrives makes the consumers' bounded wait expire)
+            const uint8_t* src = c.pages + ((size_t)(ib * Hkv + ih) * g.n_pages + ipage) * (size_t)g.page_bytes;
+            mbar_expect_tx(bar0 + 8 * istage, (uint32_t)g.page_bytes);
+            bulk_load(ring + istage * sl.page_stride, src, (uint32_t)g.page_bytes, bar0 + 8 * istage, policy);
+          }
+          __syncwarp();
+          if (++istage == stages) { istage = 0; iphase ^= 1; }
+          next_of(ib, ih, ipage, ipages);
+          ++ix;
+          t_idle = 0;
+          continue;
+        }
+        if (x == ix || !__all_sync(FULL, mbar_test_wait(bar0 + 8 * stage, phase))) {
+          // neither a free stage nor a page that has landed: look again, for a bounded time
+          const unsigned long long now = __shfl_sync(FULL, globaltimer_ns(), 0);
+          if (t_idle == 0) t_idle = now;
+          if (now - t_idle > wait_ns || __any_sync(FULL, *abort_flag != 0)) { ok = false; break; }
+          continue;
+        }
+        t_idle = 0;
         if (b != cur_b || h != cur_h) {          // a new stream: its queries
           cur_b = b; cur_h = h;
 #pragma unroll
           for (int nh = 0; nh < NH; ++nh) {
-            float am = load_q_lane<D>(g, c, q, b, h, (gid >> 1) + 4 * nh, tid, qv[nh]);
+            float q_all[NR][4];
+            float am = load_q_lane<D>(g, c, q, b, h, (gid >> 1) + 4 * nh, tid, q_all);
+#pragma unroll
+            for (int r = 0; r < HR; ++r) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j) qv[nh][r][j] = (gid & 1) ? q_all[HR + r][j] : q_all[r][j];
+            }
             am = fmaxf(am, __shfl_xor_sync(FULL, am, 1));
             amaxB[nh] = fmaxf(am, __shfl_xor_sync(FULL, am, 2));
           }
         }
         const int n_tok = paged_len(c.seq_len, b, g.capacity, g.R);
         const bool tail_pg = n_tok - page * kPageTokens < kPageTokens;
-        const bool got = mbar_wait(bar0 + 8 * stage, phase, wait_ns);
-        if (!__all_sync(FULL, got) || *abort_flag) {
-          *abort_flag = 1;
-          if (lane == 0) atomicOr(c.status, KVQ_STATUS_DEVICE_TIMEOUT);
-          return;
-        }
         const uint8_t* sp = smem + stage * sl.page_stride;
         uint32_t* ops = reinterpret_cast<uint32_t*>(smem + sl.chan_off + stage * CSB);     // [NH][2][NR][32]
         float* opf = reinterpret_cast<float*>(ops + NH * 2 * NR * 32);                      // zq[8], hs[8]
@@ -499,23 +536,23 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
 #pragma unroll
           for (int nh = 0; nh < NH; ++nh) {
 #pragma unroll
-            for (int r = 0; r < NR; ++r) {
+            for (int r = 0; r < HR; ++r) {
               uint32_t h0, l0_, h1, l1_;
               split_h2(qv[nh][r][0], qv[nh][r][2], h0, l0_);
               split_h2(qv[nh][r][1], qv[nh][r][3], h1, l1_);
-              ops[((nh * 2 + 0) * NR + r) * 32 + lane] = (gid & 1) ? l0_ : h0;
-              ops[((nh * 2 + 1) * NR + r) * 32 + lane] = (gid & 1) ? l1_ : h1;
+              uint32_t* o = ops + (nh * 2 * NR + r0 + r) * 32 + even;
+              o[0] = h0; o[4] = l0_;
+              o[NR * 32] = h1; o[NR * 32 + 4] = l1_;
             }
           }
         } else {
           const uint32_t* km = reinterpret_cast<const uint32_t*>(sp + K_META_OFF);
-          float smax = 0.f;
+          uint32_t top = 0u;               // (scales are not negative: their bits are in the order of their values)
           if (4 * lane < D) {
             const uint4 mm = *reinterpret_cast<const uint4*>(km + 4 * lane);
-            smax = fmaxf(fmaxf(meta_s(mm.x), meta_s(mm.y)), fmaxf(meta_s(mm.z), meta_s(mm.w)));
+            top = max(max(mm.x & 0xFFFFu, mm.y & 0xFFFFu), max(mm.z & 0xFFFFu, mm.w & 0xFFFFu));
           }
-#pragma unroll
-          for (int off = 1; off < 32; off <<= 1) smax = fmaxf(smax, __shfl_xor_sync(FULL, smax, off));
+          const float smax = meta_s(__reduce_max_sync(FULL, top));
 #pragma unroll
           for (int nh = 0; nh < NH; ++nh) {
             const int hb = (gid >> 1) + 4 * nh;
@@ -523,8 +560,8 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
             const float scale = am > 0.f ? kQFix3 / am : 0.f;
             float zsum = 0.f;
 #pragma unroll
-            for (int r = 0; r < NR; ++r) {
-              const uint4 mm = *reinterpret_cast<const uint4*>(km + 16 * r + 4 * tid);     // (s, z) of 4 channels
+            for (int r = 0; r < HR; ++r) {
+              const uint4 mm = *reinterpret_cast<const uint4*>(km + 16 * (r0 + r) + 4 * tid);     // (s, z) of 4 channels
               const uint32_t mw[4] = {mm.x, mm.y, mm.z, mm.w};
               float t[4];
 #pragma unroll
@@ -533,11 +570,13 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
                 t[j] = qv[nh][r][j] * sz.x;
                 zsum = fmaf(qv[nh][r][j], sz.y, zsum);
               }
-              uint32_t w0, w1;
-              fixed_point_bytes3(t, scale, gid & 1, w0, w1);
-              ops[((nh * 2 + 0) * NR + r) * 32 + lane] = w0;
-              ops[((nh * 2 + 1) * NR + r) * 32 + lane] = w1;
+              uint32_t w[3];
+              fixed_point_bytes3(t, scale, w);
+              uint32_t* o = ops + (nh * 2 * NR + r0 + r) * 32 + even;
+              o[0] = w[2]; o[4] = 0u;
+              o[NR * 32] = w[1]; o[NR * 32 + 4] = w[0];
             }
+            zsum += __shfl_xor_sync(FULL, zsum, 4);
             zsum += __shfl_xor_sync(FULL, zsum, 1);
             zsum += __shfl_xor_sync(FULL, zsum, 2);
             if (tid == 0 && (gid & 1) == 0) {
@@ -549,13 +588,16 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
         __syncwarp();
         if (lane == 0) mbar_arrive(bar0 + 8 * (2 * stages + stage));
         if (++stage == stages) { stage = 0; phase ^= 1; }
-        if (++page == pages_b) {
-          page = 0;
-          if (++h == Hkv) {
-            h = 0;
-            do { ++b; } while (b < B && sPref[b + 1] == sPref[b]);
-            if (b < B) pages_b = (sPref[b + 1] - sPref[b]) / Hkv;
-          }
+        next_of(b, h, page, pages_b);
+        ++x;
+      }
+      if (!ok) {
+        *abort_flag = 1;
+        if (lane == 0) atomicOr(c.status, KVQ_STATUS_DEVICE_TIMEOUT);
+        // never leave while a copy may still be writing this CTA's shared memory: wait (bounded) for those not seen yet
+        for (; x < ix; ++x) {
+          mbar_wait(bar0 + 8 * stage, phase, wait_ns);
+          if (++stage == stages) { stage = 0; phase ^= 1; }
         }
       }
       return;
@@ -648,7 +690,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
     for (int nh = 0; nh < NH; ++nh) {
       const int hb = (gid >> 1) + 4 * nh;                          // head of this lane's operand column
       hs[nh] = 0.f;
-      if constexpr (KAXIS == 0) {       // (channel-wise keys: the preparation warp makes the operands, per page)
+      if constexpr (KAXIS == 0) {       // (channel-wise keys: the producer warp makes the operands, per page)
         float qv[NR][4];
         float amax = load_q_lane<D>(g, c, q, b, h, hb, tid, qv);
         amax = fmaxf(amax, __shfl_xor_sync(FULL, amax, 1));
@@ -736,7 +778,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
                 if (v1) rb = *reinterpret_cast<const uint2*>(tl + 8 * D + 16 * r + 4 * tid);
                 const uint32_t a0 = __byte_perm(ra.x, ra.y, 0x5410), a1 = __byte_perm(rb.x, rb.y, 0x5410);
                 const uint32_t a2 = __byte_perm(ra.x, ra.y, 0x7632), a3 = __byte_perm(rb.x, rb.y, 0x7632);
-                mma16816(S, a0, a1, a2, a3, qB[nh][0][r], qB[nh][NTK - 1][r]);    // q's fp16 parts, made by the preparation warp
+                mma16816(S, a0, a1, a2, a3, qB[nh][0][r], qB[nh][NTK - 1][r]);    // q's fp16 parts, made by the producer warp
               }
               L[u][0][nh] = c1 * (S[0] + S[1]);
               L[u][1][nh] = c1 * (S[2] + S[3]);
@@ -1130,7 +1172,7 @@ int launch_mma_inst(const Geom& g, const CachePtrs& c, const void* q, float c1, 
   auto kern = decode_mma_kernel<D, KB, VB, KAXIS, NGK, NGV, NH, MINB>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sl.total) != cudaSuccess)
     return KVQ_ERR_CUDA_LAUNCH;
-  const cudaError_t e = launch_dependent(kern, dim3(148 * MINB), (kConsumerWarps + 1 + (KAXIS == 1 ? 1 : 0)) * 32, sl.total, stream, 1, g, c,
+  const cudaError_t e = launch_dependent(kern, dim3(148 * MINB), (kConsumerWarps + 1) * 32, sl.total, stream, 1, g, c,
                                          static_cast<const uint16_t*>(q), c1, ws, s_cap, stages, out, out_dtype, call_id, wait_ns, skip_x);
   return e == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
 }
