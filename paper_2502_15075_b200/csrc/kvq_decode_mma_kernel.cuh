@@ -102,12 +102,12 @@ constexpr int kGapPages = 8, kGapPagesChan = 2;
 constexpr float kQFix = 32512.0f;          // largest |Q| of the 16-bit fixed-point q (hi limb stays within +-127)
 constexpr float kQFix3 = 8300000.0f;       // ... of the 24-bit fixed-point q * s of channel-wise keys (three limbs)
 
-// Four values times `scale` rounded to integers |Q| <= kQFix3 and taken apart as two's-complement bytes,
+// Four values |t| <= kQFix3 rounded to integers Q and taken apart as two's-complement bytes,
 // Q = b2 * 65536 + b1 * 256 + b0 with b2 signed and b1, b0 unsigned; byte j of w[k] is b_k of t[j].  The even operand
 // columns carry b2 in n-tile 0 (signed bytes) and b1 in n-tile 1 (unsigned bytes), the odd ones nothing in n-tile 0 and b0 in n-tile 1.
-__device__ __forceinline__ void fixed_point_bytes3(const float (&t)[4], float scale, uint32_t (&w)[3]) {
-  const uint32_t q0 = (uint32_t)__float2int_rn(t[0] * scale), q1 = (uint32_t)__float2int_rn(t[1] * scale);
-  const uint32_t q2 = (uint32_t)__float2int_rn(t[2] * scale), q3 = (uint32_t)__float2int_rn(t[3] * scale);
+__device__ __forceinline__ void fixed_point_bytes3(const float (&t)[4], uint32_t (&w)[3]) {
+  const uint32_t q0 = (uint32_t)__float2int_rn(t[0]), q1 = (uint32_t)__float2int_rn(t[1]);
+  const uint32_t q2 = (uint32_t)__float2int_rn(t[2]), q3 = (uint32_t)__float2int_rn(t[3]);
   const uint32_t lo01 = prmt(q0, q1, 0x5140u), lo23 = prmt(q2, q3, 0x5140u);      // bytes (0, 0), (1, 1) of a pair
   w[0] = prmt(lo01, lo23, 0x5410u);
   w[1] = prmt(lo01, lo23, 0x7632u);
@@ -282,6 +282,8 @@ static __host__ __device__ __forceinline__ bool weighted_shares(const FlatPlan& 
 // replayed graph: 8B shape 32k K4V2 80.0 -> 78.5 us (16k: 48.7 -> 45.4, K2V4 49.6 -> 45.8, K4V4 54.8 -> 51.5, K8V4 75.2 -> 70.7, groups of
 // 32 / 64 57.9 / 59.4 -> 52.4 / 52.7); 8 heads per KV head 16 x 16,384 tokens 84 -> 68; channel-wise 16 x 32,768 tokens K4V2 183 -> 154,
 // 16,384 tokens K8V2 101.6 -> 88.4; 4 x 8 streams of 4,000 tokens 22.5 -> 18.0.
+// The two token rows of a lane share every fp32 operation on logits and weights that has a packed form: two 70B-shaped layers at 128k
+// tokens, step 256 -> 251 us, 8B shape 181 -> 179.
 constexpr int kConsumerWarps = 4;
 template <int D, int KB, int VB, int KAXIS, int NGK, int NGV, int NH, int MINB>
 __global__ void __launch_bounds__((kConsumerWarps + 1) * 32, MINB)
@@ -558,24 +560,27 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
             const int hb = (gid >> 1) + 4 * nh;
             const float am = amaxB[nh] * smax;
             const float scale = am > 0.f ? kQFix3 / am : 0.f;
-            float zsum = 0.f;
+            f32x2 zsum2 = pack2(0.f, 0.f);
 #pragma unroll
             for (int r = 0; r < HR; ++r) {
               const uint4 mm = *reinterpret_cast<const uint4*>(km + 16 * (r0 + r) + 4 * tid);     // (s, z) of 4 channels
               const uint32_t mw[4] = {mm.x, mm.y, mm.z, mm.w};
               float t[4];
 #pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const float2 sz = __half22float2(as_h2(mw[j]));
-                t[j] = qv[nh][r][j] * sz.x;
-                zsum = fmaf(qv[nh][r][j], sz.y, zsum);
+              for (int j = 0; j < 4; j += 2) {
+                const float2 a = __half22float2(as_h2(mw[j])), d = __half22float2(as_h2(mw[j + 1]));
+                const f32x2 q2 = pack2(qv[nh][r][j], qv[nh][r][j + 1]);
+                zsum2 = fma2(q2, pack2(a.y, d.y), zsum2);
+                const float2 x = unpack2(mul2(mul2(q2, pack2(a.x, d.x)), pack2(scale, scale)));
+                t[j] = x.x; t[j + 1] = x.y;
               }
               uint32_t w[3];
-              fixed_point_bytes3(t, scale, w);
+              fixed_point_bytes3(t, w);
               uint32_t* o = ops + (nh * 2 * NR + r0 + r) * 32 + even;
               o[0] = w[2]; o[4] = 0u;
               o[NR * 32] = w[1]; o[NR * 32 + 4] = w[0];
             }
+            float zsum = unpack2(zsum2).x + unpack2(zsum2).y;
             zsum += __shfl_xor_sync(FULL, zsum, 4);
             zsum += __shfl_xor_sync(FULL, zsum, 1);
             zsum += __shfl_xor_sync(FULL, zsum, 2);
@@ -735,8 +740,8 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       const uint8_t* sp = smem + stage * sl.page_stride;
       uint8_t* wbuf = smem + sl.w_off + (page_no & 1) * (NGV * 4 * WB);
       // ---- logits of the warp's 32 tokens, two tiles of 16; (scale, zero) of their values
-      float L[2][2][NH];                 // [tile][row gid / gid + 8][head]
-      float sv[2][2][NGV], zv[2][2][NGV];
+      f32x2 L[2][NH];                    // [tile][head], of rows gid and gid + 8
+      f32x2 sv[2][NGV], zv[2][NGV];
       const bool active = FULL_PAGE || warp * 32 < nv;
       const bool masked = !FULL_PAGE && (page + pp) * kPageTokens + warp * 32 + 32 > n_unmasked;
       bool trig = false;
@@ -780,8 +785,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
                 const uint32_t a2 = __byte_perm(ra.x, ra.y, 0x7632), a3 = __byte_perm(rb.x, rb.y, 0x7632);
                 mma16816(S, a0, a1, a2, a3, qB[nh][0][r], qB[nh][NTK - 1][r]);    // q's fp16 parts, made by the producer warp
               }
-              L[u][0][nh] = c1 * (S[0] + S[1]);
-              L[u][1][nh] = c1 * (S[2] + S[3]);
+              L[u][nh] = pack2(c1 * (S[0] + S[1]), c1 * (S[2] + S[3]));
             }
           } else {
             uint32_t ka[KW], kb2[KW];
@@ -810,25 +814,23 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
             if constexpr (KAXIS == 1) {
 #pragma unroll
               for (int nh = 0; nh < NH; ++nh) {
-                const float t0 = fmaf((float)S[0][nh][0][0], 65536.f, fmaf((float)S[0][nh][NTK - 1][0], 256.f, (float)S[0][nh][NTK - 1][1]));
-                const float t1 = fmaf((float)S[0][nh][0][2], 65536.f, fmaf((float)S[0][nh][NTK - 1][2], 256.f, (float)S[0][nh][NTK - 1][3]));
-                L[u][0][nh] = fmaf(t0, hs[nh], zq[nh]);
-                L[u][1][nh] = fmaf(t1, hs[nh], zq[nh]);
+                // (the two lower bytes' sums fit 32 bits together: 128 x 255 x 255 x 257 < 2^31)
+                const f32x2 lo = pack2((float)(S[0][nh][NTK - 1][0] * 256 + S[0][nh][NTK - 1][1]), (float)(S[0][nh][NTK - 1][2] * 256 + S[0][nh][NTK - 1][3]));
+                const f32x2 t = fma2(pack2((float)S[0][nh][0][0], (float)S[0][nh][0][2]), pack2(65536.f, 65536.f), lo);
+                L[u][nh] = fma2(t, pack2(hs[nh], hs[nh]), pack2(zq[nh], zq[nh]));
               }
             } else {
               const uint32_t* km = reinterpret_cast<const uint32_t*>(sp + lane_km + u * (16 * 4 * NGK));   // row tok0
 #pragma unroll
-              for (int nh = 0; nh < NH; ++nh) { L[u][0][nh] = 0.f; L[u][1][nh] = 0.f; }
-#pragma unroll
               for (int j = 0; j < NGK; ++j) {
                 const float2 ma = __half22float2(as_h2(km[j]));                       // (scale, zero) of row tok0
                 const float2 mb = __half22float2(as_h2(km[8 * NGK + j]));             // ... of row tok0 + 8
+                const f32x2 s2 = pack2(ma.x, mb.x), z2 = pack2(ma.y, mb.y);
 #pragma unroll
                 for (int nh = 0; nh < NH; ++nh) {
-                  const float t0 = (float)(S[j][nh][0][0] * 256 + S[j][nh][0][1]);
-                  const float t1 = (float)(S[j][nh][0][2] * 256 + S[j][nh][0][3]);
-                  L[u][0][nh] += fmaf(ma.x * hs[nh], t0, ma.y * qsum[nh][j]);
-                  L[u][1][nh] += fmaf(mb.x * hs[nh], t1, mb.y * qsum[nh][j]);
+                  const f32x2 t = pack2((float)(S[j][nh][0][0] * 256 + S[j][nh][0][1]), (float)(S[j][nh][0][2] * 256 + S[j][nh][0][3]));
+                  const f32x2 x = fma2(mul2(s2, pack2(hs[nh], hs[nh])), t, mul2(z2, pack2(qsum[nh][j], qsum[nh][j])));
+                  L[u][nh] = j == 0 ? x : add2(L[u][nh], x);
                 }
               }
             }
@@ -837,34 +839,37 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
 #pragma unroll
           for (int j = 0; j < NGV; ++j) {
             const float2 fa = __half22float2(as_h2(vm[j])), fb = __half22float2(as_h2(vm[8 * NGV + j]));
-            sv[u][0][j] = fa.x; zv[u][0][j] = fa.y;
-            sv[u][1][j] = fb.x; zv[u][1][j] = fb.y;
+            sv[u][j] = pack2(fa.x, fb.x);
+            zv[u][j] = pack2(fa.y, fb.y);
           }
           if (masked) {
             const int tokg = (page + pp) * kPageTokens + tok0;        // position of row tok0 in the sequence
+            const bool there0 = tok0 < nv, there1 = tok0 + 8 < nv;
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-              const bool there = tok0 + 8 * r < nv;
+            for (int nh = 0; nh < NH; ++nh) {
+              // tokens the lane's head may attend to: the causal limit of its query row
+              const int lim = n_all - (g.rows - 1 - min((tid + 4 * nh) / Gq, g.rows - 1));
+              float2 x = unpack2(L[u][nh]);
+              if (!there0 || tokg >= lim) x.x = -INFINITY;
+              if (!there1 || tokg + 8 >= lim) x.y = -INFINITY;
+              L[u][nh] = pack2(x.x, x.y);
+            }
 #pragma unroll
-              for (int nh = 0; nh < NH; ++nh) {
-                // tokens the lane's head may attend to: the causal limit of its query row
-                const int lim = n_all - (g.rows - 1 - min((tid + 4 * nh) / Gq, g.rows - 1));
-                if (!there || tokg + 8 * r >= lim) L[u][r][nh] = -INFINITY;
-              }
-#pragma unroll
-              for (int j = 0; j < NGV; ++j) {
-                if (!there) sv[u][r][j] = zv[u][r][j] = 0.f;
-              }
+            for (int j = 0; j < NGV; ++j) {
+              const float2 x = unpack2(sv[u][j]), y = unpack2(zv[u][j]);
+              sv[u][j] = pack2(there0 ? x.x : 0.f, there1 ? x.y : 0.f);
+              zv[u][j] = pack2(there0 ? y.x : 0.f, there1 ? y.y : 0.f);
             }
           }
 #pragma unroll
-          for (int j = 0; j < NGV; ++j) smax = fmaxf(smax, fmaxf(sv[u][0][j], sv[u][1][j]));
+          for (int j = 0; j < NGV; ++j) smax = fmaxf(smax, fmaxf(unpack2(sv[u][j]).x, unpack2(sv[u][j]).y));
         }
         // ---- softmax reference / scale check (rarely true)
         trig = smax * sscale >= PONE;
 #pragma unroll
         for (int nh = 0; nh < NH; ++nh) {
-          bmax[nh] = fmaxf(fmaxf(L[0][0][nh], L[0][1][nh]), fmaxf(L[1][0][nh], L[1][1][nh]));
+          const float2 x = unpack2(L[0][nh]), y = unpack2(L[1][nh]);
+          bmax[nh] = fmaxf(fmaxf(x.x, x.y), fmaxf(y.x, y.y));
           trig |= bmax[nh] > m_ref[nh];
         }
       }
@@ -873,39 +878,33 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       // the B operands of the block; the sums over the warp's own tokens are kept apart until the reference holds
       float psum[NH], zsum[NH][NGV];
       auto make_weights = [&]() {
-#pragma unroll
-        for (int nh = 0; nh < NH; ++nh) {
-          psum[nh] = 0.f;
-#pragma unroll
-          for (int j = 0; j < NGV; ++j) zsum[nh][j] = 0.f;
-        }
+        f32x2 psum2[NH], zsum2[NH][NGV];          // over the even and the odd rows of the tiles
         uint32_t bV[NGV][NTV][2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          float p[2][NH];
+          f32x2 p[NH];
 #pragma unroll
           for (int nh = 0; nh < NH; ++nh) {
-            p[0][nh] = ex2(L[u][0][nh] - m_ref[nh]);
-            p[1][nh] = ex2(L[u][1][nh] - m_ref[nh]);
-          }
-          if (masked) {       // a head that has seen no token yet has no reference: its weights are zero
-#pragma unroll
-            for (int nh = 0; nh < NH; ++nh) {
-              if (L[u][0][nh] == -INFINITY) p[0][nh] = 0.f;
-              if (L[u][1][nh] == -INFINITY) p[1][nh] = 0.f;
+            const float2 x = unpack2(add2(L[u][nh], pack2(-m_ref[nh], -m_ref[nh])));
+            float2 e = make_float2(ex2(x.x), ex2(x.y));
+            if (masked) {       // a head that has seen no token yet has no reference: its weights are zero
+              const float2 y = unpack2(L[u][nh]);
+              if (y.x == -INFINITY) e.x = 0.f;
+              if (y.y == -INFINITY) e.y = 0.f;
             }
+            p[nh] = pack2(e.x, e.y);
+            psum2[nh] = u == 0 ? p[nh] : add2(psum2[nh], p[nh]);
           }
-#pragma unroll
-          for (int nh = 0; nh < NH; ++nh) psum[nh] += p[0][nh] + p[1][nh];
 #pragma unroll
           for (int j = 0; j < NGV; ++j) {
-            const float sa = sv[u][0][j] * sscale, sb = sv[u][1][j] * sscale;
+            const f32x2 ss = mul2(sv[u][j], pack2(sscale, sscale));
             uint32_t Pa[NH], Pb[NH];
 #pragma unroll
             for (int nh = 0; nh < NH; ++nh) {
-              zsum[nh][j] = fmaf(p[0][nh], zv[u][0][j], fmaf(p[1][nh], zv[u][1][j], zsum[nh][j]));
-              Pa[nh] = __float2uint_rn(p[0][nh] * sa);      // token tok0
-              Pb[nh] = __float2uint_rn(p[1][nh] * sb);      // token tok0 + 8
+              zsum2[nh][j] = u == 0 ? mul2(p[nh], zv[u][j]) : fma2(p[nh], zv[u][j], zsum2[nh][j]);
+              const float2 x = unpack2(mul2(p[nh], ss));
+              Pa[nh] = __float2uint_rn(x.x);      // token tok0
+              Pb[nh] = __float2uint_rn(x.y);      // token tok0 + 8
             }
             // one 16-bit element per (column, lane row) = that column's limb of tokens (tok0, tok0 + 8); the 8x8
             // transpose turns lane columns into the B operand (column = lane/4, tokens 2t, 2t+8, 2t+1, 2t+9)
@@ -915,6 +914,12 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
               bV[j][2 * nh + 1][u] = movmatrix_trans(prmt(Pa[nh], Pb[nh], 0x4051));     // limbs (1, 0): bytes a1 b1 a0 b0
             }
           }
+        }
+#pragma unroll
+        for (int nh = 0; nh < NH; ++nh) {
+          psum[nh] = unpack2(psum2[nh]).x + unpack2(psum2[nh]).y;
+#pragma unroll
+          for (int j = 0; j < NGV; ++j) zsum[nh][j] = unpack2(zsum2[nh][j]).x + unpack2(zsum2[nh][j]).y;
         }
 #pragma unroll
         for (int j = 0; j < NGV; ++j) {
