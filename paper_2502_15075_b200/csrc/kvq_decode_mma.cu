@@ -87,7 +87,7 @@ void host_plan(const Geom& g, int gap, const int32_t* seq_len, int32_t* parts, i
   const bool waves = mma::weighted_shares<WAVES>(plan, gap, WAVES * 148, pmax, slots);
   info[0] = slots; info[1] = plan.c_eff; info[2] = waves;
   for (int c = 0; c <= plan.c_eff && plan.N; ++c)
-    starts[c] = mma::first_page<WAVES>(plan, waves, c, pref, vpref, g.B, g.Hkv, gap);
+    starts[c] = mma::share_start<WAVES>(plan, waves, c, pref, vpref, g.B, g.Hkv, gap).x;
   for (int b = 0; b < g.B; ++b) {
     const int pages = (pref[b + 1] - pref[b]) / g.Hkv;
     for (int h = 0; h < g.Hkv; ++h) {

@@ -190,21 +190,36 @@ __device__ __forceinline__ float meta_z(uint32_t m) { return __half2float(__usho
 // ------------------------------------------------------------------ flat split and merge bookkeeping
 constexpr int kMaxBatchFlat = 1024;   // the flat partition keeps a per-batch prefix in shared memory
 
+// n / d of 64-bit integers (n >= 0, d > 0, quotient below 2^31), exact: an fp32 estimate of the quotient and of what it leaves, then
+// whole steps.  A 64-bit division in software is several times as long, and the split of a decode call waits for three of them (with
+// them, a second search for the sequence and queries that were not yet in L2: 16 layers of the 1B shape 354 us, 350 without, two
+// 70B-shaped layers 251 and 246, 14B 230 and 226).
+__host__ __device__ __forceinline__ long long divide(long long n, long long d) {
+  const float df = (float)d;
+  long long q = (long long)((float)n / df), r = n - q * d;
+  const long long e = (long long)((float)r / df);
+  q += e;
+  r -= e * d;
+  while (r < 0) { --q; r += d; }
+  while (r >= d) { ++q; r -= d; }
+  return q;
+}
+
 // Flat split of all pages over the grid.
 struct FlatPlan {
   long long N;       // total pages over all streams
   int c_eff;         // CTAs that take part
-  __host__ __device__ __forceinline__ int cta_of(long long x) const { return (int)(((x + 1) * c_eff - 1) / N); }
-  __host__ __device__ __forceinline__ long long lo(int c) const { return (long long)c * N / c_eff; }
+  __host__ __device__ __forceinline__ int cta_of(long long x) const { return (int)divide((x + 1) * c_eff - 1, N); }
+  __host__ __device__ __forceinline__ long long lo(int c) const { return divide((long long)c * N, c_eff); }
 };
 
 __host__ __device__ __forceinline__ FlatPlan make_plan(long long N, int pages_max, int grid, int s_cap) {
   FlatPlan p;
   p.N = N;
-  long long cap = pages_max > 0 ? (long long)(s_cap - 1) * N / pages_max : 0;
-  long long ce = grid;
+  long long ce = grid;                        // the smallest of grid, N and (s_cap - 1) N / pages_max
   if (ce > N) ce = N;
-  if (ce > cap) ce = cap;
+  if (pages_max <= 0) ce = 0;
+  else if ((long long)(s_cap - 1) * N < ce * pages_max) ce = divide((long long)(s_cap - 1) * N, pages_max);
   p.c_eff = (int)ce;
   return p;
 }

@@ -216,35 +216,31 @@ static __host__ __device__ __forceinline__ int cta_of_virtual(const FlatPlan& pl
   const long long b1 = plan.N * (148ll * W0), b2 = plan.N * (148ll * (W0 + W1));
   const int k = (WAVES == 3 && a >= b2) ? 2 : a >= b1 ? 1 : 0;
   const long long base = k == 2 ? b2 : k == 1 ? b1 : 0;
-  const long long r = (a - base) / (plan.N * (k == 2 ? W2 : k == 1 ? W1 : W0));
+  const long long r = divide(a - base, plan.N * (k == 2 ? W2 : k == 1 ? W1 : W0));
   return 148 * k + (int)(r < 147 ? r : 147);
 }
-// Flat index of the first real page at or after the start of a CTA's share (sPref: pages, sVPref: pages + gaps).
+// Where a CTA's share starts: its first real page, flat and as (sequence, KV head, page).  sPref, sVPref: pages per sequence over all KV
+// heads, and pages with gaps, as prefixes over the batch.  The CTA behind the last one that takes part starts where the pages end.
+struct ShareStart { long long x; int b, h, page; };
 template <int WAVES>
-static __host__ __device__ __forceinline__ long long share_start(const FlatPlan& plan, bool waves, int cta, const int* sPref,
+static __host__ __device__ __forceinline__ ShareStart share_start(const FlatPlan& plan, bool waves, int cta, const int* sPref,
                                                      const int* sVPref, int B, int Hkv, int gap) {
   const long long v = share_start_virtual<WAVES>(plan, waves, cta);
-  if (v >= plan.N) return sPref[B];
+  if (v >= plan.N) return {sPref[B], 0, 0, 0};
   int lo_ = 0, hi_ = B - 1;                        // last batch entry with sVPref <= v
   while (lo_ < hi_) {
     const int mid = (lo_ + hi_ + 1) >> 1;
     if (sVPref[mid] <= v) lo_ = mid; else hi_ = mid - 1;
   }
-  const int pb = (sPref[lo_ + 1] - sPref[lo_]) / Hkv, len = pb + gap;
-  const int vs = (int)(v - sVPref[lo_]), hh = vs / len, off = vs % len;
-  return (long long)sPref[lo_] + (long long)hh * pb + (off > gap ? off - gap : 0);
+  const int len = (sVPref[lo_ + 1] - sVPref[lo_]) / Hkv, pb = len - gap;
+  const int vs = (int)v - sVPref[lo_], hh = vs / len, off = vs - hh * len, pg = off > gap ? off - gap : 0;
+  return {(long long)sPref[lo_] + (long long)hh * pb + pg, lo_, hh, pg};
 }
 // The CTAs that hold pages of a stream: the first one, and how many (its partials).  xs: the stream's first page, virtual axis.
 template <int WAVES>
 static __host__ __device__ __forceinline__ void stream_ctas(const FlatPlan& plan, bool waves, long long xs, int pages, int* first, int* count) {
   *first = cta_of_virtual<WAVES>(plan, waves, xs);
   *count = cta_of_virtual<WAVES>(plan, waves, xs + pages - 1) - *first + 1;
-}
-// First page (real, flat) of a CTA's share; the CTA behind the last one that takes part starts where the pages end.
-template <int WAVES>
-static __host__ __device__ __forceinline__ long long first_page(const FlatPlan& plan, bool waves, int cta, const int* sPref,
-                                                             const int* sVPref, int B, int Hkv, int gap) {
-  return gap == 0 ? plan.lo(cta) : share_start<WAVES>(plan, waves, cta, sPref, sVPref, B, Hkv, gap);
 }
 // The time-balanced split (stream gaps) pays where the arithmetic per page limits the kernel (token-wise and
 // channel-wise keys alike); pages of 10 bits per element pair and more lose with it and keep the plain split by pages.
@@ -349,6 +345,9 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
     __syncwarp();
   }
   begin_after_predecessor();
+  // the queries, which a stream's start waits for, come to L2 while the split is worked out
+  for (long long i = ((long long)blockIdx.x * blockDim.x + tid_) * 64; i < (long long)B * g.rows * g.Hq * D; i += (long long)gridDim.x * blockDim.x * 64)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(q + i));
   if (warp == 0) {
     int carry = 0, vcarry = 0, pmax = 0;
     for (int base = 0; base < B; base += 32) {
@@ -371,24 +370,10 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       // lane 0: the share's first page, the CTAs that take part and the cursor; lane 1: the share's end
       const FlatPlan p0 = make_plan(vcarry, pmax + GAP, gridDim.x, s_plan);
       const bool w0 = weighted_shares<WAVES>(p0, GAP, gridDim.x, pmax, s_plan);
-      long long x0 = 0;
-      if (p0.N != 0 && (int)blockIdx.x < p0.c_eff)
-        x0 = first_page<WAVES>(p0, w0, (int)blockIdx.x + lane, sPref, sVPref, B, Hkv, GAP);
-      *reinterpret_cast<long long*>(sMisc + 4 + 2 * lane) = x0;
-      if (lane == 0) {
-        int cb = 0, ch = 0, cp = 0;
-        if (x0 < carry) {                      // a real page: (sequence, kv head, page) of the share's first page
-          int lo_ = 0, hi_ = B - 1;            // last sequence with sPref <= x0
-          while (lo_ < hi_) {
-            int mid = (lo_ + hi_ + 1) >> 1;
-            if (sPref[mid] <= x0) lo_ = mid; else hi_ = mid - 1;
-          }
-          cb = lo_;
-          const int pb = (sPref[cb + 1] - sPref[cb]) / Hkv, r = (int)x0 - sPref[cb];
-          if (pb > 0) { ch = r / pb; cp = r % pb; }
-        }
-        sMisc[10] = p0.c_eff; sMisc[11] = cb; sMisc[12] = ch; sMisc[13] = cp; sMisc[14] = w0;
-      }
+      ShareStart at{0, 0, 0, 0};
+      if (p0.N != 0 && (int)blockIdx.x < p0.c_eff) at = share_start<WAVES>(p0, w0, (int)blockIdx.x + lane, sPref, sVPref, B, Hkv, GAP);
+      *reinterpret_cast<long long*>(sMisc + 4 + 2 * lane) = at.x;
+      if (lane == 0) { sMisc[10] = p0.c_eff; sMisc[11] = at.b; sMisc[12] = at.h; sMisc[13] = at.page; sMisc[14] = w0; }
     }
   }
   __syncthreads();
