@@ -39,14 +39,31 @@ append_rows_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, cons
     const int R = g.R, end = t0 + t_new;
     const int qa = R ? (t0 / R) * R : t0, qb = R ? (end / R) * R : end;      // tokens to quantize now
     const int nq = qb - qa, total = nh * (CHAN ? 1 : 2) * nq;
-    for (int base = (tid >> 5) * RPW; base < total; base += (blockDim.x >> 5) * RPW) {
+    // the next row's loads are in flight while this one is quantized (16 layers of the 1B shape that take in 128 tokens, four turns of
+    // rows a warp, and decode: 351 -> 338 us)
+    struct Row { uint4 raw; int hs, t; };
+    auto fetch = [&](int base) {
+      const int idx = base + lane / LPR < total ? base + lane / LPR : base;
+      Row r;
+      r.hs = idx / nq;
+      r.t = qa + idx - r.hs * nq;
+      const bool is_v = CHAN || (r.hs & 1) == 0;
+      const int h = rank + ranks * (CHAN ? r.hs : r.hs >> 1);
+      const uint16_t* src = (is_v ? v_new : k_new) + (int64_t)b * sb + (int64_t)h * sh + (int64_t)(r.t - t0) * st;
+      if (r.t < t0) src = c.kv_win + (((size_t)b * g.Hkv + h) * R + r.t % R) * (2 * D) + (is_v ? D : 0);       // still in the residual window
+      r.raw = *reinterpret_cast<const uint4*>(src + 8 * l);
+      return r;
+    };
+    const int first = (tid >> 5) * RPW, step = (blockDim.x >> 5) * RPW;
+    Row next{};
+    if (first < total) next = fetch(first);
+    for (int base = first; base < total; base += step) {
       const bool active = base + lane / LPR < total;
-      const int idx = active ? base + lane / LPR : base, hs = idx / nq, t = qa + idx % nq;
+      const int hs = next.hs, t = next.t;
       const bool is_v = CHAN || (hs & 1) == 0;
       const int h = rank + ranks * (CHAN ? hs : hs >> 1), bh = b * g.Hkv + h;
-      const uint16_t* src = (is_v ? v_new : k_new) + (int64_t)b * sb + (int64_t)h * sh + (int64_t)(t - t0) * st;
-      if (t < t0) src = c.kv_win + (((size_t)bh * R + t % R) * 2 + (is_v ? 1 : 0)) * D;       // still in the residual window
-      const uint4 raw = *reinterpret_cast<const uint4*>(src + 8 * l);
+      const uint4 raw = next.raw;
+      if (base + step < total) next = fetch(base + step);
       const uint32_t rw[4] = {raw.x, raw.y, raw.z, raw.w};
       float x[8];
 #pragma unroll
