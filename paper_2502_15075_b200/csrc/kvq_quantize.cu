@@ -228,7 +228,8 @@ __device__ __forceinline__ void quantize_task(const RowSrc& rsrc, int gsz, int l
 
 // Rotated keys (y = H (signs * x) / sqrt(D), then token-wise groups): tokens [lo, hi) of a task, one token of a lane at a time with
 // the next one's loads in flight (bound by fetching instructions beside the value side's code; two tokens at a time were slower, 32
-// streams x 2,047 tokens 24.8 us against 24; with the signs converted for every token and lanes' own divisions 36 us).
+// streams x 2,047 tokens 24.8 us against 24; with the signs converted for every token and lanes' own divisions 36 us).  The transform and
+// the codes take two neighbouring channels per operation: four such chunks 90.9 -> 86.2 us.
 // Lanes and fields as in quantize_task; butterfly stages in the order h = 1, 2, 4, ...: bits of i in the lane, rh across
 // lanes, bits of f in the lane, bits of mw across lanes.
 template <int BITS, int D, int DTYPE>
@@ -260,28 +261,40 @@ __device__ __forceinline__ void quantize_task_rotated(const RowSrc& rsrc, int gs
 #pragma unroll 1
   for (int base = lo; base < hi; base += RS) {
     const int tau = base + rs;
-    float x[FPB][8];
+    // (two neighbouring channels share an operation; differences as sums with a product by -1, which is exact)
+    const f32x2 minus = pack2(-1.0f, -1.0f);
+    f32x2 y[FPB][4];
 #pragma unroll
     for (int f = 0; f < FPB; ++f) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) x[f][i] = __fmul_rn(piece_value<DTYPE>(next[f], i), sg[f][i]);
+      for (int i = 0; i < 4; ++i)
+        y[f][i] = mul2(pack2(piece_value<DTYPE>(next[f], 2 * i), piece_value<DTYPE>(next[f], 2 * i + 1)), pack2(sg[f][2 * i], sg[f][2 * i + 1]));
     }
     fetch(tau + RS);
 #pragma unroll
     for (int f = 0; f < FPB; ++f) {
 #pragma unroll
-      for (int h = 1; h < 8; h <<= 1) {
+      for (int i = 0; i < 4; ++i) {
+        const float2 a = unpack2(y[f][i]);
+        y[f][i] = pack2(__fadd_rn(a.x, a.y), __fsub_rn(a.x, a.y));
+      }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+      for (int h = 1; h < 4; h <<= 1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
           if ((i & h) == 0) {
-            const float a = x[f][i], c = x[f][i + h];
-            x[f][i] = __fadd_rn(a, c);
-            x[f][i + h] = __fsub_rn(a, c);
+            const f32x2 a = y[f][i], c = y[f][i + h];
+            y[f][i] = add2(a, c);
+            y[f][i + h] = fma2(c, minus, a);
           }
         }
       }
 #pragma unroll
-      for (int i = 0; i < 8; ++i) x[f][i] = __fmaf_rn(srh, x[f][i], __shfl_xor_sync(FULL, x[f][i], 1));
+      for (int i = 0; i < 4; ++i) {
+        float2 o = unpack2(y[f][i]);
+        o.x = __shfl_xor_sync(FULL, o.x, 1); o.y = __shfl_xor_sync(FULL, o.y, 1);
+        y[f][i] = fma2(pack2(srh, srh), y[f][i], pack2(o.x, o.y));
+      }
     }
 #pragma unroll
     for (int hf = 1; hf < FPB; hf <<= 1) {
@@ -289,10 +302,10 @@ __device__ __forceinline__ void quantize_task_rotated(const RowSrc& rsrc, int gs
       for (int f = 0; f < FPB; ++f) {
         if ((f & hf) == 0) {
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const float a = x[f][i], c = x[f + hf][i];
-            x[f][i] = __fadd_rn(a, c);
-            x[f + hf][i] = __fsub_rn(a, c);
+          for (int i = 0; i < 4; ++i) {
+            const f32x2 a = y[f][i], c = y[f + hf][i];
+            y[f][i] = add2(a, c);
+            y[f + hf][i] = fma2(c, minus, a);
           }
         }
       }
@@ -303,7 +316,20 @@ __device__ __forceinline__ void quantize_task_rotated(const RowSrc& rsrc, int gs
 #pragma unroll
       for (int f = 0; f < FPB; ++f) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) x[f][i] = __fmaf_rn(sm, x[f][i], __shfl_xor_sync(FULL, x[f][i], 2 * hm));
+        for (int i = 0; i < 4; ++i) {
+          float2 o = unpack2(y[f][i]);
+          o.x = __shfl_xor_sync(FULL, o.x, 2 * hm); o.y = __shfl_xor_sync(FULL, o.y, 2 * hm);
+          y[f][i] = fma2(pack2(sm, sm), y[f][i], pack2(o.x, o.y));
+        }
+      }
+    }
+    float x[FPB][8];
+#pragma unroll
+    for (int f = 0; f < FPB; ++f) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 a = unpack2(mul2(y[f][i], pack2(inv_sqrt_dim<D>(), inv_sqrt_dim<D>())));
+        x[f][2 * i] = a.x; x[f][2 * i + 1] = a.y;
       }
     }
     // (from the first value on, as everywhere: a row of NaN has the same parameters in every kernel)
@@ -313,7 +339,6 @@ __device__ __forceinline__ void quantize_task_rotated(const RowSrc& rsrc, int gs
       const int e = NSET == 2 ? f >> 1 : 0;
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        x[f][i] = __fmul_rn(x[f][i], inv_sqrt_dim<D>());
         const bool first = i == 0 && f == (FPB / NSET) * e;
         mn[e] = first ? x[f][i] : fminf(mn[e], x[f][i]);
         mx[e] = first ? x[f][i] : fmaxf(mx[e], x[f][i]);
@@ -344,10 +369,10 @@ __device__ __forceinline__ void quantize_task_rotated(const RowSrc& rsrc, int gs
 #pragma unroll
       for (int f = FPB - 1; f >= 0; --f) {
         const int e = NSET == 2 ? f >> 1 : 0;
-        float v[4], zz[4], ii[4];
+        float v[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) { v[j] = x[f][4 * hh + j]; zz[j] = z[e]; ii[j] = inv[e]; }
-        w = w * (1u << BITS) + code_word4<BITS>(v, zz, ii);
+        for (int j = 0; j < 4; ++j) v[j] = x[f][4 * hh + j];
+        w = w * (1u << BITS) + code_word4_packed<BITS>(v, z[e], inv[e]);
       }
       if (tau < hi)
         *reinterpret_cast<uint32_t*>(codes + (size_t)tau * K_ROW_BYTES + chunk_word_byte(2 * rh + hh, mw, wpc, 4)) = w;
