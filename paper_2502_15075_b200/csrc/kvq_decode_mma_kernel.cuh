@@ -890,7 +890,11 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       // the B operands of the block; the sums over the warp's own tokens are kept apart until the reference holds
       float psum[NH], zsum[NH][NGV];
       auto make_weights = [&]() {
-        f32x2 psum2[NH], zsum2[NH][NGV];          // over the even and the odd rows of the tiles
+        // One head a lane: sums in one chain, token tok0 + 8 before tok0, tile after tile (neighbouring tokens that cancel do so
+        // exactly; the last bits of every output follow this order).  Two heads: two chains, over tok0 and over tok0 + 8, in packed
+        // operations; one chain costs two 70B-shaped layers at 128k tokens 4.5 us (246.5 -> 251), one-head shapes nothing.
+        constexpr bool CHAINS = NH == 2;
+        [[maybe_unused]] f32x2 psum2[NH], zsum2[NH][NGV];
         uint32_t bV[NGV][NTV][2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
@@ -905,7 +909,8 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
               if (y.y == -INFINITY) e.y = 0.f;
             }
             p[nh] = pack2(e.x, e.y);
-            psum2[nh] = u == 0 ? p[nh] : add2(psum2[nh], p[nh]);
+            if constexpr (CHAINS) psum2[nh] = u == 0 ? p[nh] : add2(psum2[nh], p[nh]);
+            else psum[nh] = u == 0 ? e.x + e.y : psum[nh] + (e.x + e.y);
           }
 #pragma unroll
           for (int j = 0; j < NGV; ++j) {
@@ -913,7 +918,12 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
             uint32_t Pa[NH], Pb[NH];
 #pragma unroll
             for (int nh = 0; nh < NH; ++nh) {
-              zsum2[nh][j] = u == 0 ? mul2(p[nh], zv[u][j]) : fma2(p[nh], zv[u][j], zsum2[nh][j]);
+              if constexpr (CHAINS) {
+                zsum2[nh][j] = u == 0 ? mul2(p[nh], zv[u][j]) : fma2(p[nh], zv[u][j], zsum2[nh][j]);
+              } else {
+                const float2 e = unpack2(p[nh]), z = unpack2(zv[u][j]);
+                zsum[nh][j] = fmaf(e.x, z.x, u == 0 ? e.y * z.y : fmaf(e.y, z.y, zsum[nh][j]));
+              }
               const float2 x = unpack2(mul2(p[nh], ss));
               Pa[nh] = __float2uint_rn(x.x);      // token tok0
               Pb[nh] = __float2uint_rn(x.y);      // token tok0 + 8
@@ -927,11 +937,13 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
             }
           }
         }
+        if constexpr (CHAINS) {
 #pragma unroll
-        for (int nh = 0; nh < NH; ++nh) {
-          psum[nh] = unpack2(psum2[nh]).x + unpack2(psum2[nh]).y;
+          for (int nh = 0; nh < NH; ++nh) {
+            psum[nh] = unpack2(psum2[nh]).x + unpack2(psum2[nh]).y;
 #pragma unroll
-          for (int j = 0; j < NGV; ++j) zsum[nh][j] = unpack2(zsum2[nh][j]).x + unpack2(zsum2[nh][j]).y;
+            for (int j = 0; j < NGV; ++j) zsum[nh][j] = unpack2(zsum2[nh][j]).x + unpack2(zsum2[nh][j]).y;
+          }
         }
 #pragma unroll
         for (int j = 0; j < NGV; ++j) {

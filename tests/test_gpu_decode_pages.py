@@ -79,6 +79,22 @@ def test_streams_of_very_different_values_share_a_cta(kvq, form, heads):
     assert err.max() <= tl.REL_L2_TOL, f"stream {err.argmax()}: rel-L2 {err.max():.2e}"
 
 
+@pytest.mark.parametrize("form", ["k4v2", "k4v4", "k2v4", "k8v4", "k4v2-g64", "d64", "channel-k4v2"])
+@pytest.mark.parametrize("T", [32, 256, 1536])
+def test_neighbouring_tokens_cancel_exactly(kvq, form, T):
+    """Equal weights, values 2^27 apart that cancel between tokens t and t + 8: a lane adds the two before it goes on to the next
+    tile, so what is left is exact.  (Values are constant over a row: codes and scales are 0, a token adds weight x zero-point.)"""
+    w = FORMS[form].with_(n_kv_heads=2, n_q_heads=8)
+    big, small = 2.0 ** 15, 2.0 ** -12
+    t = torch.arange(T) % 32
+    row = torch.where(t < 8, big, torch.where(t < 16, -big, small))
+    k, v = wl.make_kv(w, tokens=T, batch=2)
+    v = row.view(1, 1, T, 1).expand(v.shape).to(w.torch_dtype).contiguous()
+    cfg, gc, _ = tl.build_both(kvq, w, k, v, [T], 1536)
+    got = tl.gpu_decode(kvq, cfg, gc, torch.zeros((2, 8, w.head_dim), dtype=w.torch_dtype))      # every logit is 0
+    assert np.array_equal(got, np.full(got.shape, small / 2))
+
+
 def test_value_sums_over_more_pages_than_an_integer_accumulator_holds(kvq):
     """Over 350 pages per CTA of equal weights and largest codes: without the fold every 128 pages the 32-bit sums would overflow
     (the second weight byte is 254, the upper code field 192: 344 pages of 128 tokens).  All values of a head are equal, so the
