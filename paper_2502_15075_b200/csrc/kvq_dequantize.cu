@@ -139,7 +139,8 @@ __device__ __forceinline__ void fast_keys(const Geom& g, const uint8_t* __restri
 // Rotated keys of one page: as fast_keys, rotated back (x = signs * H y / sqrt(D)) before they are rounded.  A thread has channels
 // 16 r + 4 chunk + j of its token, so of the butterfly stages h = 1, 2, 4, ..., in this order, only h = 4 and 8 cross lanes (two shuffles
 // per element instead of the four of eight consecutive channels a lane).  32 streams x 30,000 tokens K4V2, both sides: 213 us with
-// the page staged in shared memory and element-wise expansion, 135 now.
+// the page staged in shared memory and element-wise expansion, 135 now.  The signs may lie at any address: they are read byte by byte,
+// once per CTA, and a row takes them as words of shared memory (four bytes a word from global memory for every row: 142.)
 template <int B, int D, int AXIS, int DTYPE>
 __device__ __forceinline__ void fast_keys_rotated(const Geom& g, const uint8_t* __restrict__ pg, const uint16_t* __restrict__ tail,
                                                   const int8_t* __restrict__ signs, uint16_t* __restrict__ out, int lo, int hi, int tid) {
@@ -148,6 +149,9 @@ __device__ __forceinline__ void fast_keys_rotated(const Geom& g, const uint8_t* 
   const uint32_t* meta = reinterpret_cast<const uint32_t*>(pg + g.k_meta_off);
   const int lgk = ilog2(g.gk), ngk = D >> lgk, chunk = tid & 3;
   const float s4 = (chunk & 1) ? -1.0f : 1.0f, s8 = (chunk & 2) ? -1.0f : 1.0f;      // a butterfly between lanes: o + s x (exact product)
+  __shared__ char4 sign[D / 4];
+  if (tid < D) reinterpret_cast<int8_t*>(sign)[tid] = __ldg(signs + tid);
+  __syncthreads();
   for (int item = tid; item < kPageTokens * 4; item += kThreads) {
     const int t = item >> 2;
     const bool active = t >= lo && t < hi;
@@ -229,7 +233,7 @@ __device__ __forceinline__ void fast_keys_rotated(const Geom& g, const uint8_t* 
     constexpr float NORM = inv_sqrt_dim<D>();
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-      const char4 s = __ldg(reinterpret_cast<const char4*>(signs + 16 * r + 4 * chunk));
+      const char4 s = sign[4 * r + chunk];
       const uint32_t a = pack16<DTYPE>(mul2(mul2(x[r][0], pack2(NORM, NORM)), pack2((float)s.x, (float)s.y)));
       const uint32_t b = pack16<DTYPE>(mul2(mul2(x[r][1], pack2(NORM, NORM)), pack2((float)s.z, (float)s.w)));
       __stcs(reinterpret_cast<uint2*>(orow + 16 * r), make_uint2(a, b));

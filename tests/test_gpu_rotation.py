@@ -60,6 +60,34 @@ def test_rotated_keys_parity(kvq, name):
         tl.assert_attention_close(tl.gpu_decode(kvq, cfg, gc, q), oc2.decode(tl.bits_of(q)))
 
 
+@pytest.mark.parametrize("name,T", [("8b-k4v2", 300), ("8b-k8v4", 131), ("14b-k4v2", 300), ("1b", 200)])
+def test_signs_at_any_address(kvq, name, T):
+    """The signs as a view into a larger tensor, at every distance from a 4-byte boundary: every call as with a tensor of their own."""
+    w = CASES[name][0].with_(n_kv_heads=2, n_q_heads=8)
+    D, B, cap = w.head_dim, 2, 384
+    signs = torch.from_numpy(signs_for(D, 5))
+    k, v = (x.cuda() for x in wl.make_kv(w, tokens=T, batch=B))
+    q = wl.make_q(w, batch=B)
+    cfg = tl.gpu_config_for(kvq, w, B, cap)
+
+    def calls(k_signs):
+        gc = kvq.Cache(cfg, k_signs=k_signs)
+        for lo, hi in ((0, T - 3), (T - 3, T)):                   # a long append and a short one
+            kvq.kvq_quantize_append(cfg, gc, k[:, :, lo:hi], v[:, :, lo:hi])
+        out = [gc.pages] + ([] if gc.k_tail is None else [gc.k_tail])
+        for sides in ((True, True), (True, False)):
+            back = [torch.zeros((B, 2, cap, D), dtype=w.torch_dtype, device="cuda") if s else None for s in sides]
+            kvq.kvq_dequantize(cfg, gc, back[0], back[1], 0, T)
+            out += [b for b in back if b is not None]
+        return gc, out, tl.gpu_decode(kvq, cfg, gc, q)
+
+    _, want, want_out = calls(signs)
+    for offset in range(1, 5):
+        gc, got, got_out = calls(torch.cat((torch.zeros(offset, dtype=torch.int8), signs)).cuda()[offset:])
+        assert gc.k_signs.data_ptr() % 4 == offset % 4            # the view itself, not a copy
+        assert all(torch.equal(a, b) for a, b in zip(got, want)) and np.array_equal(got_out, want_out)
+
+
 def test_rotation_lowers_attention_error_on_outlier_keys(kvq):
     """Keys with 8 heavy channels per head: rotating them before 4-bit quantization lowers the error of the
     attention output against exact attention on the unquantized cache (Sec. 4.4, key-only rotation)."""
