@@ -107,12 +107,21 @@ def _dtype_code(dt: torch.dtype) -> int:
     return _DTYPE_CODES[dt]
 
 
+def _stream_reader(c=torch._C):
+    """How the current device's current stream is read: its handle as a number where torch has the two (private) calls for it -
+    making a torch.cuda.Stream object took 3.1 of the 10 us of a library call - else through such an object."""
+    raw, device = getattr(c, "_cuda_getCurrentRawStream", None), getattr(c, "_cuda_getDevice", None)
+    if raw is None or device is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(device())
+
+
+_current_stream_ptr = _stream_reader()
+
+
 def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> int:
-    """The stream's handle: the given one's, or the current device's current stream's (read as a number; making a
-    torch.cuda.Stream object for it took 3.1 of the 10 us of a call; the CUDA tensors of the call have initialised CUDA)."""
-    if stream is not None:
-        return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    """The stream's handle: the given one's, or the current device's current stream's."""
+    return stream.cuda_stream if stream is not None else _current_stream_ptr()
 
 
 def kvq_strerror(code: int) -> str:

@@ -3,6 +3,7 @@ host-only layout queries agree with the oracle's layout.  No GPU needed."""
 import ctypes
 import os
 import re
+import types
 
 import pytest
 
@@ -90,6 +91,15 @@ def test_null_and_misaligned_arguments_fail_before_any_launch(kvq):
     assert lib.kvq_quantize_append(ctypes.byref(cfg), ctypes.byref(ok), 4096, 4096, 0, 0, 128, 257, None) == -5  # > capacity
     assert lib.kvq_decode_attention(ctypes.byref(cfg), ctypes.byref(ok), 4096, 4096, 2, 0.0, 4096, 8, None) == -4
     assert lib.kvq_decode_attention(ctypes.byref(cfg), ctypes.byref(ok), 4096, 4096, 9, 0.0, 4096, 1 << 20, None) == -1
+
+
+def test_a_torch_without_the_private_stream_calls_is_served(kvq, monkeypatch):
+    monkeypatch.setattr(kvq.torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=11))
+    both = dict(_cuda_getCurrentRawStream=lambda device: 100 + device, _cuda_getDevice=lambda: 3)
+    assert kvq._stream_reader(types.SimpleNamespace(**both))() == 103
+    for name in both:
+        assert kvq._stream_reader(types.SimpleNamespace(**{name: both[name]}))() == 11
+    assert kvq._stream_ptr(types.SimpleNamespace(cuda_stream=7)) == 7
 
 
 def test_bit_balance_is_the_log_ratio_of_the_frobenius_norms(kvq):
