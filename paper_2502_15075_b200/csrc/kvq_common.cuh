@@ -50,7 +50,8 @@ __device__ __forceinline__ int paged_len(const int32_t* seq_len, int b, int capa
 
 // Dependent launches: a kernel started by launch_dependent may begin before the one in front of it on the stream has ended, so
 // every thread waits here before it touches global memory; behind the wait everything that the stream ran before is complete and
-// visible.  No kernel lets the next one in earlier than its own end (griddepcontrol.launch_dependents): blocks that wait beside a
+// visible.  (decode_generic_kernel, merge_kernel and decode_tc_kernel are launched plainly and wait for the whole of the kernel before
+// them.)  No kernel lets the next one in earlier than its own end (griddepcontrol.launch_dependents): blocks that wait beside a
 // running kernel take places on its multiprocessors, and those of a decode call then no longer spread one launch wave after the
 // other (16 layers of the 1B shape, append and decode 424 us; with dependent launches 357; with the signal at each kernel's start 392;
 // channel-wise 14B shape, two layers 272, 265, 277; twelve error analyses 223, 191, 198).
@@ -177,14 +178,6 @@ __device__ __forceinline__ void rotate_row8(float (&x)[8], const int8_t* signs, 
   for (int i = 0; i < 8; ++i) x[i] = __fmul_rn(x[i], inv_sqrt_dim<D>());
 }
 
-// x = signs * (H y / sqrt(D))
-template <int D>
-__device__ __forceinline__ void unrotate_row8(float (&x)[8], const int8_t* signs, int l) {
-  fwht_row8<D>(x, l);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) x[i] = __fmul_rn(__fmul_rn(x[i], inv_sqrt_dim<D>()), (float)signs[8 * l + i]);
-}
-
 // ---------------------------------------------------------------- layout index functions
 // Byte offset (inside the K-code region of a page) of the 32-bit word holding
 // channel d of page-local token t, and the field's bit offset inside that word.
@@ -215,20 +208,11 @@ __host__ __device__ __forceinline__ void v_code_pos(int t, int d, int D, int b, 
   bit = 8 * j + b * f;
 }
 
-// Inverse maps: which channel (and tile-local token) sits in field f of a word.
+// Inverse map: which channel sits in field f of a word.
 __device__ __forceinline__ int k_field_channel(int chunk, int word, int f, int b) {
   int fpb = 8 / b;
   int r = word * fpb + (f % fpb);
   return 16 * r + 4 * chunk + (f / fpb);
-}
-
-// Word number w (0 .. D*b-1) of a value block: which block-local token and channel sit in byte j, field f.
-__device__ __forceinline__ void v_field_pos(int w, int j, int f, int b, int& tau, int& d) {
-  const int fpb = 8 / b;
-  const int mw = w >> 7, lane = (w >> 2) & 31, sub = w & 3;
-  const int gq = lane >> 2, tq = lane & 3, rh = sub >> 1, kh = sub & 1;
-  tau = 16 * kh + 2 * tq + (j >> 1) + 8 * (j & 1);
-  d = 16 * (fpb * mw + f) + 8 * rh + gq;
 }
 
 // Code widths 1, 3 and 6 are stored as bit planes: a high plane of 2 (4) bits followed by a low plane of 1 (2)
@@ -261,11 +245,6 @@ __device__ __forceinline__ uint32_t load_code_any(const uint8_t* region, bool is
     c = (c << lo) | ((*reinterpret_cast<const uint32_t*>(region + wb) >> bit) & ((1u << lo) - 1u));
   }
   return c;
-}
-
-__device__ __forceinline__ uint32_t load_code(const uint8_t* region, int word_byte, int bit, int b) {
-  uint32_t w = *reinterpret_cast<const uint32_t*>(region + word_byte);
-  return (w >> bit) & ((1u << b) - 1u);
 }
 
 }  // namespace kvq

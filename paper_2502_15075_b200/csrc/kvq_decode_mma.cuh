@@ -185,7 +185,6 @@ __device__ __forceinline__ void load_words(const uint8_t* p, int quad_stride, ui
 }
 
 __device__ __forceinline__ float meta_s(uint32_t m) { return __half2float(__ushort_as_half((uint16_t)(m & 0xFFFF))); }
-__device__ __forceinline__ float meta_z(uint32_t m) { return __half2float(__ushort_as_half((uint16_t)(m >> 16))); }
 
 // ------------------------------------------------------------------ flat split and merge bookkeeping
 constexpr int kMaxBatchFlat = 1024;   // the flat partition keeps a per-batch prefix in shared memory

@@ -92,7 +92,7 @@ __device__ __forceinline__ uint32_t fixed_point_limb(const float (&t)[4], float 
 }
 
 // The split balances time, not pages.  Ending one stream and starting the next costs a CTA about as much as six to eight pages
-// (load and convert the next queries, publish a partial, perhaps merge), so every stream is given kGapPages virtual pages in front
+// (load and convert the next queries, publish a partial, perhaps merge), so every stream is given a gap of virtual pages in front
 // of its real ones and the split is taken on that virtual axis; with many CTAs per stream the gap also keeps shares from
 // crossing into the next stream for a page or two (40 ragged streams of 36 to 70 K4V4 pages: gap 8 16.5 us, 6 19.8, 0 28).
 // Channel-wise keys, whose pages take longer: gap 2 (two ragged 14B-shaped layers 226 us; 5: 228, 8: 233).  At head_dim 64 a page is
@@ -318,7 +318,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   const SmemLayout sl = smem_layout(g.page_bytes, stages, g.B, D, NH, NGV, KAXIS == 1);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + sl.bar_off);   // full[0..stages), empty[0..stages)
   int* sPref = reinterpret_cast<int*>(smem + sl.pref_off);
-  int* sVPref = sPref + (g.B + 1);                                   // the same prefix with kGapPages more per stream
+  int* sVPref = sPref + (g.B + 1);                                   // the same prefix with GAP more per stream
   int* sMisc = reinterpret_cast<int*>(smem + sl.misc_off);           // [1] abort flag, [2] published count, [4..7] share ends, [8..9] segment slot / partials, [10..13] CTAs taking part, cursor, [14] weighted shares
   double* sZ = reinterpret_cast<double*>(smem + sl.red_off);         // [NW][8][NGV] sums of weight x zero-point
   float* sMax = reinterpret_cast<float*>(sZ + NW * 8 * NGV);         // [NW][8] block maxima
@@ -822,7 +822,8 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
               }
             }
             // accumulator columns 2 tid, 2 tid + 1 = (hi, lo) limbs of head tid + 4 nh: sum_d code_d Q_d = 256 hi + lo
-            // (channel-wise keys: the signed top byte in n-tile 0, the two unsigned lower bytes in n-tile 1, combined in fp32)
+            // (channel-wise keys: the signed top byte in n-tile 0, the two unsigned lower bytes in n-tile 1; these two meet as integers,
+            // the top byte joins them in fp32)
             if constexpr (KAXIS == 1) {
 #pragma unroll
               for (int nh = 0; nh < NH; ++nh) {
