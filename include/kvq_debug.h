@@ -46,11 +46,12 @@ int kvq_debug_decode_stall_impl(const kvq_config* cfg, const kvq_cache* cache, c
 /* Host only, no GPU work: how the warp-level kernel of the fast path splits the pages of sequences of the given lengths
  * (HOST memory, [batch]) over its CTAs.  info[0] = partial slots per stream, info[1] = CTAs that take part, info[2] = 1 if
  * their shares are weighted; starts[0 .. info[1]] = first page of every CTA's share (flat page numbers in (batch,
- * kv-head, page) order; starts has room for 445 entries); parts[2 s], parts[2 s + 1] = first CTA and number of partials of
+ * kv-head, page) order; starts has room for 445 entries), cursors[3 i ..] the same page as (batch, kv-head, page of the stream)
+ * for i < info[1] (0, 0, 0 where the pages end); parts[2 s], parts[2 s + 1] = first CTA and number of partials of
  * stream s = batch * n_kv_heads + kv-head (0, 0 for an empty one).  KVQ_ERR_UNSUPPORTED where that kernel does not serve the
  * configuration. */
 int kvq_debug_decode_plan(const kvq_config* cfg, int32_t n_rows, const int32_t* seq_len, int32_t* parts, int64_t* starts,
-                          int32_t* info);
+                          int32_t* cursors, int32_t* info);
 
 #ifdef __cplusplus
 }

@@ -72,7 +72,7 @@ bool decode_mma_supported(const Geom& g) {
 namespace {
 // The kernel's plan for given lengths, worked out on the host by the same functions.
 template <int WAVES>
-void host_plan(const Geom& g, int gap, const int32_t* seq_len, int32_t* parts, int64_t* starts, int32_t* info) {
+void host_plan(const Geom& g, int gap, const int32_t* seq_len, int32_t* parts, int64_t* starts, int32_t* cursors, int32_t* info) {
   int pref[mma::kMaxBatchFlat + 1] = {}, vpref[mma::kMaxBatchFlat + 1] = {};
   int pmax = 0;
   for (int b = 0; b < g.B; ++b) {
@@ -86,8 +86,11 @@ void host_plan(const Geom& g, int gap, const int32_t* seq_len, int32_t* parts, i
   const mma::FlatPlan plan = mma::make_plan(vpref[g.B], pmax + gap, WAVES * 148, slots);
   const bool waves = mma::weighted_shares<WAVES>(plan, gap, WAVES * 148, pmax, slots);
   info[0] = slots; info[1] = plan.c_eff; info[2] = waves;
-  for (int c = 0; c <= plan.c_eff && plan.N; ++c)
-    starts[c] = mma::share_start<WAVES>(plan, waves, c, pref, vpref, g.B, g.Hkv, gap).x;
+  for (int c = 0; c <= plan.c_eff && plan.N; ++c) {
+    const mma::ShareStart at = mma::share_start<WAVES>(plan, waves, c, pref, vpref, g.B, g.Hkv, gap);
+    starts[c] = at.x;
+    if (c < plan.c_eff) { cursors[3 * c] = at.b; cursors[3 * c + 1] = at.h; cursors[3 * c + 2] = at.page; }
+  }
   for (int b = 0; b < g.B; ++b) {
     const int pages = (pref[b + 1] - pref[b]) / g.Hkv;
     for (int h = 0; h < g.Hkv; ++h) {
@@ -99,15 +102,15 @@ void host_plan(const Geom& g, int gap, const int32_t* seq_len, int32_t* parts, i
 }
 }  // namespace
 
-int decode_mma_plan(const Geom& g, const int32_t* seq_len, int32_t* parts, int64_t* starts, int32_t* info) {
+int decode_mma_plan(const Geom& g, const int32_t* seq_len, int32_t* parts, int64_t* starts, int32_t* cursors, int32_t* info) {
   CachePtrs none{};
   int grid = 0;
   if (g.B > mma::kMaxBatchFlat) return KVQ_ERR_UNSUPPORTED;
   const int rc = pick(g, none, nullptr, 0.f, nullptr, 0, nullptr, 0, DecodeDebug{}, nullptr, true, &grid);
   if (rc != KVQ_OK) return rc;
   const int gap = mma::gap_pages(g.D, g.kb, g.vb, g.k_axis);
-  if (grid == 3 * 148) host_plan<3>(g, gap, seq_len, parts, starts, info);
-  else host_plan<2>(g, gap, seq_len, parts, starts, info);
+  if (grid == 3 * 148) host_plan<3>(g, gap, seq_len, parts, starts, cursors, info);
+  else host_plan<2>(g, gap, seq_len, parts, starts, cursors, info);
   return KVQ_OK;
 }
 

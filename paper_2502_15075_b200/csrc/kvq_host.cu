@@ -325,14 +325,14 @@ int kvq_debug_decode_stall_impl(const kvq_config* cfg, const kvq_cache* cache, c
 }
 
 int kvq_debug_decode_plan(const kvq_config* cfg, int32_t n_rows, const int32_t* seq_len, int32_t* parts, int64_t* starts,
-                          int32_t* info) {
+                          int32_t* cursors, int32_t* info) {
   Geom g;
   int rc = make_geom(cfg, &g);
   if (rc != KVQ_OK) return rc;
-  if (!seq_len || !parts || !starts || !info || n_rows < 1) return KVQ_ERR_INVALID_ARG;
+  if (!seq_len || !parts || !starts || !cursors || !info || n_rows < 1) return KVQ_ERR_INVALID_ARG;
   if (n_rows * g.G > kMaxGroupHeads) return KVQ_ERR_UNSUPPORTED;
   g.rows = n_rows;
-  return decode_mma_plan(g, seq_len, parts, starts, info);
+  return decode_mma_plan(g, seq_len, parts, starts, cursors, info);
 }
 
 int kvq_dequantize(const kvq_config* cfg, const kvq_cache* cache, void* k_out, void* v_out, int32_t t_begin,

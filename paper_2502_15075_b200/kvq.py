@@ -71,8 +71,7 @@ _lib.kvq_debug_decode_impl.argtypes = [_P(kvq_config), _P(kvq_cache), ctypes.c_v
 _lib.kvq_debug_decode_stall_impl.argtypes = [_P(kvq_config), _P(kvq_cache), ctypes.c_void_p, ctypes.c_void_p,
                                              ctypes.c_int32, ctypes.c_float, ctypes.c_void_p, ctypes.c_size_t,
                                              ctypes.c_int64, ctypes.c_uint32, ctypes.c_int32, ctypes.c_void_p]
-_lib.kvq_debug_decode_plan.argtypes = [_P(kvq_config), ctypes.c_int32, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
-                                       ctypes.c_void_p]
+_lib.kvq_debug_decode_plan.argtypes = [_P(kvq_config), ctypes.c_int32] + [ctypes.c_void_p] * 5
 _lib.kvq_check_status.argtypes = [_P(kvq_cache), ctypes.c_void_p]
 _lib.kvq_strerror.argtypes = [ctypes.c_int]
 _lib.kvq_strerror.restype = ctypes.c_char_p
@@ -341,16 +340,26 @@ def kvq_debug_decode_stall_impl(cfg: kvq_config, cache: Cache, q: torch.Tensor, 
                                             int(impl), _stream_ptr(None)), "kvq_debug_decode_stall_impl")
 
 
-def kvq_debug_decode_plan(cfg: kvq_config, seq_len, n_rows: int = 1):
-    """Test hook, host only: the split of the fast decode kernel for a list of lengths.  Returns (partial slots per stream,
-    weighted shares?, first page of every share [CTAs + 1], (first CTA, partials) per stream)."""
+def _decode_plan(cfg: kvq_config, seq_len, n_rows: int):
     lens = torch.tensor(list(seq_len), dtype=torch.int32)
     assert lens.numel() == cfg.batch
     parts = torch.zeros((cfg.batch * cfg.n_kv_heads, 2), dtype=torch.int32)
-    starts, info = torch.zeros(512, dtype=torch.int64), torch.zeros(3, dtype=torch.int32)
+    starts, cursors, info = torch.zeros(512, dtype=torch.int64), torch.zeros((512, 3), dtype=torch.int32), torch.zeros(3, dtype=torch.int32)
     _check(_lib.kvq_debug_decode_plan(ctypes.byref(cfg), int(n_rows), lens.data_ptr(), parts.data_ptr(), starts.data_ptr(),
-                                      info.data_ptr()), "kvq_debug_decode_plan")
-    return int(info[0]), bool(info[2]), starts[:int(info[1]) + 1].numpy(), parts.numpy()
+                                      cursors.data_ptr(), info.data_ptr()), "kvq_debug_decode_plan")
+    n = int(info[1])
+    return int(info[0]), bool(info[2]), starts[:n + 1].numpy(), parts.numpy(), cursors[:n].numpy()
+
+
+def kvq_debug_decode_plan(cfg: kvq_config, seq_len, n_rows: int = 1):
+    """Test hook, host only: the split of the fast decode kernel for a list of lengths.  Returns (partial slots per stream,
+    weighted shares?, first page of every share [CTAs + 1], (first CTA, partials) per stream)."""
+    return _decode_plan(cfg, seq_len, n_rows)[:4]
+
+
+def kvq_debug_decode_cursors(cfg: kvq_config, seq_len, n_rows: int = 1):
+    """Test hook, host only: first page of every share of that split as (sequence, KV head, page of the stream) [CTAs, 3]."""
+    return _decode_plan(cfg, seq_len, n_rows)[4]
 
 
 def kvq_check_status(cache: Cache, stream: Optional[torch.cuda.Stream] = None) -> int:

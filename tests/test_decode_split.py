@@ -22,6 +22,10 @@ def check_split(kvq, cfg, pages, rows=1):
     lens = [PAGE * p - (7 * i) % PAGE if p else 0 for i, p in enumerate(pages)]        # p pages, the last one incomplete
     slots, weighted, starts, parts = kvq.kvq_debug_decode_plan(cfg, lens, rows)
     H, first = cfg.n_kv_heads, 0
+    cursors, before = kvq.kvq_debug_decode_cursors(cfg, lens, rows), np.cumsum([0] + [H * p for p in pages])
+    for (b, h, page), start in zip(cursors, starts[:-1]):               # the share's first page, said twice
+        assert 0 <= h < H and 0 <= page < pages[b] and before[b] + h * pages[b] + page == start
+    assert len(cursors) == len(starts) - 1
     assert starts[0] == 0 and starts[-1] == H * sum(pages) and np.all(np.diff(starts) >= 0)
     for b, p in enumerate(pages):
         for h in range(H):
@@ -36,21 +40,24 @@ def check_split(kvq, cfg, pages, rows=1):
     return weighted
 
 
-# (key bits, value bits, key axis, query heads per KV head): three weighted waves with the stream gap of token-wise and of
-# channel-wise keys, two weighted waves, equal shares
-FORMS = {"token": (4, 2, 0, 4), "channel": (4, 2, 1, 4), "eight heads": (4, 2, 0, 8), "wide pages": (8, 4, 0, 4)}
+# (key bits, value bits, key axis, query heads per KV head, head_dim, group): three weighted waves with the stream gap of token-wise
+# and of channel-wise keys, two weighted waves, equal shares, the gap of head_dim 64
+FORMS = {"token": (4, 2, 0, 4, 128, 128), "channel": (4, 2, 1, 4, 128, 128), "eight heads": (4, 2, 0, 8, 128, 128),
+         "wide pages": (8, 4, 0, 4, 128, 128), "d64": (4, 2, 0, 4, 64, 64), "d64-g32": (4, 2, 0, 2, 64, 32)}
 
 
 def config(kvq, form, batch, heads, max_pages, residual=0):
-    kb, vb, axis, group = FORMS[form]
-    return kvq.make_config(batch, heads * group, heads, 128, kb, vb, 128, 128, axis, "bf16", PAGE * max_pages, residual)
+    kb, vb, axis, q_heads, D, group = FORMS[form]
+    return kvq.make_config(batch, heads * q_heads, heads, D, kb, vb, group, group, axis, "bf16", PAGE * max_pages, residual)
 
 
 @pytest.mark.parametrize("form,heads,pages", [
     ("channel", 10, [95, 63, 37, 57, 58, 70, 35, 110, 117, 93]),
     ("token", 8, [472, 1024]),
     ("token", 1, [3000, 900, 5]),
-    ("wide pages", 8, [472, 1024])])
+    ("wide pages", 8, [472, 1024]),
+    ("d64", 8, [31, 0, 1, 250, 33]),
+    ("d64-g32", 3, [1, 1, 700, 2])])
 def test_long_streams_of_uneven_batches(kvq, form, heads, pages):
     check_split(kvq, config(kvq, form, len(pages), heads, max(pages)), pages)
 
