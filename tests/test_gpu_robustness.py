@@ -83,6 +83,36 @@ def test_a_wait_that_runs_out_sets_the_status_and_leaves_the_context_usable(kvq)
     assert np.array_equal(again, good)
 
 
+@pytest.mark.parametrize("name,w,tokens", [
+    ("token", wl.LLAMA_8B.with_(n_kv_heads=8, n_q_heads=32), 128 * 120),
+    ("channel", wl.SHAPED_14B.with_(n_kv_heads=8, n_q_heads=32), 128 * 120 - 58),
+    ("channel-k8", wl.SHAPED_14B.with_(n_kv_heads=8, n_q_heads=32, kb=8), 128 * 120 - 58)])
+def test_a_withheld_page_anywhere_in_a_share_of_several_ring_turns(kvq, name, w, tokens):
+    """Shares of more pages than the ring has stages; the page that never arrives is the first of a share, one of its first turn, one
+    behind it, its last one, and a stream's last (for channel-wise keys the incomplete one): the call returns, the status says so, and
+    the next call on the same cache and workspace gives the bytes it gave before."""
+    B, cap = 4, 128 * 120
+    cfg = tl.gpu_config_for(kvq, w, B, cap)
+    gc = kvq.Cache(cfg)
+    kvq.kvq_quantize_append(cfg, gc, *wl.make_kv(w, 0, "cuda", tokens=tokens, batch=B))
+    q = wl.make_q(w, batch=B).cuda()
+    ws = torch.empty(kvq.kvq_workspace_bytes(cfg), dtype=torch.uint8, device="cuda")
+    good, out = (torch.zeros(tuple(q.shape), dtype=torch.float32, device="cuda") for _ in range(2))
+    kvq.kvq_decode_attention(cfg, gc, q, good, ws)
+    assert kvq.kvq_check_status(gc) == 0
+    starts = kvq.kvq_debug_decode_plan(cfg, [tokens] * B)[2]
+    share = int(np.diff(starts).argmax())
+    first, last = int(starts[share]), int(starts[share + 1]) - 1
+    assert last - first >= 5                                    # (the ring has at most four stages)
+    for page in (first, first + 2, first + 5, last, 120 * 3 - 1):
+        kvq.kvq_debug_decode_stall(cfg, gc, q, out, ws, page, 2000)
+        assert kvq.kvq_check_status(gc) == -7                   # KVQ_ERR_DEVICE_TIMEOUT
+        gc.status.zero_()
+        out.fill_(7.0)
+        kvq.kvq_decode_attention(cfg, gc, q, out, ws)
+        assert kvq.kvq_check_status(gc) == 0 and torch.equal(out, good)
+
+
 def test_append_and_dequantize_stay_inside_their_buffers(kvq):
     w = wl.LLAMA_8B.with_(n_kv_heads=2, n_q_heads=8)
     B, cap, T = 2, 256, 200
