@@ -96,11 +96,14 @@ __device__ __forceinline__ uint32_t fixed_point_limb(const float (&t)[4], float 
 // of its real ones and the split is taken on that virtual axis; with many CTAs per stream the gap also keeps shares from
 // crossing into the next stream for a page or two (40 ragged streams of 36 to 70 K4V4 pages: gap 8 16.5 us, 6 19.8, 0 28).
 // Channel-wise keys, whose pages take longer: gap 2 (two ragged 14B-shaped layers 226 us; 5: 228, 8: 233).  At head_dim 64 a page is
-// half the work: gap 18 (1B shape, append 128 and decode, 16 layers: gap 8 335 us, 10 330, 14 337, 18 327, 24 331; eight layers, one new
-// token: 1 x 4,000 tokens 199 -> 179, 4 x 1,000 113 -> 107, 8 x 2,000 126 -> 122).  Eight heads per KV head: as many shapes lose with 14 as win.  Of the CTAs that
-// share an SM the hardware favours the older ones (0.85 / 0.91 / 0.99 us per page at three per SM, 0.96 / 1.01 at two),
+// half the work: gap 18 (1B shape, append 128 and decode, 16 layers: gap 8 335 us, 10 330, 14 337, 18 327, 24 331), but only up to 64
+// streams: with more of them a share is not much longer than such a gap, and some are left with nothing else (steps of six 1B-shaped
+// layers, gap 8 / 18: 8 streams x 4,000 tokens 147 / 135 us, 32 x 1,200 90.4 / 86.1, 64 x 1,200 89.5 / 86.5, 64 x 4,000 106 / 102.5, 64 x
+// 16,000 157 / 158; 72 x 1,200 89.7 / 92.9, 72 x 4,000 110 / 108, 96 x 1,200 90.3 / 97.5, 128 x 4,000 122 / 131, 256 x 1,200 113.6 /
+// 109, 256 x 4,000 167 / 184, 512 x 4,000 259 / 264; groups of 32 alike).  Eight heads per KV head: as many shapes lose with 14 as win.
+// Of the CTAs that share an SM the hardware favours the older ones (0.85 / 0.91 / 0.99 us per page at three per SM, 0.96 / 1.01 at two),
 // so the launch waves are weighted (8B shape K4V2 when the weights were chosen: 1040 76.1 us, 1080 77.3, equal 80.4).
-constexpr int kGapPages = 8, kGapPages64 = 18, kGapPagesChan = 2;
+constexpr int kGapPages = 8, kGapPages64 = 18, kGapStreams64 = 64, kGapPagesChan = 2;
 constexpr float kQFix = 32512.0f;          // largest |Q| of the 16-bit fixed-point q (hi limb stays within +-127)
 constexpr float kQFix3 = 8300000.0f;       // ... of the 24-bit fixed-point q * s of channel-wise keys (three limbs)
 
@@ -246,8 +249,8 @@ static __host__ __device__ __forceinline__ void stream_ctas(const FlatPlan& plan
 }
 // The time-balanced split (stream gaps) pays where the arithmetic per page limits the kernel (token-wise and
 // channel-wise keys alike); pages of 10 bits per element pair and more lose with it and keep the plain split by pages.
-__host__ __device__ constexpr int gap_pages(int D, int kb, int vb, int k_axis) {
-  return kb + vb <= 8 ? (k_axis == 1 ? kGapPagesChan : D == 64 ? kGapPages64 : kGapPages) : 0;
+__host__ __device__ constexpr int gap_pages(int D, int kb, int vb, int k_axis, int streams) {
+  return kb + vb <= 8 ? (k_axis == 1 ? kGapPagesChan : D == 64 && streams <= kGapStreams64 ? kGapPages64 : kGapPages) : 0;
 }
 // Whether the shares of a full grid are weighted by launch wave: only where every stream's partials fit its slots all the
 // same.  A stream of P pages touches fewer than 2 + (P - 1) / s CTAs when no share is smaller than s virtual pages (the shares
@@ -307,7 +310,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   constexpr int V_META_OFF = V_CODES_OFF + 4 * V_BLOCK_BYTES;
   constexpr int NCONS = NW * 32;
   constexpr uint32_t FULL = 0xffffffffu;
-  constexpr int GAP = gap_pages(D, KB, VB, KAXIS);
+  const int GAP = gap_pages(D, KB, VB, KAXIS, g.B * g.Hkv);      // (known at compile time at head_dim 128)
   constexpr int WAVES = MINB;               // CTAs per SM = launch waves (the weights apply to a grid of 148 * WAVES)
   static_assert(MT % NW == 0 && (MT / NGV) % MTW == 0, "a warp's channels are whole m-tiles of one value group");
   static_assert(KAXIS == 0 || KB != 2, "channel-wise 2-bit keys are not instantiated");

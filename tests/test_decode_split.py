@@ -80,6 +80,15 @@ def test_random_uneven_batches(kvq, form):
     assert (weighted > 0) == (form != "wide pages")         # the weighted split is among what was checked
 
 
+@pytest.mark.parametrize("form,batch,heads", [("d64", 14, 8), ("d64", 16, 8), ("d64-g32", 130, 1), ("d64", 64, 8)])
+def test_shares_of_many_streams_hold_pages(kvq, form, batch, heads):
+    """head_dim 64, more than 64 streams of 4,096 tokens: a share is not swallowed by the gap in front of a stream, and the largest is
+    not far from the mean."""
+    starts = kvq.kvq_debug_decode_plan(config(kvq, form, batch, heads, 32), [PAGE * 32] * batch)[2]
+    pages = np.diff(starts)
+    assert pages.max() <= 1.55 * pages.mean() and (pages == 0).sum() <= len(pages) // 20
+
+
 def test_empty_caches_have_no_split(kvq):
     slots, weighted, starts, parts = kvq.kvq_debug_decode_plan(config(kvq, "token", 3, 2, 4), [0, 0, 0])
     assert len(starts) == 1 and not parts.any() and not weighted
