@@ -5,8 +5,8 @@
 // (cluster barrier) one thread stores the new one.  A token row is spread over D / 8 lanes, eight consecutive channels each; lanes whose
 // codes share bytes merge them with shuffles.  The call is bound by latency, not by bytes: the code is kept short and is
 // the same for every width, because in a step the instructions come from L2 each time.  The task kernels of
-// kvq_quantize.cu (32 tokens a warp, several thousand instructions) and a launch for the lengths take 7 to 8 us for one token
-// (9 to 10 with channel-wise keys), this kernel 3.0 to 3.5 (4).
+// kvq_quantize.cu (32 tokens a warp, several thousand instructions) and a launch for the lengths take 4.2 us at the least and 6 to 7 for a
+// few tokens, this kernel 2.9 at the least and 4.5.
 #include "kvq_quantize.cuh"
 
 namespace kvq {
@@ -159,16 +159,20 @@ append_rows_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, cons
 }  // namespace
 
 // A sequence has at most eight CTAs, so the time goes with the rows of one of them: its KV heads x new tokens.  Both sides measured
-// from an uneven position, one call alone on the GPU, rows / tasks + lengths, for 1 and 16 sequences (K4V2, head_dim 128):
-//    8 KV heads:  64 tokens 7.4 / 8.7 us, 10.3 / 13.4;   96 tokens 9.5 / 8.8, 14.0 / 13.5
-//   16 KV heads:  32 tokens 7.3 / 8.3, 10.2 / 9.8;       48 tokens 9.5 / 8.7, 13.9 / 12.5
-//   32 KV heads:  16 tokens 7.2 / 7.8, 10.2 / 13.1;      32 tokens 11.7 / 8.0, 17.6 / 14.0
-//   64 KV heads:   8 tokens 7.0 / 7.8, 10.0 / 17.3;      16 tokens 11.2 / 8.0, 17.2 / 18.3
-// so 64 rows a CTA at head_dim 128 and 128 at head_dim 64 (16 heads, 64 tokens 7.2 / 7.5; 128 tokens 11.1 / 8.7).  Rotated keys and a
-// residual window cost more a row: 40 rows beyond eight heads (16 heads, 16 tokens rotated 5.8 / 7.1, 8.1 / 8.0, 32 tokens
-// 8.8 / 8.3, 13.2 / 9.4; with a window 16 tokens 6.2 / 7.2, 8.5 / 8.2, 32 tokens 8.8 / 8.8, 13.1 / 10.2).  Channel-wise keys also
-// pay for a block a head (10 heads, 1 and 32 sequences: 48 tokens 10.7 / 12.7, 14.5 / 14.8, 64 tokens 13.8 / 12.9, 17.5 / 16.3; 32
-// heads: 16 tokens 9.0 / 9.4, 11.5 / 18.1, 32 tokens 14.9 / 10.6, 19.4 / 21.8; 64 heads: 4 tokens 7.5 / 9.6, 8 tokens 11.4 / 9.7).
+// behind 613 cached tokens, one of sixteen calls in a row in a replayed graph, us rows / tasks + lengths, for 1 and 16 sequences (K4V2,
+// head_dim 128):
+//    8 KV heads:  48 tokens 5.4 / 6.5, 7.9 / 8.5;     64 tokens 6.3 / 6.6, 10.0 / 12.3;   96 tokens 8.5 / 6.8, 14.2 / 12.6
+//   16 KV heads:  16 tokens 4.5 / 7.0, 6.2 / 9.0;     32 tokens 6.5 / 7.0, 10.1 / 8.9;    48 tokens 8.5 / 7.2, 14.2 / 9.5
+//   32 KV heads:   8 tokens 4.5 / 6.5, 6.2 / 11.5;    16 tokens 6.4 / 7.2, 10.1 / 12.6;   32 tokens 10.6 / 7.4, 18.1 / 13.3
+//   64 KV heads:   4 tokens 4.5 / 6.1, 6.4 / 15.3;     8 tokens 6.5 / 6.3, 10.2 / 15.9;   16 tokens 10.6 / 7.2, 18.2 / 17.6
+// so 64 rows a CTA at head_dim 128 and 128 at head_dim 64 (8 heads: 128 tokens 6.4 / 7.3, 9.9 / 11.2, 192 tokens 8.5 / 7.4, 14.0 / 11.2;
+// 16 heads: 64 tokens 6.5 / 6.4, 9.9 / 9.2, 128 tokens 10.4 / 7.5, 17.7 / 11.7).  Rotated keys and a residual window cost more a row: 40
+// rows beyond eight heads (16 heads rotated: 16 tokens 5.3 / 6.0, 7.8 / 6.8, 20 tokens 6.4 / 6.7, 9.3 / 7.6, 32 tokens 8.3 / 8.5, 13.2 / 9.9;
+// with a window: 20 tokens 3.3 / 5.1, 5.1 / 8.0, 32 tokens, which complete a block, 12.8 / 7.9, 22.6 / 10.6; eight heads: 64 tokens rotated
+// 8.2 / 8.9, 13.1 / 10.6, with a window 8.0 / 9.6, 14.0 / 15.8).  Channel-wise keys also pay for a block a head (1 and 32 sequences; 32
+// heads: 16 tokens 7.4 / 8.0, 11.2 / 16.8, 20 tokens 9.4 / 8.5, 14.3 / 18.7; 64 heads: 4 tokens 7.0 / 7.9, 11.2 / 21.8, 8 tokens 9.0 / 8.0,
+// 13.9 / 22.1).  The lines were drawn when neither kernel overlapped the launch before it; they no longer lie best for several rotated
+// sequences (above) and for 30 to 52 tokens of ten channel-wise heads (32 tokens 9.8 / 9.2, 16.1 / 15.8, 52 tokens 12.6 / 9.7, 20.4 / 17.1).
 // An append of at most 64 tokens of channel-wise keys completes at most one block.
 bool append_rows_serves(const Geom& g, bool rotated, int t_new) {
   auto width = [](int b) { return b == 2 || b == 4 || b == 8; };
