@@ -42,7 +42,7 @@ NOMINAL_HBM_GBS = 8000.0
 
 # DRAM traffic of one launch of the dominant kernel from an ncu capture (bytes), keyed by the sha256 of the
 # kernel source it was taken from; reported as null once that source has changed.
-NCU_TRAFFIC = {"3cdb9daea50696da3caaeeacd9ead45e887266667e0a91db5f561032cc09c6cd": 440328448}   # dram read 436.43 MB + write 3.90 MB
+NCU_TRAFFIC = {"6e482c7e38ba6c6b569a53db26d11e20b5cddbe167d3fe92c712627a69638991": 440414464}   # dram read 436.44 MB + write 3.98 MB
 DECODE_KERNEL_SOURCES = ("kvq_decode_mma.cuh", "kvq_decode_mma_kernel.cuh", "kvq_decode_mma_list.inc")
 
 WORKLOADS = {"tiny": wl.TINY, "1b": wl.LLAMA_1B, "8b": wl.LLAMA_8B, "14b": wl.SHAPED_14B, "70b": wl.LLAMA_70B}
@@ -490,16 +490,13 @@ def run_workload(kvq, w: wl.Workload, dev, rank: int, world: int, steps: int, wa
     roof_q = hbm_block("kvq_quantize_append, bulk build of one layer (reads 16-bit K and V, writes the packed layer)",
                        src_bulk + packed_bulk, q_us, peak, peak_src)
     roof_dq = hbm_block("kvq_dequantize of one whole layer (reads the packed layer, writes 16-bit K and V)",
-                        decode_bytes_per_layer(w, T) + source_bytes_per_layer(w, T), dq_us, peak, peak_src)
+                        (decode_bytes_per_layer(w, T) + source_bytes_per_layer(w, T)) * (n_tok / T), dq_us, peak, peak_src)
 
     cpu = oracle_leg(kvq, w, cfg, caches[0], qs[0], outs[0], oracle_budget_s)
     fast_bits = lambda b: b in (2, 4, 8)  # noqa: E731
-    deq_launches = ((1 if w.head_dim == 128 and fast_bits(w.vb) else 0) +
-                    (1 if w.head_dim == 128 and w.k_axis == 0 and fast_bits(w.kb) else 0))
-    if deq_launches == 2:
-        deq_launches = 1 if B * w.n_kv_heads <= 148 * 8 else 2     # a short range takes both sides in one launch
-    else:
-        deq_launches += 1                                           # the general kernel serves what is left
+    # 2/4/8-bit sides: one launch for both when the range is short, else one each; other widths share a launch of the general kernel
+    deq_launches = (1 if B * w.n_kv_heads <= 148 * 8 else 2) if fast_bits(w.kb) and fast_bits(w.vb) else \
+        1 + (fast_bits(w.kb) or fast_bits(w.vb))
     # append of one token (one launch for 2/4/8-bit codes; else quantize [+ channel-wise K] + lengths), decode, dequantize of
     # the newest page
     short = fast_bits(w.kb) and fast_bits(w.vb) and (w.k_axis == 0 or (w.head_dim == 128 and w.kb != 2))
