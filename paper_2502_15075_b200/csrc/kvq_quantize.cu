@@ -10,7 +10,9 @@
 // word, is then assembled in that lane's registers and stored directly - no shared memory, no
 // atomics, no read-modify-write; a token that is not new is simply not stored (byte stores for
 // values).  Group minima and maxima are reduced with a few shuffles between the lanes of a row.
-// Bound by instruction issue and load latency in long calls, by fetching instructions in short ones.
+// Long calls are bound by the memory system and the length of a warp's chain, short ones by fetching instructions.
+#include <algorithm>
+
 #include "kvq_quantize.cuh"
 
 namespace kvq {
@@ -45,34 +47,40 @@ __device__ __forceinline__ float piece_value(const uint4& r, int e) {
   else { const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w)); return (e & 1) ? f.y : f.x; }
 }
 
-// Quantize one side of a task of TT tokens, four tokens of a lane per pass.  rsrc: the task's rows; tokens [lo, hi) of the
-// task are new (FULLBLK: all of them).  codes: keys - the page's key row of the task's first token; values - the page's
-// value block of the task's first token.  meta_out: metadata row of the task's first token.
+// Task-local token of token slot k: of the four of a value word (slots 4 i .. 4 i + 3), or of a key row.
+template <bool IS_V, int RS>
+__device__ __forceinline__ int token_slot(int k, int rs) {
+  if constexpr (IS_V) {
+    const int cmb = (k >> 2) * RS + rs, j = k & 3;         // cmb = (block, half, t) of the word; j = byte
+    return 32 * (cmb >> 3) + 16 * ((cmb >> 2) & 1) + 2 * (cmb & 3) + (j >> 1) + 8 * (j & 1);
+  } else {
+    return k * RS + rs;
+  }
+}
+
+// One pass over four tokens of every lane, one side of a task of TT tokens; tokens [lo, hi) of the task are new.  load(kk, f): the
+// lane's piece f of its token kk.  next is called when the pieces have been read.  codes: keys - the page's key row of the task's first
+// token; values - the page's value block of the task's first token.  meta_out: metadata row of the task's first token.
 //
 // Lane = (row slot rs, word column mw, row half rh): it owns, for each of its tokens, the FPB pieces of 8 channels
 // 16 (FPB mw + f) + 8 rh + {0..7}, f < FPB, whose codes share bytes.  The minima / maxima of the four tokens are reduced
 // with a shuffle reduce-scatter, so that the group parameters (two divisions) are computed once per group rather than once
-// per lane, and are then broadcast to the lanes of the group.  Minimum and negated maximum travel as one pair of the 16-bit type,
-// the clamp is the saturation of a multiplication: 10.6 instructions per element instead of 14.  K and V of 64 streams x
-// 32,768 tokens (K4V2, 1.29 GB) 333 -> 272 us; in a replayed graph 335 -> 250 us at five CTAs per SM (four 259, three 298, six 270;
-// registers spill at five as well, 168 / 368 bytes); bound by issue (60 %) and load latency.  8-byte pieces at 2 bits (half
-// the registers, twice the loads): 276 us.  A short call is bound by fetching instructions (6.6 of 10 cycles between two of a warp), so
-// a value word's two ways of leaving, whole or byte by byte, are one branch behind all eight words: a branch per word made the
-// partial tasks longer (8 streams x 500 tokens K4V2 11.8 -> 8.7 us, K2V4 11.1 -> 8.3, head_dim 64 12.2 -> 8.7; 64 x 2,047 19.5 -> 18.9).
-template <int BITS, bool IS_V, int D, int DTYPE, bool FULLBLK>
-__device__ __forceinline__ void quantize_task(const RowSrc& rsrc, int gsz, int lo, int hi, uint8_t* __restrict__ codes,
-                                              uint32_t* __restrict__ meta_out, int lane) {
+// per lane, and are then broadcast to the lanes of the group.  Minimum and negated maximum travel as one pair of the 16-bit type.
+// PLAIN: if all groups of the warp are plain (see plain_group; all but those with values beyond the fp16 range or scales and minima
+// below its normal numbers are), codes need no clamp and two values share every operation: 8.7 instructions per element instead of
+// 10.6; else nothing is stored and the answer is false.  A value word's two ways of leaving, whole or byte by byte, are one branch behind
+// all eight words (a branch per word: 8 streams x 500 tokens K4V2 11.8 us against 8.7).
+template <int BITS, bool IS_V, int D, int DTYPE, bool PLAIN, typename Load, typename Next>
+__device__ __forceinline__ bool quantize_pass(Load&& load, Next&& next, int gsz, int lo, int hi, uint8_t* __restrict__ codes,
+                                              uint32_t* __restrict__ meta_out, int lane, int pass) {
   using H2 = typename Pair16<DTYPE>::type;
   constexpr int FPB = 8 / BITS;
   constexpr int NMW = (D / 16) / FPB;        // word columns per row half
   constexpr int LR = 2 * NMW;                // lanes per token row
   constexpr int RS = 32 / LR;                // token rows per load instruction
-  constexpr int TT = task_tokens(D, BITS);
-  constexpr int TPL = TT / RS;               // tokens per lane
   constexpr int K_ROW_BYTES = D * BITS / 8;
   constexpr int NSET = FPB == 4 ? 2 : 1;      // a lane's fields may belong to two groups (groups of 32 at 2 bits)
   constexpr float DOWN = 1.0f / (float)(1 << BITS);
-  static_assert(TPL % 4 == 0, "a lane holds whole groups of four tokens");
   const int rs = lane / LR, cs = lane % LR, mw = cs >> 1, rh = cs & 1;
   const float qmax = (float)((1 << BITS) - 1);
   const int spg = gsz >> 4;                                  // 16-channel slices per group
@@ -82,146 +90,222 @@ __device__ __forceinline__ void quantize_task(const RowSrc& rsrc, int gsz, int l
   const int b0 = cs & 1, b1 = (cs >> 1) & 1;
   const int gbase = lane & ~(lpg - 1);                       // first lane of this lane's group
 
-  // block-local token of token slot k
-  auto token_of = [&](int k) {
-    if constexpr (IS_V) {
-      const int cmb = (k >> 2) * RS + rs, j = k & 3;         // cmb = (block, half, t) of the word; j = byte
-      return 32 * (cmb >> 3) + 16 * ((cmb >> 2) & 1) + 2 * (cmb & 3) + (j >> 1) + 8 * (j & 1);
-    } else {
-      return k * RS + rs;
-    }
-  };
+  auto token_of = [&](int k) { return token_slot<IS_V, RS>(k, rs); };
   auto swap = [](H2 x, int off) {
     const uint32_t o = __shfl_xor_sync(FULL, *reinterpret_cast<uint32_t*>(&x), off);
     return *reinterpret_cast<const H2*>(&o);
   };
 
-#pragma unroll 1
-  for (int pass = 0; pass < TPL / 4; ++pass) {
-    uint4 raw[4][FPB];
-    bool valid[4];
+  uint4 raw[4][FPB];
+  bool valid[4];
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-      const int tau = token_of(4 * pass + kk);
-      valid[kk] = FULLBLK || (tau >= lo && tau < hi);
+  for (int kk = 0; kk < 4; ++kk) {
+    const int tau = token_of(4 * pass + kk);
+    valid[kk] = tau >= lo && tau < hi;
 #pragma unroll
-      for (int f = 0; f < FPB; ++f) {
-        raw[kk][f] = make_uint4(0u, 0u, 0u, 0u);
-        if (valid[kk]) raw[kk][f] = __ldcs(reinterpret_cast<const uint4*>(rsrc.row(tau) + 16 * (FPB * mw + f) + 8 * rh));
-      }
+    for (int f = 0; f < FPB; ++f) raw[kk][f] = load(kk, f);
+  }
+  // ---- minima / maxima of the lane's fields, per token and per set
+  H2 m[NSET][4];
+#pragma unroll
+  for (int kk = 0; kk < 4; ++kk) {
+    m[0][kk] = minmax8<DTYPE, PLAIN>(raw[kk][0]);
+    if constexpr (FPB == 2) m[0][kk] = min_pair(m[0][kk], minmax8<DTYPE, PLAIN>(raw[kk][1]), PLAIN);
+    if constexpr (FPB == 4) {
+      m[0][kk] = min_pair(m[0][kk], minmax8<DTYPE, PLAIN>(raw[kk][1]), PLAIN);
+      m[1][kk] = min_pair(minmax8<DTYPE, PLAIN>(raw[kk][2]), minmax8<DTYPE, PLAIN>(raw[kk][3]), PLAIN);
+      if (!split) m[0][kk] = min_pair(m[0][kk], m[1][kk], PLAIN);
     }
-    // ---- minima / maxima of the lane's fields, per token and per set
-    H2 m[NSET][4];
+  }
+  // ---- reduce-scatter over the lanes of the group: after lane bit 0 a lane holds tokens 2 b0 + {0, 1}, after
+  // bit 1 (groups of 4 lanes or more) token 2 b0 + b1; higher bits are plain butterflies
+  float pz[NSET][2], pinv[NSET][2];
+  uint32_t pmeta[NSET][2];
+  bool plain = true;
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-      m[0][kk] = minmax8<DTYPE>(raw[kk][0]);
-      if constexpr (FPB == 2) m[0][kk] = __hmin2(m[0][kk], minmax8<DTYPE>(raw[kk][1]));
-      if constexpr (FPB == 4) {
-        m[0][kk] = __hmin2(m[0][kk], minmax8<DTYPE>(raw[kk][1]));
-        m[1][kk] = __hmin2(minmax8<DTYPE>(raw[kk][2]), minmax8<DTYPE>(raw[kk][3]));
-        if (!split) m[0][kk] = __hmin2(m[0][kk], m[1][kk]);
-      }
+  for (int e = 0; e < NSET; ++e) {
+    if (e == 1 && !split) break;
+    H2 a0 = min_pair(b0 ? m[e][2] : m[e][0], swap(b0 ? m[e][0] : m[e][2], 1), PLAIN);
+    H2 a1 = min_pair(b0 ? m[e][3] : m[e][1], swap(b0 ? m[e][1] : m[e][3], 1), PLAIN);
+    if (lpg >= 4) a0 = min_pair(b1 ? a1 : a0, swap(b1 ? a0 : a1, 2), PLAIN);
+    if (lpg >= 8) a0 = min_pair(a0, swap(a0, 4), PLAIN);
+    if (lpg >= 16) a0 = min_pair(a0, swap(a0, 8), PLAIN);
+    const float2 f0 = pair_to_f32(a0);
+    const GroupParams p0 = group_params(f0.x, -f0.y, qmax);
+    if constexpr (PLAIN) plain &= plain_group(f0.x, -f0.y, p0, qmax);
+    pz[e][0] = p0.z; pinv[e][0] = p0.inv * DOWN; pmeta[e][0] = p0.meta;
+    pz[e][1] = 0.f; pinv[e][1] = 0.f; pmeta[e][1] = 0u;
+    if (lpg == 2) {
+      const float2 f1 = pair_to_f32(a1);
+      const GroupParams p1 = group_params(f1.x, -f1.y, qmax);
+      if constexpr (PLAIN) plain &= plain_group(f1.x, -f1.y, p1, qmax);
+      pz[e][1] = p1.z; pinv[e][1] = p1.inv * DOWN; pmeta[e][1] = p1.meta;
     }
-    // ---- reduce-scatter over the lanes of the group: after lane bit 0 a lane holds tokens 2 b0 + {0, 1}, after
-    // bit 1 (groups of 4 lanes or more) token 2 b0 + b1; higher bits are plain butterflies
-    float pz[NSET][2], pinv[NSET][2];
+  }
+  next();                                   // (the shuffles above have seen all of `raw`: its place may be filled again)
+  if constexpr (PLAIN) {
+    if (!__all_sync(FULL, plain)) return false;
+  }
+  // the lane (one per group) that holds a token's parameters stores its metadata word
+  if ((cs & (lpg - 1) & ~3) == 0) {
 #pragma unroll
     for (int e = 0; e < NSET; ++e) {
       if (e == 1 && !split) break;
-      H2 a0 = __hmin2(b0 ? m[e][2] : m[e][0], swap(b0 ? m[e][0] : m[e][2], 1));
-      H2 a1 = __hmin2(b0 ? m[e][3] : m[e][1], swap(b0 ? m[e][1] : m[e][3], 1));
-      if (lpg >= 4) a0 = __hmin2(b1 ? a1 : a0, swap(b1 ? a0 : a1, 2));
-      if (lpg >= 8) a0 = __hmin2(a0, swap(a0, 4));
-      if (lpg >= 16) a0 = __hmin2(a0, swap(a0, 8));
-      uint32_t pmeta[2];
-      const float2 f0 = pair_to_f32(a0);
-      const GroupParams p0 = group_params(f0.x, -f0.y, qmax);
-      pz[e][0] = p0.z; pinv[e][0] = p0.inv * DOWN; pmeta[0] = p0.meta;
-      pz[e][1] = 0.f; pinv[e][1] = 0.f; pmeta[1] = 0u;
-      if (lpg == 2) {
-        const float2 f1 = pair_to_f32(a1);
-        const GroupParams p1 = group_params(f1.x, -f1.y, qmax);
-        pz[e][1] = p1.z; pinv[e][1] = p1.inv * DOWN; pmeta[1] = p1.meta;
-      }
-      // the lane (one per group) that holds a token's parameters stores its metadata word
-      if ((cs & (lpg - 1) & ~3) == 0) {
-        const int gi = (16 * FPB * mw) / gsz + e;
+      const int gi = (16 * FPB * mw) / gsz + e;
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          if (i == 1 && lpg != 2) break;
-          const int kk = 2 * b0 + (lpg >= 4 ? b1 : i);
-          const int tau = token_of(4 * pass + kk);
-          if (FULLBLK || (tau >= lo && tau < hi)) meta_out[tau * ng + gi] = pmeta[i];
-        }
+      for (int i = 0; i < 2; ++i) {
+        if (i == 1 && lpg != 2) break;
+        const int kk = 2 * b0 + (lpg >= 4 ? b1 : i);
+        const int tau = token_of(4 * pass + kk);
+        if (tau >= lo && tau < hi) meta_out[tau * ng + gi] = pmeta[e][i];
       }
     }
-    // ---- the group's parameters, fetched from the lane that made them
-    float z[NSET][4], inv[NSET][4];
+  }
+  // ---- the group's parameters, fetched from the lane that made them
+  float z[NSET][4], inv[NSET][4];
+#pragma unroll
+  for (int kk = 0; kk < 4; ++kk) {
+    const int srcl = gbase + (lpg >= 4 ? (kk >> 1) + 2 * (kk & 1) : (kk >> 1));
+    const int el = (lpg >= 4) ? 0 : (kk & 1);
+    z[0][kk] = __shfl_sync(FULL, el ? pz[0][1] : pz[0][0], srcl);
+    inv[0][kk] = __shfl_sync(FULL, el ? pinv[0][1] : pinv[0][0], srcl);
+    if constexpr (NSET == 2) {
+      z[1][kk] = z[0][kk]; inv[1][kk] = inv[0][kk];
+      if (split) {
+        z[1][kk] = __shfl_sync(FULL, el ? pz[1][1] : pz[1][0], srcl);
+        inv[1][kk] = __shfl_sync(FULL, el ? pinv[1][1] : pinv[1][0], srcl);
+      }
+    }
+  }
+  if constexpr (!IS_V) {
+    // ---- keys: the four bytes of a word are channels 4 hh + {0..3} of this lane's 8, chunk 2 rh + hh, word mw of the row
+    constexpr int wpc = D * BITS / 128;
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
-      const int srcl = gbase + (lpg >= 4 ? (kk >> 1) + 2 * (kk & 1) : (kk >> 1));
-      const int el = (lpg >= 4) ? 0 : (kk & 1);
-      z[0][kk] = __shfl_sync(FULL, el ? pz[0][1] : pz[0][0], srcl);
-      inv[0][kk] = __shfl_sync(FULL, el ? pinv[0][1] : pinv[0][0], srcl);
-      if constexpr (NSET == 2) {
-        z[1][kk] = z[0][kk]; inv[1][kk] = inv[0][kk];
-        if (split) {
-          z[1][kk] = __shfl_sync(FULL, el ? pz[1][1] : pz[1][0], srcl);
-          inv[1][kk] = __shfl_sync(FULL, el ? pinv[1][1] : pinv[1][0], srcl);
-        }
-      }
-    }
-    if constexpr (!IS_V) {
-      // ---- keys: the four bytes of a word are channels 4 hh + {0..3} of this lane's 8, chunk 2 rh + hh, word mw of the row
-      constexpr int wpc = D * BITS / 128;
+      const int tau = token_of(4 * pass + kk);
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        const int tau = token_of(4 * pass + kk);
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-          uint32_t w = 0;
-#pragma unroll
-          for (int f = FPB - 1; f >= 0; --f) {
-            const int e = NSET == 2 ? f >> 1 : 0;
-            float x[4], zz[4], ii[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) { x[j] = piece_value<DTYPE>(raw[kk][f], 4 * hh + j); zz[j] = z[e][kk]; ii[j] = inv[e][kk]; }
-            w = w * (1u << BITS) + code_word4<BITS>(x, zz, ii);
-          }
-          if (valid[kk])
-            *reinterpret_cast<uint32_t*>(codes + (size_t)tau * K_ROW_BYTES + chunk_word_byte(2 * rh + hh, mw, wpc, 4)) = w;
-        }
-      }
-    } else {
-      // ---- values: the four bytes of a word are this lane's four tokens; word of channel slot i at lane chunk 4 i + t
-      const int cmb = pass * RS + rs;
-      uint8_t* wbase = codes + (size_t)(cmb >> 3) * (4 * D * BITS) + mw * 512 + (cmb & 3) * 16 +
-                       4 * (2 * rh + ((cmb >> 2) & 1));
-      uint32_t w[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        w[i] = 0;
+      for (int hh = 0; hh < 2; ++hh) {
+        uint32_t w = 0;
 #pragma unroll
         for (int f = FPB - 1; f >= 0; --f) {
           const int e = NSET == 2 ? f >> 1 : 0;
           float x[4];
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) x[kk] = piece_value<DTYPE>(raw[kk][f], i);
-          w[i] = w[i] * (1u << BITS) + code_word4<BITS>(x, z[e], inv[e]);
-        }
-      }
-      if (FULLBLK || (valid[0] && valid[1] && valid[2] && valid[3])) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) *reinterpret_cast<uint32_t*>(wbase + 64 * i) = w[i];
-      } else {
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          if (valid[kk]) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) wbase[64 * i + kk] = (uint8_t)(w[i] >> (8 * kk));
+          for (int j = 0; j < 4; ++j) x[j] = piece_value<DTYPE>(raw[kk][f], 4 * hh + j);
+          if constexpr (PLAIN) {
+            const f32x2 nz = pack2(-z[e][kk], -z[e][kk]), ii = pack2(inv[e][kk], inv[e][kk]);
+            w = w * (1u << BITS) + code_word4_plain<BITS>(pack2(x[0], x[1]), pack2(x[2], x[3]), nz, nz, ii, ii);
+          } else {
+            const float zz[4] = {z[e][kk], z[e][kk], z[e][kk], z[e][kk]}, ii[4] = {inv[e][kk], inv[e][kk], inv[e][kk], inv[e][kk]};
+            w = w * (1u << BITS) + code_word4<BITS>(x, zz, ii);
           }
         }
+        if (valid[kk])
+          *reinterpret_cast<uint32_t*>(codes + (size_t)tau * K_ROW_BYTES + chunk_word_byte(2 * rh + hh, mw, wpc, 4)) = w;
       }
+    }
+  } else {
+    // ---- values: the four bytes of a word are this lane's four tokens; word of channel slot i at lane chunk 4 i + t
+    const int cmb = pass * RS + rs;
+    uint8_t* wbase = codes + (size_t)(cmb >> 3) * (4 * D * BITS) + mw * 512 + (cmb & 3) * 16 +
+                     4 * (2 * rh + ((cmb >> 2) & 1));
+    uint32_t w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      w[i] = 0;
+#pragma unroll
+      for (int f = FPB - 1; f >= 0; --f) {
+        const int e = NSET == 2 ? f >> 1 : 0;
+        float x[4];
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) x[kk] = piece_value<DTYPE>(raw[kk][f], i);
+        if constexpr (PLAIN)
+          w[i] = w[i] * (1u << BITS) + code_word4_plain<BITS>(pack2(x[0], x[1]), pack2(x[2], x[3]), pack2(-z[e][0], -z[e][1]), pack2(-z[e][2], -z[e][3]),
+                                                        pack2(inv[e][0], inv[e][1]), pack2(inv[e][2], inv[e][3]));
+        else
+          w[i] = w[i] * (1u << BITS) + code_word4<BITS>(x, z[e], inv[e]);
+      }
+    }
+    if (valid[0] && valid[1] && valid[2] && valid[3]) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) *reinterpret_cast<uint32_t*>(wbase + 64 * i) = w[i];
+    } else {
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        if (valid[kk]) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) wbase[64 * i + kk] = (uint8_t)(w[i] >> (8 * kk));
+        }
+      }
+    }
+  }
+  return true;
+}
+
+// The same with clamped codes, out of line: few passes need it.
+template <int BITS, bool IS_V, int D, int DTYPE>
+__device__ __noinline__ void quantize_pass_clamped(RowSrc rsrc, int gsz, int lo, int hi, uint8_t* __restrict__ codes,
+                                                   uint32_t* __restrict__ meta_out, int lane, int pass) {
+  constexpr int FPB = 8 / BITS, LR = 2 * (D / 16) / FPB, RS = 32 / LR;
+  const int rs = lane / LR, cs = lane % LR;
+  auto load = [&](int kk, int f) {
+    const int tau = token_slot<IS_V, RS>(4 * pass + kk, rs);
+    return *reinterpret_cast<const uint4*>(rsrc.row(min(max(tau, lo), hi - 1)) + 16 * (FPB * (cs >> 1) + f) + 8 * (cs & 1));
+  };
+  quantize_pass<BITS, IS_V, D, DTYPE, false>(load, [] {}, gsz, lo, hi, codes, meta_out, lane, pass);
+}
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// The passes of one side of a stream that fall to a warp: first, first + step, ... of all passes over the 32- or 64-token blocks that
+// hold tokens [qa, qb).  slot: 16 bytes per lane and piece of a pass in shared memory.  Every lane copies the pieces that it will read
+// itself and needs no barrier; those of the next pass are on their way while this one is quantized.  K and V of 64 streams x 32,767
+// tokens (K4V2, 1.29 GB), loads into registers and clamped codes before / now: 262 / 252 us on one box, 250 / 243 on another (four CTAs
+// per SM; three 248, five 248; two passes ahead at three CTAs per SM 256; pieces read twice instead of held, for more warps: 252 to 325).
+// The same loads and stores without the arithmetic between them take 220 us; one grid that goes through all streams pass by pass 299.
+template <int BITS, bool IS_V, int D, int DTYPE>
+__device__ __forceinline__ void quantize_passes(const Geom& g, const CachePtrs& c, const uint16_t* __restrict__ in, int64_t st, int bh, int t0, int qa,
+                                                int qb, int first, int step, uint4* slot, int lane) {
+  constexpr int FPB = 8 / BITS, LR = 2 * (D / 16) / FPB, RS = 32 / LR, TT = task_tokens(D, BITS), NP = TT / RS / 4;
+  static_assert(TT % (4 * RS) == 0, "a lane holds whole groups of four tokens");
+  const int rs = lane / LR, cs = lane % LR;
+  const int gsz = IS_V ? g.gv : g.gk, R = g.R;
+  const int first_task = qa / TT, n = ((qb + TT - 1) / TT - first_task) * NP;
+  const uint16_t* win = R ? c.kv_win + (size_t)bh * R * (2 * D) + (IS_V ? D : 0) : nullptr;
+  in += 16 * FPB * (cs >> 1) + 8 * (cs & 1) - (int64_t)t0 * st;
+  slot += lane;
+  const uint32_t slot_s = (uint32_t)__cvta_generic_to_shared(slot);
+  auto issue = [&](int u) {
+    const int tk0 = (first_task + u / NP) * TT;
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+      const int t = min(max(tk0 + token_slot<IS_V, RS>(4 * (u % NP) + kk, rs), qa), qb - 1);     // (tokens that are not new: any that is)
+      const uint16_t* p = in + (int64_t)t * st;
+      if (R && t < t0) p = win + (size_t)(t % R) * (2 * D) + 16 * FPB * (cs >> 1) + 8 * (cs & 1);
+#pragma unroll
+      for (int f = 0; f < FPB; ++f) cp_async16(slot_s + 512 * (kk * FPB + f), p + 16 * f);
+    }
+  };
+  auto load = [&](int kk, int f) { return slot[32 * (kk * FPB + f)]; };
+  if (first < n) issue(first);
+#pragma unroll 1
+  for (int u = first; u < n; u += step) {
+    const int tk0 = (first_task + u / NP) * TT, tp0 = tk0 & 127;
+    const int lo = max(qa, tk0) - tk0, hi = min(qb, tk0 + TT) - tk0;
+    uint8_t* pg = c.pages + ((size_t)bh * g.n_pages + (tk0 >> 7)) * g.page_bytes;
+    uint8_t* codes = IS_V ? pg + g.v_codes_off + (size_t)(tp0 >> 5) * (4 * D * BITS) : pg + tp0 * (D * BITS / 8);
+    uint32_t* meta = reinterpret_cast<uint32_t*>(pg + (IS_V ? g.v_meta_off : g.k_meta_off)) + tp0 * (D / gsz);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (!quantize_pass<BITS, IS_V, D, DTYPE, true>(load, [&] { if (u + step < n) issue(u + step); }, gsz, lo, hi, codes, meta, lane, u % NP)) {
+      RowSrc rsrc;
+      rsrc.in = in - (16 * FPB * (cs >> 1) + 8 * (cs & 1)) + (int64_t)tk0 * st;
+      rsrc.st = st;
+      rsrc.n_win = R ? max(0, min(TT, t0 - tk0)) : 0;
+      rsrc.wst = 2 * D;
+      rsrc.win = R ? win + (size_t)(tk0 % R) * (2 * D) : nullptr;
+      quantize_pass_clamped<BITS, IS_V, D, DTYPE>(rsrc, gsz, lo, hi, codes, meta, lane, u % NP);
     }
   }
 }
@@ -230,7 +314,7 @@ __device__ __forceinline__ void quantize_task(const RowSrc& rsrc, int gsz, int l
 // the next one's loads in flight (bound by fetching instructions beside the value side's code; two tokens at a time were slower, 32
 // streams x 2,047 tokens 24.8 us against 24; with the signs converted for every token and lanes' own divisions 36 us).  The transform and
 // the codes take two neighbouring channels per operation: four such chunks 90.9 -> 86.2 us.
-// Lanes and fields as in quantize_task; butterfly stages in the order h = 1, 2, 4, ...: bits of i in the lane, rh across
+// Lanes and fields as in quantize_pass; butterfly stages in the order h = 1, 2, 4, ...: bits of i in the lane, rh across
 // lanes, bits of f in the lane, bits of mw across lanes.
 template <int BITS, int D, int DTYPE>
 __device__ __forceinline__ void quantize_task_rotated(const RowSrc& rsrc, int gsz, int lo, int hi, uint8_t* __restrict__ codes,
@@ -446,95 +530,74 @@ __device__ __forceinline__ void copy_task_side(const RowSrc& rsrc, int D, int lo
         *reinterpret_cast<const uint4*>(rsrc.row(row) + l * 8);
 }
 
-// Token-wise quantization of V (blockIdx.z == 0) and of K (blockIdx.z == 1).  grid.y = stream, grid.x strides
-// over the warp tasks touched by this append.
+// Token-wise quantization of V and of K, a side per blockIdx.z.  grid.y = stream, grid.x strides over the passes (or, for 16-bit
+// rows, bit planes and rotated keys, over the warp tasks) touched by this append.  Rotated keys take longer than the values beside them
+// and come first: four chunks of 32 streams x 2,047 tokens 80 us with the values first, 75 now (87 before the passes were pipelined).
+__host__ __device__ constexpr int slot_bytes(int bits) { return bits == 2 ? 8192 : bits == 4 ? 4096 : 2048; }        // 16-byte pieces of a warp's pass
 template <int D, int DTYPE, bool ROT>
-__global__ void __launch_bounds__(kThreads, ROT ? 4 : 5)
+__global__ void __launch_bounds__(kThreads, 4)
 quant_token_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
                    int64_t sb, int64_t sh, int64_t st, int t_new) {
+  extern __shared__ __align__(16) uint8_t smem[];
   begin_after_predecessor();
-  const bool is_v = blockIdx.z == 0;
+  const bool is_v = blockIdx.z == (ROT ? 1 : 0);           // rotated keys take longer and come first
   const int bh = blockIdx.y;
   const int b = bh / g.Hkv, h = bh % g.Hkv;
   const int t0 = c.seq_len[b];
   if (!append_fits(t0, t_new, g.capacity)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int bits = is_v ? g.vb : g.kb;
-  const int TT = (bits == 16 || is_plane_width(bits)) ? 32 : task_tokens(D, bits);
   // tokens to quantize: the new ones, or - with a residual window of R tokens - the blocks of R that this append
   // completes (their first tokens may come from the window, the rest from the input)
   const int R = g.R;
   const int qa = R ? (t0 / R) * R : t0, qb = R ? ((t0 + t_new) / R) * R : t0 + t_new;
   if (qb <= qa) return;
+  const uint16_t* in = (is_v ? v_new : k_new) + (int64_t)b * sb + (int64_t)h * sh;
+  const int gsz = is_v ? g.gv : g.gk;
+  const int first = blockIdx.x * kWarps + warp, step = gridDim.x * kWarps;
+
+  if ((bits == 2 || bits == 4 || bits == 8) && (is_v || !ROT)) {
+    uint4* slot = reinterpret_cast<uint4*>(smem + warp * slot_bytes(bits));
+#define KVQ_PASSES(BITS_, V_) quantize_passes<BITS_, V_, D, DTYPE>(g, c, in, st, bh, t0, qa, qb, first, step, slot, lane)
+    if (is_v) {
+      if (bits == 2) KVQ_PASSES(2, true);
+      else if (bits == 4) KVQ_PASSES(4, true);
+      else KVQ_PASSES(8, true);
+    } else if constexpr (!ROT) {
+      if (bits == 2) KVQ_PASSES(2, false);
+      else if (bits == 4) KVQ_PASSES(4, false);
+      else KVQ_PASSES(8, false);
+    }
+#undef KVQ_PASSES
+    return;
+  }
+  // 16-bit rows, bit planes, rotated keys: a warp per task
+  const int TT = (bits == 16 || is_plane_width(bits)) ? 32 : task_tokens(D, bits);
   const int first_task = qa / TT;
   const int n_tasks = (qb + TT - 1) / TT - first_task;
-  const uint16_t* in = is_v ? v_new : k_new;
-  const int gsz = is_v ? g.gv : g.gk;
-
-  for (int j = blockIdx.x * kWarps + warp; j < n_tasks; j += gridDim.x * kWarps) {
+  for (int j = first; j < n_tasks; j += step) {
     const int tk0 = (first_task + j) * TT;                     // first token of the task
     const int lo = max(qa, tk0) - tk0, hi = min(qb, tk0 + TT) - tk0;
     const int page = tk0 >> 7, tp0 = tk0 & 127;                // page-local token of the task's first row
     uint8_t* pg = c.pages + ((size_t)bh * g.n_pages + page) * g.page_bytes;
     // row 0 of the task in the input (may lie before the first new token; never dereferenced there)
     RowSrc rs;
-    rs.in = in + (int64_t)b * sb + (int64_t)h * sh + (int64_t)(tk0 - t0) * st;
+    rs.in = in + (int64_t)(tk0 - t0) * st;
     rs.st = st;
     rs.n_win = R ? max(0, min(TT, t0 - tk0)) : 0;
     rs.wst = 2 * D;
     rs.win = R ? c.kv_win + ((size_t)bh * R + (tk0 % R)) * (2 * D) + (is_v ? D : 0) : nullptr;
-    if (is_v) {
-      if (bits == 16) {
-        copy_task_side(rs, D, lo, hi, reinterpret_cast<uint16_t*>(pg + g.v_codes_off) + (size_t)tp0 * D, lane);
-        continue;
-      }
-      if (is_plane_width(bits)) {
-        quantize_task_planes<D, DTYPE>(rs, gsz, bits, true, lo, hi, tp0, pg + g.v_codes_off,
-                                       reinterpret_cast<uint32_t*>(pg + g.v_meta_off) + tp0 * (D / gsz), lane);
-        continue;
-      }
-      uint8_t* vb = pg + g.v_codes_off + (size_t)(tp0 >> 5) * (4 * D * bits);
-      uint32_t* vm = reinterpret_cast<uint32_t*>(pg + g.v_meta_off) + tp0 * (D / gsz);
-      const bool full = lo == 0 && hi == TT;
-      if (bits == 2) {
-        if (full) quantize_task<2, true, D, DTYPE, true>(rs, gsz, lo, hi, vb, vm, lane);
-        else quantize_task<2, true, D, DTYPE, false>(rs, gsz, lo, hi, vb, vm, lane);
-      } else if (bits == 4) {
-        if (full) quantize_task<4, true, D, DTYPE, true>(rs, gsz, lo, hi, vb, vm, lane);
-        else quantize_task<4, true, D, DTYPE, false>(rs, gsz, lo, hi, vb, vm, lane);
-      } else {
-        if (full) quantize_task<8, true, D, DTYPE, true>(rs, gsz, lo, hi, vb, vm, lane);
-        else quantize_task<8, true, D, DTYPE, false>(rs, gsz, lo, hi, vb, vm, lane);
-      }
-    } else {
-      if (bits == 16) {
-        copy_task_side(rs, D, lo, hi, reinterpret_cast<uint16_t*>(pg) + (size_t)tp0 * D, lane);
-        continue;
-      }
-      if (is_plane_width(bits)) {
-        quantize_task_planes<D, DTYPE>(rs, gsz, bits, false, lo, hi, tp0, pg,
-                                       reinterpret_cast<uint32_t*>(pg + g.k_meta_off) + tp0 * (D / gsz), lane);
-        continue;
-      }
+    uint8_t* region = pg + (is_v ? g.v_codes_off : 0);
+    uint32_t* meta = reinterpret_cast<uint32_t*>(pg + (is_v ? g.v_meta_off : g.k_meta_off)) + (bits == 16 ? 0 : tp0 * (D / gsz));
+    if (bits == 16) {
+      copy_task_side(rs, D, lo, hi, reinterpret_cast<uint16_t*>(region) + (size_t)tp0 * D, lane);
+    } else if (is_plane_width(bits)) {
+      quantize_task_planes<D, DTYPE>(rs, gsz, bits, is_v, lo, hi, tp0, region, meta, lane);
+    } else if constexpr (ROT) {
       uint8_t* kr = pg + (size_t)tp0 * (D * bits / 8);
-      uint32_t* km = reinterpret_cast<uint32_t*>(pg + g.k_meta_off) + tp0 * (D / gsz);
-      if constexpr (ROT) {
-        if (bits == 2) quantize_task_rotated<2, D, DTYPE>(rs, gsz, lo, hi, kr, km, lane, c.k_signs);
-        else if (bits == 4) quantize_task_rotated<4, D, DTYPE>(rs, gsz, lo, hi, kr, km, lane, c.k_signs);
-        else quantize_task_rotated<8, D, DTYPE>(rs, gsz, lo, hi, kr, km, lane, c.k_signs);
-      } else {
-        const bool full = lo == 0 && hi == TT;
-        if (bits == 2) {
-          if (full) quantize_task<2, false, D, DTYPE, true>(rs, gsz, lo, hi, kr, km, lane);
-          else quantize_task<2, false, D, DTYPE, false>(rs, gsz, lo, hi, kr, km, lane);
-        } else if (bits == 4) {
-          if (full) quantize_task<4, false, D, DTYPE, true>(rs, gsz, lo, hi, kr, km, lane);
-          else quantize_task<4, false, D, DTYPE, false>(rs, gsz, lo, hi, kr, km, lane);
-        } else {
-          if (full) quantize_task<8, false, D, DTYPE, true>(rs, gsz, lo, hi, kr, km, lane);
-          else quantize_task<8, false, D, DTYPE, false>(rs, gsz, lo, hi, kr, km, lane);
-        }
-      }
+      if (bits == 2) quantize_task_rotated<2, D, DTYPE>(rs, gsz, lo, hi, kr, meta, lane, c.k_signs);
+      else if (bits == 4) quantize_task_rotated<4, D, DTYPE>(rs, gsz, lo, hi, kr, meta, lane, c.k_signs);
+      else quantize_task_rotated<8, D, DTYPE>(rs, gsz, lo, hi, kr, meta, lane, c.k_signs);
     }
   }
 }
@@ -723,12 +786,14 @@ int launch_quantize_append(const Geom& g, const CachePtrs& c, const void* k_new,
   if (gx > want) gx = want;
   dim3 grid1(gx, streams, g.k_axis == 0 ? 2 : 1);            // z = 0 values, z = 1 token-wise keys
   const bool rot = c.k_signs != nullptr && g.k_axis == 0;
+  auto side_slots = [](int bits) { return bits == 2 || bits == 4 || bits == 8 ? kWarps * slot_bytes(bits) : 0; };
+  const size_t smem1 = std::max(side_slots(g.vb), g.k_axis == 0 && !rot ? side_slots(g.kb) : 0);
   cudaError_t e = cudaSuccess;
   auto run = [&](auto kern, dim3 grid, unsigned threads, size_t smem, auto... args) {      // (the first failure ends the call)
     if (e == cudaSuccess) e = launch_dependent(kern, grid, threads, smem, stream, 1, args...);
   };
 #define KVQ_QLAUNCH(D_, T_) \
-  run(rot ? quant_token_kernel<D_, T_, true> : quant_token_kernel<D_, T_, false>, grid1, kThreads, 0, g, c, k, v, sb, sh, st, t_new)
+  run(rot ? quant_token_kernel<D_, T_, true> : quant_token_kernel<D_, T_, false>, grid1, kThreads, smem1, g, c, k, v, sb, sh, st, t_new)
   if (g.D == 128 && g.in_dtype == KVQ_BF16) KVQ_QLAUNCH(128, KVQ_BF16);
   else if (g.D == 128) KVQ_QLAUNCH(128, KVQ_FP16);
   else if (g.in_dtype == KVQ_BF16) KVQ_QLAUNCH(64, KVQ_BF16);

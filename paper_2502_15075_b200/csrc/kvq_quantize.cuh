@@ -25,14 +25,18 @@ __device__ __forceinline__ __half2 highs(__half2 a, __half2 b) { return __highs2
 __device__ __forceinline__ __nv_bfloat162 lows(__nv_bfloat162 a, __nv_bfloat162 b) { return __lows2bfloat162(a, b); }
 __device__ __forceinline__ __nv_bfloat162 highs(__nv_bfloat162 a, __nv_bfloat162 b) { return __highs2bfloat162(a, b); }
 
-// (minimum, - maximum) of the eight values of a 16-byte piece.
-template <int DTYPE>
+// (minimum, - maximum) of the eight values of a 16-byte piece.  NANS: a NaN among them makes both NaN, else it is passed over.
+__device__ __forceinline__ __half2 min_pair(__half2 a, __half2 b, bool nans) { return nans ? __hmin2_nan(a, b) : __hmin2(a, b); }
+__device__ __forceinline__ __half2 max_pair(__half2 a, __half2 b, bool nans) { return nans ? __hmax2_nan(a, b) : __hmax2(a, b); }
+__device__ __forceinline__ __nv_bfloat162 min_pair(__nv_bfloat162 a, __nv_bfloat162 b, bool nans) { return nans ? __hmin2_nan(a, b) : __hmin2(a, b); }
+__device__ __forceinline__ __nv_bfloat162 max_pair(__nv_bfloat162 a, __nv_bfloat162 b, bool nans) { return nans ? __hmax2_nan(a, b) : __hmax2(a, b); }
+template <int DTYPE, bool NANS = false>
 __device__ __forceinline__ typename Pair16<DTYPE>::type minmax8(const uint4& r) {
   using H2 = typename Pair16<DTYPE>::type;
   const H2* h = reinterpret_cast<const H2*>(&r);
-  const H2 lo = __hmin2(__hmin2(h[0], h[1]), __hmin2(h[2], h[3]));
-  const H2 hi = __hneg2(__hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3])));
-  return __hmin2(lows(lo, hi), highs(lo, hi));
+  const H2 lo = min_pair(min_pair(h[0], h[1], NANS), min_pair(h[2], h[3], NANS), NANS);
+  const H2 hi = __hneg2(max_pair(max_pair(h[0], h[1], NANS), max_pair(h[2], h[3], NANS), NANS));
+  return min_pair(lows(lo, hi), highs(lo, hi), NANS);
 }
 
 // An append of t_new tokens at position t0 fits the cache; written without a sum that could overflow.
@@ -84,6 +88,23 @@ __device__ __forceinline__ uint32_t code_word4(const float (&x)[4], const float 
   constexpr uint32_t TOP = ((1u << BITS) - 1u) * 0x00010001u;
   const uint32_t even = __vminu2(prmt(n[0], n[2], 0x5410), TOP), odd = __vminu2(prmt(n[1], n[3], 0x5410), TOP);
   return even + odd * 256u;
+}
+
+// Whether no value of a group needs a clamp: the values of its codes before rounding grow with x, so they all round to 0 .. qmax when
+// those of its minimum and maximum do.  True for every group of 16-bit values whose minimum and scale are normal fp16 numbers (the
+// zero-point is then the minimum itself, and a scale rounded down takes the maximum to qmax (1 + 2^-11) at most); false for a NaN.
+__device__ __forceinline__ bool plain_group(float mn, float mx, const GroupParams& p, float qmax) {
+  return __fmul_rn(__fsub_rn(mn, p.z), p.inv) >= -0.5f && __fmul_rn(__fsub_rn(mx, p.z), p.inv) < qmax + 0.5f;
+}
+
+// Codes of four values of plain groups as the four bytes of a word, two values per operation: rint((x - z) * inv) in the low bits of
+// the sum with 1.5 * 2^23.  nz: minus the zero-points; inv_q: inv * 2^-BITS, as above (a product by inv itself and the sum behind it
+// would be contracted to one operation with one rounding, although both ask for their own).
+template <int BITS>
+__device__ __forceinline__ uint32_t code_word4_plain(f32x2 x01, f32x2 x23, f32x2 nz01, f32x2 nz23, f32x2 inv01, f32x2 inv23) {
+  const f32x2 magic = pack2(kRoundMagic, kRoundMagic), up = pack2((float)(1 << BITS), (float)(1 << BITS));
+  const float2 a = unpack2(fma2(mul2(add2(x01, nz01), inv01), up, magic)), b = unpack2(fma2(mul2(add2(x23, nz23), inv23), up, magic));
+  return prmt(prmt(__float_as_uint(a.x), __float_as_uint(a.y), 0x0040), prmt(__float_as_uint(b.x), __float_as_uint(b.y), 0x0040), 0x5410);
 }
 
 // The same in packed operations, two values each, of one group.  (For rotated keys; the other kernels gain nothing, and

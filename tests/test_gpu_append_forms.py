@@ -160,3 +160,47 @@ def test_append_to_sequences_of_different_lengths(kvq, shape, kb, n):
     oc.append(tl.bits_of(k)[:, :, 120:], tl.bits_of(v)[:, :, 120:])
     assert kvq.kvq_check_status(gc) == 0
     tl.assert_caches_equal(gc, oc)
+
+
+@pytest.mark.parametrize("axis,kb,vb", [("token", 4, 2), ("token", 2, 8), ("token", 8, 4), ("channel", 4, 2), ("channel", 8, 4)])
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+def test_values_below_the_normal_fp16_numbers(kvq, axis, kb, vb, dtype):
+    """Magnitudes from 2^-26 to 2^3 side by side (a bf16 key of a channel-wise block is rounded to fp16 in the sum), groups that
+    need no clamp next to groups that do: one block of three, and single rows, reach the ends of the 16-bit type."""
+    w = (wl.SHAPED_14B if axis == "channel" else wl.LLAMA_8B).with_(n_kv_heads=2, n_q_heads=2, kb=kb, vb=vb, dtype=dtype)
+    T, B = 405, 2
+    g = torch.Generator().manual_seed(7)
+    k, v = wl.make_kv(w, tokens=T, batch=B)
+    for x in (k, v):
+        x *= torch.exp2(torch.randint(-24, 2, x.shape, generator=g).to(torch.float32)).to(x.dtype)
+        x[:, :, 50:60] = (x[:, :, 50:60].float() * 2.0 ** -10).to(x.dtype)
+        for t in (140, 141, 200):
+            x[:, 0, t, 3:5] = torch.tensor([65504.0, -65504.0]).to(x.dtype)
+    cfg, gc, oc = tl.build_both(kvq, w, k, v, [3, 402], 512)
+    assert kvq.kvq_check_status(gc) == 0
+    tl.assert_caches_equal(gc, oc)
+    _, gc, oc = tl.build_both(kvq, w, k, v, [405], 512)
+    tl.assert_caches_equal(gc, oc)
+
+
+@pytest.mark.parametrize("axis,kb,vb,D", [("token", 4, 2, 128), ("token", 2, 8, 128), ("token", 8, 4, 64), ("channel", 4, 2, 128), ("channel", 8, 4, 128)])
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+def test_a_long_append_gives_the_bytes_of_its_pieces(kvq, axis, kb, vb, D, dtype):
+    """60 streams x 5,989 tokens: several passes or blocks per warp or CTA, the next one's loads in flight; pieces have one each."""
+    w = (wl.SHAPED_14B if axis == "channel" else wl.LLAMA_8B).with_(n_kv_heads=20, n_q_heads=20, kb=kb, vb=vb, dtype=dtype, head_dim=D, gk=64, gv=64)
+    if axis == "channel":
+        w = w.with_(gk=128)
+    T, B = 5989, 3
+    k, v = wl.make_kv(w, tokens=T, batch=B, device="cuda")
+    for t in (40, 1000, 2500, 2501, 5980):
+        k[:, t % 20, t, 3] = v[:, t % 20, t, 5] = 60000.0
+    pages = []
+    for piece in (T, 640):
+        cfg = tl.gpu_config_for(kvq, w, B, 6144)
+        gc = kvq.Cache(cfg)
+        for t in range(0, T, piece):
+            kvq.kvq_quantize_append(cfg, gc, k[:, :, t:t + piece], v[:, :, t:t + piece])
+        assert kvq.kvq_check_status(gc) == 0 and gc.seq_len.tolist() == [T] * B
+        pages.append((gc.pages.cpu(), gc.tail_view()[:, :, :T % 128].cpu() if axis == "channel" else None))
+    assert torch.equal(pages[0][0], pages[1][0])
+    assert axis == "token" or torch.equal(pages[0][1], pages[1][1])
