@@ -620,29 +620,56 @@ __device__ __forceinline__ void pack_k_rows(const uint8_t* codes, int code_strid
   }
 }
 
-// Channel-wise quantization of K, head_dim 128, 4- or 8-bit codes: CTA j of a stream takes the j-th 128-token block that the
-// append touches; CTA 0 also takes the last one when that stays incomplete (its rows go to the tail, which CTA 0 must
-// have finished reading first).  A complete block never passes through shared memory: every thread has eight 16-byte
-// loads in flight and keeps them, which is what the kernel is bound by (reading the 16-bit rows).  K and V of 120 streams x
-// 16,383 tokens (values by the kernel above included): 605 us with the block staged in shared memory (48 KB a CTA,
-// one load in flight per thread, 7 instructions more per element), 292 us now.
+// Channel-wise quantization of K, head_dim 128, 4- or 8-bit codes: CTA j of a stream takes every grid.x-th of the 128-token blocks that
+// this append completes; CTA 0, which alone reads the tail (for the first block), also writes the rows of the block that stays
+// incomplete to it.  A block stays in the registers of 256 threads; the next one is on its way to shared memory meanwhile, each
+// thread's own pieces, so that no barrier is needed for them.  K and V of 120 streams x 16,383 tokens (values by the kernel above): 286 us
+// with one block per CTA, converted to fp16, clamped and packed value by value (15 instructions per element, issue 68 %), 251 now (four
+// CTAs per SM 250, but 171 us against 147 for rotated keys of 130 streams x 330 tokens; CTAs for 6, 12 or 24 blocks per SM at a time 255, 251, 251).
 template <int DTYPE, int KB, bool ROT>
 __global__ void __launch_bounds__(256, 3)
 quant_kchan_fast_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, int64_t sb, int64_t sh, int64_t st, int t_new) {
+  extern __shared__ __align__(16) uint8_t smem[];
   __shared__ KchanShared scratch;
   begin_after_predecessor();
   const int bh = blockIdx.y, b = bh / g.Hkv, h = bh % g.Hkv;
   const int t0 = c.seq_len[b];
   if (!append_fits(t0, t_new, g.capacity)) return;
-  const int end = t0 + t_new, first_page = t0 >> 7;
-  const int nblk = ((end + 127) >> 7) - first_page;
-  const bool last_partial = (end & 127) != 0;
+  const int end = t0 + t_new, first_page = t0 >> 7, complete = (end >> 7) - first_page;      // blocks that are complete after this append
   const int tid = threadIdx.x;
-  const int j = blockIdx.x;
-  if (j >= nblk) return;
   const uint16_t* in = k_new + (int64_t)b * sb + (int64_t)h * sh - (int64_t)t0 * st + (tid & 15) * 8;
-  if (j < nblk - 1 || !last_partial) kchan_complete_block<DTYPE, KB, ROT>(g, c, bh, first_page + j, t0, in, st, scratch, tid);
-  if (j == 0 && last_partial) kchan_tail_rows<DTYPE, ROT>(c, bh, first_page + nblk - 1, t0, end, in, st, tid);
+  int j = blockIdx.x;
+  if (j < complete && (ROT || (j == 0 && (t0 & 127) != 0))) {        // rows from the tail, or to be rotated
+    kchan_complete_block<DTYPE, KB, ROT>(g, c, bh, first_page + j, t0, in, st, scratch, tid);
+    j += gridDim.x;
+  }
+  if constexpr (ROT) {
+    for (; j < complete; j += gridDim.x) kchan_complete_block<DTYPE, KB, ROT>(g, c, bh, first_page + j, t0, in, st, scratch, tid);
+  } else {
+    // a thread copies the pieces that it will read itself; those of the next block are on their way while this one is quantized
+    uint4* slot = reinterpret_cast<uint4*>(smem) + tid;
+    const uint32_t slot_s = (uint32_t)__cvta_generic_to_shared(slot);
+    auto issue = [&](int block) {
+      const uint16_t* p = in + (int64_t)(((first_page + block) << 7) + (tid >> 4)) * st;
+#pragma unroll
+      for (int i = 0; i < 8; ++i, p += 16 * st) cp_async16(slot_s + 4096 * i, p);
+    };
+    if (j < complete) issue(j);
+#pragma unroll 1
+    for (; j < complete; j += gridDim.x) {
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      uint4 val[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) val[i] = slot[256 * i];
+      uint8_t* pg = c.pages + ((size_t)bh * g.n_pages + first_page + j) * g.page_bytes;
+      if (!kchan_block_plain<DTYPE, KB>(val, scratch, pg, g, tid, [&] { if (j + (int)gridDim.x < complete) issue(j + gridDim.x); })) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) val[i] = key_row_fp16<DTYPE, false>(val[i], nullptr, tid & 15);
+        kchan_block<KB>(val, scratch, pg, g, tid);
+      }
+    }
+  }
+  if (blockIdx.x == 0 && (end & 127) != 0) kchan_tail_rows<DTYPE, ROT>(c, bh, end >> 7, t0, end, in, st, tid);
 }
 
 // Channel-wise quantization of K over 128-token blocks with the fp16 tail, the shapes that the kernel above does not
@@ -799,10 +826,11 @@ int launch_quantize_append(const Geom& g, const CachePtrs& c, const void* k_new,
   else if (g.in_dtype == KVQ_BF16) KVQ_QLAUNCH(64, KVQ_BF16);
   else KVQ_QLAUNCH(64, KVQ_FP16);
 #undef KVQ_QLAUNCH
-  const dim3 grid2((t_new + 127) / 128 + 1, streams);
+  dim3 grid2((t_new + 127) / 128 + 1, streams);
   if (g.k_axis == 1 && g.D == 128 && (g.kb == 4 || g.kb == 8)) {
+    grid2.x = std::min<unsigned>(grid2.x, (148 * 12 + streams - 1) / streams);
 #define KVQ_KCHAN(T_, KB_)                                                                                           \
-  run(c.k_signs ? quant_kchan_fast_kernel<T_, KB_, true> : quant_kchan_fast_kernel<T_, KB_, false>, grid2, 256, 0, g, c, k, \
+  run(c.k_signs ? quant_kchan_fast_kernel<T_, KB_, true> : quant_kchan_fast_kernel<T_, KB_, false>, grid2, 256, c.k_signs ? 0 : 32768, g, c, k, \
       sb, sh, st, t_new)
     if (g.in_dtype == KVQ_BF16) { if (g.kb == 4) KVQ_KCHAN(KVQ_BF16, 4); else KVQ_KCHAN(KVQ_BF16, 8); }
     else { if (g.kb == 4) KVQ_KCHAN(KVQ_FP16, 4); else KVQ_KCHAN(KVQ_FP16, 8); }

@@ -133,7 +133,7 @@ __device__ __forceinline__ uint32_t code_word4_packed(const float (&x)[4], float
 // per token, and each stores one word of the row: the 16 lanes of a row write its 64 (8 bits: 128) bytes whole.
 struct KchanShared {
   uint4 mn[8][16], mx[8][16];       // per warp: the eight channels of each v
-  float2 par[128];                  // (zero, 2^-KB / scale) per channel
+  __align__(16) float2 par[128];    // (zero, 2^-KB / scale) per channel, or both for two channels at a time
 };
 template <int KB>
 __device__ __forceinline__ void kchan_block(const uint4 (&val)[8], KchanShared& sh, uint8_t* __restrict__ pg, const Geom& g, int tid) {
@@ -203,6 +203,104 @@ __device__ __forceinline__ void kchan_block(const uint4 (&val)[8], KchanShared& 
     }
   }
   __syncthreads();                       // the scratch may be used for another block
+}
+
+// The same from the input rows as they are, without conversions, clamps or scalar operations: true, or false with nothing settled where
+// a channel of the block is not plain (see plain_group; here also: beyond the fp16 range).  The quantizer sees the keys as fp16 values.
+// fp16 inputs are those; a bf16 value within the range is one too unless it lies below the normal fp16 numbers, where it has to be
+// rounded to a multiple of 2^-24: the sum with 0.75 does that (its last place is 2^-24 there, and above it holds all of a bf16 value),
+// and 0.75 leaves again with the zero-point, whose sum with it is exact as well.  `next` is called when `val` has been read.
+template <int DTYPE, int KB, typename Next>
+__device__ __forceinline__ bool kchan_block_plain(const uint4 (&val)[8], KchanShared& sh, uint8_t* __restrict__ pg, const Geom& g, int tid, Next&& next) {
+  using H2 = typename Pair16<DTYPE>::type;
+  constexpr int ROW = 128 * KB / 8;
+  constexpr float SHIFT = DTYPE == KVQ_BF16 ? 0.75f : 0.0f, UP = (float)(1 << KB);
+  const int tr = tid >> 4, v = tid & 15, warp = tid >> 5, lane = tid & 31;
+  auto h2 = [](uint32_t u) { return *reinterpret_cast<const H2*>(&u); };
+  auto u32 = [](H2 h) { return *reinterpret_cast<const uint32_t*>(&h); };
+  {
+    H2 mn[4], mx[4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t w[4] = {val[i].x, val[i].y, val[i].z, val[i].w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        mn[j] = i ? min_pair(mn[j], h2(w[j]), true) : h2(w[j]);
+        mx[j] = i ? max_pair(mx[j], h2(w[j]), true) : h2(w[j]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      mn[j] = min_pair(mn[j], h2(__shfl_xor_sync(FULL, u32(mn[j]), 16)), true);
+      mx[j] = max_pair(mx[j], h2(__shfl_xor_sync(FULL, u32(mx[j]), 16)), true);
+    }
+    if (lane < 16) {
+      sh.mn[warp][v] = make_uint4(u32(mn[0]), u32(mn[1]), u32(mn[2]), u32(mn[3]));
+      sh.mx[warp][v] = make_uint4(u32(mx[0]), u32(mx[1]), u32(mx[2]), u32(mx[3]));
+    }
+  }
+  __syncthreads();
+  next();
+  bool plain = true;
+  if (tid < 64) {                        // two channels a thread
+    const uint32_t* a = reinterpret_cast<const uint32_t*>(sh.mn) + tid;
+    const uint32_t* b = reinterpret_cast<const uint32_t*>(sh.mx) + tid;
+    H2 lo = h2(a[0]), hi = h2(b[0]);
+#pragma unroll
+    for (int w = 1; w < 8; ++w) { lo = min_pair(lo, h2(a[64 * w]), true); hi = max_pair(hi, h2(b[64 * w]), true); }
+    const float2 l2 = pair_to_f32(lo), u2 = pair_to_f32(hi);
+    const float qmax = (float)((1 << KB) - 1);
+    uint2 meta;
+    float4 par;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const float l = e ? l2.y : l2.x, u = e ? u2.y : u2.x;
+      plain &= l >= -65504.0f && u <= 65504.0f;
+      const float l16 = __half2float(__ushort_as_half(f32_to_fp16_sat_bits(l))), u16 = __half2float(__ushort_as_half(f32_to_fp16_sat_bits(u)));
+      const GroupParams p = group_params(l16, u16, qmax);
+      plain &= plain_group(l16, u16, p, qmax);
+      (e ? meta.y : meta.x) = p.meta;
+      (e ? par.z : par.x) = -(p.z + SHIFT);
+      (e ? par.w : par.y) = p.inv * (1.0f / UP);
+    }
+    reinterpret_cast<uint2*>(pg + g.k_meta_off)[tid] = meta;
+    reinterpret_cast<float4*>(sh.par)[tid] = make_float4(par.x, par.z, par.y, par.w);      // (- zero, - zero, 2^-KB / scale, 2^-KB / scale)
+  }
+  if (!__syncthreads_and(plain)) return false;
+  f32x2 nz[4], inv_q[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float4 p = reinterpret_cast<const float4*>(sh.par)[4 * v + j];
+    nz[j] = pack2(p.x, p.y); inv_q[j] = pack2(p.z, p.w);
+  }
+  const f32x2 up = pack2(UP, UP), magic = pack2(kRoundMagic, kRoundMagic), shift = pack2(SHIFT, SHIFT);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t w[4] = {val[i].x, val[i].y, val[i].z, val[i].w};
+    uint32_t pair[4];                    // two codes each, bytes 0 and 1
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 f = pair_to_f32(h2(w[j]));
+      f32x2 x = pack2(f.x, f.y);
+      if constexpr (DTYPE == KVQ_BF16) x = add2(x, shift);
+      const float2 r = unpack2(fma2(mul2(add2(x, nz[j]), inv_q[j]), up, magic));
+      pair[j] = prmt(__float_as_uint(r.x), __float_as_uint(r.y), 0x0040);
+    }
+    const uint32_t word[2] = {prmt(pair[0], pair[1], 0x5410), prmt(pair[2], pair[3], 0x5410)};
+    uint8_t* row = pg + (tr + 16 * i) * ROW;
+    if constexpr (KB == 4) {
+      const int rh = v & 1, f = (v >> 1) & 1, mw = v >> 2;
+      const uint32_t other = __shfl_xor_sync(FULL, f ? word[0] : word[1], 2);       // the partner's half of the word this lane stores
+      *reinterpret_cast<uint32_t*>(row + (2 * rh + f) * 16 + mw * 4) = f ? (other | (word[1] << 4)) : (word[0] | (other << 4));
+    } else {
+      const int rh = v & 1, mw = v >> 1;
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh)
+        *reinterpret_cast<uint32_t*>(row + (mw >> 2) * 64 + (2 * rh + hh) * 16 + (mw & 3) * 4) = word[hh];
+    }
+  }
+  __syncthreads();                       // the scratch may be used for another block
+  return true;
 }
 
 // Block `page` of a stream, complete after this append: slots [0, t0 - 128 page) from the tail, the rest from the input.
