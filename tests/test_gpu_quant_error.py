@@ -108,3 +108,19 @@ def test_error_sums_of_values_far_from_zero(kvq, D, gk, gv, dtype):
         kvq.kvq_quant_error(cfg, k.cuda(), v.cuda(), sums)
         want = oe.quant_error_sums(tl.bits_of(k), tl.bits_of(v), w.dtype, w.kb, w.vb, w.gk, w.gv)
         assert np.allclose(sums.cpu().numpy(), want, rtol=1e-5, atol=0.0), (sums.cpu().numpy() / want - 1)
+
+
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+@pytest.mark.parametrize("kb,vb", [(2, 8), (3, 4)])
+def test_error_sums_of_groups_that_clamp(kvq, dtype, kb, vb):
+    """Rows beyond the fp16 range, below its normal numbers and around a minimum that fp16 rounds, next to ordinary ones."""
+    w = wl.LLAMA_8B.with_(n_kv_heads=2, n_q_heads=2, gk=32, gv=128, dtype=dtype, kb=kb, vb=vb)
+    k, v = wl.make_kv(w, tokens=130, batch=1)
+    for x in (k, v):
+        x[:, :, 7] *= 2.0 ** -18
+        x[:, 0, 40, :2] = torch.tensor([65504.0, -65504.0] if dtype == "fp16" else [3.0e8, -1.0e8]).to(x.dtype)
+    cfg = tl.gpu_config_for(kvq, w, 1, 128)
+    sums = torch.zeros((1, 2, 4), dtype=torch.float64, device="cuda")
+    kvq.kvq_quant_error(cfg, k.cuda(), v.cuda(), sums)
+    want = oe.quant_error_sums(tl.bits_of(k), tl.bits_of(v), w.dtype, w.kb, w.vb, w.gk, w.gv)
+    assert np.allclose(sums.cpu().numpy(), want, rtol=1e-5, atol=0.0), (sums.cpu().numpy() / want - 1)
