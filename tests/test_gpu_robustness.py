@@ -154,3 +154,26 @@ def test_append_guard_rejects_lengths_near_int_max(kvq):
     kvq.kvq_quantize_append(cfg, gc, k.cuda(), v.cuda())
     assert kvq.kvq_check_status(gc) == -5
     assert gc.seq_len.tolist() == [2 ** 31 - 1, 2 ** 31 - 8] and torch.equal(gc.pages, before)
+
+
+@pytest.mark.parametrize("B,heads,T,window", [(1, 1, 128 * 60, 0), (1, 8, 30000, 0), (3, 8, 2001, 64), (1, 2, 129, 64)])
+def test_whatever_the_workspace_holds(kvq, B, heads, T, window):
+    """The count words of a stream's partials start right from any contents: zeros (as a merge leaves them), all ones (one addition
+    wraps them), other bytes, other values in every word, and what the call before left; streams of many partials and of one."""
+    w = wl.LLAMA_8B.with_(n_kv_heads=heads, n_q_heads=4 * heads)
+    k, v = wl.make_kv(w, tokens=T, batch=B, device="cuda")
+    cfg = tl.gpu_config_for(kvq, w, B, -(-T // 128) * 128, window)
+    gc = kvq.Cache(cfg)
+    kvq.kvq_quantize_append(cfg, gc, k, v)
+    q = wl.make_q(w, batch=B).cuda()
+    ws = torch.zeros(kvq.kvq_workspace_bytes(cfg), dtype=torch.uint8, device="cuda")
+    outs = []
+    for fill in (0, 255, 0xA5, "ramp", None, 0, None, None):
+        if fill == "ramp":
+            ws.copy_((torch.arange(ws.numel(), device="cuda") * 37 % 251).to(torch.uint8))
+        elif fill is not None:
+            ws.fill_(fill)
+        outs.append(torch.zeros(tuple(q.shape), dtype=torch.float32, device="cuda"))
+        kvq.kvq_decode_attention(cfg, gc, q, outs[-1], ws)
+    assert kvq.kvq_check_status(gc) == 0
+    assert all(torch.equal(o, outs[0]) for o in outs[1:]) and bool(torch.isfinite(outs[0]).all())
