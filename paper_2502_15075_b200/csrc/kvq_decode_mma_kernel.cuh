@@ -75,20 +75,16 @@ __device__ __forceinline__ bool named_bar_any(int id, int nthreads, bool p) {
   return r != 0;
 }
 
-// Four values times `scale` rounded to integers |Q| <= 32512 and split into two balanced signed bytes,
-// Q = hi * 256 + lo; returns the four hi bytes (lo_limb = 0) or the four lo bytes (lo_limb = 1) as one word
-// and adds the four Q to `qsum`.
-__device__ __forceinline__ uint32_t fixed_point_limb(const float (&t)[4], float scale, int lo_limb, int& qsum) {
-  uint32_t w = 0;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int Q = __float2int_rn(t[j] * scale);
-    const int lo = (int)(int8_t)(Q & 0xFF);
-    const int hi = (Q - lo) >> 8;
-    w |= (uint32_t)((lo_limb ? lo : hi) & 0xFF) << (8 * j);
-    qsum += Q;
-  }
-  return w;
+// Four values times `scale` rounded to integers |Q| <= 32512 and split into two balanced signed bytes, Q = hi * 256 + lo: the four hi
+// bytes or the four lo bytes as one word.  The sum with 1.5 * 2^23 (+ 128 for the hi bytes: hi = (Q + 128) >> 8) leaves Q as the low bits
+// of n; the caller gets them all added up.  scale_q: scale * 2^-8 (the product is rounded before it is rounded to an integer, by a fused
+// operation that takes the 2^8 back).  sel: bytes 1 (hi) or 0 (lo) of two words.
+__device__ __forceinline__ uint32_t fixed_point_limb(const float (&t)[4], f32x2 scale_q, f32x2 magic, uint32_t sel, uint32_t& nsum) {
+  const f32x2 up = pack2(256.0f, 256.0f);
+  const float2 a = unpack2(fma2(mul2(pack2(t[0], t[1]), scale_q), up, magic)), b = unpack2(fma2(mul2(pack2(t[2], t[3]), scale_q), up, magic));
+  const uint32_t n0 = __float_as_uint(a.x), n1 = __float_as_uint(a.y), n2 = __float_as_uint(b.x), n3 = __float_as_uint(b.y);
+  nsum += n0 + n1 + n2 + n3;
+  return prmt(prmt(n0, n1, sel), prmt(n2, n3, sel), 0x5410);
 }
 
 // The split balances time, not pages.  Ending one stream and starting the next costs a CTA about as much as six to eight pages
@@ -131,21 +127,32 @@ constexpr int kFlushPages = 128;           // fold the int32 value accumulators 
 // 16 r + 4 tid + {0..3} for every slot r, in fp32, rotated like the keys if the cache rotates them; heads >= G are
 // zero.  Returns max |q| over the lane's values (the caller reduces over the quad).
 template <int D>
-__device__ __forceinline__ float load_q_lane(const Geom& g, const CachePtrs& c, const uint16_t* __restrict__ q, int b,
-                                             int h, int hb, int tid, float (&qv)[D / 16][4]) {
+__device__ __forceinline__ void load_q_raw(const Geom& g, const uint16_t* __restrict__ q, int b, int h, int hb, int tid, uint2 (&raw)[D / 16]) {
+  const int Gq = g.G, G = g.G * g.rows;
+  const uint16_t* qrow = q + (((size_t)b * g.rows + hb / Gq) * g.Hq + (size_t)h * Gq + hb % Gq) * D;
+#pragma unroll
+  for (int r = 0; r < D / 16; ++r) {
+    raw[r] = make_uint2(0u, 0u);
+    if (hb < G) raw[r] = *reinterpret_cast<const uint2*>(qrow + 16 * r + 4 * tid);
+  }
+}
+template <int D>
+__device__ __forceinline__ float convert_q_lane(const Geom& g, const CachePtrs& c, const uint2 (&raw)[D / 16], int tid, float (&qv)[D / 16][4]) {
   constexpr int NR = D / 16;
   constexpr uint32_t FULL = 0xffffffffu;
-  const int Gq = g.G, G = g.G * g.rows;
-        const uint16_t* qrow = q + (((size_t)b * g.rows + hb / Gq) * g.Hq + (size_t)h * Gq + hb % Gq) * D;
+  if (g.in_dtype == KVQ_FP16) {
 #pragma unroll
-        for (int r = 0; r < NR; ++r) {
-          uint2 raw = make_uint2(0u, 0u);
-          if (hb < G) raw = *reinterpret_cast<const uint2*>(qrow + 16 * r + 4 * tid);
-          qv[r][0] = bits16_to_f32((uint16_t)(raw.x & 0xFFFF), g.in_dtype);
-          qv[r][1] = bits16_to_f32((uint16_t)(raw.x >> 16), g.in_dtype);
-          qv[r][2] = bits16_to_f32((uint16_t)(raw.y & 0xFFFF), g.in_dtype);
-          qv[r][3] = bits16_to_f32((uint16_t)(raw.y >> 16), g.in_dtype);
-        }
+    for (int r = 0; r < NR; ++r) {
+      const float2 x = __half22float2(as_h2(raw[r].x)), y = __half22float2(as_h2(raw[r].y));
+      qv[r][0] = x.x; qv[r][1] = x.y; qv[r][2] = y.x; qv[r][3] = y.y;
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      qv[r][0] = __uint_as_float(raw[r].x << 16); qv[r][1] = __uint_as_float(raw[r].x & 0xFFFF0000u);
+      qv[r][2] = __uint_as_float(raw[r].y << 16); qv[r][3] = __uint_as_float(raw[r].y & 0xFFFF0000u);
+    }
+  }
         if (c.k_signs != nullptr) {
           // rotated keys: give q the same rotation, q' = H (signs * q) / sqrt(D); channel 16 r + 4 tid + j,
           // so the butterflies run over j inside the lane, over tid across lanes, over r inside the lane
@@ -510,7 +517,9 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
 #pragma unroll
           for (int nh = 0; nh < NH; ++nh) {
             float q_all[NR][4];
-            float am = load_q_lane<D>(g, c, q, b, h, (gid >> 1) + 4 * nh, tid, q_all);
+            uint2 q_raw[NR];
+            load_q_raw<D>(g, q, b, h, (gid >> 1) + 4 * nh, tid, q_raw);
+            float am = convert_q_lane<D>(g, c, q_raw, tid, q_all);
 #pragma unroll
             for (int r = 0; r < HR; ++r) {
 #pragma unroll
@@ -665,6 +674,12 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
     // row r sees the first n - (rows - 1 - r) tokens of the n the sequence holds, window included)
     const int n_unmasked = min(n_tok, n_all - (g.rows - 1));
     const int stream = b * Hkv + h;
+    // the queries are on their way while one thread works out
+    [[maybe_unused]] uint2 q_raw[NH][NR];
+    if constexpr (KAXIS == 0) {
+#pragma unroll
+      for (int nh = 0; nh < NH; ++nh) load_q_raw<D>(g, q, b, h, (gid >> 1) + 4 * nh, tid, q_raw[nh]);
+    }
     // which of the stream's partials this CTA writes, and how many there are: one thread works it out now, everybody
     // reads it after the barrier at the segment's end (the barrier that closed the last segment keeps its readers apart)
     if (tid_ == 0) {
@@ -690,27 +705,30 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
     sscale = SSCALE0;
 #pragma unroll
     for (int nh = 0; nh < NH; ++nh) {
-      const int hb = (gid >> 1) + 4 * nh;                          // head of this lane's operand column
       hs[nh] = 0.f;
       if constexpr (KAXIS == 0) {       // (channel-wise keys: the producer warp makes the operands, per page)
         float qv[NR][4];
-        float amax = load_q_lane<D>(g, c, q, b, h, hb, tid, qv);
+        float amax = convert_q_lane<D>(g, c, q_raw[nh], tid, qv);
         amax = fmaxf(amax, __shfl_xor_sync(FULL, amax, 1));
         amax = fmaxf(amax, __shfl_xor_sync(FULL, amax, 2));
         // 16-bit fixed point relative to the head's largest entry: Q = rint(q * scale), |Q| <= 32512
         const float scale = amax > 0.f ? kQFix / amax : 0.f;
         const float hsb = amax > 0.f ? c1 / scale : 0.f;
-        int qs[NGK];
+        const f32x2 scale_q = pack2(scale * 0.00390625f, scale * 0.00390625f);
+        const float magicf = 12582912.0f + ((gid & 1) ? 0.0f : 128.0f);
+        const f32x2 magic = pack2(magicf, magicf);
+        const uint32_t sel = (gid & 1) ? 0x0040u : 0x0051u;
+        uint32_t qs[NGK];
 #pragma unroll
-        for (int j = 0; j < NGK; ++j) qs[j] = 0;
+        for (int j = 0; j < NGK; ++j) qs[j] = 0u - (uint32_t)(4 * (NR / NGK)) * __float_as_uint(magicf);      // (what the words carry besides Q)
 #pragma unroll
-        for (int r = 0; r < NR; ++r) qB[nh][0][r] = fixed_point_limb(qv[r], scale, gid & 1, qs[r / (NR / NGK)]);
+        for (int r = 0; r < NR; ++r) qB[nh][0][r] = fixed_point_limb(qv[r], scale_q, magic, sel, qs[r / (NR / NGK)]);
         hs[nh] = __shfl_sync(FULL, hsb, 8 * tid);
         // the zero-point term uses the sum of the same fixed-point q the MMAs see: the two large terms
         // s (q . c) and z sum(q) of a logit then cancel exactly as they do for the exact q
 #pragma unroll
         for (int j = 0; j < NGK; ++j) {
-          int v = qs[j];
+          int v = (int)qs[j];
           v += __shfl_xor_sync(FULL, v, 1);
           v += __shfl_xor_sync(FULL, v, 2);
           qsum[nh][j] = hs[nh] * (float)__shfl_sync(FULL, v, 8 * tid);
