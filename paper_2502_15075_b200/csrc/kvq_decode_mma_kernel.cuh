@@ -692,12 +692,6 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       stream_ctas<WAVES>(plan, waves, xs, pages_b, &first, &count);
       sMisc[8] = (int)blockIdx.x - first;
       sMisc[9] = count;
-      // Start the stream's count word for this launch, unless another CTA has: the last merge cleared it, so that counting a partial
-      // takes one addition at the segment's end.  Started there, by whoever came first, the CTAs of a stream that finished together
-      // swapped against one another: one sequence of 30,000 tokens (8B shape, four layers) 168 -> 88 us, 16 layers of the 1B shape that
-      // take in 128 tokens 328 -> 315, eight ragged K4V4 layers 165 -> 154, 70B-shaped 246 -> 243.  (A word with other contents is
-      // started when it is counted in, see tagged_count.)
-      if (count > 1 || n_all > n_tok) atomicCAS(reinterpret_cast<unsigned long long*>(ws + tag_offset_floats(B * Hkv, s_cap, G, D)) + stream, 0ull, id40 << 24);
     }
 
     // ---- segment start: q operands, group sums and a clean state for this stream's heads (the scale limit too: under one
@@ -748,6 +742,14 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
 #pragma unroll
       for (int nt = 0; nt < NTV; ++nt) { Oi[nt][i][0] = Oi[nt][i][1] = Oi[nt][i][2] = Oi[nt][i][3] = 0; }
     }
+
+    // Start the stream's count word for this launch, unless another CTA has: the last merge cleared it, so that counting a partial takes
+    // one addition at the segment's end.  Started there, by whoever came first, the CTAs of a stream that finished together swapped
+    // against one another: one sequence of 30,000 tokens (8B shape, four layers) 162 -> 85 us, 16 layers of the 1B shape that take in 128
+    // tokens 328 -> 313, eight ragged K4V4 layers 166 -> 150, 70B-shaped 247 -> 239.  (By another thread than the bookkeeping's and
+    // behind the queries: 1 to 2 % of a short step.  A word with other contents is started when it is counted in, see tagged_count.)
+    if (tid_ == 32 && (seg_pages < pages_b || n_all > n_tok))
+      atomicCAS(reinterpret_cast<unsigned long long*>(ws + tag_offset_floats(B * Hkv, s_cap, G, D)) + stream, 0ull, id40 << 24);
 
     auto process = [&](auto full_tag, int pp) {
       constexpr bool FULL_PAGE = decltype(full_tag)::value;
