@@ -118,16 +118,15 @@ int launch_decode_mma(const Geom& g, const CachePtrs& c, const void* q, void* ou
                       float* ws, const DecodeDebug& dbg, cudaStream_t stream) {
   const int s_cap = flat_slot_cap(g);
   int grid = 0;
-  if (g.R) {      // the residual window first: its partial (or, for sequences without pages, the output) is ready
-                  // when the main kernel's last finisher merges
-    int rc = launch_decode_window(g, c, q, out, out_dtype, c1, ws, s_cap, stream);
-    if (rc != KVQ_OK) return rc;
-  }
-  const bool tc_ok = decode_tc_supported(g, c);
-  if (dbg.fast_impl == 2 && !tc_ok) return KVQ_ERR_UNSUPPORTED;
-  if (tc_ok && dbg.fast_impl == 2)
+  if (dbg.fast_impl == 2) {
+    if (!decode_tc_supported(g, c)) return KVQ_ERR_UNSUPPORTED;
+    if (g.R) {      // the residual window first: its partial (or, for sequences without pages, the output) is ready when the last partial is merged
+      const int rc = launch_decode_window(g, c, q, out, out_dtype, c1, ws, s_cap, stream);
+      if (rc != KVQ_OK) return rc;
+    }
     return launch_decode_tc(g, c, q, c1, ws, s_cap, out, out_dtype, next_call_id(),
                             dbg.wait_us ? 1000ull * dbg.wait_us : mma::kWaitTimeoutNs, dbg.skip_page, stream);
+  }
   return pick(g, c, q, c1, ws, s_cap, out, out_dtype, dbg, stream, false, &grid);
 }
 

@@ -270,6 +270,134 @@ static __host__ __device__ __forceinline__ bool weighted_shares(const FlatPlan& 
          (pages_max - 1) * 1000ll * grid <= (slots - 1) * plan.N * WMIN;
 }
 
+// D += A(16x16, row) * B(16x8, col), bf16 operands, fp32 accumulate.
+__device__ __forceinline__ void mma16816_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// Attention over the residual window (Sec. 4.1's buffer of recent full-precision tokens) of one stream, by the four consumer warps: the
+// newest nw <= 127 tokens are 16-bit rows in a ring (key row, value row of slot i side by side), positions f .. f + nw - 1.  Leaves the
+// partial (m, l, o) at `part`, or the output of a stream that has no pages (part = nullptr).  Run once per stream, it is bound by
+// fetching its instructions and by latency, so it is kept short: a thread sums two channels over every 128 / (D / 2)-th token.  Logits are
+// exact products of the 16-bit keys and queries, summed in fp32 by the tensor cores, 16 tokens a warp and step, a column per (row,
+// head) pair; weights and the sums of weighted values are fp32.  scratch: 128 x 4 NH floats; red_max, red_sum: 4 x 8 each; win: the rows,
+// in global or shared memory.  As a kernel of its own in front of this one (32 CTAs on 148 SMs, then a launch that waits for it) the window
+// cost 7 us a layer: eight layers of 4 x 8 streams of 2,000 tokens with two drafted rows 192 us, 154 here; always by the CTA with the
+// stream's first page 182.
+template <int D, int NH>
+__device__ __forceinline__ void window_partial(const Geom& g, const uint16_t* win, const uint16_t* __restrict__ q, float c1, int n, int f, int nw,
+                                               float* scratch, float* red_max, float* red_sum, float* __restrict__ part, void* __restrict__ out,
+                                               size_t out0, int out_dtype) {
+  constexpr int NC = 128, NR = D / 16, VH = 4 * NH, TG = NC / (D / 2);       // token groups of the weighted values
+  constexpr uint32_t FULL = 0xffffffffu;
+  const int tid_ = threadIdx.x, lane = tid_ & 31, warp = tid_ >> 5, gid = lane >> 2, tid = lane & 3;
+  const int Gq = g.G, nvh = g.G * g.rows;
+  const bool bf = g.in_dtype == KVQ_BF16;
+  const int cp = tid_ % (D / 2), tg = tid_ / (D / 2);
+  // ---- logits: warp w takes tokens 16 w .. 16 w + 15 and, of a window of 128, those 64 behind
+  uint2 qf[NR];
+  {
+    const uint16_t* qrow = q + (size_t)(gid / Gq) * g.Hq * D + (size_t)(gid % Gq) * D;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) qf[r] = gid < nvh ? *reinterpret_cast<const uint2*>(qrow + 16 * r + 4 * tid) : make_uint2(0u, 0u);
+  }
+  float m0 = -INFINITY, m1 = -INFINITY;          // of (row, head) pairs 2 tid, 2 tid + 1
+  const int lim0 = n - f - (g.rows - 1 - min(2 * tid / Gq, g.rows - 1)), lim1 = n - f - (g.rows - 1 - min((2 * tid + 1) / Gq, g.rows - 1));
+#pragma unroll 1
+  for (int t0 = 16 * warp; t0 < nw; t0 += 64) {
+    const uint16_t* ka = win + (size_t)(t0 + gid) * 2 * D + 4 * tid;       // (slots beyond nw are there, their logits are dropped)
+    float S[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const uint2 a = *reinterpret_cast<const uint2*>(ka + 16 * r), b = *reinterpret_cast<const uint2*>(ka + 16 * D + 16 * r);
+      if (bf) mma16816_bf16(S, a.x, b.x, a.y, b.y, qf[r].x, qf[r].y);
+      else mma16816(S, a.x, b.x, a.y, b.y, qf[r].x, qf[r].y);
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int t = t0 + gid + 8 * e;
+      const float x = t < min(nw, lim0) ? c1 * S[2 * e] : -INFINITY, y = t < min(nw, lim1) ? c1 * S[2 * e + 1] : -INFINITY;
+      m0 = fmaxf(m0, x); m1 = fmaxf(m1, y);
+      if (2 * tid < VH) *reinterpret_cast<float2*>(scratch + t * VH + 2 * tid) = make_float2(x, y);
+    }
+  }
+#pragma unroll
+  for (int off = 4; off < 32; off <<= 1) {
+    m0 = fmaxf(m0, __shfl_xor_sync(FULL, m0, off));
+    m1 = fmaxf(m1, __shfl_xor_sync(FULL, m1, off));
+  }
+  if (gid == 0) { red_max[warp * 8 + 2 * tid] = m0; red_max[warp * 8 + 2 * tid + 1] = m1; }
+  named_bar_sync(1, NC);
+  // ---- weights: thread (token, pair) by pairs; sums per warp
+  {
+    const int vh = tid_ % VH;
+    const float m = fmaxf(fmaxf(red_max[vh], red_max[8 + vh]), fmaxf(red_max[16 + vh], red_max[24 + vh]));
+    float sum = 0.f;
+    for (int t = tid_ / VH; t < nw; t += NC / VH) {
+      const float p = m == -INFINITY ? 0.f : exp2f(scratch[t * VH + vh] - m);
+      scratch[t * VH + vh] = p;
+      sum += p;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int off = VH; off < 32; off <<= 1) sum += __shfl_xor_sync(FULL, sum, off);
+    if (lane < VH) red_sum[warp * 8 + lane] = sum;
+  }
+  named_bar_sync(1, NC);
+  // ---- weighted values
+  float o[VH][2];
+#pragma unroll
+  for (int e = 0; e < VH; ++e) o[e][0] = o[e][1] = 0.f;
+#pragma unroll 8
+  for (int t = tg; t < nw; t += TG) {
+    const uint32_t raw = *reinterpret_cast<const uint32_t*>(win + ((size_t)t * 2 + 1) * D + 2 * cp);
+    const float2 v = bf ? make_float2(__uint_as_float(raw << 16), __uint_as_float(raw & 0xFFFF0000u)) : __half22float2(as_h2(raw));
+#pragma unroll
+    for (int e = 0; e < VH; e += 4) {
+      const float4 w = *reinterpret_cast<const float4*>(scratch + t * VH + e);
+      o[e][0] = fmaf(w.x, v.x, o[e][0]); o[e][1] = fmaf(w.x, v.y, o[e][1]);
+      o[e + 1][0] = fmaf(w.y, v.x, o[e + 1][0]); o[e + 1][1] = fmaf(w.y, v.y, o[e + 1][1]);
+      o[e + 2][0] = fmaf(w.z, v.x, o[e + 2][0]); o[e + 2][1] = fmaf(w.z, v.y, o[e + 2][1]);
+      o[e + 3][0] = fmaf(w.w, v.x, o[e + 3][0]); o[e + 3][1] = fmaf(w.w, v.y, o[e + 3][1]);
+    }
+  }
+  named_bar_sync(1, NC);                         // the weights have been read: their place takes the other groups' sums
+  if (tg > 0) {
+#pragma unroll
+    for (int e = 0; e < VH; ++e) *reinterpret_cast<float2*>(scratch + ((tg - 1) * VH + e) * D + 2 * cp) = make_float2(o[e][0], o[e][1]);
+  }
+  named_bar_sync(1, NC);
+  if (tg == 0) {
+#pragma unroll
+    for (int e = 0; e < VH; ++e) {
+#pragma unroll
+      for (int k = 0; k < TG - 1; ++k) {
+        const float2 x = *reinterpret_cast<const float2*>(scratch + (k * VH + e) * D + 2 * cp);
+        o[e][0] += x.x; o[e][1] += x.y;
+      }
+      if (e < nvh) {
+        const float l = (red_sum[e] + red_sum[8 + e]) + (red_sum[16 + e] + red_sum[24 + e]);
+        if (part != nullptr) {
+          float* dst = part + e * (D + 2);
+          if (cp == 0) {
+            dst[0] = fmaxf(fmaxf(red_max[e], red_max[8 + e]), fmaxf(red_max[16 + e], red_max[24 + e]));
+            dst[1] = l;
+          }
+          *reinterpret_cast<float2*>(dst + 2 + 2 * cp) = make_float2(o[e][0], o[e][1]);
+        } else {
+          const size_t oi = out0 + ((size_t)(e / Gq) * g.Hq + e % Gq) * D + 2 * cp;
+          const float x = l > 0.f ? o[e][0] / l : 0.f, y = l > 0.f ? o[e][1] / l : 0.f;
+          if (out_dtype == KVQ_FP32) *reinterpret_cast<float2*>(static_cast<float*>(out) + oi) = make_float2(x, y);
+          else *reinterpret_cast<uint32_t*>(static_cast<uint16_t*>(out) + oi) = (uint32_t)f32_to_bits16(x, out_dtype) | ((uint32_t)f32_to_bits16(y, out_dtype) << 16);
+        }
+      }
+    }
+  }
+  named_bar_sync(1, NC);                         // the scratch may be used again
+}
+
 // Template parameters: head_dim, key bits, value bits, key axis (0 token-wise, 1 channel-wise), key / value groups
 // per row, NH = query heads per lane (1: up to 4 heads per KV head, 2: up to 8), resident CTAs per SM.
 //
@@ -293,7 +421,7 @@ static __host__ __device__ __forceinline__ bool weighted_shares(const FlatPlan& 
 // The two token rows of a lane share every fp32 operation on logits and weights that has a packed form: two 70B-shaped layers at 128k
 // tokens, step 256 -> 251 us, 8B shape 181 -> 179.
 constexpr int kConsumerWarps = 4;
-template <int D, int KB, int VB, int KAXIS, int NGK, int NGV, int NH, int MINB>
+template <int D, int KB, int VB, int KAXIS, int NGK, int NGV, int NH, int MINB, bool WIN>
 __global__ void __launch_bounds__((kConsumerWarps + 1) * 32, MINB)
 decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1, float* __restrict__ ws,
                   int s_cap, int stages, void* __restrict__ out, int out_dtype, unsigned long long call_id,
@@ -389,10 +517,9 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
     }
   }
   __syncthreads();
-  // an empty sequence has no page and therefore no CTA of its own: its output rows are zero (with a residual
-  // window the window kernel, which runs first, has written the rows of sequences without pages)
-  for (int bb = blockIdx.x; bb < B && g.R == 0; bb += gridDim.x) {
-    if (sPref[bb + 1] == sPref[bb]) {
+  // a sequence without pages has no CTA of its own: its output rows are zero, or the attention over its residual window
+  for (int bb = blockIdx.x; bb < B; bb += gridDim.x) {
+    if (sPref[bb + 1] == sPref[bb] && (!WIN || clamped_len(c.seq_len, bb, g.capacity) == 0)) {
       for (int i = tid_; i < g.rows * g.Hq * D; i += blockDim.x) {
         const size_t oi = (size_t)bb * g.rows * g.Hq * D + i;
         if (out_dtype == KVQ_FP32) static_cast<float*>(out)[oi] = 0.f;
@@ -400,9 +527,45 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       }
     }
   }
+  [[maybe_unused]] auto window_of = [&](int bb, int hh, int n, const uint16_t* rows, float* part) {
+    const int f = n / g.R * g.R;
+    const size_t first = ((size_t)bb * g.rows * g.Hq + (size_t)hh * Gq) * D;
+    window_partial<D, NH>(g, rows, q + first, c1, n, f, n - f, reinterpret_cast<float*>(smem + sl.w_off), sMax, sSum,
+                          part, out, first, out_dtype);
+  };
+  if constexpr (WIN) {
+    if (warp < NW) {
+#pragma unroll 1
+      for (int st = blockIdx.x; st < B * Hkv; st += gridDim.x) {
+        const int bb = st / Hkv, n = clamped_len(c.seq_len, bb, g.capacity);
+        if (sPref[bb + 1] == sPref[bb] && n > 0) window_of(bb, st - bb * Hkv, n, c.kv_win + (size_t)st * g.R * (2 * D), nullptr);
+      }
+    }
+  }
   if (sVPref[B] == 0 || (int)blockIdx.x >= sMisc[10]) return;
   const int x_lo = (int)*reinterpret_cast<const long long*>(sMisc + 4), x_hi = (int)*reinterpret_cast<const long long*>(sMisc + 6);
-  if (x_lo >= x_hi) return;                          // a share that lies inside a gap (tiny problems only)
+  // A share that lies inside a gap (short contexts) has nothing to do; the first of them in front of a stream takes its residual window.
+  [[maybe_unused]] bool win_only = false;
+  auto window_owner = [&](int bb, int hh, int pages, int first) {       // the CTA that computes the window's partial
+    const FlatPlan plan{(long long)sVPref[B], sMisc[10]};
+    const long long v = (long long)sVPref[bb] + (long long)hh * (pages + GAP);
+    const int w = v > 0 ? cta_of_virtual<WAVES>(plan, GAP != 0 && sMisc[14] != 0, v - 1) + 1 : 0;
+    return w < first ? w : first;
+  };
+  if (x_lo >= x_hi) {
+    if constexpr (!WIN) return;
+    if (tid_ == 0) {
+      const int bb = sMisc[11], hh = sMisc[12], pages = (sPref[bb + 1] - sPref[bb]) / Hkv;
+      const FlatPlan plan{(long long)sVPref[B], sMisc[10]};
+      int first, count;
+      stream_ctas<WAVES>(plan, GAP != 0 && sMisc[14] != 0, (long long)sVPref[bb] + (long long)hh * (pages + GAP) + GAP, pages, &first, &count);
+      const int n = clamped_len(c.seq_len, bb, g.capacity);
+      sMisc[0] = n % g.R != 0 && window_owner(bb, hh, pages, first) == (int)blockIdx.x;
+    }
+    __syncthreads();
+    if (sMisc[0] == 0) return;
+    win_only = true;
+  }
 
   // ---- cursor: first page of this CTA -> (b, h, page)
   int b = sMisc[11], h = sMisc[12], page = sMisc[13];
@@ -666,8 +829,8 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
     }
   };
 
-  for (int x = x_lo; x < x_hi;) {
-    const int seg_pages = min(pages_b - page, x_hi - x);
+  for (int x = x_lo; x < x_hi || (WIN && win_only);) {
+    const int seg_pages = WIN && win_only ? 0 : min(pages_b - page, x_hi - x);
     const int n_all = clamped_len(c.seq_len, b, g.capacity);
     const int n_tok = g.R ? (n_all / g.R) * g.R : n_all;          // tokens of the sequence that are in the pages
     // a block is unmasked when all of its 32 tokens exist and every query row may see them (several causal rows:
@@ -692,6 +855,31 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       stream_ctas<WAVES>(plan, waves, xs, pages_b, &first, &count);
       sMisc[8] = (int)blockIdx.x - first;
       sMisc[9] = count;
+      if constexpr (WIN) {
+        sMisc[0] = window_owner(b, h, pages_b, first);
+        sMisc[3] = count + (n_all > n_tok && sMisc[0] < first ? 1 : 0);          // CTAs that count themselves
+      }
+    }
+
+    // the stream's residual window: one more partial, in the slot behind the page partials', by a CTA whose share lies in the gap in
+    // front of the stream (its ring is free for the rows), else by the one that has its first page, counted with that one's own
+    if constexpr (WIN) {
+      if (page == 0 && n_all > n_tok) {
+        named_bar_sync(1, NCONS);
+        if (sMisc[0] == (int)blockIdx.x) {
+          const uint16_t* rows = c.kv_win + (size_t)stream * g.R * (2 * D);
+          const int bytes = (n_all - n_tok) * 4 * D;
+          if (win_only && bytes <= sl.ring_bytes) {
+            if (tid_ == 0) {
+              mbar_expect_tx(bar0, (uint32_t)bytes);
+              bulk_load(ring, rows, (uint32_t)bytes, bar0, l2_evict_first_policy());
+            }
+            if (!__all_sync(FULL, mbar_try_wait(bar0, 0))) wait_slowly(bar0);
+            rows = reinterpret_cast<const uint16_t*>(smem);
+          }
+          window_of(b, h, n_all, rows, ws + ((size_t)stream * s_cap + (s_cap - 1)) * G * (D + 2));
+        }
+      }
     }
 
     // ---- segment start: q operands, group sums and a clean state for this stream's heads (the scale limit too: under one
@@ -1101,13 +1289,13 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       // whole stream writes the output at once; otherwise it stores its partial, counts itself in, and the CTA
       // that completes the count merges all partials of the stream by log-sum-exp and stores the output.
       const int slot = sMisc[8], n_part = sMisc[9];
-      const bool has_win = n_all > n_tok;                 // the window kernel left a partial in slot s_cap - 1
-      if (slot >= 0 && slot < s_plan) {
+      const bool has_win = WIN && n_all > n_tok;                 // its partial is in slot s_cap - 1
+      if ((slot >= 0 && slot < s_plan) || (WIN && win_only)) {
         const bool direct = n_part == 1 && !has_win;
 #pragma unroll
         for (int nh = 0; nh < NH; ++nh) {
           const int head = tid + 4 * nh;
-          if (head < G) {
+          if (head < G && !(WIN && win_only)) {
             float lsum = 0.f;
             double zsum = 0.0;
 #pragma unroll
@@ -1141,7 +1329,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
           unsigned long long* counts = reinterpret_cast<unsigned long long*>(ws + tag_offset_floats(B * Hkv, s_cap, G, D));
           if (tid_ == 0) *n_published = (int)tagged_count(counts + stream, id40);
           named_bar_sync(1, NCONS);
-          if (*n_published == n_part) {
+          if (*n_published == (WIN ? sMisc[3] : n_part)) {
             __threadfence();
             // a warp per head, two or four channels per lane; eight partials' loads are in flight at a time
             constexpr int C2 = D / 64;
@@ -1200,6 +1388,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       named_bar_sync(1, NCONS);
     }
 
+    if (WIN && win_only) return;
     // ---- advance the cursor past this segment
     x += seg_pages;
     page += seg_pages;
@@ -1228,7 +1417,10 @@ int launch_mma_inst(const Geom& g, const CachePtrs& c, const void* q, float c1, 
   if (stages > 2 && stages * ((g.page_bytes + 127) & ~127) > 54 * 1024) stages = 3;
   if (stages < 2) return KVQ_ERR_UNSUPPORTED;
   const SmemLayout sl = smem_layout(g.page_bytes, stages, g.B, D, NH, NGV, KAXIS == 1);
-  auto kern = decode_mma_kernel<D, KB, VB, KAXIS, NGK, NGV, NH, MINB>;
+  auto kern = decode_mma_kernel<D, KB, VB, KAXIS, NGK, NGV, NH, MINB, false>;
+  if constexpr (KAXIS == 0) {
+    if (g.R) kern = decode_mma_kernel<D, KB, VB, KAXIS, NGK, NGV, NH, MINB, true>;
+  }
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sl.total) != cudaSuccess)
     return KVQ_ERR_CUDA_LAUNCH;
   const cudaError_t e = launch_dependent(kern, dim3(148 * MINB), (kConsumerWarps + 1) * 32, sl.total, stream, 1, g, c,

@@ -3,6 +3,7 @@
 // softmax-attention partials (m, l, o) of all (row, head) pairs over those at most R - 1 tokens in fp32 and leaves
 // them in the stream's last partial slot, where the main kernel's merge picks them up; a stream without pages gets
 // its output written here.
+// Runs in front of the tcgen05 kernel only; the warp-level kernel takes the window itself (window_partial in kvq_decode_mma_kernel.cuh).
 //
 // At most 64 KB per stream, so latency is all there is: every thread loads its share of the keys and of the values (16-byte
 // pieces) before it computes anything.  Logits: four lanes per token, a quarter of the channels each, four heads at once.  Values:

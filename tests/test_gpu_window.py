@@ -104,3 +104,41 @@ def test_window_tokens_only_and_with_pages(kvq, D, heads, rows, dtype, R, T):
     cfg, gc, oc = tl.build_both(kvq, w, k, v, [T], 384, residual=R)
     q = make_q_rows(w, 2, rows, T)
     tl.assert_attention_close(decode_rows(kvq, cfg, gc, q), oc.decode_rows(tl.bits_of(q)))
+
+
+@pytest.mark.parametrize("w,R,rows,lens", [
+    (W8, 64, 1, [0, 40, 64 * 3 + 9, 128 * 20 + 70, 128 * 70 + 13, 128]),        # windows in gaps, with first pages, without pages, empty
+    (W8, 64, 2, [2, 63, 65, 1000, 1001]),
+    (W8.with_(kb=8, vb=4), 128, 1, [127, 300, 128 * 9 + 127]),                   # no gaps between the streams
+    (wl.LLAMA_70B.with_(n_kv_heads=2, n_q_heads=16), 128, 1, [50, 128 * 3 + 127, 128 * 40 + 1]),
+    (wl.LLAMA_1B.with_(n_kv_heads=2, n_q_heads=8), 128, 1, [50, 128 * 3 + 127, 128 * 40 + 1]),
+    (W8, 64, 1, [64 * (i % 9) + 7 * i % 64 for i in range(90)]),                  # many short streams
+    (wl.LLAMA_8B.with_(n_kv_heads=1, n_q_heads=4), 128, 1, [128 * 60 + 99]),      # one stream over many shares
+])
+def test_windows_of_uneven_batches(kvq, w, R, rows, lens):
+    """Whoever takes a stream's window - a share inside the gap in front of it, the share with its first page, or a stream without
+    pages - and whatever the other streams do: each sequence gives what it gives alone, checked against the oracle."""
+    T, cap = max(lens), -(-max(lens) // 128) * 128
+    cfg = tl.gpu_config_for(kvq, w, len(lens), cap, R)
+    gc = kvq.Cache(cfg)
+    cfg1 = tl.gpu_config_for(kvq, w, 1, cap, R)
+    k, v = wl.make_kv(w, tokens=T, batch=1, device="cuda")
+    pages, win = gc.pages_view(), gc.window_view()
+    win.fill_(-1)                                  # rows that hold no token are NaN
+    for b, n in enumerate(lens):
+        one = kvq.Cache(cfg1)
+        one.window_view().fill_(-1)
+        if n:
+            kvq.kvq_quantize_append(cfg1, one, k[:, :, T - n:], v[:, :, T - n:])
+        pages[b], win[b] = one.pages_view()[0], one.window_view()[0]
+    gc.seq_len.copy_(torch.tensor(lens, dtype=torch.int32))
+    q = make_q_rows(w, len(lens), rows, 3)
+    got = decode_rows(kvq, cfg, gc, q)
+    assert np.array_equal(got, decode_rows(kvq, cfg, gc, q))
+    check = range(len(lens)) if len(lens) < 10 else range(0, len(lens), 7)
+    for b in check:
+        sub = kvq.Cache(cfg1)
+        sub.pages_view()[0], sub.window_view()[0] = pages[b], win[b]
+        sub.seq_len.fill_(lens[b])
+        oc = tl.oracle_on_gpu_codes(sub, w)
+        tl.assert_attention_close(got[b:b + 1], oc.decode_rows(tl.bits_of(q[b:b + 1])))
