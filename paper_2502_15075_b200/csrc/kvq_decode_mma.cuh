@@ -195,8 +195,15 @@ constexpr int kMaxBatchFlat = 1024;   // the flat partition keeps a per-batch pr
 // 70B-shaped layers 251 and 246, 14B 230 and 226).
 __host__ __device__ __forceinline__ long long divide(long long n, long long d) {
   const float df = (float)d;
-  long long q = (long long)((float)n / df), r = n - q * d;
-  const long long e = (long long)((float)r / df);
+  auto estimate = [df](long long x) {
+#ifdef __CUDA_ARCH__
+    return (long long)__fdividef((float)x, df);
+#else
+    return (long long)((float)x / df);
+#endif
+  };
+  long long q = estimate(n), r = n - q * d;
+  const long long e = estimate(r);
   q += e;
   r -= e * d;
   while (r < 0) { --q; r += d; }
