@@ -13,7 +13,7 @@ namespace kvq {
 
 namespace {
 
-constexpr int kMaxThreads = 512;
+constexpr int kMaxThreads = 1024;
 inline int heads_per_cta(int n_kv_heads) { return (n_kv_heads + 7) / 8; }
 constexpr int kChanThreads = 256;       // channel-wise keys: what a block's registers are laid out for
 
@@ -158,28 +158,28 @@ append_rows_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, cons
 
 }  // namespace
 
-// A sequence has at most eight CTAs, so the time goes with the rows of one of them: its KV heads x new tokens.  Both sides measured
-// behind 613 cached tokens, one of sixteen calls in a row in a replayed graph, us rows / tasks + lengths, for 1 and 16 sequences (K4V2,
-// head_dim 128):
-//    8 KV heads:  48 tokens 5.4 / 6.5, 7.9 / 8.5;     64 tokens 6.3 / 6.6, 10.0 / 12.3;   96 tokens 8.5 / 6.8, 14.2 / 12.6
-//   16 KV heads:  16 tokens 4.5 / 7.0, 6.2 / 9.0;     32 tokens 6.5 / 7.0, 10.1 / 8.9;    48 tokens 8.5 / 7.2, 14.2 / 9.5
-//   32 KV heads:   8 tokens 4.5 / 6.5, 6.2 / 11.5;    16 tokens 6.4 / 7.2, 10.1 / 12.6;   32 tokens 10.6 / 7.4, 18.1 / 13.3
-//   64 KV heads:   4 tokens 4.5 / 6.1, 6.4 / 15.3;     8 tokens 6.5 / 6.3, 10.2 / 15.9;   16 tokens 10.6 / 7.2, 18.2 / 17.6
-// so 64 rows a CTA at head_dim 128 and 128 at head_dim 64 (8 heads: 128 tokens 6.4 / 7.3, 9.9 / 11.2, 192 tokens 8.5 / 7.4, 14.0 / 11.2;
-// 16 heads: 64 tokens 6.5 / 6.4, 9.9 / 9.2, 128 tokens 10.4 / 7.5, 17.7 / 11.7).  Rotated keys and a residual window cost more a row: 40
-// rows beyond eight heads (16 heads rotated: 16 tokens 5.3 / 6.0, 7.8 / 6.8, 20 tokens 6.4 / 6.7, 9.3 / 7.6, 32 tokens 8.3 / 8.5, 13.2 / 9.9;
-// with a window: 20 tokens 3.3 / 5.1, 5.1 / 8.0, 32 tokens, which complete a block, 12.8 / 7.9, 22.6 / 10.6; eight heads: 64 tokens rotated
-// 8.2 / 8.9, 13.1 / 10.6, with a window 8.0 / 9.6, 14.0 / 15.8).  Channel-wise keys also pay for a block a head (1 and 32 sequences; 32
-// heads: 16 tokens 7.4 / 8.0, 11.2 / 16.8, 20 tokens 9.4 / 8.5, 14.3 / 18.7; 64 heads: 4 tokens 7.0 / 7.9, 11.2 / 21.8, 8 tokens 9.0 / 8.0,
-// 13.9 / 22.1).  The lines were drawn when neither kernel overlapped the launch before it; they no longer lie best for several rotated
-// sequences (above) and for 30 to 52 tokens of ten channel-wise heads (32 tokens 9.8 / 9.2, 16.1 / 15.8, 52 tokens 12.6 / 9.7, 20.4 / 17.1).
+// A sequence has at most eight CTAs, so the time goes with the rows of one of them: its KV heads x new tokens; beyond twelve sequences
+// two clusters share SMs and it goes up once more.  Both sides measured behind 613 cached tokens, one of sixteen calls in a row in a
+// replayed graph, us rows / tasks + lengths, for 8, 16 and 32 sequences (K4V2):
+//    8 KV heads, head_dim 128:   24 tokens 3.9 / 4.3, 5.4 / 5.2, 5.6 / 5.8;   32 tokens 4.6 / 4.5, 6.3 / 5.5, 6.4 / 6.3;
+//                                48 tokens 5.5 / 4.5, 8.1 / 5.5, 8.3 / 6.4;   64 tokens 6.3 / 4.7, 10.0 / 6.0, 10.1 / 7.3
+//   16 KV heads, head_dim 128:   16 tokens 4.6 / 5.2, 6.2 / 5.8, 6.4 / 7.8;   24 tokens 5.5 / 5.2, 8.1 / 5.8, 8.3 / 7.7
+//    8 KV heads, head_dim 64:    64 tokens 4.2 / 4.9, 6.2 / 5.7, 6.3 / 6.5;  128 tokens 6.0 / 6.0, 9.8 / 7.4, 9.9 / 8.5
+//    8 KV heads, rotated:        32 tokens 5.5 / 7.3, 7.9 / 7.7, 8.2 / 8.5;   64 tokens 7.9 / 7.8, 13.0 / 8.6, 13.3 / 10.1
+//    8 KV heads, window of 64:   24 tokens 3.0 / 5.5, 3.7 / 5.6, 4.0 / 6.2;   32 tokens, which complete a block, 7.8 / 6.8, 11.8 / 7.6, 12.7 / 10.1
+//   10 channel-wise heads:       24 tokens 6.0 / 6.8, 6.1 / 7.0, 7.1 / 7.7;   32 tokens, which complete a block, 10.4 / 9.7, 12.6 / 12.5, 15.4 / 14.5;
+//                                48 tokens, which complete a block, 12.8 / 9.9, 15.5 / 12.5, 19.0 / 15.3
+// Two or three launches cost the host 8 to 10 us a call, this one 6, so up to twelve sequences the line stays at 64 rows a CTA at head_dim
+// 128 and 128 at head_dim 64, where tasks would save the GPU 1.5 us; beyond, at 32 and 64.  Rotated keys and a residual window cost more a
+// row: 40 rows beyond eight heads (16 heads rotated: 20 tokens 6.4 / 6.7, 32 tokens 8.3 / 8.5; with a window 32 tokens, which complete a
+// block, 12.8 / 7.9).  Channel-wise keys also pay for a block a head: 36 tokens at ten heads.
 // An append of at most 64 tokens of channel-wise keys completes at most one block.
 bool append_rows_serves(const Geom& g, bool rotated, int t_new) {
   auto width = [](int b) { return b == 2 || b == 4 || b == 8; };
   if (t_new > 64 * 128 / g.D || !width(g.kb) || !width(g.vb)) return false;
   const long long heads = heads_per_cta(g.Hkv);
-  if (g.k_axis == 1) return g.D == 128 && g.kb != 2 && heads * (t_new + 12) <= 128;
-  const int limit = heads > 1 && (rotated || g.R) ? 40 : 64;
+  if (g.k_axis == 1) return g.D == 128 && g.kb != 2 && heads * (t_new + 12) <= 96;
+  const int limit = g.B > 12 ? 32 : heads > 1 && (rotated || g.R) ? 40 : 64;
   return heads * t_new * g.D <= limit * 128;
 }
 
@@ -188,7 +188,10 @@ int launch_append_rows(const Geom& g, const CachePtrs& c, const void* k_new, con
   const int per_cta = heads_per_cta(g.Hkv), ranks = (g.Hkv + per_cta - 1) / per_cta;        // at most 8 CTAs, evenly loaded
   const bool chan = g.k_axis == 1, rot = c.k_signs != nullptr;
   int threads = per_cta * 2 * (t_new + g.R) * (g.D / 8);
-  threads = chan ? kChanThreads : threads > kMaxThreads ? kMaxThreads : (threads + 31) / 32 * 32;
+  // 1,024 threads where every cluster finds SMs of its own (8 sequences x 128 tokens at head_dim 64: 6.5 us with 512, 6.0; 16 sequences
+  // of 50 tokens, whose CTAs then no longer share SMs, 9.1 and 10.5), and no window (a block's rows only when one is completed)
+  const int most = g.R || g.B > 8 ? kMaxThreads / 2 : kMaxThreads;
+  threads = chan ? kChanThreads : threads > most ? most : (threads + 31) / 32 * 32;
   const uint16_t* k = static_cast<const uint16_t*>(k_new);
   const uint16_t* v = static_cast<const uint16_t*>(v_new);
   cudaError_t e;

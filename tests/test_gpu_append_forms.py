@@ -204,3 +204,19 @@ def test_a_long_append_gives_the_bytes_of_its_pieces(kvq, axis, kb, vb, D, dtype
         pages.append((gc.pages.cpu(), gc.tail_view()[:, :, :T % 128].cpu() if axis == "channel" else None))
     assert torch.equal(pages[0][0], pages[1][0])
     assert axis == "token" or torch.equal(pages[0][1], pages[1][1])
+
+
+@pytest.mark.parametrize("B,D,heads,n", [(8, 128, 8, 64), (9, 128, 8, 64), (12, 64, 8, 128), (13, 128, 8, 32), (13, 64, 8, 64), (14, 128, 16, 16)])
+@pytest.mark.parametrize("form", ["plain", "rotated"])
+def test_the_short_append_of_several_sequences(kvq, B, D, heads, n, form):
+    """More threads per CTA up to eight sequences, fewer tokens beyond twelve: the largest append of one launch and the one beyond it."""
+    if form == "rotated" and heads > 8:
+        n = min(n, 20)
+    w = wl.LLAMA_8B.with_(n_kv_heads=heads, n_q_heads=heads, head_dim=D, gk=64, gv=64)
+    check(kvq, w, B, [13, n, n + 1], SIGNS[:D] if form == "rotated" else None)
+
+
+@pytest.mark.parametrize("heads,n", [(8, 64), (10, 36), (17, 20)])
+def test_the_short_append_of_channelwise_keys_and_the_one_beyond(kvq, heads, n):
+    w = wl.SHAPED_14B.with_(n_kv_heads=heads, n_q_heads=heads)
+    check(kvq, w, 2, [13, n, n + 1, 3, n, n + 1])
