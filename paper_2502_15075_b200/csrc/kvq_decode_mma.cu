@@ -108,7 +108,7 @@ int decode_mma_plan(const Geom& g, const int32_t* seq_len, int32_t* parts, int64
   if (g.B > mma::kMaxBatchFlat) return KVQ_ERR_UNSUPPORTED;
   const int rc = pick(g, none, nullptr, 0.f, nullptr, 0, nullptr, 0, DecodeDebug{}, nullptr, true, &grid);
   if (rc != KVQ_OK) return rc;
-  const int gap = mma::gap_pages(g.D, g.kb, g.vb, g.k_axis, g.G * g.rows <= 4 ? 1 : 2, g.R != 0, g.B * g.Hkv);
+  const int gap = mma::gap_pages(g.D, g.kb, g.vb, g.k_axis, g.B * g.Hkv);
   if (grid == 3 * 148) host_plan<3>(g, gap, seq_len, parts, starts, cursors, info);
   else host_plan<2>(g, gap, seq_len, parts, starts, cursors, info);
   return KVQ_OK;

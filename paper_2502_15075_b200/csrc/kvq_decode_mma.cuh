@@ -18,7 +18,7 @@
 //    and  o = sum_t (p_t s_t) c_t + sum_t p_t z_t ;
 //  * the sequence is split flat over the grid: CTA i takes the i-th share of all pages
 //    of all streams (shares balanced by time where the arithmetic limits the kernel: a
-//    stream boundary counts as six or eight pages, twelve at head_dim 64 up to 64 streams, two with channel-wise keys; the launch waves of
+//    stream boundary counts as eight pages, twelve at head_dim 64 up to 64 streams, two with channel-wise keys; the launch waves of
 //    an SM are weighted where every stream's partials fit its slots all the same) and
 //    writes one unnormalised partial (m, l, o) per stream it touches; the CTA that
 //    publishes the last partial of a stream merges them by log-sum-exp and writes the

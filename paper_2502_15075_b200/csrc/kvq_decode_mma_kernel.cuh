@@ -90,17 +90,16 @@ __device__ __forceinline__ uint32_t fixed_point_limb(const float (&t)[4], f32x2 
 // The split balances time, not pages.  Ending one stream and starting the next costs a CTA about as much as several pages
 // (load and convert the next queries, publish a partial, perhaps merge), so every stream is given a gap of virtual pages in front
 // of its real ones and the split is taken on that virtual axis; with many CTAs per stream the gap also keeps shares from
-// crossing into the next stream for a page or two.  One head a lane at head_dim 128: gap 6 (eight layers of 40 ragged K4V4 streams gap 8
-// 145.9 us, 6 145.2, 4 143.3; four layers of 80 ragged streams of 4,000 tokens 73.2, 70.6, 70.0; 64 x 700 tokens 53.7, 52.2, 53.4; two of
-// 128 x 32,767 174.7, 174.6, 175.6).  Two heads a lane, or a window to be taken besides: 8 (70B shape at 128k tokens 237 us, 6 239.5, 4 242; 64
-// windowed streams of 16,000 tokens 63.6, 65.3, 68.0).  Channel-wise keys, whose pages take longer: 2 (two ragged 14B-shaped layers 226 us; 5:
-// 228, 8: 233).  At head_dim 64 a page is half the work: 12 (1B shape, append 128 and decode, 16 layers: 18 301.6 us, 15 297.0, 12 296.4;
+// crossing into the next stream for a page or two.  Eight pages at head_dim 128 (70B shape at 128k tokens 237 us, gap 6 239.5, 4 242; 64
+// windowed streams of 16,000 tokens 63.6, 65.3, 68.0; two layers of 128 x 32,767 174.7, 174.6, 175.6; short ragged ones of one head a lane
+// gain: 80 streams of 4,000 tokens 73.2, 70.6, 70.0).  Channel-wise keys, whose pages take longer: 2 (two ragged 14B-shaped layers 226
+// us; 5: 228, 8: 233).  At head_dim 64 a page is half the work: 12 (1B shape, append 128 and decode, 16 layers: 18 301.6 us, 15 297.0, 12 296.4;
 // eight layers of 64 streams of 1,000 tokens 103.5, 102.9, 99.6, 64 ragged ones of 4,000 122.2, 120.3, 118.9), but only up to 64 streams: with
 // more of them a share is not much longer than such a gap, and some are left with nothing else (steps of six 1B-shaped layers, gap 8 / 18
 // when it was 18: 72 x 1,200 89.7 / 92.9, 96 x 1,200 90.3 / 97.5, 128 x 4,000 122 / 131, 256 x 4,000 167 / 184).
 // Of the CTAs that share an SM the hardware favours the older ones (0.85 / 0.91 / 0.99 us per page at three per SM, 0.96 / 1.01 at two),
 // so the launch waves are weighted (8B shape K4V2 when the weights were chosen: 1040 76.1 us, 1080 77.3, equal 80.4).
-constexpr int kGapPages = 8, kGapPagesShort = 6, kGapPages64 = 12, kGapStreams64 = 64, kGapPagesChan = 2;
+constexpr int kGapPages = 8, kGapPages64 = 12, kGapStreams64 = 64, kGapPagesChan = 2;
 constexpr float kQFix = 32512.0f;          // largest |Q| of the 16-bit fixed-point q (hi limb stays within +-127)
 constexpr float kQFix3 = 8300000.0f;       // ... of the 24-bit fixed-point q * s of channel-wise keys (three limbs)
 
@@ -257,11 +256,8 @@ static __host__ __device__ __forceinline__ void stream_ctas(const FlatPlan& plan
 }
 // The time-balanced split (stream gaps) pays where the arithmetic per page limits the kernel (token-wise and
 // channel-wise keys alike); pages of 10 bits per element pair and more lose with it and keep the plain split by pages.
-__host__ __device__ constexpr int gap_pages(int D, int kb, int vb, int k_axis, int heads, bool window, int streams) {
-  if (kb + vb > 8) return 0;
-  if (k_axis == 1) return kGapPagesChan;
-  if (D == 64) return streams <= kGapStreams64 ? kGapPages64 : kGapPages;
-  return heads == 1 && !window ? kGapPagesShort : kGapPages;
+__host__ __device__ constexpr int gap_pages(int D, int kb, int vb, int k_axis, int streams) {
+  return kb + vb <= 8 ? (k_axis == 1 ? kGapPagesChan : D == 64 && streams <= kGapStreams64 ? kGapPages64 : kGapPages) : 0;
 }
 // Whether the shares of a full grid are weighted by launch wave: only where every stream's partials fit its slots all the
 // same.  A stream of P pages touches fewer than 2 + (P - 1) / s CTAs when no share is smaller than s virtual pages (the shares
@@ -449,7 +445,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   constexpr int V_META_OFF = V_CODES_OFF + 4 * V_BLOCK_BYTES;
   constexpr int NCONS = NW * 32;
   constexpr uint32_t FULL = 0xffffffffu;
-  const int GAP = gap_pages(D, KB, VB, KAXIS, NH, WIN, g.B * g.Hkv);      // (known at compile time at head_dim 128)
+  const int GAP = gap_pages(D, KB, VB, KAXIS, g.B * g.Hkv);      // (known at compile time at head_dim 128)
   constexpr int WAVES = MINB;               // CTAs per SM = launch waves (the weights apply to a grid of 148 * WAVES)
   static_assert(MT % NW == 0 && (MT / NGV) % MTW == 0, "a warp's channels are whole m-tiles of one value group");
   static_assert(KAXIS == 0 || KB != 2, "channel-wise 2-bit keys are not instantiated");
