@@ -3,11 +3,11 @@
 // groups along head_dim, or channel-wise groups over a 128-token block with an
 // fp16 residual tail) and packing into the page layout.
 //
-// Token-wise kernel: one warp per block of 32 tokens (64 for head_dim 64 at 2 bits) of one
-// stream and one side (keys or values).  A byte of the packed page holds codes of channels that
+// Token-wise kernel: a warp takes passes of four tokens a lane over blocks of 32 tokens (64 for head_dim 64 at 2
+// bits) of one stream and one side (keys or values).  A byte of the packed page holds codes of channels that
 // lie 16 apart, so a lane loads, for each of its tokens, the 8/b 16-byte pieces whose codes share
 // bytes: every output byte, and with four tokens (values) or four channels (keys) every output
-// word, is then assembled in that lane's registers and stored directly - no shared memory, no
+// word, is then assembled in that lane's registers and stored directly - codes need no shared memory, no
 // atomics, no read-modify-write; a token that is not new is simply not stored (byte stores for
 // values).  Group minima and maxima are reduced with a few shuffles between the lanes of a row.
 // Long calls are bound by the memory system and the length of a warp's chain, short ones by fetching instructions.
@@ -262,7 +262,7 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
 // The passes of one side of a stream that fall to a warp: first, first + step, ... of all passes over the 32- or 64-token blocks that
 // hold tokens [qa, qb).  slot: 16 bytes per lane and piece of a pass in shared memory.  Every lane copies the pieces that it will read
 // itself and needs no barrier; those of the next pass are on their way while this one is quantized.  K and V of 64 streams x 32,767
-// tokens (K4V2, 1.29 GB), loads into registers and clamped codes before / now: 262 / 252 us on one box, 250 / 243 on another (four CTAs
+// tokens (K4V2, 1.29 GB), loads into registers and clamped codes before / now: 262 / 252 us on one GPU, 250 / 243 on another (four CTAs
 // per SM; three 248, five 248; two passes ahead at three CTAs per SM 256; pieces read twice instead of held, for more warps: 252 to 325).
 // The same loads and stores without the arithmetic between them take 220 us; one grid that goes through all streams pass by pass 299.
 template <int BITS, bool IS_V, int D, int DTYPE>
@@ -535,7 +535,7 @@ __device__ __forceinline__ void copy_task_side(const RowSrc& rsrc, int D, int lo
 // and come first: four chunks of 32 streams x 2,047 tokens 80 us with the values first, 75 now (87 before the passes were pipelined).
 __host__ __device__ constexpr int slot_bytes(int bits) { return bits == 2 ? 8192 : bits == 4 ? 4096 : 2048; }        // 16-byte pieces of a warp's pass
 template <int D, int DTYPE, bool ROT>
-__global__ void __launch_bounds__(kThreads, 4)
+__global__ void __launch_bounds__(kThreads, D == 64 && !ROT ? 5 : 4)
 quant_token_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
                    int64_t sb, int64_t sh, int64_t st, int t_new) {
   extern __shared__ __align__(16) uint8_t smem[];
@@ -807,12 +807,15 @@ int launch_quantize_append(const Geom& g, const CachePtrs& c, const void* k_new,
   const uint16_t* v = static_cast<const uint16_t*>(v_new);
   // warp tasks touched per stream: at most ceil(t_new / 32) + 1; one warp per task, CTAs stride over them
   const int max_tasks = (t_new + 31) / 32 + 1;
-  int gx = (max_tasks + kWarps - 1) / kWarps;
+  // (head_dim 64: two passes a warp and five CTAs per SM, four layers of 64 streams x 4,096 tokens 99 us, one pass 102, at four CTAs 106;
+  // at head_dim 128 one pass a warp up to that many, 40 streams x 3,000 tokens K4V4 89 us, two 93)
+  const bool rot = c.k_signs != nullptr && g.k_axis == 0;
+  const int per_cta = g.D == 64 && !rot ? 2 * kWarps : kWarps;
+  int gx = (max_tasks + per_cta - 1) / per_cta;
   const int streams = g.B * g.Hkv;
   const int want = (148 * 16 + streams - 1) / streams;       // enough CTAs to fill the GPU, not one per task
   if (gx > want) gx = want;
   dim3 grid1(gx, streams, g.k_axis == 0 ? 2 : 1);            // z = 0 values, z = 1 token-wise keys
-  const bool rot = c.k_signs != nullptr && g.k_axis == 0;
   auto side_slots = [](int bits) { return bits == 2 || bits == 4 || bits == 8 ? kWarps * slot_bytes(bits) : 0; };
   const size_t smem1 = std::max(side_slots(g.vb), g.k_axis == 0 && !rot ? side_slots(g.kb) : 0);
   cudaError_t e = cudaSuccess;
