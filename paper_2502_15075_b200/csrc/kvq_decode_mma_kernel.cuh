@@ -457,7 +457,10 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + sl.bar_off);   // full[0..stages), empty[0..stages)
   int* sPref = reinterpret_cast<int*>(smem + sl.pref_off);
   int* sVPref = sPref + (g.B + 1);                                   // the same prefix with GAP more per stream
-  int* sMisc = reinterpret_cast<int*>(smem + sl.misc_off);           // [1] abort flag, [2] published count, [4..7] share ends, [8..9] segment slot / partials, [10..13] CTAs taking part, cursor, [14] weighted shares
+  // [0] CTA that takes the segment's window, [1] abort flag, [2] published count, [3] CTAs that count themselves, [4..7] share ends, [8..9] segment
+  // slot / partials, [10] CTAs taking part, [11..13] cursor, [14] weighted shares, [15] free.  A word has one meaning and one place that sets it
+  // (besides the abort flag's start): whoever reads it is a barrier away from that place on both sides.
+  int* sMisc = reinterpret_cast<int*>(smem + sl.misc_off);
   double* sZ = reinterpret_cast<double*>(smem + sl.red_off);         // [NW][8][NGV] sums of weight x zero-point
   float* sMax = reinterpret_cast<float*>(sZ + NW * 8 * NGV);         // [NW][8] block maxima
   float* sLim = sMax + NW * 8;                                       // [NW][4] value scales (one used)
@@ -563,14 +566,14 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   [[maybe_unused]] bool win_only = false;
   if (x_lo >= x_hi) {                                // a share that lies inside a gap
     if constexpr (!WIN) return;
+    bool takes = false;
     if (warp == 0) {
       const int bb = sMisc[11], hh = sMisc[12], n = clamped_len(c.seq_len, bb, g.capacity);
       int first, last, window;
       stream_range(bb, hh, (sPref[bb + 1] - sPref[bb]) / Hkv, first, last, window);
-      if (lane == 0) sMisc[0] = n % g.R != 0 && window == (int)blockIdx.x;
+      takes = n % g.R != 0 && window == (int)blockIdx.x;
     }
-    __syncthreads();
-    if (sMisc[0] == 0) return;
+    if (!__syncthreads_or(takes)) return;            // (all warps leave or none: the answer comes with the barrier, not through a word)
     win_only = true;
   }
 
