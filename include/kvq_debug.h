@@ -53,6 +53,10 @@ int kvq_debug_decode_stall_impl(const kvq_config* cfg, const kvq_cache* cache, c
 int kvq_debug_decode_plan(const kvq_config* cfg, int32_t n_rows, const int32_t* seq_len, int32_t* parts, int64_t* starts,
                           int32_t* cursors, int32_t* info);
 
+/* Host only, no GPU work: info[0] = bytes of a CTA's ring of pages in that kernel, info[1] = tokens of the longest residual window
+ * that is read from the ring (0 without a window). */
+int kvq_debug_decode_ring(const kvq_config* cfg, int32_t n_rows, int32_t* info);
+
 #ifdef __cplusplus
 }
 #endif

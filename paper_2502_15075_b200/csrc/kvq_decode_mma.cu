@@ -42,9 +42,10 @@ static unsigned long long next_call_id() {
   return v ? v : counter.fetch_add(1, std::memory_order_relaxed);
 }
 
-// Finds the instantiation for this geometry; launches it unless `probe`.  *grid = CTAs of the launch.
+// Finds the instantiation for this geometry; launches it unless `probe`.  *grid = CTAs of the launch, *ring (may be null) = its ring.
 static int pick(const Geom& g, const CachePtrs& c, const void* q, float c1, float* ws, int s_cap, void* out,
-                int out_dtype, const DecodeDebug& dbg, cudaStream_t stream, bool probe, int* grid) {
+                int out_dtype, const DecodeDebug& dbg, cudaStream_t stream, bool probe, int* grid,
+                mma::SmemLayout* ring = nullptr) {
   const int ngk = (g.k_axis == 1 || g.kb == 16) ? 1 : g.D / g.gk;
   const int ngv = (g.vb == 16) ? 1 : g.D / g.gv;
   const int nh = g.G * g.rows <= 4 ? 1 : 2;                                // (virtual) query heads per lane
@@ -52,6 +53,7 @@ static int pick(const Geom& g, const CachePtrs& c, const void* q, float c1, floa
   if (g.D == D_ && g.kb == KB_ && g.vb == VB_ && g.k_axis == KAXIS_ && ngk == NGK_ && ngv == NGV_ &&          \
       NH_ == nh) {                                                                                            \
     *grid = 148 * MINB_;                                                                                      \
+    if (ring) *ring = mma::smem_layout(g.page_bytes, mma::ring_stages(g, NH_, NGV_, KAXIS_ == 1, MINB_), g.B, D_, NH_, NGV_, KAXIS_ == 1); \
     if (probe) return KVQ_OK;                                                                                 \
     return mma::launch_mma_inst<D_, KB_, VB_, KAXIS_, NGK_, NGV_, NH_, MINB_>(                          \
         g, c, q, c1, ws, s_cap, out, out_dtype, next_call_id(),                                               \
@@ -111,6 +113,18 @@ int decode_mma_plan(const Geom& g, const int32_t* seq_len, int32_t* parts, int64
   const int gap = mma::gap_pages(g.D, g.kb, g.vb, g.k_axis, g.B * g.Hkv);
   if (grid == 3 * 148) host_plan<3>(g, gap, seq_len, parts, starts, cursors, info);
   else host_plan<2>(g, gap, seq_len, parts, starts, cursors, info);
+  return KVQ_OK;
+}
+
+int decode_mma_ring(const Geom& g, int32_t* info) {
+  CachePtrs none{};
+  int grid = 0;
+  mma::SmemLayout ring{};
+  if (g.B > mma::kMaxBatchFlat) return KVQ_ERR_UNSUPPORTED;
+  const int rc = pick(g, none, nullptr, 0.f, nullptr, 0, nullptr, 0, DecodeDebug{}, nullptr, true, &grid, &ring);
+  if (rc != KVQ_OK) return rc;
+  info[0] = ring.ring_bytes;
+  for (info[1] = g.R ? g.R - 1 : 0; info[1] > 0 && !mma::window_fits_ring(ring, info[1], g.D);) --info[1];
   return KVQ_OK;
 }
 

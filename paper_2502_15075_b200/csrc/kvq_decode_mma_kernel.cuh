@@ -33,6 +33,21 @@ __host__ __device__ inline SmemLayout smem_layout(int page_bytes, int stages, in
   return s;
 }
 
+// Stages of the ring for `minb` resident CTAs per SM, or fewer than two where a configuration does not fit.
+// Deeper rings do not help, and more bytes in flight cost DRAM efficiency: at most four stages and 54 KB (K4V4, 17 KB pages, 8B
+// shape: four stages 97.9 us, three 89.8 us; K4V2, 13 KB pages: four 76.8 us, three 77.3 us).
+inline int ring_stages(const Geom& g, int nh, int ngv, bool chan, int minb) {
+  const int budget = (227 * 1024) / minb - 1024;            // shared memory per CTA
+  int stages = (budget - smem_layout(0, 0, g.B, g.D, nh, ngv, chan).total) /
+               (((g.page_bytes + 127) & ~127) + (chan ? chan_stage_bytes(g.D, nh) : 0));
+  if (stages > 4) stages = 4;
+  if (stages > 2 && stages * ((g.page_bytes + 127) & ~127) > 54 * 1024) stages = 3;
+  return stages;
+}
+// Whether a residual window of nw tokens may be read from the ring: its logits read whole tiles of 16 rows (key row, value row), the
+// last one beyond the rows that were copied.
+__host__ __device__ inline bool window_fits_ring(const SmemLayout& sl, int nw, int D) { return ((nw + 15) & ~15) * 4 * D <= sl.ring_bytes; }
+
 // prmt.b32 with the full selector semantics (a selector nibble with bit 3 set replicates the sign of the byte).
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
   uint32_t d;
@@ -876,7 +891,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
         if (sMisc[0] == (int)blockIdx.x) {
           const uint16_t* rows = c.kv_win + (size_t)stream * g.R * (2 * D);
           const int bytes = (n_all - n_tok) * 4 * D;
-          if (win_only && bytes <= sl.ring_bytes) {
+          if (win_only && window_fits_ring(sl, n_all - n_tok, D)) {
             if (tid_ == 0) {
               mbar_expect_tx(bar0, (uint32_t)bytes);
               bulk_load(ring, rows, (uint32_t)bytes, bar0, l2_evict_first_policy());
@@ -1415,13 +1430,7 @@ template <int D, int KB, int VB, int KAXIS, int NGK, int NGV, int NH, int MINB>
 int launch_mma_inst(const Geom& g, const CachePtrs& c, const void* q, float c1, float* ws, int s_cap,
                     void* out, int out_dtype, unsigned long long call_id, unsigned long long wait_ns, long long skip_x,
                     cudaStream_t stream) {
-  const int budget = (227 * 1024) / MINB - 1024;            // shared memory per CTA for MINB resident CTAs per SM
-  int stages = (budget - smem_layout(0, 0, g.B, D, NH, NGV, KAXIS == 1).total) /
-               (((g.page_bytes + 127) & ~127) + (KAXIS == 1 ? chan_stage_bytes(D, NH) : 0));
-  // Deeper rings do not help, and more bytes in flight cost DRAM efficiency: at most four stages and 54 KB (K4V4, 17 KB pages, 8B
-  // shape: four stages 97.9 us, three 89.8 us; K4V2, 13 KB pages: four 76.8 us, three 77.3 us).
-  if (stages > 4) stages = 4;
-  if (stages > 2 && stages * ((g.page_bytes + 127) & ~127) > 54 * 1024) stages = 3;
+  const int stages = ring_stages(g, NH, NGV, KAXIS == 1, MINB);
   if (stages < 2) return KVQ_ERR_UNSUPPORTED;
   const SmemLayout sl = smem_layout(g.page_bytes, stages, g.B, D, NH, NGV, KAXIS == 1);
   auto kern = decode_mma_kernel<D, KB, VB, KAXIS, NGK, NGV, NH, MINB, false>;

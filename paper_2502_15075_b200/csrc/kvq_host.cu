@@ -335,6 +335,16 @@ int kvq_debug_decode_plan(const kvq_config* cfg, int32_t n_rows, const int32_t* 
   return decode_mma_plan(g, seq_len, parts, starts, cursors, info);
 }
 
+int kvq_debug_decode_ring(const kvq_config* cfg, int32_t n_rows, int32_t* info) {
+  Geom g;
+  int rc = make_geom(cfg, &g);
+  if (rc != KVQ_OK) return rc;
+  if (!info || n_rows < 1) return KVQ_ERR_INVALID_ARG;
+  if (n_rows * g.G > kMaxGroupHeads) return KVQ_ERR_UNSUPPORTED;
+  g.rows = n_rows;
+  return decode_mma_ring(g, info);
+}
+
 int kvq_dequantize(const kvq_config* cfg, const kvq_cache* cache, void* k_out, void* v_out, int32_t t_begin,
                    int32_t t_end, void* cuda_stream) {
   Geom g;

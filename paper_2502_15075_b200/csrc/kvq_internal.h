@@ -75,6 +75,8 @@ int launch_decode_mma(const Geom& g, const CachePtrs& c, const void* q, void* ou
                       float scale_log2e, float* ws, const DecodeDebug& dbg, cudaStream_t stream);
 // The split that launch_decode_mma's kernel would take for given lengths (host memory; test hook, see kvq_debug.h).
 int decode_mma_plan(const Geom& g, const int32_t* seq_len, int32_t* parts, int64_t* starts, int32_t* cursors, int32_t* info);
+// Its ring of pages and the longest residual window that is read from it (test hook, see kvq_debug.h).
+int decode_mma_ring(const Geom& g, int32_t* info);
 // tcgen05 / tensor-memory variant of the fast path (same split, workspace and merge)
 bool decode_tc_supported(const Geom& g, const CachePtrs& c);
 int launch_decode_tc(const Geom& g, const CachePtrs& c, const void* q, float scale_log2e, float* ws, int s_cap,

@@ -72,13 +72,14 @@ _lib.kvq_debug_decode_stall_impl.argtypes = [_P(kvq_config), _P(kvq_cache), ctyp
                                              ctypes.c_int32, ctypes.c_float, ctypes.c_void_p, ctypes.c_size_t,
                                              ctypes.c_int64, ctypes.c_uint32, ctypes.c_int32, ctypes.c_void_p]
 _lib.kvq_debug_decode_plan.argtypes = [_P(kvq_config), ctypes.c_int32] + [ctypes.c_void_p] * 5
+_lib.kvq_debug_decode_ring.argtypes = [_P(kvq_config), ctypes.c_int32, ctypes.c_void_p]
 _lib.kvq_check_status.argtypes = [_P(kvq_cache), ctypes.c_void_p]
 _lib.kvq_strerror.argtypes = [ctypes.c_int]
 _lib.kvq_strerror.restype = ctypes.c_char_p
 for _f in ("kvq_page_bytes", "kvq_cache_bytes", "kvq_workspace_bytes", "kvq_quantize_append",
            "kvq_decode_attention", "kvq_decode_attention_static", "kvq_dequantize", "kvq_check_status",
            "kvq_quant_error", "kvq_bit_balance", "kvq_debug_decode_generic", "kvq_debug_decode_stall",
-           "kvq_debug_decode_impl", "kvq_debug_decode_stall_impl", "kvq_debug_decode_plan", "kvq_workspace_bytes_rows", "kvq_decode_attention_rows"):
+           "kvq_debug_decode_impl", "kvq_debug_decode_stall_impl", "kvq_debug_decode_plan", "kvq_debug_decode_ring", "kvq_workspace_bytes_rows", "kvq_decode_attention_rows"):
     getattr(_lib, _f).restype = ctypes.c_int
 
 EXPORTS = ("kvq_layout_version", "kvq_page_bytes", "kvq_cache_bytes", "kvq_workspace_bytes",
@@ -360,6 +361,13 @@ def kvq_debug_decode_plan(cfg: kvq_config, seq_len, n_rows: int = 1):
 def kvq_debug_decode_cursors(cfg: kvq_config, seq_len, n_rows: int = 1):
     """Test hook, host only: first page of every share of that split as (sequence, KV head, page of the stream) [CTAs, 3]."""
     return _decode_plan(cfg, seq_len, n_rows)[4]
+
+
+def kvq_debug_decode_ring(cfg: kvq_config, n_rows: int = 1):
+    """Test hook, host only: (bytes of the fast decode kernel's ring of pages, tokens of the longest residual window read from it)."""
+    info = torch.zeros(2, dtype=torch.int32)
+    _check(_lib.kvq_debug_decode_ring(ctypes.byref(cfg), int(n_rows), info.data_ptr()), "kvq_debug_decode_ring")
+    return int(info[0]), int(info[1])
 
 
 def kvq_check_status(cache: Cache, stream: Optional[torch.cuda.Stream] = None) -> int:

@@ -142,3 +142,10 @@ def test_windows_of_uneven_batches(kvq, w, R, rows, lens):
         sub.seq_len.fill_(lens[b])
         oc = tl.oracle_on_gpu_codes(sub, w)
         tl.assert_attention_close(got[b:b + 1], oc.decode_rows(tl.bits_of(q[b:b + 1])))
+
+
+@pytest.mark.parametrize("kb,vb", [(4, 4), (4, 2), (8, 4)])
+def test_windows_longer_than_the_ring(kvq, kb, vb):
+    """Windows around what fits a CTA's ring of pages (96 tokens), taken by shares inside the gaps of a short batch (none at K8V4)."""
+    lens = [128 * 3 + 96, 97, 128 * 20 + 102, 128 * 9 + 111, 128 * 2 + 103, 128 + 104, 128 * 5 + 112, 128 * 4 + 95]
+    test_windows_of_uneven_batches(kvq, W8.with_(kb=kb, vb=vb), 128, 1, lens)
