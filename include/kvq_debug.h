@@ -27,7 +27,8 @@ int kvq_debug_decode_impl(const kvq_config* cfg, const kvq_cache* cache, const v
 
 /* kvq_decode_attention on the fast path with every device-side wait limited to wait_us microseconds
  * (1 .. 100000) and the copy of flat page number skip_page (counted over all streams in (batch, kv-head, page)
- * order; -1: none) never issued.  The warps that wait for that page give up after wait_us, set
+ * order; -1: none; -2 - p: the copy of the residual window of the stream whose first page is p, where a CTA with
+ * an empty share of the pages takes it) never issued.  The warps that wait for that page give up after wait_us, set
  * KVQ_STATUS_DEVICE_TIMEOUT in the cache's status word, keep their barrier protocol and return: the call
  * never hangs, kvq_check_status then reports KVQ_ERR_DEVICE_TIMEOUT, the output is undefined, and after the
  * caller clears the status word the next call on the same cache works.  Configurations that the fast path

@@ -892,7 +892,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
           const uint16_t* rows = c.kv_win + (size_t)stream * g.R * (2 * D);
           const int bytes = (n_all - n_tok) * 4 * D;
           if (win_only && window_fits_ring(sl, n_all - n_tok, D)) {
-            if (tid_ == 0) {
+            if (tid_ == 0 && skip_x != -2 - (long long)x_lo) {          // (test hook, as for pages)
               mbar_expect_tx(bar0, (uint32_t)bytes);
               bulk_load(ring, rows, (uint32_t)bytes, bar0, l2_evict_first_policy());
             }
@@ -1410,7 +1410,10 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
       named_bar_sync(1, NCONS);
     }
 
-    if (WIN && win_only) return;
+    if (WIN && win_only) {
+      if (aborted) mbar_wait(bar0, 0, wait_ns);      // never leave while the copy may still be writing this CTA's shared memory (bounded)
+      return;
+    }
     // ---- advance the cursor past this segment
     x += seg_pages;
     page += seg_pages;

@@ -149,3 +149,26 @@ def test_windows_longer_than_the_ring(kvq, kb, vb):
     """Windows around what fits a CTA's ring of pages (96 tokens), taken by shares inside the gaps of a short batch (none at K8V4)."""
     lens = [128 * 3 + 96, 97, 128 * 20 + 102, 128 * 9 + 111, 128 * 2 + 103, 128 + 104, 128 * 5 + 112, 128 * 4 + 95]
     test_windows_of_uneven_batches(kvq, W8.with_(kb=kb, vb=vb), 128, 1, lens)
+
+
+def test_a_window_that_never_arrives_sets_the_status(kvq):
+    """The copy of a window taken by a share inside a gap: its wait runs out, the call returns (after it has waited once more for what may
+    be on its way), the status says so, and the next call on the same cache and workspace gives the bytes it gave before."""
+    B, T, R = 3, 64 * 5 + 37, 64
+    cfg = tl.gpu_config_for(kvq, W8, B, 384, R)
+    gc = kvq.Cache(cfg)
+    kvq.kvq_quantize_append(cfg, gc, *wl.make_kv(W8, 0, "cuda", tokens=T, batch=B))
+    q = wl.make_q(W8, batch=B).cuda()
+    ws = torch.empty(kvq.kvq_workspace_bytes(cfg), dtype=torch.uint8, device="cuda")
+    good, out = (torch.zeros(tuple(q.shape), dtype=torch.float32, device="cuda") for _ in range(2))
+    kvq.kvq_decode_attention(cfg, gc, q, good, ws)
+    assert kvq.kvq_check_status(gc) == 0
+    for stream in range(B * W8.n_kv_heads):
+        kvq.kvq_debug_decode_stall(cfg, gc, q, out, ws, -2 - 3 * stream, 2000)        # (three pages a stream)
+        assert kvq.kvq_check_status(gc) == -7                   # KVQ_ERR_DEVICE_TIMEOUT
+        gc.status.zero_()
+        out.fill_(7.0)
+        kvq.kvq_decode_attention(cfg, gc, q, out, ws)
+        assert kvq.kvq_check_status(gc) == 0 and torch.equal(out, good)
+    kvq.kvq_debug_decode_stall(cfg, gc, q, out, ws, -2 - 1, 50000)                  # no stream starts with page 1
+    assert kvq.kvq_check_status(gc) == 0 and torch.equal(out, good)
