@@ -58,12 +58,17 @@ __device__ __forceinline__ int token_slot(int k, int rs) {
   }
 }
 
-// One pass over four tokens of every lane, one side of a task of TT tokens; tokens [lo, hi) of the task are new.  load(kk, f): the
+// Tokens of a lane per pass: four make up a word of value codes.  Keys at 2 bits, whose pieces of four tokens would take 64 registers
+// beside those of the arithmetic, go by two and in passes of 4 KB, as most sides do: four layers of 40 streams x 3,000 tokens K2V4 92 us by
+// four, 87.5 by two; two of 64 x 4,000 81.7 and 78.8.
+__host__ __device__ constexpr int pass_tokens(int bits, bool is_v) { return bits == 2 && !is_v ? 2 : 4; }
+
+// One pass over pass_tokens tokens of every lane, one side of a task of TT tokens; tokens [lo, hi) of the task are new.  load(kk, f): the
 // lane's piece f of its token kk.  next is called when the pieces have been read.  codes: keys - the page's key row of the task's first
 // token; values - the page's value block of the task's first token.  meta_out: metadata row of the task's first token.
 //
 // Lane = (row slot rs, word column mw, row half rh): it owns, for each of its tokens, the FPB pieces of 8 channels
-// 16 (FPB mw + f) + 8 rh + {0..7}, f < FPB, whose codes share bytes.  The minima / maxima of the four tokens are reduced
+// 16 (FPB mw + f) + 8 rh + {0..7}, f < FPB, whose codes share bytes.  The minima / maxima of its tokens are reduced
 // with a shuffle reduce-scatter, so that the group parameters (two divisions) are computed once per group rather than once
 // per lane, and are then broadcast to the lanes of the group.  Minimum and negated maximum travel as one pair of the 16-bit type.
 // PLAIN: if all groups of the warp are plain (see plain_group; all but those with values beyond the fp16 range or scales and minima
@@ -74,7 +79,7 @@ template <int BITS, bool IS_V, int D, int DTYPE, bool PLAIN, typename Load, type
 __device__ __forceinline__ bool quantize_pass(Load&& load, Next&& next, int gsz, int lo, int hi, uint8_t* __restrict__ codes,
                                               uint32_t* __restrict__ meta_out, int lane, int pass) {
   using H2 = typename Pair16<DTYPE>::type;
-  constexpr int FPB = 8 / BITS;
+  constexpr int FPB = 8 / BITS, TK = pass_tokens(BITS, IS_V);
   constexpr int NMW = (D / 16) / FPB;        // word columns per row half
   constexpr int LR = 2 * NMW;                // lanes per token row
   constexpr int RS = 32 / LR;                // token rows per load instruction
@@ -96,19 +101,19 @@ __device__ __forceinline__ bool quantize_pass(Load&& load, Next&& next, int gsz,
     return *reinterpret_cast<const H2*>(&o);
   };
 
-  uint4 raw[4][FPB];
-  bool valid[4];
+  uint4 raw[TK][FPB];
+  bool valid[TK];
 #pragma unroll
-  for (int kk = 0; kk < 4; ++kk) {
-    const int tau = token_of(4 * pass + kk);
+  for (int kk = 0; kk < TK; ++kk) {
+    const int tau = token_of(TK * pass + kk);
     valid[kk] = tau >= lo && tau < hi;
 #pragma unroll
     for (int f = 0; f < FPB; ++f) raw[kk][f] = load(kk, f);
   }
   // ---- minima / maxima of the lane's fields, per token and per set
-  H2 m[NSET][4];
+  H2 m[NSET][TK];
 #pragma unroll
-  for (int kk = 0; kk < 4; ++kk) {
+  for (int kk = 0; kk < TK; ++kk) {
     m[0][kk] = minmax8<DTYPE, PLAIN>(raw[kk][0]);
     if constexpr (FPB == 2) m[0][kk] = min_pair(m[0][kk], minmax8<DTYPE, PLAIN>(raw[kk][1]), PLAIN);
     if constexpr (FPB == 4) {
@@ -118,16 +123,22 @@ __device__ __forceinline__ bool quantize_pass(Load&& load, Next&& next, int gsz,
     }
   }
   // ---- reduce-scatter over the lanes of the group: after lane bit 0 a lane holds tokens 2 b0 + {0, 1}, after
-  // bit 1 (groups of 4 lanes or more) token 2 b0 + b1; higher bits are plain butterflies
+  // bit 1 (groups of 4 lanes or more) token 2 b0 + b1; of two tokens it holds token b0; higher bits are plain butterflies
   float pz[NSET][2], pinv[NSET][2];
   uint32_t pmeta[NSET][2];
   bool plain = true;
 #pragma unroll
   for (int e = 0; e < NSET; ++e) {
     if (e == 1 && !split) break;
-    H2 a0 = min_pair(b0 ? m[e][2] : m[e][0], swap(b0 ? m[e][0] : m[e][2], 1), PLAIN);
-    H2 a1 = min_pair(b0 ? m[e][3] : m[e][1], swap(b0 ? m[e][1] : m[e][3], 1), PLAIN);
-    if (lpg >= 4) a0 = min_pair(b1 ? a1 : a0, swap(b1 ? a0 : a1, 2), PLAIN);
+    H2 a0, a1;
+    if constexpr (TK == 4) {
+      a0 = min_pair(b0 ? m[e][2] : m[e][0], swap(b0 ? m[e][0] : m[e][2], 1), PLAIN);
+      a1 = min_pair(b0 ? m[e][3] : m[e][1], swap(b0 ? m[e][1] : m[e][3], 1), PLAIN);
+      if (lpg >= 4) a0 = min_pair(b1 ? a1 : a0, swap(b1 ? a0 : a1, 2), PLAIN);
+    } else {
+      a0 = a1 = min_pair(b0 ? m[e][1] : m[e][0], swap(b0 ? m[e][0] : m[e][1], 1), PLAIN);
+      if (lpg >= 4) a0 = min_pair(a0, swap(a0, 2), PLAIN);
+    }
     if (lpg >= 8) a0 = min_pair(a0, swap(a0, 4), PLAIN);
     if (lpg >= 16) a0 = min_pair(a0, swap(a0, 8), PLAIN);
     const float2 f0 = pair_to_f32(a0);
@@ -135,7 +146,7 @@ __device__ __forceinline__ bool quantize_pass(Load&& load, Next&& next, int gsz,
     if constexpr (PLAIN) plain &= plain_group(f0.x, -f0.y, p0, qmax);
     pz[e][0] = p0.z; pinv[e][0] = p0.inv * DOWN; pmeta[e][0] = p0.meta;
     pz[e][1] = 0.f; pinv[e][1] = 0.f; pmeta[e][1] = 0u;
-    if (lpg == 2) {
+    if (TK == 4 && lpg == 2) {
       const float2 f1 = pair_to_f32(a1);
       const GroupParams p1 = group_params(f1.x, -f1.y, qmax);
       if constexpr (PLAIN) plain &= plain_group(f1.x, -f1.y, p1, qmax);
@@ -147,26 +158,26 @@ __device__ __forceinline__ bool quantize_pass(Load&& load, Next&& next, int gsz,
     if (!__all_sync(FULL, plain)) return false;
   }
   // the lane (one per group) that holds a token's parameters stores its metadata word
-  if ((cs & (lpg - 1) & ~3) == 0) {
+  if ((cs & (lpg - 1) & -TK) == 0) {
 #pragma unroll
     for (int e = 0; e < NSET; ++e) {
       if (e == 1 && !split) break;
       const int gi = (16 * FPB * mw) / gsz + e;
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
-        if (i == 1 && lpg != 2) break;
-        const int kk = 2 * b0 + (lpg >= 4 ? b1 : i);
-        const int tau = token_of(4 * pass + kk);
+        if (i == 1 && (TK == 2 || lpg != 2)) break;
+        const int kk = TK == 2 ? b0 : 2 * b0 + (lpg >= 4 ? b1 : i);
+        const int tau = token_of(TK * pass + kk);
         if (tau >= lo && tau < hi) meta_out[tau * ng + gi] = pmeta[e][i];
       }
     }
   }
   // ---- the group's parameters, fetched from the lane that made them
-  float z[NSET][4], inv[NSET][4];
+  float z[NSET][TK], inv[NSET][TK];
 #pragma unroll
-  for (int kk = 0; kk < 4; ++kk) {
-    const int srcl = gbase + (lpg >= 4 ? (kk >> 1) + 2 * (kk & 1) : (kk >> 1));
-    const int el = (lpg >= 4) ? 0 : (kk & 1);
+  for (int kk = 0; kk < TK; ++kk) {
+    const int srcl = gbase + (TK == 2 ? kk : lpg >= 4 ? (kk >> 1) + 2 * (kk & 1) : (kk >> 1));
+    const int el = TK == 2 || lpg >= 4 ? 0 : kk & 1;
     z[0][kk] = __shfl_sync(FULL, el ? pz[0][1] : pz[0][0], srcl);
     inv[0][kk] = __shfl_sync(FULL, el ? pinv[0][1] : pinv[0][0], srcl);
     if constexpr (NSET == 2) {
@@ -181,8 +192,8 @@ __device__ __forceinline__ bool quantize_pass(Load&& load, Next&& next, int gsz,
     // ---- keys: the four bytes of a word are channels 4 hh + {0..3} of this lane's 8, chunk 2 rh + hh, word mw of the row
     constexpr int wpc = D * BITS / 128;
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-      const int tau = token_of(4 * pass + kk);
+    for (int kk = 0; kk < TK; ++kk) {
+      const int tau = token_of(TK * pass + kk);
 #pragma unroll
       for (int hh = 0; hh < 2; ++hh) {
         uint32_t w = 0;
@@ -218,7 +229,7 @@ __device__ __forceinline__ bool quantize_pass(Load&& load, Next&& next, int gsz,
         const int e = NSET == 2 ? f >> 1 : 0;
         float x[4];
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) x[kk] = piece_value<DTYPE>(raw[kk][f], i);
+        for (int kk = 0; kk < TK; ++kk) x[kk] = piece_value<DTYPE>(raw[kk][f], i);
         if constexpr (PLAIN)
           w[i] = w[i] * (1u << BITS) + code_word4_plain<BITS>(pack2(x[0], x[1]), pack2(x[2], x[3]), pack2(-z[e][0], -z[e][1]), pack2(-z[e][2], -z[e][3]),
                                                         pack2(inv[e][0], inv[e][1]), pack2(inv[e][2], inv[e][3]));
@@ -231,7 +242,7 @@ __device__ __forceinline__ bool quantize_pass(Load&& load, Next&& next, int gsz,
       for (int i = 0; i < 8; ++i) *reinterpret_cast<uint32_t*>(wbase + 64 * i) = w[i];
     } else {
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
+      for (int kk = 0; kk < TK; ++kk) {
         if (valid[kk]) {
 #pragma unroll
           for (int i = 0; i < 8; ++i) wbase[64 * i + kk] = (uint8_t)(w[i] >> (8 * kk));
@@ -249,7 +260,7 @@ __device__ __noinline__ void quantize_pass_clamped(RowSrc rsrc, int gsz, int lo,
   constexpr int FPB = 8 / BITS, LR = 2 * (D / 16) / FPB, RS = 32 / LR;
   const int rs = lane / LR, cs = lane % LR;
   auto load = [&](int kk, int f) {
-    const int tau = token_slot<IS_V, RS>(4 * pass + kk, rs);
+    const int tau = token_slot<IS_V, RS>(pass_tokens(BITS, IS_V) * pass + kk, rs);
     return *reinterpret_cast<const uint4*>(rsrc.row(min(max(tau, lo), hi - 1)) + 16 * (FPB * (cs >> 1) + f) + 8 * (cs & 1));
   };
   quantize_pass<BITS, IS_V, D, DTYPE, false>(load, [] {}, gsz, lo, hi, codes, meta_out, lane, pass);
@@ -276,8 +287,9 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint64
 template <int BITS, bool IS_V, int D, int DTYPE>
 __device__ __forceinline__ void quantize_passes(const Geom& g, const CachePtrs& c, const uint16_t* __restrict__ in, int64_t st, int bh, int t0, int qa,
                                                 int qb, int first, int step, uint4* slot, int lane) {
-  constexpr int FPB = 8 / BITS, LR = 2 * (D / 16) / FPB, RS = 32 / LR, TT = task_tokens(D, BITS), NP = TT / RS / 4;
-  static_assert(TT % (4 * RS) == 0, "a lane holds whole groups of four tokens");
+  constexpr int FPB = 8 / BITS, LR = 2 * (D / 16) / FPB, RS = 32 / LR, TT = task_tokens(D, BITS);
+  constexpr int TK = pass_tokens(BITS, IS_V), NP = TT / RS / TK;
+  static_assert(TT % (TK * RS) == 0, "a lane's tokens of a task make up whole passes");
   const int rs = lane / LR, cs = lane % LR;
   const int gsz = IS_V ? g.gv : g.gk, R = g.R;
   const int first_task = qa / TT, n = ((qb + TT - 1) / TT - first_task) * NP;
@@ -289,8 +301,8 @@ __device__ __forceinline__ void quantize_passes(const Geom& g, const CachePtrs& 
   auto issue = [&](int u) {
     const int tk0 = (first_task + u / NP) * TT;
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-      const int t = min(max(tk0 + token_slot<IS_V, RS>(4 * (u % NP) + kk, rs), qa), qb - 1);     // (tokens that are not new: any that is)
+    for (int kk = 0; kk < TK; ++kk) {
+      const int t = min(max(tk0 + token_slot<IS_V, RS>(TK * (u % NP) + kk, rs), qa), qb - 1);     // (tokens that are not new: any that is)
       const uint16_t* p = in + (int64_t)t * st;
       if (R && t < t0) p = win + (size_t)(t % R) * (2 * D) + 16 * FPB * (cs >> 1) + 8 * (cs & 1);
 #pragma unroll
@@ -542,7 +554,7 @@ __device__ __forceinline__ void copy_task_side(const RowSrc& rsrc, int D, int lo
 // Token-wise quantization of V and of K, a side per blockIdx.z.  grid.y = stream, grid.x strides over the passes (or, for 16-bit
 // rows, bit planes and rotated keys, over the warp tasks) touched by this append.  Rotated keys take longer than the values beside them
 // and come first: four chunks of 32 streams x 2,047 tokens 80 us with the values first, 75 now (87 before the passes were pipelined).
-__host__ __device__ constexpr int slot_bytes(int bits) { return bits == 2 ? 8192 : bits == 4 ? 4096 : 2048; }        // 16-byte pieces of a warp's pass
+__host__ __device__ constexpr int slot_bytes(int bits, bool is_v) { return 32 * 16 * pass_tokens(bits, is_v) * (8 / bits); }        // a warp's pieces of a pass
 template <int D, int DTYPE, bool ROT>
 __global__ void __launch_bounds__(kThreads, D == 64 && !ROT ? 5 : 4)
 quant_token_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
@@ -566,7 +578,7 @@ quant_token_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, cons
   const int first = blockIdx.x * kWarps + warp, step = gridDim.x * kWarps;
 
   if ((bits == 2 || bits == 4 || bits == 8) && (is_v || !ROT)) {
-    uint4* slot = reinterpret_cast<uint4*>(smem + warp * slot_bytes(bits));
+    uint4* slot = reinterpret_cast<uint4*>(smem + warp * slot_bytes(bits, is_v));
 #define KVQ_PASSES(BITS_, V_) quantize_passes<BITS_, V_, D, DTYPE>(g, c, in, st, bh, t0, qa, qb, first, step, slot, lane)
     if (is_v) {
       if (bits == 2) KVQ_PASSES(2, true);
@@ -826,8 +838,8 @@ int launch_quantize_append(const Geom& g, const CachePtrs& c, const void* k_new,
   const int want = (148 * 16 + streams - 1) / streams;       // enough CTAs to fill the GPU, not one per task
   if (gx > want) gx = want;
   dim3 grid1(gx, streams, g.k_axis == 0 ? 2 : 1);            // z = 0 values, z = 1 token-wise keys
-  auto side_slots = [](int bits) { return bits == 2 || bits == 4 || bits == 8 ? kWarps * slot_bytes(bits) : 0; };
-  const size_t smem1 = std::max(side_slots(g.vb), g.k_axis == 0 && !rot ? side_slots(g.kb) : 0);
+  auto side_slots = [](int bits, bool is_v) { return bits == 2 || bits == 4 || bits == 8 ? kWarps * slot_bytes(bits, is_v) : 0; };
+  const size_t smem1 = std::max(side_slots(g.vb, true), g.k_axis == 0 && !rot ? side_slots(g.kb, false) : 0);
   cudaError_t e = cudaSuccess;
   auto run = [&](auto kern, dim3 grid, unsigned threads, size_t smem, auto... args) {      // (the first failure ends the call)
     if (e == cudaSuccess) e = launch_dependent(kern, grid, threads, smem, stream, 1, args...);

@@ -220,3 +220,16 @@ def test_the_short_append_of_several_sequences(kvq, B, D, heads, n, form):
 def test_the_short_append_of_channelwise_keys_and_the_one_beyond(kvq, heads, n):
     w = wl.SHAPED_14B.with_(n_kv_heads=heads, n_q_heads=heads)
     check(kvq, w, 2, [13, n, n + 1, 3, n, n + 1])
+
+
+@pytest.mark.parametrize("D,gk", [(128, 32), (128, 64), (128, 128), (64, 32), (64, 64)])
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+def test_keys_at_two_bits_of_long_appends(kvq, D, gk, dtype):
+    """Two tokens of a lane per pass: parts of tasks and whole ones, groups of two and four lanes and two groups a lane, and groups that clamp."""
+    w = wl.LLAMA_8B.with_(n_kv_heads=3, n_q_heads=3, head_dim=D, kb=2, vb=4, gk=gk, gv=D, dtype=dtype)
+    k, v = wl.make_kv(w, tokens=613, batch=2)
+    k[:, 1, 300:330, 5:7] = torch.tensor([60000.0, -60000.0]).to(k.dtype)
+    k[:, 2, 100:140] *= 2.0 ** -18
+    _, gc, oc = tl.build_both(kvq, w, k, v, [129, 1, 483], 640)
+    assert kvq.kvq_check_status(gc) == 0
+    tl.assert_caches_equal(gc, oc)
