@@ -837,6 +837,26 @@ int launch_quantize_append(const Geom& g, const CachePtrs& c, const void* k_new,
   const int streams = g.B * g.Hkv;
   const int want = (148 * 16 + streams - 1) / streams;       // enough CTAs to fill the GPU, not one per task
   if (gx > want) gx = want;
+  // Both sides token-wise and by passes, head_dim 128: whole waves of the four CTAs that an SM holds, so that no last wave is nearly empty and a
+  // warp has passes to load ahead.  One wave where a warp then has at most eight pieces of 4 KB and both sides take about as long (values of 4
+  // bits, keys of 2 or 4), two up to sixty with keys of 4 and values of 2 or 4 bits, else up to thirty, beyond that a warp per task up to eight waves.
+  // As many CTAs as tasks / two waves / one, us, before the rows left the L2 first (streams x tokens, layers):
+  //            40 x 3,000, 4          16 x 8,000, 4          64 x 4,000, 2          64 x 8,000, 1          64 x 16,000, 1
+  //   K4V4     88.6 / 84.0 / 79.9     91.7 / 88.6 / 80.8     81.3 / 76.4 / 80.0     73.1 / 72.6 / 76.0     138.5 / 140.3 / 146.3
+  //   K2V4     89.6 / 87.2 / 82.8     93.3 / 91.4 / 84.1     81.7 / 78.2 / 84.0     75.0 / 72.8 / 78.5     140.5 / 139.1 / 151.6
+  //   K4V2     88.8 / 85.3 / 87.3     92.0 / 89.2 / 89.7     79.7 / 75.7 / 84.7     73.1 / 71.5 / 78.1     135.5 / 133.7 / 147.5
+  //   K8V4    102.7 / 96.6 / 102.1   106.2 / 100.3 / 103.7   94.6 / 88.7 / 104.7    86.9 / 83.1 / 99.3     164.9 / 158.7 / 189.8
+  // (pieces of one wave: 6, 7, 14, 27, 54; since the rows leave the L2 first 48 x 16,000 K4V2 104.0 / 99.6 and K4V4 108.1 / 104.3 with as many
+  // CTAs as tasks / two waves, K2V4 106.4 / 108.4, 64 x 16,000 K8V8 184 / 193).
+  // Fewer than four CTAs of a wave for each stream and side: no rule, the waves would not be whole.  At head_dim 64 whole waves lose (64
+  // streams x 4,096 tokens, 4 layers, 96.5 / 95.0 / 105.4; 40 x 2,500 52.6 / 52.4 / 58.7).
+  const int per_x = 2 * streams, resident = 4 * 148;
+  auto by_passes = [](int bits) { return bits == 2 || bits == 4 || bits == 8; };
+  if (g.D == 128 && g.k_axis == 0 && !rot && by_passes(g.kb) && by_passes(g.vb) && 4 * per_x <= resident) {
+    const long long pieces = 2ll * max_tasks * per_x / (kWarps * resident);        // per warp of a single wave
+    const int waves = pieces <= 8 && g.kb <= 4 && g.vb == 4 ? 1 : pieces <= (g.kb == 4 && g.vb <= 4 ? 60 : 30) ? 2 : 0;
+    if (waves != 0) gx = std::min(gx, waves * resident / per_x);
+  }
   dim3 grid1(gx, streams, g.k_axis == 0 ? 2 : 1);            // z = 0 values, z = 1 token-wise keys
   auto side_slots = [](int bits, bool is_v) { return bits == 2 || bits == 4 || bits == 8 ? kWarps * slot_bytes(bits, is_v) : 0; };
   const size_t smem1 = std::max(side_slots(g.vb, true), g.k_axis == 0 && !rot ? side_slots(g.kb, false) : 0);
