@@ -268,14 +268,19 @@ __device__ __noinline__ void quantize_pass_clamped(RowSrc rsrc, int gsz, int lo,
 
 // The rows of a long append are read once: they leave the L2 first, as with a streaming load, and what else is there stays (the rows that
 // a residual window takes behind the same call, the pages just written, other tensors).  Four layers of 32 streams x 2,000 tokens K4V2,
-// evict-normal / evict-first: with a window of 128 117 / 95 us, without one 57 / 55; one of 64 streams x 32,767 tokens 262 / 262.
-__device__ __forceinline__ uint64_t read_once_policy() {
+// default / evict-first: with a window of 128 118 / 96 us, without one 57 / 55; one of 64 x 8,000 70 / 68.5, 64 x 16,000 132 / 132.  A call of
+// more than four times the L2 has nothing there to keep, and the hint costs it: 64 x 32,767 255 / 259.  (policy: 0 = no hint.)
+__device__ __forceinline__ uint64_t read_once_policy(int t_new, int D) {
+  if ((long long)gridDim.y * t_new * D * 4 > (512ll << 20)) return 0;
   uint64_t policy;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
   return policy;
 }
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint64_t policy) {
-  asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "l"(policy) : "memory");
+  if (policy != 0)
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "l"(policy) : "memory");
+  else
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 
 // The passes of one side of a stream that fall to a warp: first, first + step, ... of all passes over the 32- or 64-token blocks that
@@ -286,7 +291,7 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint64
 // The same loads and stores without the arithmetic between them take 220 us; one grid that goes through all streams pass by pass 299.
 template <int BITS, bool IS_V, int D, int DTYPE>
 __device__ __forceinline__ void quantize_passes(const Geom& g, const CachePtrs& c, const uint16_t* __restrict__ in, int64_t st, int bh, int t0, int qa,
-                                                int qb, int first, int step, uint4* slot, int lane) {
+                                                int qb, int t_new, int first, int step, uint4* slot, int lane) {
   constexpr int FPB = 8 / BITS, LR = 2 * (D / 16) / FPB, RS = 32 / LR, TT = task_tokens(D, BITS);
   constexpr int TK = pass_tokens(BITS, IS_V), NP = TT / RS / TK;
   static_assert(TT % (TK * RS) == 0, "a lane's tokens of a task make up whole passes");
@@ -297,7 +302,7 @@ __device__ __forceinline__ void quantize_passes(const Geom& g, const CachePtrs& 
   in += 16 * FPB * (cs >> 1) + 8 * (cs & 1) - (int64_t)t0 * st;
   slot += lane;
   const uint32_t slot_s = (uint32_t)__cvta_generic_to_shared(slot);
-  const uint64_t policy = read_once_policy();
+  const uint64_t policy = read_once_policy(t_new, D);
   auto issue = [&](int u) {
     const int tk0 = (first_task + u / NP) * TT;
 #pragma unroll
@@ -579,7 +584,7 @@ quant_token_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, cons
 
   if ((bits == 2 || bits == 4 || bits == 8) && (is_v || !ROT)) {
     uint4* slot = reinterpret_cast<uint4*>(smem + warp * slot_bytes(bits, is_v));
-#define KVQ_PASSES(BITS_, V_) quantize_passes<BITS_, V_, D, DTYPE>(g, c, in, st, bh, t0, qa, qb, first, step, slot, lane)
+#define KVQ_PASSES(BITS_, V_) quantize_passes<BITS_, V_, D, DTYPE>(g, c, in, st, bh, t0, qa, qb, t_new, first, step, slot, lane)
     if (is_v) {
       if (bits == 2) KVQ_PASSES(2, true);
       else if (bits == 4) KVQ_PASSES(4, true);
@@ -670,7 +675,7 @@ quant_kchan_fast_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new,
     // a thread copies the pieces that it will read itself; those of the next block are on their way while this one is quantized
     uint4* slot = reinterpret_cast<uint4*>(smem) + tid;
     const uint32_t slot_s = (uint32_t)__cvta_generic_to_shared(slot);
-    const uint64_t policy = read_once_policy();
+    const uint64_t policy = read_once_policy(t_new, 128);
     auto issue = [&](int block) {
       const uint16_t* p = in + (int64_t)(((first_page + block) << 7) + (tid >> 4)) * st;
 #pragma unroll
