@@ -158,28 +158,32 @@ append_rows_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ k_new, cons
 
 }  // namespace
 
-// A sequence has at most eight CTAs, so the time goes with the rows of one of them: its KV heads x new tokens; beyond twelve sequences
-// two clusters share SMs and it goes up once more.  Both sides measured behind 613 cached tokens, one of sixteen calls in a row in a
-// replayed graph, us rows / tasks + lengths, for 8, 16 and 32 sequences (K4V2):
-//    8 KV heads, head_dim 128:   24 tokens 3.9 / 4.3, 5.4 / 5.2, 5.6 / 5.8;   32 tokens 4.6 / 4.5, 6.3 / 5.5, 6.4 / 6.3;
-//                                48 tokens 5.5 / 4.5, 8.1 / 5.5, 8.3 / 6.4;   64 tokens 6.3 / 4.7, 10.0 / 6.0, 10.1 / 7.3
-//   16 KV heads, head_dim 128:   16 tokens 4.6 / 5.2, 6.2 / 5.8, 6.4 / 7.8;   24 tokens 5.5 / 5.2, 8.1 / 5.8, 8.3 / 7.7
-//    8 KV heads, head_dim 64:    64 tokens 4.2 / 4.9, 6.2 / 5.7, 6.3 / 6.5;  128 tokens 6.0 / 6.0, 9.8 / 7.4, 9.9 / 8.5
-//    8 KV heads, rotated:        32 tokens 5.5 / 7.3, 7.9 / 7.7, 8.2 / 8.5;   64 tokens 7.9 / 7.8, 13.0 / 8.6, 13.3 / 10.1
-//    8 KV heads, window of 64:   24 tokens 3.0 / 5.5, 3.7 / 5.6, 4.0 / 6.2;   32 tokens, which complete a block, 7.8 / 6.8, 11.8 / 7.6, 12.7 / 10.1
-//   10 channel-wise heads:       24 tokens 6.0 / 6.8, 6.1 / 7.0, 7.1 / 7.7;   32 tokens, which complete a block, 10.4 / 9.7, 12.6 / 12.5, 15.4 / 14.5;
-//                                48 tokens, which complete a block, 12.8 / 9.9, 15.5 / 12.5, 19.0 / 15.3
-// Two or three launches cost the host 8 to 10 us a call, this one 6, so up to twelve sequences the line stays at 64 rows a CTA at head_dim
-// 128 and 128 at head_dim 64, where tasks would save the GPU 1.5 us; beyond, at 32 and 64.  Rotated keys and a residual window cost more a
-// row: 40 rows beyond eight heads (16 heads rotated: 20 tokens 6.4 / 6.7, 32 tokens 8.3 / 8.5; with a window 32 tokens, which complete a
-// block, 12.8 / 7.9).  Channel-wise keys also pay for a block a head: 36 tokens at ten heads.
+// A sequence has at most eight CTAs, so the time goes with the rows of one of them: its KV heads x new tokens.  Up to 120 CTAs (fifteen
+// sequences of eight heads) every cluster finds SMs of its own; beyond, two clusters share them and a row costs more.
+inline bool own_sms(const Geom& g) {
+  const int per_cta = heads_per_cta(g.Hkv);
+  return (long long)g.B * ((g.Hkv + per_cta - 1) / per_cta) <= 120;
+}
+
+// Both sides measured as a layer's append and decode behind 1,000 tokens, replayed graph, us of four layers, this launch / tasks + lengths
+// (K4V2; in eager steps the second costs another 3 to 5 us):
+//    8 KV heads, head_dim 128:   48 tokens: 8 sequences 62.5 / 68.7, 14 72.5 / 81.4, 15 74.5 / 84.2;   64 tokens: 65.1 / 68.4, 75.4 / 81.6, 77.6 / 84.2
+//                                40 tokens: 16 sequences 80.0 / 78.9, 18 87.3 / 87.5, 20 83.1 / 83.5, 28 90.0 / 90.4;   56 tokens: 88.0 / 82.6, 95.9 / 91.8
+//    8 KV heads, head_dim 64:    128 tokens: 8 sequences 61.9 / 66.6, 15 70.4 / 76.7;   80 tokens: 16 73.3 / 72.0, 18 78.4 / 78.1, 24 81.9 / 81.9
+//    8 KV heads, rotated:        48 tokens: 14 sequences 80.3 / 91.0, 15 83.3 / 95.5;   40 tokens: 16 92.6 / 93.9, 20 96.0 / 99.1;   64 tokens: 16 107 / 95
+//    8 KV heads, window of 64:   48 tokens: 14 sequences 66.7 / 85.0, 16 72.6 / 91.3;   64 tokens, a block for sure: 8 76.6 / 89.3, 16 107 / 107, 32 141 / 149
+//   10 channel-wise heads:       24 tokens: 8 sequences 75.7 / 82.3, 16 94.3 / 101;   36 tokens: 85.2 / 84.3, 104 / 104;   48 tokens: 90.2 / 85.5, 108 / 104
+// (a layer of 16 heads: 20 tokens, 16 sequences 23.2 / 23.3, 32 30.9 / 33.9; 32 tokens, 15 sequences 22.5 / 23.6, 16 25.9 / 23.5; with a window 32
+// tokens, 8 sequences 18.5 / 21.5, 16 26.3 / 27.9.)  So 64 rows a CTA at head_dim 128 and 128 at head_dim 64 while clusters have their own SMs
+// or with a residual window, else 40 and 80.  Rotated keys cost more a row: 40 rows beyond eight heads (one call of sixteen in a row: 16 heads
+// rotated, 20 tokens 6.4 / 6.7, 32 tokens 8.3 / 8.5).  Channel-wise keys also pay for a block a head: 36 tokens at ten heads.
 // An append of at most 64 tokens of channel-wise keys completes at most one block.
 bool append_rows_serves(const Geom& g, bool rotated, int t_new) {
   auto width = [](int b) { return b == 2 || b == 4 || b == 8; };
   if (t_new > 64 * 128 / g.D || !width(g.kb) || !width(g.vb)) return false;
   const long long heads = heads_per_cta(g.Hkv);
   if (g.k_axis == 1) return g.D == 128 && g.kb != 2 && heads * (t_new + 12) <= 96;
-  const int limit = g.B > 12 ? 32 : heads > 1 && (rotated || g.R) ? 40 : 64;
+  const int limit = g.R ? 64 : !own_sms(g) || (heads > 1 && rotated) ? 40 : 64;
   return heads * t_new * g.D <= limit * 128;
 }
 
@@ -188,9 +192,9 @@ int launch_append_rows(const Geom& g, const CachePtrs& c, const void* k_new, con
   const int per_cta = heads_per_cta(g.Hkv), ranks = (g.Hkv + per_cta - 1) / per_cta;        // at most 8 CTAs, evenly loaded
   const bool chan = g.k_axis == 1, rot = c.k_signs != nullptr;
   int threads = per_cta * 2 * (t_new + g.R) * (g.D / 8);
-  // 1,024 threads where every cluster finds SMs of its own (8 sequences x 128 tokens at head_dim 64: 6.5 us with 512, 6.0; 16 sequences
-  // of 50 tokens, whose CTAs then no longer share SMs, 9.1 and 10.5), and no window (a block's rows only when one is completed)
-  const int most = g.R || g.B > 8 ? kMaxThreads / 2 : kMaxThreads;
+  // 1,024 threads where every cluster finds SMs of its own (64 tokens as above, 512 / 1,024 threads: 8 sequences 67.1 / 65.1, 12 76.6 / 74.5, 15
+  // 79.6 / 77.6; 16 sequences, whose CTAs then no longer share SMs, 90.9 / 97.1), and no window (a block's rows only when one is completed)
+  const int most = g.R || !own_sms(g) ? kMaxThreads / 2 : kMaxThreads;
   threads = chan ? kChanThreads : threads > most ? most : (threads + 31) / 32 * 32;
   const uint16_t* k = static_cast<const uint16_t*>(k_new);
   const uint16_t* v = static_cast<const uint16_t*>(v_new);

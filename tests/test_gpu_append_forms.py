@@ -233,3 +233,22 @@ def test_keys_at_two_bits_of_long_appends(kvq, D, gk, dtype):
     _, gc, oc = tl.build_both(kvq, w, k, v, [129, 1, 483], 640)
     assert kvq.kvq_check_status(gc) == 0
     tl.assert_caches_equal(gc, oc)
+
+
+@pytest.mark.parametrize("B,D,heads,n,form", [
+    (15, 128, 8, 64, "plain"), (16, 128, 8, 40, "plain"), (15, 64, 8, 128, "plain"), (16, 64, 8, 80, "plain"), (16, 128, 16, 20, "plain"),
+    (15, 128, 8, 64, "rotated"), (16, 128, 8, 40, "rotated"), (61, 128, 2, 40, "plain"), (60, 128, 2, 64, "plain")])
+def test_the_short_append_where_clusters_begin_to_share_sms(kvq, B, D, heads, n, form):
+    """The largest append of one launch and the one beyond it, on both sides of 120 CTAs."""
+    w = wl.LLAMA_8B.with_(n_kv_heads=heads, n_q_heads=heads, head_dim=D, gk=64, gv=64)
+    check(kvq, w, B, [13, n, n + 1], SIGNS[:D] if form == "rotated" else None)
+
+
+@pytest.mark.parametrize("B,heads,n", [(16, 8, 64), (3, 8, 64), (4, 16, 32)])
+def test_the_short_append_with_a_window(kvq, B, heads, n):
+    """Up to 64 rows a CTA with a window, however many sequences; the longest of one launch completes a block."""
+    w = wl.LLAMA_8B.with_(n_kv_heads=heads, n_q_heads=heads)
+    k, v = wl.make_kv(w, tokens=13 + 2 * n + 1, batch=B)
+    _, gc, oc = tl.build_both(kvq, w, k, v, [13, n, n + 1], 384, residual=64)
+    assert kvq.kvq_check_status(gc) == 0
+    tl.assert_caches_equal(gc, oc)
