@@ -58,6 +58,14 @@ int kvq_debug_decode_plan(const kvq_config* cfg, int32_t n_rows, const int32_t* 
  * that is read from the ring (0 without a window). */
 int kvq_debug_decode_ring(const kvq_config* cfg, int32_t n_rows, int32_t* info);
 
+/* Host only, no GPU work: who takes the residual windows in that kernel.  windows[2 s] = the CTA that takes the window of stream s
+ * (-1 where it has none, or no pages: then any CTA takes it), windows[2 s + 1] = the CTAs that count themselves in before its partials
+ * are merged (0 for a stream without pages). */
+int kvq_debug_decode_windows(const kvq_config* cfg, int32_t n_rows, const int32_t* seq_len, int32_t* windows);
+
+/* The division that the split uses, on the device (DEVICE memory): q[i] = n[i] / d[i] for n >= 0, d > 0 and quotients below 2^31. */
+int kvq_debug_divide(const int64_t* n, const int64_t* d, int64_t* q, int32_t count, void* cuda_stream);
+
 #ifdef __cplusplus
 }
 #endif

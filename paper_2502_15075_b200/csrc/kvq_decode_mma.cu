@@ -72,14 +72,15 @@ bool decode_mma_supported(const Geom& g) {
 }
 
 namespace {
-// The kernel's plan for given lengths, worked out on the host by the same functions.
-template <int WAVES>
-void host_plan(const Geom& g, int gap, const int32_t* seq_len, int32_t* parts, int64_t* starts, int32_t* cursors, int32_t* info) {
+// The kernel's plan for given lengths, worked out on the host by the same functions.  Each stream's CTAs go to `each`(stream, CTAs, whether it
+// has a residual window), null for a stream without pages.
+template <int WAVES, typename Each>
+void host_plan(const Geom& g, int gap, const int32_t* seq_len, int64_t* starts, int32_t* cursors, int32_t* info, Each&& each) {
+  auto len = [&](int b) { return seq_len[b] < 0 ? 0 : seq_len[b] > g.capacity ? g.capacity : seq_len[b]; };
   int pref[mma::kMaxBatchFlat + 1] = {}, vpref[mma::kMaxBatchFlat + 1] = {};
   int pmax = 0;
   for (int b = 0; b < g.B; ++b) {
-    const int n = seq_len[b] < 0 ? 0 : seq_len[b] > g.capacity ? g.capacity : seq_len[b];
-    const int pages = ((g.R ? n / g.R * g.R : n) + kPageTokens - 1) / kPageTokens;
+    const int n = len(b), pages = ((g.R ? n / g.R * g.R : n) + kPageTokens - 1) / kPageTokens;
     pmax = pages > pmax ? pages : pmax;
     pref[b + 1] = pref[b] + pages * g.Hkv;
     vpref[b + 1] = vpref[b] + (pages ? (pages + gap) * g.Hkv : 0);
@@ -96,24 +97,47 @@ void host_plan(const Geom& g, int gap, const int32_t* seq_len, int32_t* parts, i
   for (int b = 0; b < g.B; ++b) {
     const int pages = (pref[b + 1] - pref[b]) / g.Hkv;
     for (int h = 0; h < g.Hkv; ++h) {
-      int32_t* p = parts + 2 * (b * g.Hkv + h);
-      p[0] = p[1] = 0;
-      if (pages) mma::stream_ctas<WAVES>(plan, waves, (long long)vpref[b] + (long long)h * (pages + gap) + gap, pages, p, p + 1);
+      const long long xs = (long long)vpref[b] + (long long)h * (pages + gap) + gap;
+      auto cta = [&](int which) { return pages ? mma::stream_cta<WAVES>(plan, waves, xs, pages, gap, which) : -1; };
+      const mma::StreamCtas ctas(cta(0), cta(1), cta(2));
+      each(b * g.Hkv + h, pages ? &ctas : nullptr, len(b) % (g.R ? g.R : 1) != 0);
     }
   }
 }
 }  // namespace
 
-int decode_mma_plan(const Geom& g, const int32_t* seq_len, int32_t* parts, int64_t* starts, int32_t* cursors, int32_t* info) {
+int decode_mma_plan(const Geom& g, const int32_t* seq_len, int32_t* parts, int32_t* windows, int64_t* starts, int32_t* cursors, int32_t* info) {
   CachePtrs none{};
   int grid = 0;
   if (g.B > mma::kMaxBatchFlat) return KVQ_ERR_UNSUPPORTED;
   const int rc = pick(g, none, nullptr, 0.f, nullptr, 0, nullptr, 0, DecodeDebug{}, nullptr, true, &grid);
   if (rc != KVQ_OK) return rc;
   const int gap = mma::gap_pages(g.D, g.kb, g.vb, g.k_axis, g.B * g.Hkv);
-  if (grid == 3 * 148) host_plan<3>(g, gap, seq_len, parts, starts, cursors, info);
-  else host_plan<2>(g, gap, seq_len, parts, starts, cursors, info);
+  auto each = [&](int stream, const mma::StreamCtas* ctas, bool has_window) {
+    if (parts) {
+      parts[2 * stream] = ctas ? ctas->first : 0;
+      parts[2 * stream + 1] = ctas ? ctas->partials() : 0;
+    }
+    if (windows) {
+      windows[2 * stream] = ctas && has_window ? ctas->window : -1;
+      windows[2 * stream + 1] = ctas ? ctas->counted(has_window) : 0;
+    }
+  };
+  if (grid == 3 * 148) host_plan<3>(g, gap, seq_len, starts, cursors, info, each);
+  else host_plan<2>(g, gap, seq_len, starts, cursors, info, each);
   return KVQ_OK;
+}
+
+namespace {
+__global__ void divide_kernel(const long long* n, const long long* d, long long* q, int count) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) q[i] = mma::divide(n[i], d[i]);
+}
+}  // namespace
+
+int debug_divide(const int64_t* n, const int64_t* d, int64_t* q, int count, cudaStream_t stream) {
+  divide_kernel<<<(count + 255) / 256, 256, 0, stream>>>(reinterpret_cast<const long long*>(n), reinterpret_cast<const long long*>(d),
+                                                        reinterpret_cast<long long*>(q), count);
+  return cudaGetLastError() == cudaSuccess ? KVQ_OK : KVQ_ERR_CUDA_LAUNCH;
 }
 
 int decode_mma_ring(const Geom& g, int32_t* info) {

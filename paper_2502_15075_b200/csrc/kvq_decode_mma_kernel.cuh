@@ -263,12 +263,23 @@ static __host__ __device__ __forceinline__ ShareStart share_start(const FlatPlan
   const int vs = (int)v - sVPref[lo_], hh = vs / len, off = vs - hh * len, pg = off > gap ? off - gap : 0;
   return {(long long)sPref[lo_] + (long long)hh * pb + pg, lo_, hh, pg};
 }
-// The CTAs that hold pages of a stream: the first one, and how many (its partials).  xs: the stream's first page, virtual axis.
+// The CTA that holds a virtual page of a stream whose first page is xs: which = 0 its first page, 1 its last one, 2 the page before the gap
+// in front of it (-1 where there is none).
 template <int WAVES>
-static __host__ __device__ __forceinline__ void stream_ctas(const FlatPlan& plan, bool waves, long long xs, int pages, int* first, int* count) {
-  *first = cta_of_virtual<WAVES>(plan, waves, xs);
-  *count = cta_of_virtual<WAVES>(plan, waves, xs + pages - 1) - *first + 1;
+static __host__ __device__ __forceinline__ int stream_cta(const FlatPlan& plan, bool waves, long long xs, int pages, int gap, int which) {
+  const long long v = which == 0 ? xs : which == 1 ? xs + pages - 1 : xs - gap - 1;
+  return v < 0 ? -1 : cta_of_virtual<WAVES>(plan, waves, v);
 }
+// The CTAs of a stream, from those three: its partials are those of first .. last.  window: the one that takes its residual window - the
+// first whose share lies in the gap in front of the stream (short contexts), else the one with the first page.
+struct StreamCtas {
+  int first, last, window;
+  __host__ __device__ __forceinline__ StreamCtas(int first_, int last_, int before_gap)
+      : first(first_), last(last_), window(before_gap + 1 < first_ ? before_gap + 1 : first_) {}
+  __host__ __device__ __forceinline__ int partials() const { return last - first + 1; }
+  // CTAs that count themselves in when they are through with the stream
+  __host__ __device__ __forceinline__ int counted(bool has_window) const { return partials() + (has_window && window < first ? 1 : 0); }
+};
 // The time-balanced split (stream gaps) pays where the arithmetic per page limits the kernel (token-wise and
 // channel-wise keys alike); pages of 10 bits per element pair and more lose with it and keep the plain split by pages.
 __host__ __device__ constexpr int gap_pages(int D, int kb, int vb, int k_axis, int streams) {
@@ -562,21 +573,17 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
   }
   if (sVPref[B] == 0 || (int)blockIdx.x >= sMisc[10]) return;
   const int x_lo = (int)*reinterpret_cast<const long long*>(sMisc + 4), x_hi = (int)*reinterpret_cast<const long long*>(sMisc + 6);
-  // The CTAs that hold a stream's first and last page, and the one that takes its residual window: the first whose share lies in the gap in
-  // front of the stream (short contexts), else the one with the first page.  A warp works them out together, a lane each: one thread
-  // after the other's divisions held up the first page (16 layers of the 1B shape 312 -> 309 us, eight ragged K4V4 layers 147.8 -> 146, window
-  // of drafts, with three such lookups, 153.5 -> 145.5; 16 windowed sequences of 30,000 tokens 139 -> 135).
-  auto stream_range = [&](int bb, int hh, int pages, int& first, int& last, int& window) {
+  // The CTAs of a stream.  A warp works them out together, a lane each: one thread after the other's divisions held up the first page (16
+  // layers of the 1B shape 312 -> 309 us, eight ragged K4V4 layers 147.8 -> 146, window of drafts, with three such lookups, 153.5 -> 145.5; 16
+  // windowed sequences of 30,000 tokens 139 -> 135).
+  auto stream_ctas = [&](int bb, int hh, int pages) {
     FlatPlan plan;                         // on the virtual axis (pages + a gap in front of every stream); kept in shared memory
     plan.N = sVPref[B];
     plan.c_eff = sMisc[10];
     const long long xs = (long long)sVPref[bb] + (long long)hh * (pages + GAP) + GAP;   // the stream's first real page, virtual axis
-    const long long v = lane == 0 ? xs : lane == 1 ? xs + pages - 1 : xs - GAP - 1;
     int cta = -1;
-    if (lane < (WIN ? 3 : 2) && v >= 0) cta = cta_of_virtual<WAVES>(plan, GAP != 0 && sMisc[14] != 0, v);
-    first = __shfl_sync(FULL, cta, 0);
-    last = __shfl_sync(FULL, cta, 1);
-    window = min(__shfl_sync(FULL, cta, 2) + 1, first);
+    if (lane < (WIN ? 3 : 2)) cta = stream_cta<WAVES>(plan, GAP != 0 && sMisc[14] != 0, xs, pages, GAP, lane);
+    return StreamCtas(__shfl_sync(FULL, cta, 0), __shfl_sync(FULL, cta, 1), __shfl_sync(FULL, cta, 2));
   };
   [[maybe_unused]] bool win_only = false;
   if (x_lo >= x_hi) {                                // a share that lies inside a gap
@@ -584,9 +591,7 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
     bool takes = false;
     if (warp == 0) {
       const int bb = sMisc[11], hh = sMisc[12], n = clamped_len(c.seq_len, bb, g.capacity);
-      int first, last, window;
-      stream_range(bb, hh, (sPref[bb + 1] - sPref[bb]) / Hkv, first, last, window);
-      takes = n % g.R != 0 && window == (int)blockIdx.x;
+      takes = n % g.R != 0 && stream_ctas(bb, hh, (sPref[bb + 1] - sPref[bb]) / Hkv).window == (int)blockIdx.x;
     }
     if (!__syncthreads_or(takes)) return;            // (all warps leave or none: the answer comes with the barrier, not through a word)
     win_only = true;
@@ -868,17 +873,16 @@ decode_mma_kernel(Geom g, CachePtrs c, const uint16_t* __restrict__ q, float c1,
 #pragma unroll
       for (int nh = 0; nh < NH; ++nh) load_q_raw<D>(g, q, b, h, (gid >> 1) + 4 * nh, tid, q_raw[nh]);
     }
-    // which of the stream's partials this CTA writes, and how many there are: one thread works it out now, everybody
+    // which of the stream's partials this CTA writes, and how many there are: one warp works it out now, everybody
     // reads it after the barrier at the segment's end (the barrier that closed the last segment keeps its readers apart)
     if (warp == 0) {
-      int first, last, window;
-      stream_range(b, h, pages_b, first, last, window);
+      const StreamCtas ctas = stream_ctas(b, h, pages_b);
       if (lane == 0) {
-        sMisc[8] = (int)blockIdx.x - first;
-        sMisc[9] = last - first + 1;
+        sMisc[8] = (int)blockIdx.x - ctas.first;
+        sMisc[9] = ctas.partials();
         if constexpr (WIN) {
-          sMisc[0] = window;
-          sMisc[3] = last - first + 1 + (n_all > n_tok && window < first ? 1 : 0);          // CTAs that count themselves
+          sMisc[0] = ctas.window;
+          sMisc[3] = ctas.counted(n_all > n_tok);
         }
       }
     }

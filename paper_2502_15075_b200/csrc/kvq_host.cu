@@ -332,7 +332,24 @@ int kvq_debug_decode_plan(const kvq_config* cfg, int32_t n_rows, const int32_t* 
   if (!seq_len || !parts || !starts || !cursors || !info || n_rows < 1) return KVQ_ERR_INVALID_ARG;
   if (n_rows * g.G > kMaxGroupHeads) return KVQ_ERR_UNSUPPORTED;
   g.rows = n_rows;
-  return decode_mma_plan(g, seq_len, parts, starts, cursors, info);
+  return decode_mma_plan(g, seq_len, parts, nullptr, starts, cursors, info);
+}
+
+int kvq_debug_decode_windows(const kvq_config* cfg, int32_t n_rows, const int32_t* seq_len, int32_t* windows) {
+  Geom g;
+  int rc = make_geom(cfg, &g);
+  if (rc != KVQ_OK) return rc;
+  if (!seq_len || !windows || n_rows < 1) return KVQ_ERR_INVALID_ARG;
+  if (n_rows * g.G > kMaxGroupHeads) return KVQ_ERR_UNSUPPORTED;
+  g.rows = n_rows;
+  int64_t starts[445];
+  int32_t cursors[3 * 445], info[3];
+  return decode_mma_plan(g, seq_len, nullptr, windows, starts, cursors, info);
+}
+
+int kvq_debug_divide(const int64_t* n, const int64_t* d, int64_t* q, int32_t count, void* cuda_stream) {
+  if (!n || !d || !q || count < 1) return KVQ_ERR_INVALID_ARG;
+  return debug_divide(n, d, q, count, static_cast<cudaStream_t>(cuda_stream));
 }
 
 int kvq_debug_decode_ring(const kvq_config* cfg, int32_t n_rows, int32_t* info) {

@@ -74,7 +74,10 @@ int launch_decode_window(const Geom& g, const CachePtrs& c, const void* q, void*
 int launch_decode_mma(const Geom& g, const CachePtrs& c, const void* q, void* out, int out_dtype,
                       float scale_log2e, float* ws, const DecodeDebug& dbg, cudaStream_t stream);
 // The split that launch_decode_mma's kernel would take for given lengths (host memory; test hook, see kvq_debug.h).
-int decode_mma_plan(const Geom& g, const int32_t* seq_len, int32_t* parts, int64_t* starts, int32_t* cursors, int32_t* info);
+// parts, windows (each may be null): as there and in kvq_debug_decode_windows.
+int decode_mma_plan(const Geom& g, const int32_t* seq_len, int32_t* parts, int32_t* windows, int64_t* starts, int32_t* cursors, int32_t* info);
+// The split's division on the device (test hook).
+int debug_divide(const int64_t* n, const int64_t* d, int64_t* q, int count, cudaStream_t stream);
 // Its ring of pages and the longest residual window that is read from it (test hook, see kvq_debug.h).
 int decode_mma_ring(const Geom& g, int32_t* info);
 // tcgen05 / tensor-memory variant of the fast path (same split, workspace and merge)

@@ -73,13 +73,16 @@ _lib.kvq_debug_decode_stall_impl.argtypes = [_P(kvq_config), _P(kvq_cache), ctyp
                                              ctypes.c_int64, ctypes.c_uint32, ctypes.c_int32, ctypes.c_void_p]
 _lib.kvq_debug_decode_plan.argtypes = [_P(kvq_config), ctypes.c_int32] + [ctypes.c_void_p] * 5
 _lib.kvq_debug_decode_ring.argtypes = [_P(kvq_config), ctypes.c_int32, ctypes.c_void_p]
+_lib.kvq_debug_decode_windows.argtypes = [_P(kvq_config), ctypes.c_int32, ctypes.c_void_p, ctypes.c_void_p]
+_lib.kvq_debug_divide.argtypes = [ctypes.c_void_p] * 3 + [ctypes.c_int32, ctypes.c_void_p]
 _lib.kvq_check_status.argtypes = [_P(kvq_cache), ctypes.c_void_p]
 _lib.kvq_strerror.argtypes = [ctypes.c_int]
 _lib.kvq_strerror.restype = ctypes.c_char_p
 for _f in ("kvq_page_bytes", "kvq_cache_bytes", "kvq_workspace_bytes", "kvq_quantize_append",
            "kvq_decode_attention", "kvq_decode_attention_static", "kvq_dequantize", "kvq_check_status",
            "kvq_quant_error", "kvq_bit_balance", "kvq_debug_decode_generic", "kvq_debug_decode_stall",
-           "kvq_debug_decode_impl", "kvq_debug_decode_stall_impl", "kvq_debug_decode_plan", "kvq_debug_decode_ring", "kvq_workspace_bytes_rows", "kvq_decode_attention_rows"):
+           "kvq_debug_decode_impl", "kvq_debug_decode_stall_impl", "kvq_debug_decode_plan", "kvq_debug_decode_ring", "kvq_debug_decode_windows",
+           "kvq_debug_divide", "kvq_workspace_bytes_rows", "kvq_decode_attention_rows"):
     getattr(_lib, _f).restype = ctypes.c_int
 
 EXPORTS = ("kvq_layout_version", "kvq_page_bytes", "kvq_cache_bytes", "kvq_workspace_bytes",
@@ -368,6 +371,22 @@ def kvq_debug_decode_ring(cfg: kvq_config, n_rows: int = 1):
     info = torch.zeros(2, dtype=torch.int32)
     _check(_lib.kvq_debug_decode_ring(ctypes.byref(cfg), int(n_rows), info.data_ptr()), "kvq_debug_decode_ring")
     return int(info[0]), int(info[1])
+
+
+def kvq_debug_decode_windows(cfg: kvq_config, seq_len, n_rows: int = 1):
+    """Test hook, host only: (CTA that takes the residual window or -1, CTAs that count themselves in) per stream."""
+    lens = torch.tensor(list(seq_len), dtype=torch.int32)
+    assert lens.numel() == cfg.batch
+    out = torch.zeros((cfg.batch * cfg.n_kv_heads, 2), dtype=torch.int32)
+    _check(_lib.kvq_debug_decode_windows(ctypes.byref(cfg), int(n_rows), lens.data_ptr(), out.data_ptr()), "kvq_debug_decode_windows")
+    return out.numpy()
+
+
+def kvq_debug_divide(n: torch.Tensor, d: torch.Tensor):
+    """Test hook: the split's division on the device, of int64 tensors."""
+    q = torch.empty_like(n)
+    _check(_lib.kvq_debug_divide(n.data_ptr(), d.data_ptr(), q.data_ptr(), n.numel(), _stream_ptr(None)), "kvq_debug_divide")
+    return q
 
 
 def kvq_check_status(cache: Cache, stream: Optional[torch.cuda.Stream] = None) -> int:

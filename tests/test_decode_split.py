@@ -98,3 +98,34 @@ def test_a_split_is_refused_where_the_kernel_does_not_serve(kvq):
     with pytest.raises(kvq.KvqError) as e:
         kvq.kvq_debug_decode_plan(kvq.make_config(1, 4, 1, 128, 16, 16, 128, 128, 0, "bf16", 256), [5])
     assert e.value.code == -2
+
+
+@pytest.mark.parametrize("form", [f for f in FORMS if f != "channel"])
+def test_windows_are_taken_by_one_cta_that_is_counted(kvq, form):
+    """A stream's residual window is taken by the CTA with its first page, or by the first one whose share lies in the gap in front of
+    it: an empty share whose cursor is the stream's first page.  The CTAs that are waited for are those with pages and that one."""
+    rng, in_gaps, with_pages = random.Random(form), 0, 0
+    for _ in range(800):
+        heads, batch = rng.randint(1, 10), rng.randint(1, 24)
+        top = rng.choice([1, 4, 40, 150, 1200])
+        R = rng.choice([64, 128])
+        lens = [rng.choice([0, R, rng.randint(1, R - 1), rng.randint(1, PAGE * top), R * rng.randint(1, max(1, PAGE * top // R))]) for _ in range(batch)]
+        cfg = config(kvq, form, batch, heads, top, R)
+        starts, parts = kvq.kvq_debug_decode_plan(cfg, lens)[2:]
+        cursors, windows = kvq.kvq_debug_decode_cursors(cfg, lens), kvq.kvq_debug_decode_windows(cfg, lens)
+        empty = {}
+        for c, cursor in enumerate(cursors.tolist()):
+            if starts[c] == starts[c + 1]:
+                empty.setdefault(tuple(cursor), []).append(c)
+        for b, n in enumerate(lens):
+            for h in range(heads):
+                (first, k), (taker, counted) = parts[b * heads + h], windows[b * heads + h]
+                if n < R or n % R == 0:
+                    assert taker == -1 and counted == (k if n >= R else 0)
+                elif taker == first:
+                    assert counted == k and (b, h, 0) not in empty
+                    with_pages += 1
+                else:
+                    assert counted == k + 1 and taker == min(empty[b, h, 0]) and taker < first
+                    in_gaps += 1
+    assert with_pages > 0 and (in_gaps > 0) == (form != "wide pages")

@@ -115,3 +115,17 @@ def test_value_sums_over_more_pages_than_an_integer_accumulator_holds(kvq):
     got = tl.gpu_decode(kvq, cfg, gc, torch.ones((1, H, 64), dtype=torch.float16))[0]
     want = 3.0 * torch.tensor(scales, dtype=torch.int16).view(torch.float16).double().numpy()
     assert np.allclose(got, want[:, None], rtol=1e-5, atol=0.0)
+
+
+def test_the_splits_division_on_the_device(kvq):
+    """Exact for every quotient below 2^31, whatever the estimate that it starts from: small and large divisors, multiples and their
+    neighbours (the host's copy of the split divides the same way from another estimate)."""
+    g = torch.Generator().manual_seed(3)
+    d = torch.cat([torch.arange(1, 200), 2 ** torch.arange(0, 44), 2 ** torch.arange(1, 44) - 1,
+                   (torch.rand(20000, generator=g, dtype=torch.float64) * 43).exp2().long(), torch.tensor([148 * 1040 * 3, 148 * 1000 * 3 * 2 ** 20])])
+    q = torch.cat([torch.arange(0, 200), (torch.rand(d.numel() - 200, generator=g, dtype=torch.float64) * 31).exp2().long()]).clamp_(max=2 ** 31 - 2)
+    q = torch.minimum(q, 2 ** 62 // d - 1)
+    want = torch.cat([q, q, q])
+    n = torch.cat([q * d, q * d + d - 1, q * d + d // 2])
+    d = torch.cat([d, d, d])
+    assert torch.equal(kvq.kvq_debug_divide(n.cuda(), d.cuda()).cpu(), want) and torch.equal(n // d, want)
