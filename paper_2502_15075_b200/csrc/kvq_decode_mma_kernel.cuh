@@ -110,8 +110,10 @@ __device__ __forceinline__ uint32_t fixed_point_limb(const float (&t)[4], f32x2 
 // gain: 80 streams of 4,000 tokens 73.2, 70.6, 70.0).  Channel-wise keys, whose pages take longer: 2 (two ragged 14B-shaped layers 226
 // us; 5: 228, 8: 233).  At head_dim 64 a page is half the work: 12 (1B shape, append 128 and decode, 16 layers: 18 301.6 us, 15 297.0, 12 296.4;
 // eight layers of 64 streams of 1,000 tokens 103.5, 102.9, 99.6, 64 ragged ones of 4,000 122.2, 120.3, 118.9), but only up to 64 streams: with
-// more of them a share is not much longer than such a gap, and some are left with nothing else (steps of six 1B-shaped layers, gap 8 / 18
-// when it was 18: 72 x 1,200 89.7 / 92.9, 96 x 1,200 90.3 / 97.5, 128 x 4,000 122 / 131, 256 x 4,000 167 / 184).
+// more of them a share is not much longer than such a gap, and some are left with nothing else (steps of four 1B-shaped layers, gap 8 / 12: 72 x
+// 1,200 51.2 / 54.3, 96 x 1,200 54.7 / 57.0, 128 x 4,000 76.9 / 80.2, 256 x 4,000 106.6 / 111.7, 512 x 4,000 166 / 167).  Up to 64 streams the two
+// lie close since a stream's count word is started early: eight streams of 512 tokens 45.0 / 40.4, of 4,000
+// 50.6 / 49.2, but 48 x 2,000 50.4 / 53.1, 64 ragged ones of 4,000 57.2 / 59.4 and the 1B shape with append 128, 16 layers, 280 / 284.
 // Of the CTAs that share an SM the hardware favours the older ones (0.85 / 0.91 / 0.99 us per page at three per SM, 0.96 / 1.01 at two),
 // so the launch waves are weighted (8B shape K4V2 when the weights were chosen: 1040 76.1 us, 1080 77.3, equal 80.4).
 constexpr int kGapPages = 8, kGapPages64 = 12, kGapStreams64 = 64, kGapPagesChan = 2;
@@ -139,8 +141,7 @@ constexpr float kHeadroom = 4.0f;
 constexpr int kFlushPages = 128;           // fold the int32 value accumulators at least this often: 128 x 128 tokens x 255 x 255 < 2^31
 
 // The query values a lane needs as MMA operand: head hb (a (row, head) pair when several rows are served), channels
-// 16 r + 4 tid + {0..3} for every slot r, in fp32, rotated like the keys if the cache rotates them; heads >= G are
-// zero.  Returns max |q| over the lane's values (the caller reduces over the quad).
+// 16 r + 4 tid + {0..3} for every slot r; heads >= G are zero.  First as they are in memory, so that they can be on their way ...
 template <int D>
 __device__ __forceinline__ void load_q_raw(const Geom& g, const uint16_t* __restrict__ q, int b, int h, int hb, int tid, uint2 (&raw)[D / 16]) {
   const int Gq = g.G, G = g.G * g.rows;
@@ -151,6 +152,7 @@ __device__ __forceinline__ void load_q_raw(const Geom& g, const uint16_t* __rest
     if (hb < G) raw[r] = *reinterpret_cast<const uint2*>(qrow + 16 * r + 4 * tid);
   }
 }
+// ... then in fp32, rotated like the keys if the cache rotates them.  Returns max |q| over the lane's values (the caller reduces over the quad).
 template <int D>
 __device__ __forceinline__ float convert_q_lane(const Geom& g, const CachePtrs& c, const uint2 (&raw)[D / 16], int tid, float (&qv)[D / 16][4]) {
   constexpr int NR = D / 16;
@@ -333,7 +335,7 @@ __device__ __forceinline__ void window_partial(const Geom& g, const uint16_t* wi
   const int lim0 = n - f - (g.rows - 1 - min(2 * tid / Gq, g.rows - 1)), lim1 = n - f - (g.rows - 1 - min((2 * tid + 1) / Gq, g.rows - 1));
 #pragma unroll 1
   for (int t0 = 16 * warp; t0 < nw; t0 += 64) {
-    const uint16_t* ka = win + (size_t)(t0 + gid) * 2 * D + 4 * tid;       // (slots beyond nw are there, their logits are dropped)
+    const uint16_t* ka = win + (size_t)(t0 + gid) * 2 * D + 4 * tid;       // (rows beyond nw are there, in the window or in the ring, see window_fits_ring; their logits are dropped)
     float S[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int r = 0; r < NR; ++r) {

@@ -3,7 +3,7 @@
 // groups along head_dim, or channel-wise groups over a 128-token block with an
 // fp16 residual tail) and packing into the page layout.
 //
-// Token-wise kernel: a warp takes passes of four tokens a lane over blocks of 32 tokens (64 for head_dim 64 at 2
+// Token-wise kernel: a warp takes passes of two or four tokens a lane over blocks of 32 tokens (64 for head_dim 64 at 2
 // bits) of one stream and one side (keys or values).  A byte of the packed page holds codes of channels that
 // lie 16 apart, so a lane loads, for each of its tokens, the 8/b 16-byte pieces whose codes share
 // bytes: every output byte, and with four tokens (values) or four channels (keys) every output
@@ -832,10 +832,11 @@ int launch_quantize_append(const Geom& g, const CachePtrs& c, const void* k_new,
   if (append_rows_serves(g, c.k_signs != nullptr, t_new)) return launch_append_rows(g, c, k_new, v_new, sb, sh, st, t_new, stream);
   const uint16_t* k = static_cast<const uint16_t*>(k_new);
   const uint16_t* v = static_cast<const uint16_t*>(v_new);
-  // warp tasks touched per stream: at most ceil(t_new / 32) + 1; one warp per task, CTAs stride over them
+  // 32-token tasks touched per stream: at most ceil(t_new / 32) + 1; a CTA for every four of them, up to eight waves of CTAs, whose warps stride
+  // over the passes (16-bit rows, bit planes, rotated keys: over the tasks)
   const int max_tasks = (t_new + 31) / 32 + 1;
-  // (head_dim 64: two passes a warp and five CTAs per SM, four layers of 64 streams x 4,096 tokens 99 us, one pass 102, at four CTAs 106;
-  // at head_dim 128 one pass a warp up to that many, 40 streams x 3,000 tokens K4V4 89 us, two 93)
+  // (head_dim 64: a CTA for eight, and five CTAs per SM; when that was chosen four layers of 64 streams x 4,096 tokens 99 us, a CTA for four
+  // 102, at four CTAs 106)
   const bool rot = c.k_signs != nullptr && g.k_axis == 0;
   const int per_cta = g.D == 64 && !rot ? 2 * kWarps : kWarps;
   int gx = (max_tasks + per_cta - 1) / per_cta;
@@ -862,7 +863,7 @@ int launch_quantize_append(const Geom& g, const CachePtrs& c, const void* k_new,
     const int waves = pieces <= 8 && g.kb <= 4 && g.vb == 4 ? 1 : pieces <= (g.kb == 4 && g.vb <= 4 ? 60 : 30) ? 2 : 0;
     if (waves != 0) gx = std::min(gx, waves * resident / per_x);
   }
-  dim3 grid1(gx, streams, g.k_axis == 0 ? 2 : 1);            // z = 0 values, z = 1 token-wise keys
+  dim3 grid1(gx, streams, g.k_axis == 0 ? 2 : 1);            // which side comes first: see the kernel
   auto side_slots = [](int bits, bool is_v) { return bits == 2 || bits == 4 || bits == 8 ? kWarps * slot_bytes(bits, is_v) : 0; };
   const size_t smem1 = std::max(side_slots(g.vb, true), g.k_axis == 0 && !rot ? side_slots(g.kb, false) : 0);
   cudaError_t e = cudaSuccess;
